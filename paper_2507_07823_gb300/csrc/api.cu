@@ -59,6 +59,10 @@ __global__ void k_mx_gather(DevPlan P, const int64_t* perm, double* c);
 __global__ void k_mx_rhs(DevPlan P, const int64_t* perm, const double* u);
 __global__ void k_mx_receivers(int64_t R, const int64_t* perm, const double* u, double* uHr);
 __global__ void k_rs_local(DevPlan P, RangeDev R);
+size_t rs_local_smem(int nint, int nm);
+__global__ void k_rs_slices(DevPlan P, RangeDev R);
+__global__ void k_rs_fold(DevPlan P, RangeDev R, int s0);
+__global__ void k_rs_pairs(DevPlan P, RangeDev R, int s0, int s1);
 __global__ void k_rs_local_T(DevPlan P, RangeDev R, int64_t n, const double* cbar, double* sb);
 __global__ void k_rs_adj_init(DevPlan P, RangeDev R, double* slot_vals, double* rhs);
 __global__ void k_rs_adj_post(DevPlan P, RangeDev R, const double* sigma_next, const double* g_next, double* grad,
@@ -72,7 +76,7 @@ __global__ void k_rs_store(DevPlan P, RangeDev R);
 __global__ void k_rs_receivers(DevPlan P, RangeDev R);
 __global__ void k_rs_finish(DevPlan P, RangeDev R);
 __global__ void k_rs_count_terms(DevPlan P, RangeDev R, unsigned long long* total);
-size_t rs_local_smem(int nint, int nm);
+size_t rs_fold_smem(int nk);
 }  // namespace wave1d
 
 using namespace wave1d;
@@ -122,7 +126,7 @@ struct wave1d_plan_s {
     // from their polynomials in the distance, implicit part solved by Jacobi sweeps (range.cu)
     bool range = false;
     RangeDev rd{};
-    size_t rs_smem = 0;
+    size_t rs_smem = 0, rs_slice_smem = 0, rs_fold_smem = 0;
     int64_t info_range_pairs = 0;
     int64_t info_terms = 0;           // (pair, m) terms of the local sum per step
     bool mixed = false;
@@ -297,6 +301,44 @@ int upload_receivers(wave1d_plan_t p) {
     return WAVE1D_OK;
 }
 
+// the tables and work arrays of the range-mode local sum on the tensor cores (range.cu)
+int fold_tables(wave1d_plan_t p) {
+    const RangeTables& rt = p->hp.rt;
+    const Params& P = p->hp.P;
+    RangeDev& rd = p->rd;
+    int rc;
+    float* f32;
+    uint16_t* h16;
+    rd.nk = rt.nk;
+    rd.nivp = rt.nivp;
+    if ((rc = upload(p, rt.fold, &h16))) return rc;
+    rd.fold = h16;
+    if ((rc = upload(p, rt.fold_scale, &f32))) return rc;
+    rd.fold_scale = f32;
+    if ((rc = dalloc(p, &rd.slices, (size_t)P.M * kRsSlices * rt.nk * 16))) return rc;
+    if ((rc = dalloc(p, &rd.slice_scale, (size_t)P.M))) return rc;
+    // e-vectors of a slab of intervals at a time: 8 KB a spring (some 170 intervals) up to 2 GiB,
+    // never more than an eighth of the memory that is free, so that many plans fit beside one
+    // another; the results do not depend on the slab
+    size_t free_b = 0, all_b = 0;
+    if (cudaMemGetInfo(&free_b, &all_b) != cudaSuccess) return fail(WAVE1D_ECUDA, "cudaMemGetInfo");
+    const size_t per_iv = (size_t)P.M * kRsRecord * sizeof(float);
+    const size_t want = std::min({(size_t)8192 * P.M, (size_t)2 << 30, free_b / 8});
+    rd.slab = (int)std::min<size_t>((size_t)((rt.nint + 7) / 8) * 8, std::max<size_t>(8, want / per_iv / 8 * 8));
+    if ((rc = dalloc(p, &rd.evec, (size_t)P.M * rd.slab * kRsRecord))) return rc;
+    if ((rc = dalloc(p, &rd.cursor, (size_t)2 * P.M))) return rc;
+    if ((rc = dalloc(p, &rd.csum, (size_t)4 * P.M))) return rc;
+    p->rs_slice_smem = (size_t)(rt.nm - 1) * 64 * sizeof(float2);
+    p->rs_fold_smem = rs_fold_smem(rt.nk);
+    if (cudaFuncSetAttribute(k_rs_fold, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->rs_fold_smem) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(k_rs_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * rd.slab) != cudaSuccess ||
+        cudaFuncSetAttribute(k_rs_slices, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->rs_slice_smem) !=
+            cudaSuccess)
+        return fail(WAVE1D_ECUDA, "cannot size the shared memory of the range-mode local sum");
+    return WAVE1D_OK;
+}
+
 // items kernel: as many 8-warp blocks as are resident at once (four per SM); warps fetch items
 // dynamically
 unsigned local_grid(const wave1d_plan_t p) {
@@ -351,8 +393,20 @@ int enqueue_step(wave1d_plan_t p, int64_t n, const double* g_ext, double* sig_hi
         cudaStreamWaitEvent(p->s2, p->ev_fork, 0);
         k_local_items<<<local_grid(p), T, 0, p->s2>>>(d);
         cudaEventRecord(p->ev_join, p->s2);
-    } else if (p->range) {
+    } else if (p->range && p->mixed) {
         k_rs_local<<<p->rd.nblk, kRsTargets, p->rs_smem, s>>>(d, p->rd);
+    } else if (p->range) {
+        // local sum: the step's density slices, then per slab of intervals the e-vectors of every
+        // spring and the pairs whose distances lie in the slab
+        const RangeDev& r = p->rd;
+        k_rs_slices<<<blocks(P.M, 64), T, p->rs_slice_smem, s>>>(d, r);
+        const unsigned gx = blocks(P.M, 128);
+        for (int s0 = 0; s0 < r.nint; s0 += r.slab) {
+            const int s1 = std::min(r.nint, s0 + r.slab), tiles = (s1 - s0 + 7) / 8;
+            const unsigned gy = (unsigned)std::max(1, std::min(tiles / 2, (int)((6u * p->sms + gx - 1) / gx)));
+            k_rs_fold<<<dim3(gx, gy), T, p->rs_fold_smem, s>>>(d, r, s0);
+            k_rs_pairs<<<dim3(blocks(P.M, kRsPairTargets), 2), kRsPairTargets, (size_t)16 * (s1 - s0), s>>>(d, r, s0, s1);
+        }
     } else {
         k_local_items<<<local_grid(p), T, 0, s>>>(d);
     }
@@ -731,10 +785,14 @@ int wave1d_plan(const double* x, const double* beta, int64_t M, int bc, double d
         }
         if ((rc = zeros(p, &rd.stats, 2 * (size_t)(kRsMaxIter + 1)))) return cleanup(rc);
         if ((rc = zeros(p, &rd.iters, 1))) return cleanup(rc);
-        p->rs_smem = rs_local_smem(rt.nint, rt.nm);
-        if (cudaFuncSetAttribute(k_rs_local, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->rs_smem) !=
-            cudaSuccess)
-            return cleanup(fail(WAVE1D_ECUDA, "cannot size the shared memory of the range-mode local sum"));
+        if (o.precision == 1) {
+            p->rs_smem = rs_local_smem(rt.nint, rt.nm);
+            if (cudaFuncSetAttribute(k_rs_local, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->rs_smem) !=
+                cudaSuccess)
+                return cleanup(fail(WAVE1D_ECUDA, "cannot size the shared memory of the range-mode local sum"));
+        } else if ((rc = fold_tables(p))) {
+            return cleanup(rc);
+        }
         p->info_range_pairs = hp.range_pairs;
     }
     {

@@ -81,14 +81,36 @@ struct RangeTables {
     std::vector<float> coef;           // [iv][m][12]: monomial coefficients of z, a0 .. a3 as (hi, lo)
                                        //   pairs, a4 .. a7 single
     std::vector<double> cheb;          // [iv][m][8]: Chebyshev coefficients in z (FP64)
+    // the same polynomials as slices of kRsSliceBits bits for the tensor-core fold (fold_index below):
+    // a_{iv,m,r} = 2^(e - 10) sum_j s_j 2^(-11 j), s_j whole numbers of at most 1024, e per (iv, r)
+    int nk = 0, nivp = 0;              // steps of 16 m (m = 1 .. 16 nk), intervals with padding
+    std::vector<uint16_t> fold;        // half-precision s_j
+    std::vector<float> fold_scale;     // [nivp][8]: 2^(e - 10)
     std::vector<int32_t> cell;         // kRsCells: interval of the left end of each cell of [0, delta)
     float cell_scale = 0.f;            // kRsCells / delta: cell of a distance d is floor(d cell_scale)
 };
 void build_range_tables(const Params& P, RangeTables& out);
+// Slices of the fold: the densities carry 4, the coefficients of power r kRsSlicesOf[r] (first index
+// kRsFirstSlice[r]); products of slices i and j with i + j < kRsDiagonals[r] are kept.
+constexpr int kRsPowers = 8;
+constexpr int kRsSlices = 4;
+constexpr int kRsSlicesOf[kRsPowers] = {4, 4, 4, 4, 3, 3, 2, 2};
+constexpr int kRsDiagonals[kRsPowers] = {5, 4, 4, 4, 3, 3, 2, 2};
+constexpr int kRsFirstSlice[kRsPowers] = {0, 4, 8, 12, 16, 19, 22, 24};
+constexpr int kRsAllSlices = 26;
+// index of the half s_j of (r, j), m, iv in RangeTables::fold: per (slice, step of 16 m, interval) a
+// row of 16 halves, ordered as a lane of mma.m16n8k16 reads its B operand (lane q of four: m offsets
+// 2q, 2q + 1, 2q + 8, 2q + 9)
+inline size_t fold_index(int slice, int m, int iv, int nk, int nivp) {
+    const int k = (m - 1) & 15, ks = (m - 1) >> 4, q = (k & 7) >> 1;
+    return (((size_t)slice * nk + ks) * nivp + iv) * 16 + q * 4 + (k >> 3) * 2 + (k & 1);
+}
 // The plan's weight rule itself at each distance, Q[i * (m_max + 1) + m] (for checks).
 void local_weights_exact(const Params& P, const std::vector<double>& d, std::vector<double>& Q);
 // targets per block of the range-mode local sum (one per thread); cells of the distance lookup table
 constexpr int kRsTargets = 256;
+constexpr int kRsPairTargets = 128; // targets per block of its pair kernel
+constexpr int kRsRecord = 12;       // floats of an e-vector record in memory
 constexpr int kRsTTargets = 128;    // outputs per block of the transposed local sum (reverse march)
 constexpr int kRsCells = 2048;
 
@@ -311,6 +333,15 @@ struct RangeDev {
     const double* cheb;         // [iv][m][8] Chebyshev coefficients in z (FP64)
     const int* cell;            // kRsCells: first interval of each cell of [0, delta)
     float cell_scale;           // kRsCells / delta
+    int nk, nivp;               // steps of 16 m, padded intervals of the fold's table
+    const uint16_t* fold;       // coefficient slices (RangeTables::fold)
+    const float* fold_scale;    // [nivp][8]
+    uint16_t* slices;           // [M][kRsSlices][nk][16] halves: the step's density slices
+    float* slice_scale;         // M: their scales
+    int slab;                   // intervals whose e-vectors are held at once (a multiple of 8)
+    float* evec;                // [M][slab][kRsRecord]: e-vector records of the slab
+    int32_t* cursor;            // [2][M]: per side, each target's next source
+    float* csum;                // [2][M]: per side, each target's sum so far as a pair
     const int32_t* blk_win;     // [block][4] (see HostPlan::blk_win)
     const int32_t* nb_lo;       // M
     const int32_t* nb_cnt;      // M

@@ -1201,6 +1201,41 @@ void local_weights_exact(const Params& P, const std::vector<double>& d, std::vec
 // fl32(1 / half-width) is the scale the device uses, then written in monomials of z.
 constexpr double kRangeMaxWidth = 0.15;
 
+// half-precision bits of a whole number of magnitude at most 2048 (exact)
+static uint16_t half_bits(int v) {
+    if (v == 0) return 0;
+    const uint16_t sign = v < 0 ? 0x8000 : 0;
+    int a = std::abs(v), e = 0;
+    while ((a >> (e + 1)) != 0) e++;                      // 2^e <= a
+    return (uint16_t)(sign | ((e + 15) << 10) | (((a << 10) >> e) & 0x3ff));
+}
+
+// the coefficient slices of the tensor-core fold from a[iv][m][r] (FP64)
+static void fold_slices(const std::vector<double>& a, RangeTables& rt) {
+    const int n = rt.nint, nm = rt.nm;
+    rt.nk = (nm - 1 + 15) / 16;
+    rt.nivp = n + 8;                                      // a tile of 8 intervals may start at the last one
+    rt.fold.assign((size_t)kRsAllSlices * rt.nk * rt.nivp * 16, 0);
+    rt.fold_scale.assign((size_t)rt.nivp * kRsPowers, 0.0f);
+    for (int iv = 0; iv < n; iv++)
+        for (int r = 0; r < kRsPowers; r++) {
+            double mx = 0.0;
+            for (int m = 1; m < nm; m++) mx = std::max(mx, std::fabs(a[((size_t)iv * nm + m) * kRsPowers + r]));
+            if (mx < 1e-30) continue;                     // (far below every other term)
+            int e;
+            (void)std::frexp(mx, &e);                     // mx < 2^e
+            rt.fold_scale[(size_t)iv * kRsPowers + r] = (float)std::ldexp(1.0, e - 10);
+            for (int m = 1; m < nm; m++) {
+                double v = std::ldexp(a[((size_t)iv * nm + m) * kRsPowers + r], 10 - e);
+                for (int j = 0; j < kRsSlicesOf[r]; j++) {
+                    const double s = std::nearbyint(v);
+                    rt.fold[fold_index(kRsFirstSlice[r] + j, m, iv, rt.nk, rt.nivp)] = half_bits((int)s);
+                    v = (v - s) * 2048.0;
+                }
+            }
+        }
+}
+
 void build_range_tables(const Params& P, RangeTables& rt) {
     rt = RangeTables();
     rt.nm = P.m_max + 1;
@@ -1281,6 +1316,7 @@ void build_range_tables(const Params& P, RangeTables& rt) {
     rt.coef.assign((size_t)n * nm * 12, 0.0f);
     rt.mr.assign(2 * (size_t)n, 0);
     rt.mr0.assign(2 * (size_t)n, 0);
+    std::vector<double> mono((size_t)n * nm * np);
     for (int iv = 0; iv < n; iv++) {
         int lo = nm, hi = -1, lo1 = nm, hi1 = -1;
         for (int m = 0; m < nm; m++) {
@@ -1296,6 +1332,7 @@ void build_range_tables(const Params& P, RangeTables& rt) {
                 a[q] = 0.0;
                 for (int r = q; r < np; r++) a[q] += c[r] * T[r][q];
             }
+            std::copy(a, a + np, &mono[((size_t)iv * nm + m) * np]);
             double* cd = &rt.cheb[((size_t)iv * nm + m) * np];
             for (int r = 0; r < np; r++) cd[r] = c[r];
             float* cf = &rt.coef[((size_t)iv * nm + m) * 12];
@@ -1319,6 +1356,7 @@ void build_range_tables(const Params& P, RangeTables& rt) {
         rt.mr[2 * iv] = lo1;
         rt.mr[2 * iv + 1] = hi1;
     }
+    fold_slices(mono, rt);
 }
 
 void receiver_columns(const LocalCSR& rloc, int64_t M, ReceiverColumns& out) {

@@ -2,7 +2,12 @@
 // springs are sorted, so the sources within delta of a target are an index window, and the local
 // weights Q_m(d) (Sec. 4.1) come from their polynomials in the distance (range.cuh).  One step:
 //
-//   k_rs_local      local explicit sum c_j over m >= 1 (Sec. 4.1), compensated FP32 pairs
+//   local explicit sum c_j over m >= 1 (Sec. 4.1), compensated FP32 pairs:
+//     k_rs_slices   the step's densities as 11-bit slices (operands of the fold)
+//     per slab of intervals of the distance:
+//     k_rs_fold     e-vectors of every spring and interval on the tensor cores
+//     k_rs_pairs    the polynomials of all pairs whose distance lies in the slab
+//   (k_rs_local, range_fp32.cu, with FP32 spreading and interpolation)
 //   history pipeline (type-1 NUFFT, mode update, [projection], type-2 NUFFT): the per-stage
 //                   kernels of every plan; the interpolation leaves rhs_j = -g_j - beta_j u_H(x_j)
 //   k_rs_solve_init rhs_j -= (beta_j / 2) c_j; first iterate extrapolated from sigma^{n-7..n}
@@ -15,6 +20,7 @@
 //   k_rs_finish     u = u_L + u_H at the receivers, step counter
 //
 // Every kernel reads the step index from the device counter (graphs of steps are replayed).
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -22,34 +28,15 @@
 #include "internal.h"
 #include "phases.cuh"
 #include "range.cuh"
+#include "range_dev.cuh"
 #include "../../include/wave1d.h"
 
 namespace wave1d {
 
 namespace {
-constexpr double kPiR = 3.14159265358979323846264338327950288;
-constexpr int kRsChunk = 32;      // sources per chunk (one per lane of warp 0 in the set-up)
-constexpr int kRsIvCap = 32;      // intervals whose e-vectors are held at once (3 blocks of 256 threads per SM)
-// one interval's row of e-vector records: 32 records of 12 floats and 4 floats of padding, so the
-// rows of consecutive intervals start 4 banks apart (threads of a warp read the records of the 2-3
-// intervals their distances fall in)
-constexpr int kRsRow = kRsChunk * rs::kERecord + 4;
+constexpr int kRsChunk = 32;      // inputs per chunk of the transposed local sum
+constexpr int kRsPosChunk = 1024; // source positions staged at once by a block of k_rs_pairs
 }  // namespace
-
-// shared memory of k_rs_local (bytes): e-vector rows, the chunk's densities, the interval table
-size_t rs_local_smem(int nint, int nm) {
-    return (size_t)kRsIvCap * kRsRow * sizeof(float) + (size_t)nm * kRsChunk * sizeof(float2) +
-           (size_t)4 * nint * sizeof(float);
-}
-
-// position of extended source index e: the same expression as the host's window tests
-__device__ __forceinline__ double rs_xext(const DevPlan& P, int64_t e) {
-    if (e < 0) return P.x[e + P.M] - 2.0 * kPiR;
-    if (e >= P.M) return P.x[e - P.M] + 2.0 * kPiR;
-    return P.x[e];
-}
-
-__device__ __forceinline__ int64_t rs_spring(int64_t e, int64_t M) { return e < 0 ? e + M : (e >= M ? e - M : e); }
 
 // interval of an FP64 distance
 __device__ __forceinline__ int rs_locate64(const RangeDev& R, double d) {
@@ -82,389 +69,468 @@ __device__ __forceinline__ double rs_q0(const RangeDev& R, double d) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Local explicit sum, one block per kRsTargets consecutive targets (thread t: target j0 + t).
-// The block's sources (window [wlo, whi) of extended indices) are visited twice over as
-// "left" sources (strictly left of the target: d = x_j - x_e) and "right" sources (at or right
-// of it: d = x_e - x_j), in chunks of 32.  Per chunk:
-//   1. once per 8 chunks, one thread per source: its position on the block grid (range.cuh) and
-//      the interval range its distances to the block's targets fall in;
-//   2. the chunk's densities sigma^{n+1-m}, m = 1 .. m_max, into shared memory;
-//   3. for each interval of the chunk's range (at most kRsIvCap at a time), one warp folds the
-//      densities of all 32 sources into their e-vectors (coefficients are warp-uniform loads);
-//   4. each thread walks the 32 sources: z on the tracked interval of the side (it moves by about
-//      one interval from one source to the next), and the polynomial of the source's e-vector at z
-//      into the thread's compensated accumulator.
+// The fold e_{l,iv,r} = sum_m a_{iv,m,r} sigma_l^{n+1-m} is a contraction over m with the same
+// coefficients for every source, so it runs on the tensor cores: A = densities (16 sources x 16 m),
+// B = coefficients (16 m x 8 intervals).  To keep the pairs' precision both operands are split into
+// slices of 11 bits, whole numbers of at most 1024 that halves hold exactly (sigma = 2^(e-10)
+// sum_i s_i 2^(-11 i), one exponent per source; coefficients likewise, one per (interval, r)).  The
+// product of slices i and j is a whole number, products of equal i + j share an accumulator, and
+// every partial sum stays below 2^24 (sum_m |a_m| is about 11 times the largest |a_m|), so FP32
+// accumulation is exact; what is dropped lies below 2^-43 of the largest |a sigma| of the source and
+// interval for e_0, and by as many bits less for the higher powers as their coefficients are smaller.
+// ---------------------------------------------------------------------------------------------
+
+// the step's density slices of every spring: sigma^{n+1-m}, m = 1 .. 16 nk (zero past m_max), a row
+// of [slice][step of 16 m][16] halves in the order of RangeTables::fold.  A block takes 64 springs:
+// the ring rows are read coalesced into shared memory, then a thread makes the slices of eight m.
+constexpr int kRsSliceSprings = 64;
+__global__ void __launch_bounds__(256) k_rs_slices(DevPlan P, RangeDev R) {
+    extern __shared__ __align__(16) float2 sl_sm[];          // [m_max][kRsSliceSprings]
+    __shared__ float sUnit[kRsSliceSprings], sInv[kRsSliceSprings];
+    const int64_t n = load_step(P), l0 = (int64_t)blockIdx.x * kRsSliceSprings;
+    const int t = threadIdx.x, mm = R.nm - 1;
+    for (int i = t; i < mm * kRsSliceSprings; i += blockDim.x) {
+        const int k = i & (kRsSliceSprings - 1), m = 1 + i / kRsSliceSprings;
+        float2 v = make_float2(0.f, 0.f);
+        if (l0 + k < P.M) v = __ldg((const float2*)P.sig2 + (int64_t)ring_slot(n + 1 - m, P.ring) * P.M + l0 + k);
+        sl_sm[i] = v;
+    }
+    __syncthreads();
+    {
+        // the largest magnitude of the spring's history (as bits: a NaN sorts above every number),
+        // four threads per spring
+        const int k = t >> 2;
+        unsigned mx = 0;
+        for (int m = t & 3; m < mm; m += 4) mx = max(mx, __float_as_uint(sl_sm[m * kRsSliceSprings + k].x) & 0x7fffffffu);
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        // units of 2^(E-10); a non-finite density makes the scale NaN, so every sum it enters is NaN
+        const int E = rs::slice_exponent(mx);
+        const bool fin = mx < 0x7f800000u;
+        if ((t & 3) == 0) {
+            sInv[k] = __uint_as_float((unsigned)(127 + 10 - E) << 23);
+            sUnit[k] = fin ? __uint_as_float((unsigned)(127 + E - 10) << 23) : __uint_as_float(0x7fc00000u);
+            if (l0 + k < P.M) R.slice_scale[l0 + k] = sUnit[k];
+        }
+    }
+    __syncthreads();
+    const int per = 2 * R.nk;                                  // groups of 8 halves of a row's slice
+    for (int i = t; i < kRsSliceSprings * per; i += blockDim.x) {
+        const int k = i / per, c = i - k * per, ks = c >> 1, q0 = 2 * (c & 1);
+        if (l0 + k >= P.M) break;
+        const float inv = sInv[k];
+        const bool fin = sUnit[k] == sUnit[k];
+        unsigned short h[kRsSlices][8];
+#pragma unroll
+        for (int u = 0; u < 8; u++) {
+            const int m = ks * 16 + 2 * (q0 + (u >> 2)) + 8 * ((u >> 1) & 1) + (u & 1);      // m - 1
+            float2 v = make_float2(0.f, 0.f);
+            if (m < mm && fin) v = sl_sm[m * kRsSliceSprings + k];
+            float sl[kRsSlices];
+            rs::density_slices(v.x, v.y, inv, sl);
+#pragma unroll
+            for (int j = 0; j < kRsSlices; j++) h[j][u] = __half_as_ushort(__float2half_rn(sl[j]));
+        }
+        uint4* row = (uint4*)(R.slices + (size_t)(l0 + k) * kRsSlices * R.nk * 16);
+#pragma unroll
+        for (int j = 0; j < kRsSlices; j++)
+            row[(j * R.nk + ks) * 2 + (c & 1)] =
+                make_uint4(h[j][0] | (unsigned)h[j][1] << 16, h[j][2] | (unsigned)h[j][3] << 16,
+                           h[j][4] | (unsigned)h[j][5] << 16, h[j][6] | (unsigned)h[j][7] << 16);
+    }
+}
+
+__device__ __forceinline__ void rs_mma(float (&d)[4], const unsigned (&a)[4], uint2 b) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
+}
+
+// accumulators of power R by the weight of its products: acc[g] += sum_{i+j=g} A_i B_j
+template <int R>
+struct RsAcc {
+    float v[kRsDiagonals[R]][4] = {};
+    // tab: this lane's operand of slice 0 at the step of 16 m, slice_stride apart
+    __device__ __forceinline__ void add(const unsigned (&a)[kRsSlices][4], const uint2* tab, int slice_stride) {
+        constexpr int S = kRsSlicesOf[R], first = kRsFirstSlice[R], D = kRsDiagonals[R];
+        uint2 b[S];
+#pragma unroll
+        for (int j = 0; j < S; j++) b[j] = tab[(first + j) * slice_stride];
+#pragma unroll
+        for (int g = 0; g < D; g++)
+#pragma unroll
+            for (int i = 0; i <= g; i++)
+                if (i < kRsSlices && g - i < S) rs_mma(v[g], a[i], b[g - i]);
+    }
+    // element c as a pair or a single float, times the scale
+    __device__ __forceinline__ float2 pair(int c, float sc) const {
+        float s, e;
+        rs::two_sum(v[0][c], __fmul_rn(v[1][c], 0x1p-11f), s, e);
+        constexpr int D = kRsDiagonals[R];
+        float u = v[D - 1][c];
+#pragma unroll
+        for (int g = D - 2; g >= 2; g--) u = __fmaf_rn(u, 0x1p-11f, v[g][c]);
+        return make_float2(__fmul_rn(s, sc), __fmul_rn(__fmaf_rn(u, 0x1p-22f, e), sc));
+    }
+    __device__ __forceinline__ float single(int c, float sc) const {
+        constexpr int D = kRsDiagonals[R];
+        float u = v[D - 1][c];
+#pragma unroll
+        for (int g = D - 2; g >= 0; g--) u = __fmaf_rn(u, 0x1p-11f, v[g][c]);
+        return __fmul_rn(u, sc);
+    }
+};
+
+// The A operand of a warp: the four slices of 16 sources.  NK > 0: all steps of 16 m in registers;
+// NK = 0 (windows of more than 64 steps): read again from memory at every use.
+template <int NK>
+struct RsDensities {
+    unsigned a[NK > 0 ? NK : 1][kRsSlices][4];
+    const uint2 *r0, *r1;
+    int nk;
+    __device__ __forceinline__ void load(int slot, int ks) {
+#pragma unroll
+        for (int i = 0; i < kRsSlices; i++) {
+            const uint2 u = __ldg(r0 + (i * nk + ks) * 4), v = __ldg(r1 + (i * nk + ks) * 4);
+            a[slot][i][0] = u.x;
+            a[slot][i][1] = v.x;
+            a[slot][i][2] = u.y;
+            a[slot][i][3] = v.y;
+        }
+    }
+    // rows: the slices of the lane's two sources (g, g + 8), offset by its quarter of a row
+    __device__ __forceinline__ RsDensities(const uint2* row0, const uint2* row1, int nk_) : r0(row0), r1(row1), nk(nk_) {
+        if constexpr (NK > 0) {
+#pragma unroll
+            for (int ks = 0; ks < NK; ks++) load(ks, ks);
+        }
+    }
+    // f(operand of step ks, ks) for the steps ks0 .. nk - 1
+    template <typename F>
+    __device__ __forceinline__ void each(int ks0, F&& f) {
+        if constexpr (NK > 0) {
+#pragma unroll
+            for (int ks = 0; ks < NK; ks++)
+                if (ks >= ks0) f(a[ks], ks);
+        } else {
+            for (int ks = ks0; ks < nk; ks++) {
+                load(0, ks);
+                f(a[0], ks);
+            }
+        }
+    }
+};
+
+// What this costs, against folding in FP32 pairs inside the pair kernel (36 instructions per m, paid
+// again for each side and block of targets; range_fp32.cu): free space, 1e5 uniform springs, 676
+// intervals, 41 m: local sum 16.9 -> 3.2 ms per step (fold 1.3, bound by the tensor pipe's m16n8k16
+// rate of one per 2 cycles; pairs 1.9); a million clustered springs, 484 intervals, 33 m: 103 -> 66 ms
+// (fold 7, pairs 47-55).  Slabs hold 2 GiB of records at most, so memory grows by 8 KB a spring.
+//
+// The e-vectors of every spring for the intervals [s0, s0 + slab): a warp holds the densities of 16
+// springs and goes over tiles of 8 intervals, whose coefficient slices the block stages in shared
+// memory (two buffers, asynchronous copies).  Per tile and step of 16 m 61 products m16n8k16, in four
+// groups of powers (0, 5 | 1, 6 | 2, 7 | 3, 4) so that their accumulators fit the registers beside the
+// densities; steps of m before the tile's first m are skipped.  Records
+// (e0h e0l e5 - | e1h e1l e6 - | e2 e7 e3 e4) are staged per warp and written as whole rows.
+constexpr int kRsFoldWarps = 8;
+constexpr int kRsStageRow = 8 * kRsRecord + 4;       // floats of a spring's staged records (8 intervals)
+__host__ __device__ constexpr size_t rs_fold_tile(int nk) { return (size_t)kRsAllSlices * nk * 256; }
+size_t rs_fold_smem(int nk) { return 2 * rs_fold_tile(nk) + (size_t)kRsFoldWarps * 16 * kRsStageRow * sizeof(float); }
+
+template <int NK>
+__device__ __forceinline__ void rs_fold_block(const DevPlan& P, const RangeDev& R, int s0, unsigned char* sm) {
+    const int nk = NK > 0 ? NK : R.nk;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
+    const size_t tile_bytes = rs_fold_tile(nk);
+    float* stage = (float*)(sm + 2 * tile_bytes) + warp * 16 * kRsStageRow;
+    const int64_t l0 = ((int64_t)blockIdx.x * kRsFoldWarps + warp) * 16;
+    const int64_t la = min(l0 + g, P.M - 1), lb = min(l0 + g + 8, P.M - 1);
+    const size_t row = (size_t)kRsSlices * nk * 4;                     // uint2 of a spring's slices
+    RsDensities<NK> A((const uint2*)R.slices + la * row + q, (const uint2*)R.slices + lb * row + q, nk);
+    const float sa = __ldg(R.slice_scale + la), sb = __ldg(R.slice_scale + lb);
+    // this block's tiles of the slab
+    const int ntile = (min(R.slab, R.nint - s0) + 7) >> 3;
+    const int t0 = (int)((int64_t)ntile * blockIdx.y / gridDim.y), t1 = (int)((int64_t)ntile * (blockIdx.y + 1) / gridDim.y);
+    auto fetch = [&](int tile, int buf) {
+        const unsigned char* src = (const unsigned char*)R.fold + (size_t)(s0 + 8 * tile) * 32;
+        for (int i = threadIdx.x; i < kRsAllSlices * nk * 16; i += blockDim.x) {
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(sm + buf * tile_bytes + 16 * i);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
+                         "l"(src + (size_t)(i >> 4) * R.nivp * 32 + (i & 15) * 16));
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (t0 < t1) fetch(t0, 0);
+    for (int tile = t0; tile < t1; tile++) {
+        const int buf = (tile - t0) & 1;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();                                  // this tile has arrived, the other buffer is free
+        if (tile + 1 < t1) fetch(tile + 1, buf ^ 1);
+        const int iv0 = s0 + 8 * tile;
+        const int m0 = __reduce_min_sync(0xffffffffu, __ldg(R.mr + 2 * min(iv0 + (lane & 7), R.nint - 1)));
+        const int ks0 = min(nk - 1, max(0, (m0 - 1) >> 4));
+        const uint2* tab = (const uint2*)(sm + buf * tile_bytes) + lane;
+        const int stride = nk * 32;
+        const float* scale = R.fold_scale + (size_t)(iv0 + 2 * q) * kRsPowers;      // intervals 2q, 2q + 1
+        // element c of a fragment: spring g + 8 (c >> 1), interval 2q + (c & 1)
+        float* out = stage + g * kRsStageRow + 2 * q * kRsRecord;
+        auto at = [&](int c) { return out + (c & 1) * kRsRecord + (c >> 1) * 8 * kRsStageRow; };
+        auto sc = [&](int c, int r) { return __fmul_rn(c & 2 ? sb : sa, __ldg(scale + (c & 1) * kRsPowers + r)); };
+        {
+            RsAcc<0> x;
+            RsAcc<5> y;
+            A.each(ks0, [&](const unsigned (&a)[kRsSlices][4], int ks) {
+                x.add(a, tab + ks * 32, stride);
+                y.add(a, tab + ks * 32, stride);
+            });
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                const float2 e = x.pair(c, sc(c, 0));
+                *(float4*)at(c) = make_float4(e.x, e.y, y.single(c, sc(c, 5)), 0.f);
+            }
+        }
+        {
+            RsAcc<1> x;
+            RsAcc<6> y;
+            A.each(ks0, [&](const unsigned (&a)[kRsSlices][4], int ks) {
+                x.add(a, tab + ks * 32, stride);
+                y.add(a, tab + ks * 32, stride);
+            });
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                const float2 e = x.pair(c, sc(c, 1));
+                *(float4*)(at(c) + 4) = make_float4(e.x, e.y, y.single(c, sc(c, 6)), 0.f);
+            }
+        }
+        float2 e27[4];
+        {
+            RsAcc<2> x;
+            RsAcc<7> y;
+            A.each(ks0, [&](const unsigned (&a)[kRsSlices][4], int ks) {
+                x.add(a, tab + ks * 32, stride);
+                y.add(a, tab + ks * 32, stride);
+            });
+#pragma unroll
+            for (int c = 0; c < 4; c++) e27[c] = make_float2(x.single(c, sc(c, 2)), y.single(c, sc(c, 7)));
+        }
+        {
+            RsAcc<3> x;
+            RsAcc<4> y;
+            A.each(ks0, [&](const unsigned (&a)[kRsSlices][4], int ks) {
+                x.add(a, tab + ks * 32, stride);
+                y.add(a, tab + ks * 32, stride);
+            });
+#pragma unroll
+            for (int c = 0; c < 4; c++)
+                *(float4*)(at(c) + 8) = make_float4(e27[c].x, e27[c].y, x.single(c, sc(c, 3)), y.single(c, sc(c, 4)));
+        }
+        __syncwarp();
+        // 16 springs x 384 bytes
+        float* dst = R.evec + ((size_t)l0 * R.slab + 8 * tile) * kRsRecord;
+#pragma unroll
+        for (int i = 0; i < 12; i++) {
+            const int c = 32 * i + lane, r = c / 24, o = c - 24 * r;
+            if (l0 + r < P.M)
+                *(float4*)(dst + (size_t)r * R.slab * kRsRecord + 4 * o) = *(const float4*)(stage + r * kRsStageRow + 4 * o);
+        }
+        __syncwarp();
+    }
+}
+
+__global__ void __launch_bounds__(32 * kRsFoldWarps, 2) k_rs_fold(DevPlan P, RangeDev R, int s0) {
+    extern __shared__ __align__(16) unsigned char fold_sm[];
+    switch (R.nk) {
+        case 1: rs_fold_block<1>(P, R, s0, fold_sm); break;
+        case 2: rs_fold_block<2>(P, R, s0, fold_sm); break;
+        case 3: rs_fold_block<3>(P, R, s0, fold_sm); break;
+        case 4: rs_fold_block<4>(P, R, s0, fold_sm); break;
+        default: rs_fold_block<0>(P, R, s0, fold_sm); break;
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Pairs of one slab of intervals [s0, s1): one block per kRsPairTargets consecutive targets and side
+// (0: sources strictly left of the target, d = x_j - x_e; 1: at or right of it, d = x_e - x_j).  A
+// target meets its sources in order of distance, so those of the slab are a run that starts where the
+// last slab's ended (cursor); the warp takes the sources one by one for its 32 targets together,
+// whose records lie next to one another (same source, neighbouring intervals).  Positions on the
+// block grid (range.cuh) are staged kRsPosChunk at a time.  Each target's sum is carried from slab to
+// slab as a pair, in the order of its sources, so the result does not depend on the slabs.
 // Which side counts a source is decided by index: e < lb_j (the first spring at x_j's position) is
 // strictly left.  Q_m is continuous across the breakpoints other than dt, so a pair within
 // rounding of one takes either neighbouring interval's polynomial; at dt the spring's FP64 window
-// of near sources decides (near_side in range.cuh).
+// of near sources decides.
 // ---------------------------------------------------------------------------------------------
-template <int S>
-__device__ __forceinline__ void rs_pairs(const float* sE, const float4* sMeta, const float* ivt, const int* cell,
-                                         float cscale, int nint, int iv_dt, int k0, int k1, int W0, int W1, int lbj,
-                                         int nbl, int nbc, float bh, float bl, rs::Track& tr, float& a0h, float& a0l,
-                                         float& a1h, float& a1l) {
-    for (int k = k0; k < k1; k += 2) {
-        // the record and z of sources k and k + 1 (null where the pair does not count in this
-        // window), then both polynomials as independent chains.  z is computed for every slot
-        // (the group's meta holds 256 defined entries, so slot k + 1 >= k1 reads one); only a
-        // pair that counts moves the tracked interval.
-        const float* rec[2];
-        float zh[2], zl[2];
-#pragma unroll
-        for (int u = 0; u < 2; u++) {
-            const int kk = k + u;
-            const float4 mt = sMeta[kk];
-            const int e = __float_as_int(mt.z), lohi = __float_as_int(mt.w);
-            const int lo = max(lohi & 0x7fff, W0), hi = min(lohi >> 16, W1);
-            const bool valid = kk < k1 && lo <= hi && (S < 0 ? e < lbj : e >= lbj);
-            float h0, l0;
-            rs::z_of<S>(tr, mt.x, mt.y, h0, l0);
-            if (valid && fabsf(h0) > rs::kZTol) rs::walk<S>(ivt, cell, cscale, nint, bh, bl, mt.x, mt.y, tr, h0, l0);
-            if (valid && (lohi & 0x8000))
-                rs::near_side<S>(ivt, iv_dt, (unsigned)(e - nbl) < (unsigned)nbc, bh, bl, mt.x, mt.y, tr, h0, l0);
-            const bool ok = valid && fabsf(h0) <= rs::kZTol && tr.iv >= lo && tr.iv <= hi;
-            rec[u] = ok ? sE + (tr.iv - W0) * kRsRow + kk * rs::kERecord : nullptr;
-            zh[u] = h0;
-            zl[u] = l0;
-        }
-        if (rec[0]) rs::evec_eval(rec[0], zh[0], zl[0], a0h, a0l);
-        if (rec[1]) rs::evec_eval(rec[1], zh[1], zl[1], a1h, a1l);
-    }
+// acc += the polynomial of a record at z (record: e0h e0l e5 - | e1h e1l e6 - | e2 e7 e3 e4)
+__device__ __forceinline__ void rs_eval(const float4& a, const float4& b, const float4& c, float zh, float zl, float& ah,
+                                        float& al) {
+    rs::evec_eval4(rs::F4{a.x, a.y, b.x, b.y}, rs::F4{c.x, c.z, c.w, a.z}, rs::F4{b.z, c.y, 0.f, 0.f}, zh, zl, ah, al);
 }
 
-// The pairs of one side for one target in a chunk whose interval range takes several windows of
-// e-vectors: the sources in walk order (right: k ascending; left: k descending, so the distance
-// grows along both) from the thread's cursor cur, evaluated in the window that holds their
-// interval.  A source whose interval lies beyond the window stops the walk there (the tracked
-// interval kept, the cursor on it) until the next window; so each source is walked once per
-// thread and chunk, not once per window.  Sources beyond delta end the side.  k0 .. k1 - 1: the
-// side's sources in the chunk; par alternates the two accumulators.
-template <int S>
-__device__ __forceinline__ void rs_pairs_cursor(const float* sE, const float4* sMeta, const float* ivt, const int* cell,
-                                                float cscale, int nint, int iv_dt, int k0, int k1, int& cur, int W0,
-                                                int W1, int lbj, int nbl, int nbc, float bh, float bl, rs::Track& tr,
-                                                int& par, float& a0h, float& a0l, float& a1h, float& a1l) {
-    while (S > 0 ? cur < k1 : cur >= k0) {
-        const int k = cur;
-        const float4 mt = sMeta[k];
-        const int e = __float_as_int(mt.z), lohi = __float_as_int(mt.w);
-        const int lo = lohi & 0x7fff, hi = lohi >> 16;
-        if (lo > hi || (S < 0 ? e >= lbj : e < lbj)) {
-            cur += S;
+// the first k in [0, n) with pred(k), or n (pred monotone), by a warp: 32 probes a round
+template <typename F>
+__device__ __forceinline__ int rs_warp_first(int n, F&& pred) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0, hi = n;                      // the answer lies in [lo, hi]
+    while (hi > lo) {
+        const int step = (hi - lo + 31) / 32, k = lo + lane * step;
+        const unsigned yes = __ballot_sync(0xffffffffu, k >= hi || pred(k));
+        if (yes == 0u) {
+            lo = lo + 31 * step + 1;         // none of the probes
             continue;
         }
-        if (lo > W1) break;                                   // its interval lies in a later window
-        float zh, zl;
-        rs::z_of<S>(tr, mt.x, mt.y, zh, zl);
-        if (fabsf(zh) > rs::kZTol) rs::walk<S>(ivt, cell, cscale, nint, bh, bl, mt.x, mt.y, tr, zh, zl);
-        if (lohi & 0x8000)
-            rs::near_side<S>(ivt, iv_dt, (unsigned)(e - nbl) < (unsigned)nbc, bh, bl, mt.x, mt.y, tr, zh, zl);
-        if (tr.iv > W1 && fabsf(zh) <= rs::kZTol) break;     // a later window
-        if (fabsf(zh) <= rs::kZTol && tr.iv >= lo && tr.iv <= hi && tr.iv >= W0) {
-            const float* rec = sE + (tr.iv - W0) * kRsRow + k * rs::kERecord;
-            if (par) rs::evec_eval(rec, zh, zl, a1h, a1l);
-            else rs::evec_eval(rec, zh, zl, a0h, a0l);
-            par ^= 1;
-        } else if (zh > rs::kZTol && tr.iv == nint - 1) {
-            cur = S > 0 ? k1 : k0 - 1;                         // beyond delta, and the rest farther
-            break;
-        }
-        cur += S;
+        const int f = __ffs(yes) - 1;
+        hi = min(hi, lo + f * step);
+        if (f > 0) lo = lo + (f - 1) * step + 1;
     }
+    return hi;
 }
 
-// The pairs of one side for one target in a chunk where e-vectors would hardly be shared (the
-// chunk's interval range holds more than twice as many (source, interval) e-vectors as it has
-// pairs, as where springs lie farther apart than the intervals are wide): each pair folds its own
-// source's densities on its interval (the same e-vector, bit for bit, as the shared fold) and
-// evaluates it, with no interval windows.  Sources k0 .. k1 - 1 of the chunk.
 template <int S>
-__device__ __forceinline__ void rs_direct(const float4* sMeta, const float2* sSig, const float* ivt, const int* cell,
-                                          float cscale, int nint, int iv_dt, const float4* __restrict__ coef,
-                                          const int32_t* __restrict__ mr, int nm, int k0, int k1, int lbj, int nbl,
-                                          int nbc, float bh, float bl, rs::Track& tr, float& a0h, float& a0l,
-                                          float& a1h, float& a1l) {
-    for (int k = k0; k < k1; k++) {
-        const float4 mt = sMeta[k];
-        const int e = __float_as_int(mt.z), lohi = __float_as_int(mt.w);
-        const int lo = lohi & 0x7fff, hi = lohi >> 16;
-        if (lo > hi || (S < 0 ? e >= lbj : e < lbj)) continue;
-        float zh, zl;
-        rs::z_of<S>(tr, mt.x, mt.y, zh, zl);
-        if (fabsf(zh) > rs::kZTol) rs::walk<S>(ivt, cell, cscale, nint, bh, bl, mt.x, mt.y, tr, zh, zl);
-        if (lohi & 0x8000)
-            rs::near_side<S>(ivt, iv_dt, (unsigned)(e - nbl) < (unsigned)nbc, bh, bl, mt.x, mt.y, tr, zh, zl);
-        if (!(fabsf(zh) <= rs::kZTol && tr.iv >= lo && tr.iv <= hi)) continue;
-        rs::EVec ev;
-        rs::evec_zero(ev);
-        const int m0 = __ldg(mr + 2 * tr.iv), m1 = __ldg(mr + 2 * tr.iv + 1);
-        const float4* c = coef + (size_t)tr.iv * nm * 3;
-        const int kk = k & (kRsChunk - 1);
-#pragma unroll 1
-        for (int m = m0; m <= m1; m++) {
-            const float2 sg = sSig[m * kRsChunk + kk];
-            const float4 c01 = __ldg(c + 3 * m), c23 = __ldg(c + 3 * m + 1), c47 = __ldg(c + 3 * m + 2);
-            rs::acc_mac(ev.e0h, ev.e0l, c01.x, c01.y, sg.x, sg.y);
-            rs::acc_mac(ev.e1h, ev.e1l, c01.z, c01.w, sg.x, sg.y);
-            ev.e2 = rs::fma_(c23.y, sg.x, rs::fma_(c23.x, sg.x, ev.e2));
-            ev.e3 = rs::fma_(c23.w, sg.x, rs::fma_(c23.z, sg.x, ev.e3));
-            ev.e4 = rs::fma_(c47.x, sg.x, ev.e4);
-            ev.e5 = rs::fma_(c47.y, sg.x, ev.e5);
-            ev.e6 = rs::fma_(c47.z, sg.x, ev.e6);
-            ev.e7 = rs::fma_(c47.w, sg.x, ev.e7);
-        }
-        if (k & 1) rs::evec_eval_v(ev, zh, zl, a1h, a1l);
-        else rs::evec_eval_v(ev, zh, zl, a0h, a0l);
-    }
-}
-
-// One side of one target in a block whose targets lie farther apart than two window widths (each
-// target meets few of the block's sources): the thread walks its own sources nearest first (left:
-// e = lb_j - 1, lb_j - 2, ..; right: e = lb_j, lb_j + 1, ..) until they lie beyond delta, with the
-// shared path's per-source data (position on the block grid, interval range over the block, the
-// walk and the near/far rule) and one e-vector per pair folded from the density ring itself; no
-// shared staging, no barriers.
-template <int S>
-__device__ __forceinline__ void rs_sparse_side(const DevPlan& P, const RangeDev& R, const float* ivt, float cscale,
-                                               rs::Grid G, double xa, double span, double xj, int64_t n, int wlo,
-                                               int whi, int lbj, int nbl, int nbc, float bh, float bl, rs::Track& tr,
-                                               float& a0h, float& a0l, float& a1h, float& a1l) {
-    const double reach = R.delta * (1.0 + 8.0 * rs::kRangeMargin);
-    const float4* coef = (const float4*)R.coef;
-    for (int q = 0;; q++) {
-        const int e = S > 0 ? lbj + q : lbj - 1 - q;
-        if (S > 0 ? e >= whi : e < wlo) break;
-        const double xe = rs_xext(P, e);
-        if (!((S > 0 ? xe - xj : xj - xe) < reach)) break;     // the farther ones lie farther still
-        const double xr = xe - xa;
-        const int lohi = rs::source_range(xr, S < 0, span, R.delta, P.dt, R.bp2, R.cell, cscale, R.nint);
-        const int lo = lohi & 0x7fff, hi = lohi >> 16;
-        if (lo > hi) continue;
-        float h, l;
-        rs::grid_split(xr, G, h, l);
-        float zh, zl;
-        rs::z_of<S>(tr, h, l, zh, zl);
-        if (fabsf(zh) > rs::kZTol) rs::walk<S>(ivt, R.cell, cscale, R.nint, bh, bl, h, l, tr, zh, zl);
-        if (lohi & 0x8000) rs::near_side<S>(ivt, R.iv_dt, (unsigned)(e - nbl) < (unsigned)nbc, bh, bl, h, l, tr, zh, zl);
-        if (!(fabsf(zh) <= rs::kZTol && tr.iv >= lo && tr.iv <= hi)) continue;
-        const int64_t sp = rs_spring(e, P.M);
-        rs::EVec ev;
-        rs::evec_zero(ev);
-        const int m0 = __ldg(R.mr + 2 * tr.iv), m1 = __ldg(R.mr + 2 * tr.iv + 1);
-        const float4* c = coef + (size_t)tr.iv * R.nm * 3;
-#pragma unroll 1
-        for (int m = m0; m <= m1; m++) {
-            const float2 sg = __ldg((const float2*)P.sig2 + (int64_t)ring_slot(n + 1 - m, P.ring) * P.M + sp);
-            const float4 c01 = __ldg(c + 3 * m), c23 = __ldg(c + 3 * m + 1), c47 = __ldg(c + 3 * m + 2);
-            rs::acc_mac(ev.e0h, ev.e0l, c01.x, c01.y, sg.x, sg.y);
-            rs::acc_mac(ev.e1h, ev.e1l, c01.z, c01.w, sg.x, sg.y);
-            ev.e2 = rs::fma_(c23.y, sg.x, rs::fma_(c23.x, sg.x, ev.e2));
-            ev.e3 = rs::fma_(c23.w, sg.x, rs::fma_(c23.z, sg.x, ev.e3));
-            ev.e4 = rs::fma_(c47.x, sg.x, ev.e4);
-            ev.e5 = rs::fma_(c47.y, sg.x, ev.e5);
-            ev.e6 = rs::fma_(c47.z, sg.x, ev.e6);
-            ev.e7 = rs::fma_(c47.w, sg.x, ev.e7);
-        }
-        if (q & 1) rs::evec_eval_v(ev, zh, zl, a1h, a1l);
-        else rs::evec_eval_v(ev, zh, zl, a0h, a0l);
-    }
-}
-
-__global__ void __launch_bounds__(kRsTargets, 3) k_rs_local(DevPlan P, RangeDev R) {
-    extern __shared__ __align__(16) float rs_sm[];
-    float* sE = rs_sm;
-    float2* sSig = (float2*)(sE + kRsIvCap * kRsRow);
-    float* sIv = (float*)(sSig + (size_t)R.nm * kRsChunk);
-    // per source of a group of kRsTargets sources (8 chunks): (h, l, extended index, packed
-    // interval range), and the interval union of each chunk
-    __shared__ float4 sMeta[kRsTargets];
-    __shared__ int sU[2][kRsTargets / kRsChunk];
-    // targets' positions relative to the first (float, sorted), and per chunk an estimate of its
-    // pairs (sources' targets within delta) for the choice between shared and per-pair e-vectors
-    __shared__ float sT[kRsTargets];
-    __shared__ int sP[kRsTargets / kRsChunk];
-
+__device__ __forceinline__ void rs_pair_block(const DevPlan& P, const RangeDev& R, int s0, int s1, float* sIv, float2* sPos,
+                                              int* sRed) {
+    constexpr int side = S > 0 ? 1 : 0;
     const int64_t M = P.M;
-    const int64_t n = load_step(P);
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nwarps = blockDim.x >> 5;
-    const int b = blockIdx.x;
-    const int64_t j0 = (int64_t)b * kRsTargets;
-    const int nT = (int)min((int64_t)kRsTargets, M - j0);
-    const double xa = P.x[j0], span = P.x[j0 + nT - 1] - xa;
-    const rs::Grid G = rs::grid_of(span, R.delta);
-    for (int iv = t; iv < R.nint; iv += blockDim.x) rs::interval_on_grid(__ldg(R.mid + iv), __ldg(R.ih + iv), G, sIv + 4 * iv);
-    const float cscale = R.cell_scale;
-
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int64_t j0 = (int64_t)blockIdx.x * kRsPairTargets;
+    const int nT = (int)min((int64_t)kRsPairTargets, M - j0);
+    const double xa = P.x[j0], xb = P.x[j0 + nT - 1];
+    const rs::Grid G = rs::grid_of(xb - xa, R.delta);
+    for (int iv = s0 + t; iv < s1; iv += blockDim.x)
+        rs::interval_on_grid(__ldg(R.mid + iv), __ldg(R.ih + iv), G, sIv + 4 * (iv - s0));
     const bool valid = t < nT;
-    const int64_t j = j0 + (valid ? t : 0);
+    const int64_t j = j0 + (valid ? t : nT - 1);
     const double xj = P.x[j];
-    float hj, lj;
-    rs::grid_split(xj - xa, G, hj, lj);
-    // lb_j: the first spring at x_j's position (sources below it are strictly left of x_j)
-    int64_t lbj = j;
-    if (j > 0 && P.x[j - 1] == xj) {
-        int64_t lo = 0;
-        while (lo < lbj) {
-            const int64_t mid = (lo + lbj) >> 1;
-            if (P.x[mid] < xj) lo = mid + 1;
-            else lbj = mid;
-        }
+    float bh, bl;
+    rs::grid_split(xj - xa, G, bh, bl);
+    if (S > 0) {
+        bh = -bh;
+        bl = -bl;
     }
-    sT[t] = valid ? (float)(xj - xa) : 3.0e38f;
     const int nbl = __ldg(R.nb_lo + j), nbc = __ldg(R.nb_cnt + j);
-    const int wlo = __ldg(R.blk_win + 4 * b), inlo = __ldg(R.blk_win + 4 * b + 1);
-    const int inhi = __ldg(R.blk_win + 4 * b + 2), whi = __ldg(R.blk_win + 4 * b + 3);
-    const int nL = max(0, inhi - wlo), total = nL + max(0, whi - inlo);
-    __syncthreads();
-
-    // two accumulators (even and odd sources), so consecutive pairs are independent chains
-    float a0h = 0.f, a0l = 0.f, a1h = 0.f, a1l = 0.f;
-    rs::Track trL, trR;
-    rs::track_to(sIv, 0, hj, lj, trL);
-    rs::track_to(sIv, 0, -hj, -lj, trR);
-
-    if (span > 2.0 * R.delta) {
-        // targets farther apart than two window widths: no shared e-vectors to speak of
-        if (valid) {
-            rs_sparse_side<-1>(P, R, sIv, cscale, G, xa, span, xj, n, wlo, whi, (int)lbj, nbl, nbc, hj, lj, trL, a0h, a0l,
-                               a1h, a1l);
-            rs_sparse_side<1>(P, R, sIv, cscale, G, xa, span, xj, n, wlo, whi, (int)lbj, nbl, nbc, -hj, -lj, trR, a0h,
-                              a0l, a1h, a1l);
-            P.clocal[j] = ((double)a0h + (double)a0l) + ((double)a1h + (double)a1l);
+    int cur;
+    float ah = 0.f, al = 0.f;
+    if (s0 == 0) {
+        // lb_j: the first spring at x_j's position (sources below it are strictly left of x_j)
+        int64_t lbj = j;
+        if (j > 0 && P.x[j - 1] == xj) {
+            int64_t lo = 0;
+            while (lo < lbj) {
+                const int64_t mid = (lo + lbj) >> 1;
+                if (P.x[mid] < xj) lo = mid + 1;
+                else lbj = mid;
+            }
         }
-        return;
+        cur = (int)(S > 0 ? lbj : lbj - 1);
+    } else {
+        cur = R.cursor[side * M + j];
+        const float2 a = ((const float2*)R.csum)[side * M + j];
+        ah = a.x;
+        al = a.y;
     }
-    for (int base = 0; base < total; base += kRsChunk) {
-        const int grp = base & (kRsTargets - 1);       // the chunk's place in its group of 8
-        if (grp == 0) {
-            // set-up of the group's 256 sources, one per thread: position on the block grid and
-            // interval range; warp w reduces the union of chunk w
-            if (base > 0) __syncthreads();             // the previous group's last chunk is done
-            const int v = base + t;
-            int lohi = 1, e = 0, cnt = 0;
-            float h = 0.f, l = 0.f;
-            if (v < total) {
-                const bool left = v < nL;
-                e = left ? wlo + v : inlo + (v - nL);
-                const double xr = rs_xext(P, e) - xa;
-                rs::grid_split(xr, G, h, l);
-                lohi = rs::source_range(xr, left, span, R.delta, P.dt, R.bp2, R.cell, cscale, R.nint);
-                if ((lohi & 0x7fff) <= (lohi >> 16)) {
-                    // targets within delta of the source (an estimate: float positions)
-                    const float xf = (float)xr, df = (float)R.delta;
-                    int a = 0, bnd = nT;
-                    while (a < bnd) {
-                        const int mid = (a + bnd) >> 1;
-                        if (sT[mid] > xf - df) bnd = mid;
-                        else a = mid + 1;
-                    }
-                    int c = a;
-                    bnd = nT;
-                    while (c < bnd) {
-                        const int mid = (c + bnd) >> 1;
-                        if (sT[mid] >= xf + df) bnd = mid;
-                        else c = mid + 1;
-                    }
-                    cnt = c - a;
-                }
-            }
-            sMeta[t] = make_float4(h, l, __int_as_float(e), __int_as_float(lohi));
-            const int lo = lohi & 0x7fff, hi = lohi >> 16;
-            int u0 = lo <= hi ? lo : 0x7fffffff, u1 = lo <= hi ? hi : -1;
-            for (int o = 16; o > 0; o >>= 1) {
-                u0 = min(u0, __shfl_xor_sync(0xffffffffu, u0, o));
-                u1 = max(u1, __shfl_xor_sync(0xffffffffu, u1, o));
-                cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-            }
-            if (lane == 0) {
-                sU[0][warp] = u0;
-                sU[1][warp] = u1;
-                sP[warp] = cnt;
-            }
-        }
-        // the chunk's densities, sigma^{n+1-m} of source k at sSig[m][k] (pairs)
-        for (int i = t; i < (R.nm - 1) * kRsChunk; i += blockDim.x) {
-            const int k = i & (kRsChunk - 1), m = 1 + i / kRsChunk, v = base + k;
-            float2 s = make_float2(0.f, 0.f);
-            if (v < total) {
-                const int64_t l = rs_spring(v < nL ? wlo + v : inlo + (v - nL), M);
-                s = __ldg((const float2*)P.sig2 + (int64_t)ring_slot(n + 1 - m, P.ring) * M + l);
-            }
-            sSig[m * kRsChunk + k] = s;
+    // the block's sources of the slab: from the nearest cursor (k = 0) to the first one beyond the
+    // slab's far end of every target, inside the window of its 256-target block
+    const int* win = R.blk_win + 4 * (j0 / kRsTargets);
+    const int e0 = S > 0 ? __reduce_min_sync(0xffffffffu, cur) : __reduce_max_sync(0xffffffffu, cur);
+    if (lane == 0) sRed[warp] = e0;
+    __syncthreads();
+    int start = sRed[0];
+#pragma unroll
+    for (int w = 1; w < kRsPairTargets / 32; w++) start = S > 0 ? min(start, sRed[w]) : max(start, sRed[w]);
+    const int bound = max(0, S > 0 ? __ldg(win + 3) - start : start - __ldg(win) + 1);
+    const double reach = __ldg(R.bp + s1) + R.delta * rs::kRangeMargin;
+    if (warp == 0) {
+        const int c = rs_warp_first(bound, [&](int k) {
+            const double x = rs_xext(P, start + S * k);
+            return !((S > 0 ? x - xb : xa - x) < reach);
+        });
+        if (lane == 0) sRed[kRsPairTargets / 32] = c;
+    }
+    __syncthreads();
+    const int count = sRed[kRsPairTargets / 32];
+    int kcur = valid ? S * (cur - start) : count;         // the lane's next source
+    bool done = !valid;
+    const bool at_dt = s0 <= R.iv_dt && R.iv_dt <= s1;    // the slab touches the breakpoint dt
+    rs::Track tr;
+    rs::track_to(sIv, 0, bh, bl, tr);
+    const int ns = s1 - s0, ivd = R.iv_dt - s0;
+    for (int base = 0; base < count; base += kRsPosChunk) {
+        const int lim = min(count, base + kRsPosChunk);
+        if (base > 0) __syncthreads();
+        for (int k = base + t; k < lim; k += blockDim.x) {
+            float h, l;
+            rs::grid_split(rs_xext(P, start + S * k) - xa, G, h, l);
+            sPos[k - base] = make_float2(h, l);
         }
         __syncthreads();
-        const float4* meta = sMeta + grp;
-        const int U0 = sU[0][grp / kRsChunk], U1 = sU[1][grp / kRsChunk];
-        if (U1 >= U0 && 2 * sP[grp / kRsChunk] < kRsChunk * (U1 - U0 + 1)) {
-            // few pairs per e-vector: each pair folds its own (no windows, no shared records)
-            if (valid) {
-                const int kend = min(kRsChunk, total - base), kL = min(kend, max(0, nL - base));
-                const float4* cf = (const float4*)R.coef;
-                rs_direct<-1>(meta, sSig, sIv, R.cell, cscale, R.nint, R.iv_dt, cf, R.mr, R.nm, 0, kL, (int)lbj, nbl, nbc,
-                              hj, lj, trL, a0h, a0l, a1h, a1l);
-                rs_direct<1>(meta, sSig, sIv, R.cell, cscale, R.nint, R.iv_dt, cf, R.mr, R.nm, kL, kend, (int)lbj, nbl,
-                             nbc, -hj, -lj, trR, a0h, a0l, a1h, a1l);
-            }
-            __syncthreads();
-            continue;
-        }
-        const int lohi_lane = __float_as_int(meta[lane].w);
-        const int lo_lane = lohi_lane & 0x7fff, hi_lane = lohi_lane >> 16;
-        const bool multi = U1 - U0 + 1 > kRsIvCap;
-        const int kend_c = min(kRsChunk, total - base), kL_c = min(kend_c, max(0, nL - base));
-        int curL = kL_c - 1, curR = kL_c, par = 0;
-        for (int W0 = U0; W0 <= U1; W0 += kRsIvCap) {
-            const int W1 = min(U1, W0 + kRsIvCap - 1);
-            // e-vectors of the intervals [W0, W1]: warp per interval, lane per source
-            for (int iv = W0 + warp; iv <= W1; iv += nwarps) {
-                const bool act = lo_lane <= iv && iv <= hi_lane;
-                if (!__any_sync(0xffffffffu, act)) continue;
-                rs::EVec ev;
-                rs::evec_zero(ev);
-                const int m0 = __ldg(R.mr + 2 * iv), m1 = __ldg(R.mr + 2 * iv + 1);
-                const float4* c = (const float4*)R.coef + (size_t)iv * R.nm * 3;
-                // two m per iteration: six coefficient loads in flight (they come from L2)
-                int m = m0;
-                for (; m < m1; m += 2) {
-                    const float4 c01 = __ldg(c + 3 * m), c23 = __ldg(c + 3 * m + 1), c47 = __ldg(c + 3 * m + 2);
-                    const float4 d01 = __ldg(c + 3 * m + 3), d23 = __ldg(c + 3 * m + 4), d47 = __ldg(c + 3 * m + 5);
-                    const float2 s = sSig[m * kRsChunk + lane], s2 = sSig[(m + 1) * kRsChunk + lane];
-                    const float a01[4] = {c01.x, c01.y, c01.z, c01.w}, a23[4] = {c23.x, c23.y, c23.z, c23.w},
-                                a47[4] = {c47.x, c47.y, c47.z, c47.w};
-                    rs::evec_mac(ev, a01, a23, a47, s.x, s.y);
-                    const float b01[4] = {d01.x, d01.y, d01.z, d01.w}, b23[4] = {d23.x, d23.y, d23.z, d23.w},
-                                b47[4] = {d47.x, d47.y, d47.z, d47.w};
-                    rs::evec_mac(ev, b01, b23, b47, s2.x, s2.y);
+        int k = max(base, __reduce_min_sync(0xffffffffu, done ? count : kcur));
+        for (; k < lim; k++) {
+            const float2 ps = sPos[k - base];
+            const int e = start + S * k;
+            if (!done && k >= kcur) {
+                float zh, zl;
+                rs::z_of<S>(tr, ps.x, ps.y, zh, zl);
+                bool beyond = false;
+                if (zh > rs::kZTol) {
+                    if (zh > 4.f) {
+                        // far off: the interval of the cell of the distance, if that is farther
+                        const float d = __fadd_rn(S < 0 ? __fsub_rn(bh, ps.x) : __fadd_rn(bh, ps.x),
+                                                  S < 0 ? __fsub_rn(bl, ps.y) : __fadd_rn(bl, ps.y));
+                        const int c = min(kRsCells - 1, max(0, (int)__fmul_rn(d, R.cell_scale)));
+                        const int iv = min(__ldg(R.cell + c) - s0, ns - 1);
+                        if (iv > tr.iv) {
+                            rs::track_to(sIv, iv, bh, bl, tr);
+                            rs::z_of<S>(tr, ps.x, ps.y, zh, zl);
+                        }
+                    }
+                    while (zh > rs::kZTol) {
+                        if (tr.iv + 1 >= ns) {
+                            beyond = true;
+                            break;
+                        }
+                        rs::track_to(sIv, tr.iv + 1, bh, bl, tr);
+                        rs::z_of<S>(tr, ps.x, ps.y, zh, zl);
+                    }
                 }
-                if (m == m1) {
-                    const float4 c01 = __ldg(c + 3 * m), c23 = __ldg(c + 3 * m + 1), c47 = __ldg(c + 3 * m + 2);
-                    const float2 s = sSig[m * kRsChunk + lane];
-                    const float a01[4] = {c01.x, c01.y, c01.z, c01.w}, a23[4] = {c23.x, c23.y, c23.z, c23.w},
-                                a47[4] = {c47.x, c47.y, c47.z, c47.w};
-                    rs::evec_mac(ev, a01, a23, a47, s.x, s.y);
+                if (at_dt) {
+                    const bool near = (unsigned)(e - nbl) < (unsigned)nbc;
+                    int to = -1;
+                    if (near && (beyond || tr.iv >= ivd) && ivd - 1 < ns) to = max(0, ivd - 1);
+                    else if (!near && !beyond && tr.iv < ivd) to = ivd;
+                    if (to >= ns) {
+                        beyond = true;
+                    } else if (to >= 0) {
+                        beyond = false;
+                        rs::track_to(sIv, to, bh, bl, tr);
+                        rs::z_of<S>(tr, ps.x, ps.y, zh, zl);
+                    }
                 }
-                float4* rec = (float4*)(sE + (iv - W0) * kRsRow + lane * rs::kERecord);
-                rec[0] = make_float4(ev.e0h, ev.e0l, ev.e1h, ev.e1l);
-                rec[1] = make_float4(ev.e2, ev.e3, ev.e4, ev.e5);
-                rec[2] = make_float4(ev.e6, ev.e7, 0.f, 0.f);
+                if (beyond) {
+                    done = true;
+                    kcur = k;
+                } else {
+                    const float4* rec = (const float4*)(R.evec + ((size_t)rs_spring(e, M) * R.slab + tr.iv) * kRsRecord);
+                    const float4 r0 = __ldg(rec), r1 = __ldg(rec + 1), r2 = __ldg(rec + 2);
+                    rs_eval(r0, r1, r2, zh, zl, ah, al);
+                    kcur = k + 1;
+                }
             }
-            __syncthreads();
-            if (valid && multi) {
-                rs_pairs_cursor<-1>(sE, meta, sIv, R.cell, cscale, R.nint, R.iv_dt, 0, kL_c, curL, W0, W1, (int)lbj, nbl,
-                                    nbc, hj, lj, trL, par, a0h, a0l, a1h, a1l);
-                rs_pairs_cursor<1>(sE, meta, sIv, R.cell, cscale, R.nint, R.iv_dt, kL_c, kend_c, curR, W0, W1, (int)lbj,
-                                   nbl, nbc, -hj, -lj, trR, par, a0h, a0l, a1h, a1l);
-            } else if (valid) {
-                rs_pairs<-1>(sE, meta, sIv, R.cell, cscale, R.nint, R.iv_dt, 0, kL_c, W0, W1, (int)lbj, nbl, nbc, hj, lj,
-                             trL, a0h, a0l, a1h, a1l);
-                rs_pairs<1>(sE, meta, sIv, R.cell, cscale, R.nint, R.iv_dt, kL_c, kend_c, W0, W1, (int)lbj, nbl, nbc, -hj,
-                            -lj, trR, a0h, a0l, a1h, a1l);
-            }
-            __syncthreads();
+            if (__all_sync(0xffffffffu, done)) break;
         }
     }
-    if (valid) P.clocal[j] = ((double)a0h + (double)a0l) + ((double)a1h + (double)a1l);
+    if (!valid) return;
+    if (s1 < R.nint) R.cursor[side * M + j] = start + S * kcur;
+    ((float2*)R.csum)[side * M + j] = make_float2(ah, al);
+}
+
+__global__ void __launch_bounds__(kRsPairTargets, 8) k_rs_pairs(DevPlan P, RangeDev R, int s0, int s1) {
+    extern __shared__ __align__(16) float pair_sm[];
+    __shared__ float2 sPos[kRsPosChunk];
+    __shared__ int sRed[kRsPairTargets / 32 + 1];
+    if (blockIdx.y == 0) rs_pair_block<-1>(P, R, s0, s1, pair_sm, sPos, sRed);
+    else rs_pair_block<1>(P, R, s0, s1, pair_sm, sPos, sRed);
 }
 
 // plan time: the terms of the local sum, sum over pairs (j, l) closer than delta of the number of
@@ -526,7 +592,16 @@ __global__ void k_rs_solve_init(DevPlan P, RangeDev R) {
         for (int i = threadIdx.x; i < 2 * (kRsMaxIter + 1); i += blockDim.x) R.stats[i] = 0ull;
     const double ex[8] = {8.0, -28.0, 56.0, -70.0, 56.0, -28.0, 8.0, -1.0};
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P.M; j += (int64_t)gridDim.x * blockDim.x) {
-        const double rhs = fma(-0.5 * P.beta[j], P.clocal[j], __ldcg(P.rhs + j));
+        // the two sides of the local sum
+        double c;
+        if (R.csum) {
+            const float2 cl = ((const float2*)R.csum)[j], cr = ((const float2*)R.csum)[P.M + j];
+            c = ((double)cl.x + (double)cl.y) + ((double)cr.x + (double)cr.y);
+            P.clocal[j] = c;
+        } else {
+            c = P.clocal[j];                            // the mixed form's k_rs_local
+        }
+        const double rhs = fma(-0.5 * P.beta[j], c, __ldcg(P.rhs + j));
         P.rhs[j] = rhs;
         double x0;
         if (n >= 8) {

@@ -100,6 +100,28 @@ WAVE1D_RS_HD Pair split(double v) {
     return {h, (float)(v - (double)h)};
 }
 
+// A density hi + lo as four slices of 11 bits, whole numbers s_i of magnitude at most 1024 (2048 where
+// |hi| inv reaches it) with (hi + lo) inv = sum_i s_i 2^(-11 i) up to half a unit of the last slice;
+// inv: a power of two with |hi| inv < 1024.  The residues of hi are exact; lo (at most 2^-3 of a unit
+// of the second slice) joins the residue of that slice, with 2^-25 of its unit lost.
+WAVE1D_RS_HD void density_slices(float hi, float lo, float inv, float* s) {
+    float x = mul(hi, inv);
+    s[0] = rintf(x);
+    x = mul(sub(x, s[0]), 2048.f);
+    s[1] = rintf(x);
+    x = mul(add(sub(x, s[1]), mul(mul(lo, inv), 2048.f)), 2048.f);
+    for (int j = 2; j < kRsSlices; j++) {
+        s[j] = rintf(x);
+        x = mul(sub(x, s[j]), 2048.f);
+    }
+}
+// the power-of-two exponent E of a history whose largest |hi| has the bits mx: |hi| < 2^E, at least
+// -100 (smaller histories are 2^-144 exact), at most 127
+WAVE1D_RS_HD int slice_exponent(unsigned mx) {
+    const int e = (int)(mx >> 23) - 126;
+    return e < -100 ? -100 : (e > 127 ? 127 : e);
+}
+
 // ---------------------------------------------------------------------------------------------
 // Per-source, per-interval vector e_r (r = 0..7): e0, e1 as pairs, e2..e7 single.
 // Coefficient layout per (interval, m): three float4, (a0h, a0l, a1h, a1l), (a2h, a2l, a3h, a3l),
