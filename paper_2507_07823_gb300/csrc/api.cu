@@ -330,11 +330,11 @@ int fold_tables(wave1d_plan_t p) {
     if ((rc = dalloc(p, &rd.csum, (size_t)4 * P.M))) return rc;
     p->rs_slice_smem = (size_t)(rt.nm - 1) * 64 * sizeof(float2);
     p->rs_fold_smem = rs_fold_smem(rt.nk);
-    if (cudaFuncSetAttribute(k_rs_fold, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->rs_fold_smem) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(k_rs_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * rd.slab) != cudaSuccess ||
-        cudaFuncSetAttribute(k_rs_slices, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->rs_slice_smem) !=
-            cudaSuccess)
+    // all a block may have, for every plan: the attribute belongs to the kernel, not the plan
+    const int most = 227 * 1024;
+    if (p->rs_fold_smem > (size_t)most || p->rs_slice_smem > (size_t)most - 1024 ||
+        cudaFuncSetAttribute(k_rs_fold, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
+        cudaFuncSetAttribute(k_rs_slices, cudaFuncAttributeMaxDynamicSharedMemorySize, most - 1024) != cudaSuccess)
         return fail(WAVE1D_ECUDA, "cannot size the shared memory of the range-mode local sum");
     return WAVE1D_OK;
 }

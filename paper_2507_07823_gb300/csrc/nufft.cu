@@ -36,11 +36,6 @@
 #include "device_common.cuh"
 #include "../../include/wave1d.h"
 
-namespace wave1d {
-__global__ void k_fft_cols(const double2*, double2*, const double2*, int, int, int, int, int);
-__global__ void k_fft_rows(const double2*, double2*, const double2*, int, int, int, int, int);
-}  // namespace wave1d
-
 using namespace wave1d;
 
 namespace {
@@ -266,38 +261,128 @@ __global__ void __launch_bounds__(kUnitThreads) k_nu_spread64(const NuRange* __r
     spread64_unit<W>(ranges[blockIdx.x], runs, c, ker, grid, seg, rp);
 }
 
-// type-1 post-processing: S_k from the half-length FFT Z (E, O split) with the deconvolution
-// factors: S_k = f0 E_k + (f1 + i f2) O_k
-__global__ void k_nu_post1(const double2* __restrict__ Z, double* __restrict__ S, const double* __restrict__ modefac,
-                           int K, int L) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > K) return;
-    const double2 zk = Z[k], zm = Z[k == 0 ? 0 : L - k];
-    const double* f = modefac + 8 * (int64_t)k;
-    const double2 E = make_double2(0.5 * (zk.x + zm.x), 0.5 * (zk.y - zm.y));
-    const double2 D = make_double2(0.5 * (zk.x - zm.x), 0.5 * (zk.y + zm.y));
-    const double2 O = make_double2(D.y, -D.x);
-    const double2 s = cadd(make_double2(f[0] * E.x, f[0] * E.y), cmul(make_double2(f[1], f[2]), O));
-    S[2 * k] = s.x;
-    S[2 * k + 1] = s.y;
+// ---------------------------------------------------------------------------------------------
+// The FFTs of the transforms (L = L1 L2 complex points per instance, z[i2 + L2 i1] -> X[k1 + L1 k2]),
+// blockIdx.y = instance: one launch per pass covers all instances.  A block takes two lines at a time
+// (two adjacent columns or rows: 32-byte pieces, and two threads per butterfly of both lines,
+// fft_lines), type-1's row pass forms S_k from its pair of rows and type-2's column pass forms the
+// spectrum as it loads, so neither takes a pass over memory of its own.  Bound by the FP64 pipe: 2
+// instructions per point, component and stage; 64 instances of L = 8192 both ways about 90 us of it.
+// One instance at a time, six launches each, the 64 took 2.5 ms.
+// ---------------------------------------------------------------------------------------------
+constexpr int kFftThreads = 256;
+size_t nu_fft_smem(int N) { return (size_t)(2 * N + N / 2) * sizeof(double2); }
+
+__device__ __forceinline__ void nu_line_twiddles(double2* twN, const double2* __restrict__ tw, int L, int N, int sign) {
+    for (int j = threadIdx.x; j < N / 2; j += blockDim.x) {
+        double2 w = __ldg(tw + (int64_t)j * (L / N));
+        if (sign < 0) w.y = -w.y;
+        twN[j] = w;
+    }
 }
 
-// type-2 spectrum for the inverse real FFT: Zs[k] = alpha_k (f3 + i f4), Zs[L - k] =
-// conj(alpha_k) (f5 + i f6), zero where no mode lands
-__global__ void k_nu_pre2(const double* __restrict__ alpha, double2* __restrict__ Zs, const double* __restrict__ modefac,
-                          int K, int L) {
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < L; idx += gridDim.x * blockDim.x) {
-        double2 z = make_double2(0.0, 0.0);
-        if (idx <= K) {
-            const double* f = modefac + 8 * (int64_t)idx;
-            z = cmul(make_double2(alpha[2 * idx], alpha[2 * idx + 1]), make_double2(f[3], f[4]));
-        } else if (idx >= L - K) {
-            const int k = L - idx;
-            const double* f = modefac + 8 * (int64_t)k;
-            z = cmul(make_double2(alpha[2 * k], -alpha[2 * k + 1]), make_double2(f[5], f[6]));
-        }
-        Zs[idx] = z;
+// columns 2c, 2c + 1 (c = blockIdx.x) of z, from load(i2, i1): FFT over i1, twiddle -> Y[k1 L2 + i2]
+template <int SIGN, typename Load>
+__device__ __forceinline__ void nu_columns(Load load, double2* __restrict__ Y, const double2* __restrict__ tw, int L,
+                                           int L1, int L2, double2* sm) {
+    double2 *a = sm, *b = sm + L1, *twN = sm + 2 * L1;
+    const int logL1 = 31 - __clz(L1), c = 2 * blockIdx.x;
+    nu_line_twiddles(twN, tw, L, L1, SIGN);
+    for (int t = threadIdx.x; t < 2 * L1; t += blockDim.x)
+        (t & 1 ? b : a)[__brev(t >> 1) >> (32 - logL1)] = load(c + (t & 1), t >> 1);
+    __syncthreads();
+    fft_lines(a, b, twN, L1, logL1);
+    for (int t = threadIdx.x; t < 2 * L1; t += blockDim.x) {
+        const int i2 = c + (t & 1), k1 = t >> 1;
+        double2 w = __ldg(tw + (((int64_t)i2 * k1) & (L - 1)));
+        if (SIGN < 0) w.y = -w.y;
+        Y[(int64_t)k1 * L2 + i2] = cmul((t & 1 ? b : a)[k1], w);
     }
+}
+
+__global__ void __launch_bounds__(kFftThreads) k_nu_cols1(const double2* __restrict__ grids, double2* __restrict__ works,
+                                                          const double2* __restrict__ tw, int L, int L1, int L2) {
+    extern __shared__ __align__(16) double2 nu_sm[];
+    const double2* z = grids + (int64_t)blockIdx.y * L;
+    nu_columns<1>([&](int i2, int i1) { return __ldg(z + i2 + (int64_t)L2 * i1); }, works + (int64_t)blockIdx.y * L, tw, L,
+                  L1, L2, nu_sm);
+}
+
+// type-2 spectrum for the inverse real FFT: Zs[k] = alpha_k (f3 + i f4), Zs[L - k] = conj(alpha_k)
+// (f5 + i f6), zero where no mode lands
+__global__ void __launch_bounds__(kFftThreads) k_nu_cols2(const double* __restrict__ alphas, double2* __restrict__ works,
+                                                          const double* __restrict__ modefac,
+                                                          const double2* __restrict__ tw, int K, int L, int L1, int L2) {
+    extern __shared__ __align__(16) double2 nu_sm[];
+    const double* alpha = alphas + (int64_t)blockIdx.y * 2 * (K + 1);
+    nu_columns<-1>(
+        [&](int i2, int i1) {
+            const int idx = i2 + L2 * i1;
+            if (idx <= K) {
+                const double* f = modefac + 8 * (int64_t)idx;
+                return cmul(make_double2(alpha[2 * idx], alpha[2 * idx + 1]), make_double2(__ldg(f + 3), __ldg(f + 4)));
+            }
+            if (idx >= L - K) {
+                const int k = L - idx;
+                const double* f = modefac + 8 * (int64_t)k;
+                return cmul(make_double2(alpha[2 * k], -alpha[2 * k + 1]), make_double2(__ldg(f + 5), __ldg(f + 6)));
+            }
+            return make_double2(0.0, 0.0);
+        },
+        works + (int64_t)blockIdx.y * L, tw, L, L1, L2, nu_sm);
+}
+
+// rows k1 and L1 - k1 (k1 = blockIdx.x <= L1 / 2): FFT over i2, then S_k of the rows' modes from the
+// half-length FFT (E, O split) with the deconvolution factors, S_k = f0 E_k + (f1 + i f2) O_k; the
+// partner Z_{L-k} lies in the other row (in the same one for k1 = 0 and L1 / 2)
+__global__ void __launch_bounds__(kFftThreads) k_nu_rows1(const double2* __restrict__ works, double* __restrict__ Ss,
+                                                          const double* __restrict__ modefac,
+                                                          const double2* __restrict__ tw, int K, int L, int L1, int L2) {
+    extern __shared__ __align__(16) double2 nu_sm[];
+    double2 *a = nu_sm, *b = nu_sm + L2, *twN = nu_sm + 2 * L2;
+    const double2* Y = works + (int64_t)blockIdx.y * L;
+    double2* S = (double2*)Ss + (int64_t)blockIdx.y * (K + 1);
+    const int logL2 = 31 - __clz(L2), k1 = blockIdx.x, k1p = (L1 - k1) % L1;
+    const bool pair = k1p != k1;
+    nu_line_twiddles(twN, tw, L, L2, 1);
+    for (int i2 = threadIdx.x; i2 < L2; i2 += blockDim.x) {
+        const int rv = __brev(i2) >> (32 - logL2);
+        a[rv] = __ldg(Y + (int64_t)k1 * L2 + i2);
+        if (pair) b[rv] = __ldg(Y + (int64_t)k1p * L2 + i2);
+    }
+    __syncthreads();
+    fft_lines(a, pair ? b : nullptr, twN, L2, logL2);
+    for (int t = threadIdx.x; t < (pair ? 2 : 1) * L2; t += blockDim.x) {
+        const bool second = t >= L2;
+        const int k2 = second ? t - L2 : t, k = (second ? k1p : k1) + L1 * k2;
+        if (k > K) continue;
+        const double2 zk = (second ? b : a)[k2];
+        const double2 zm = (pair ? (second ? a : b) : a)[k1 == 0 ? (L2 - k2) & (L2 - 1) : L2 - 1 - k2];
+        const double* f = modefac + 8 * (int64_t)k;
+        const double f0 = __ldg(f);
+        const double2 E = make_double2(0.5 * (zk.x + zm.x), 0.5 * (zk.y - zm.y));
+        const double2 D = make_double2(0.5 * (zk.x - zm.x), 0.5 * (zk.y + zm.y));
+        const double2 O = make_double2(D.y, -D.x);
+        S[k] = cadd(make_double2(f0 * E.x, f0 * E.y), cmul(make_double2(__ldg(f + 1), __ldg(f + 2)), O));
+    }
+}
+
+// rows 2c, 2c + 1: FFT over i2 (sign -) -> grid points k1 + L1 k2
+__global__ void __launch_bounds__(kFftThreads) k_nu_rows2(const double2* __restrict__ works, double2* __restrict__ grids,
+                                                          const double2* __restrict__ tw, int L, int L1, int L2) {
+    extern __shared__ __align__(16) double2 nu_sm[];
+    double2 *a = nu_sm, *b = nu_sm + L2, *twN = nu_sm + 2 * L2;
+    const double2* Y = works + (int64_t)blockIdx.y * L;
+    double2* X = grids + (int64_t)blockIdx.y * L;
+    const int logL2 = 31 - __clz(L2), c = 2 * blockIdx.x;
+    nu_line_twiddles(twN, tw, L, L2, -1);
+    for (int t = threadIdx.x; t < 2 * L2; t += blockDim.x) {
+        const int r = t >= L2, i2 = r ? t - L2 : t;
+        (r ? b : a)[__brev(i2) >> (32 - logL2)] = __ldg(Y + (int64_t)(c + r) * L2 + i2);
+    }
+    __syncthreads();
+    fft_lines(a, b, twN, L2, logL2);
+    for (int t = threadIdx.x; t < 2 * L2; t += blockDim.x) X[c + (t & 1) + (int64_t)L1 * (t >> 1)] = (t & 1 ? b : a)[t >> 1];
 }
 
 // FP64 interpolation, tiles of kInterpTile consecutive points (interp64_unit, nufft_units.cuh).
@@ -422,12 +507,6 @@ bool nu_with_mixed(int w, int D, F&& f) {
            wd(I7{}, I8{}) || wd(I7{}, I10{});
 }
 
-int ilog2n(int v) {
-    int l = 0;
-    while ((1 << l) < v) l++;
-    return l;
-}
-
 }  // namespace
 
 struct wave1d_nufft_s {
@@ -454,8 +533,8 @@ struct wave1d_nufft_s {
     std::vector<int32_t> i0_host;    // points' first cells (sorted within each instance), for re-cutting
     std::vector<int64_t> off_host;   // instance offsets
     // FFT and deconvolution
-    double *grid = nullptr, *work = nullptr, *spec = nullptr, *spec2 = nullptr, *twiddle = nullptr,
-           *modefac = nullptr;
+    double *grid = nullptr, *work = nullptr, *twiddle = nullptr, *modefac = nullptr;
+    int group = 1;                   // instances whose FFTs share a launch (their work arrays fit 256 MB)
 };
 
 namespace {
@@ -656,10 +735,17 @@ int wave1d_nufft_plan_many(const double* x, const int64_t* offsets, int n_inst, 
         tw[2 * j] = std::cos(ang);
         tw[2 * j + 1] = std::sin(ang);
     }
+    h->group = std::max(1, std::min({n_inst, (1 << 25) / nf, 65535}));
     if ((rc = nu_upload(h, mf, &h->modefac)) || (rc = nu_upload(h, tw, &h->twiddle)) ||
-        (rc = nu_alloc(h, (size_t)n_inst * nf, &h->grid)) || (rc = nu_alloc(h, (size_t)nf, &h->work)) ||
-        (rc = nu_alloc(h, (size_t)nf, &h->spec)) || (rc = nu_alloc(h, (size_t)nf, &h->spec2)))
+        (rc = nu_alloc(h, (size_t)n_inst * nf, &h->grid)) || (rc = nu_alloc(h, (size_t)h->group * nf, &h->work)))
         return cleanup(rc);
+    // the largest line (2048 points) for every plan: the attribute belongs to the kernel, not the plan
+    const int most = (int)nu_fft_smem(2048);
+    if (cudaFuncSetAttribute(k_nu_cols1, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
+        cudaFuncSetAttribute(k_nu_cols2, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
+        cudaFuncSetAttribute(k_nu_rows1, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
+        cudaFuncSetAttribute(k_nu_rows2, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess)
+        return cleanup(nfail(WAVE1D_ECUDA, "cannot size the shared memory of the FFT passes"));
     if (cudaDeviceSynchronize() != cudaSuccess) return cleanup(nfail(WAVE1D_ECUDA, "upload failed"));
     *out = h;
     return WAVE1D_OK;
@@ -722,16 +808,14 @@ int wave1d_nufft_type1(wave1d_nufft_t h, const double* c, double* S) {
     int rc = wave1d_nufft_spread(h, c, h->grid);
     if (rc) return rc;
     const Params& P = h->P;
-    const int t1 = std::max(32, std::min(P.L1 / 2, 512)), t2 = std::max(32, std::min(P.L2 / 2, 512));
-    for (int b = 0; b < h->B; b++) {              // the instances' FFTs one after another
-        k_fft_cols<<<P.L2, t1, fft_smem_bytes(P.L1), h->stream>>>((const double2*)(h->grid + (size_t)b * P.nf),
-                                                                  (double2*)h->work, (const double2*)h->twiddle, P.L,
-                                                                  P.L1, P.L2, ilog2n(P.L1), +1);
-        k_fft_rows<<<P.L1, t2, fft_smem_bytes(P.L2), h->stream>>>((const double2*)h->work, (double2*)h->spec,
-                                                                  (const double2*)h->twiddle, P.L, P.L1, P.L2,
-                                                                  ilog2n(P.L2), +1);
-        k_nu_post1<<<(P.K + 1 + 127) / 128, 128, 0, h->stream>>>((const double2*)h->spec,
-                                                                 S + (size_t)b * 2 * (P.K + 1), h->modefac, P.K, P.L);
+    const double2* tw = (const double2*)h->twiddle;
+    double2* work = (double2*)h->work;
+    for (int b = 0; b < h->B; b += h->group) {
+        const unsigned nb = (unsigned)std::min(h->group, h->B - b);
+        k_nu_cols1<<<dim3(P.L2 / 2, nb), kFftThreads, nu_fft_smem(P.L1), h->stream>>>(
+            (const double2*)(h->grid + (size_t)b * P.nf), work, tw, P.L, P.L1, P.L2);
+        k_nu_rows1<<<dim3(P.L1 / 2 + 1, nb), kFftThreads, nu_fft_smem(P.L2), h->stream>>>(
+            work, S + (size_t)b * 2 * (P.K + 1), h->modefac, tw, P.K, P.L, P.L1, P.L2);
     }
     return cudaGetLastError() == cudaSuccess ? WAVE1D_OK : nfail(WAVE1D_ECUDA, "type-1 launch failed");
 }
@@ -740,17 +824,14 @@ int wave1d_nufft_type2(wave1d_nufft_t h, const double* alpha, double* u) {
     if (!h || !alpha || !u) return nfail(WAVE1D_EINVAL, "bad arguments");
     if (cudaSetDevice(h->device) != cudaSuccess) return nfail(WAVE1D_ECUDA, "cudaSetDevice");
     const Params& P = h->P;
-    const int t1 = std::max(32, std::min(P.L1 / 2, 512)), t2 = std::max(32, std::min(P.L2 / 2, 512));
-    for (int b = 0; b < h->B; b++) {
-        k_nu_pre2<<<(P.L + 255) / 256, 256, 0, h->stream>>>(alpha + (size_t)b * 2 * (P.K + 1), (double2*)h->spec2,
-                                                             h->modefac, P.K, P.L);
-        k_fft_cols<<<P.L2, t1, fft_smem_bytes(P.L1), h->stream>>>((const double2*)h->spec2, (double2*)h->work,
-                                                                  (const double2*)h->twiddle, P.L, P.L1, P.L2,
-                                                                  ilog2n(P.L1), -1);
-        k_fft_rows<<<P.L1, t2, fft_smem_bytes(P.L2), h->stream>>>((const double2*)h->work,
-                                                                  (double2*)(h->grid + (size_t)b * P.nf),
-                                                                  (const double2*)h->twiddle, P.L, P.L1, P.L2,
-                                                                  ilog2n(P.L2), -1);
+    const double2* tw = (const double2*)h->twiddle;
+    double2* work = (double2*)h->work;
+    for (int b = 0; b < h->B; b += h->group) {
+        const unsigned nb = (unsigned)std::min(h->group, h->B - b);
+        k_nu_cols2<<<dim3(P.L2 / 2, nb), kFftThreads, nu_fft_smem(P.L1), h->stream>>>(
+            alpha + (size_t)b * 2 * (P.K + 1), work, h->modefac, tw, P.K, P.L, P.L1, P.L2);
+        k_nu_rows2<<<dim3(P.L1 / 2, nb), kFftThreads, nu_fft_smem(P.L2), h->stream>>>(
+            work, (double2*)(h->grid + (size_t)b * P.nf), tw, P.L, P.L1, P.L2);
     }
     if (cudaGetLastError() != cudaSuccess) return nfail(WAVE1D_ECUDA, "type-2 launch failed");
     return wave1d_nufft_interp(h, h->grid, u);
