@@ -63,12 +63,12 @@ size_t rs_local_smem(int nint, int nm);
 __global__ void k_rs_slices(DevPlan P, RangeDev R);
 __global__ void k_rs_fold(DevPlan P, RangeDev R, int s0);
 __global__ void k_rs_pairs(DevPlan P, RangeDev R, int s0, int s1);
-__global__ void k_rs_local_T(DevPlan P, RangeDev R, int64_t n, const double* cbar, double* sb);
+__global__ void k_rs_moments(DevPlan P, RangeDev R, int s0, int s1, const double* cbar);
+__global__ void k_rs_unfold(DevPlan P, RangeDev R, int s0, int s1, int64_t n, float2* sums, double* sb);
 __global__ void k_rs_adj_init(DevPlan P, RangeDev R, double* slot_vals, double* rhs);
 __global__ void k_rs_adj_post(DevPlan P, RangeDev R, const double* sigma_next, const double* g_next, double* grad,
                               double* gbar_next, double* cbar, double* uHbar);
 __global__ void k_rs_adj_receivers(DevPlan P, RangeDev R, int64_t n, const double* ubar, double* sb);
-size_t rs_local_T_smem(int nint, int nm);
 __global__ void k_rs_nearby_weights(DevPlan P, RangeDev R);
 __global__ void k_rs_solve_init(DevPlan P, RangeDev R);
 __global__ void k_rs_jacobi(DevPlan P, RangeDev R, int it);
@@ -311,6 +311,7 @@ int fold_tables(wave1d_plan_t p) {
     uint16_t* h16;
     rd.nk = rt.nk;
     rd.nivp = rt.nivp;
+    rd.fold_shift = rt.fold_shift;
     if ((rc = upload(p, rt.fold, &h16))) return rc;
     rd.fold = h16;
     if ((rc = upload(p, rt.fold_scale, &f32))) return rc;
@@ -324,7 +325,7 @@ int fold_tables(wave1d_plan_t p) {
     if (cudaMemGetInfo(&free_b, &all_b) != cudaSuccess) return fail(WAVE1D_ECUDA, "cudaMemGetInfo");
     const size_t per_iv = (size_t)P.M * kRsRecord * sizeof(float);
     const size_t want = std::min({(size_t)8192 * P.M, (size_t)2 << 30, free_b / 8});
-    rd.slab = (int)std::min<size_t>((size_t)((rt.nint + 7) / 8) * 8, std::max<size_t>(8, want / per_iv / 8 * 8));
+    rd.slab = (int)std::min<size_t>((size_t)((rt.nint + 15) / 16) * 16, std::max<size_t>(16, want / per_iv / 16 * 16));
     if ((rc = dalloc(p, &rd.evec, (size_t)P.M * rd.slab * kRsRecord))) return rc;
     if ((rc = dalloc(p, &rd.cursor, (size_t)2 * P.M))) return rc;
     if ((rc = dalloc(p, &rd.csum, (size_t)4 * P.M))) return rc;
@@ -754,8 +755,10 @@ int wave1d_plan(const double* x, const double* beta, int64_t M, int bc, double d
         rd.bp2 = f32;
         if ((rc = upload(p, rt.ih, &f32))) return cleanup(rc);
         rd.ih = f32;
-        if ((rc = upload(p, rt.coef, &f32))) return cleanup(rc);
-        rd.coef = f32;
+        if (o.precision == 1) {
+            if ((rc = upload(p, rt.coef, &f32))) return cleanup(rc);
+            rd.coef = f32;
+        }
         if ((rc = upload(p, mr, &r32))) return cleanup(rc);
         rd.mr = r32;
         if ((rc = upload(p, mr0, &r32))) return cleanup(rc);
@@ -790,8 +793,9 @@ int wave1d_plan(const double* x, const double* beta, int64_t M, int bc, double d
             if (cudaFuncSetAttribute(k_rs_local, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->rs_smem) !=
                 cudaSuccess)
                 return cleanup(fail(WAVE1D_ECUDA, "cannot size the shared memory of the range-mode local sum"));
-        } else if ((rc = fold_tables(p))) {
-            return cleanup(rc);
+        } else {
+            if ((rc = fold_tables(p))) return cleanup(rc);
+            rd.folded = 1;
         }
         p->info_range_pairs = hp.range_pairs;
     }
@@ -1366,7 +1370,7 @@ struct Reverse {
     int npts = 0;
     size_t lsmem = 0;
     double* rrhs = nullptr;   // plans without pair lists: the transposed solve's right-hand side
-    size_t tsmem = 0;
+    float2* usum = nullptr;   // the transposed local sum's pairs between slabs
     static constexpr int kLocalWarps = 4;     // the transposed local sum: one warp per spring row
 
     int init(wave1d_plan_t pl) {
@@ -1401,10 +1405,15 @@ struct Reverse {
             return rc;
         if (p->range) {
             if ((rc = wk.zeros(&rrhs, (size_t)M))) return rc;
-            tsmem = rs_local_T_smem(p->rd.nint, p->rd.nm);
-            if (tsmem > 227 * 1024) return fail(WAVE1D_EUNSUPPORTED, "window too long for the transposed local sum");
-            CK(cudaFuncSetAttribute(k_rs_local_T, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsmem));
-            return WAVE1D_OK;
+            if (!p->rd.fold && (rc = fold_tables(p))) return rc;        // a mixed plan's first reverse march
+            if (!p->rd.unfold) {
+                uint16_t* h16;
+                if ((rc = upload(p, hp.rt.unfold, &h16))) return rc;
+                p->rd.nis = hp.rt.nis;
+                p->rd.nmp = hp.rt.nmp;
+                p->rd.unfold = h16;
+            }
+            return wk.zeros(&usum, (size_t)M * p->rd.nmp);
         }
         lsmem = adj_local_smem(P.m_max, kLocalWarps);
         if (lsmem > 227 * 1024) return fail(WAVE1D_EUNSUPPORTED, "window too long for the adjoint's local-sum accumulators");
@@ -1440,7 +1449,14 @@ struct Reverse {
                 k_rs_adj_post<<<gM, 256, 0, s>>>(d, rd, sig_rows + (n - row0) * M, g ? g + n * M : nullptr,
                                                  want_beta ? gsum : nullptr, grad_g ? grad_g + n * M : nullptr, cbar, uHbar);
                 if (n == 0) break;
-                k_rs_local_T<<<(unsigned)((M + kRsTTargets - 1) / kRsTTargets), kRsTTargets, tsmem, s>>>(d, rd, n, cbar, sb);
+                const unsigned gp = blocks_for(M, kRsPairTargets, INT32_MAX);
+                for (int s0 = 0; s0 < rd.nint; s0 += rd.slab) {
+                    const int s1 = std::min(rd.nint, s0 + rd.slab);
+                    CK(cudaMemsetAsync(rd.evec, 0, (size_t)M * rd.slab * kRsRecord * sizeof(float), s));
+                    k_rs_moments<<<gp, kRsPairTargets, (size_t)16 * (s1 - s0), s>>>(d, rd, s0, s1, cbar);
+                    k_rs_unfold<<<dim3(blocks_for(M, 64, INT32_MAX), (unsigned)(rd.nmp / 8 + 4) / 5), 128, 0, s>>>(d, rd, s0, s1, n,
+                                                                                                          usum, sb);
+                }
             } else {
                 if (have_rcv) k_adj_receivers<<<gM, 256, 0, s>>>(M, ring, n, rptr, rrcv, rmr, rwoff, rw, ub, sb);
                 k_adj_take<<<gM, 256, 0, s>>>(M, sb + (int64_t)(((n + 1) % ring)) * M, tmp);

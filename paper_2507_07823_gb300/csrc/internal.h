@@ -86,6 +86,10 @@ struct RangeTables {
     int nk = 0, nivp = 0;              // steps of 16 m (m = 1 .. 16 nk), intervals with padding
     std::vector<uint16_t> fold;        // half-precision s_j
     std::vector<float> fold_scale;     // [nivp][8]: 2^(e - 10)
+    int fold_shift = 0;                // the density slices' units are 2^shift larger, so that
+                                       //   1024 sum_m |s_0| stays below 2^(24 + shift) (long windows)
+    int nis = 0, nmp = 0;              // steps of 16 intervals, m = 1 .. nmp (a multiple of 8)
+    std::vector<uint16_t> unfold;      // the same s_j as operands of the transposed sum (unfold_index)
     std::vector<int32_t> cell;         // kRsCells: interval of the left end of each cell of [0, delta)
     float cell_scale = 0.f;            // kRsCells / delta: cell of a distance d is floor(d cell_scale)
 };
@@ -105,13 +109,19 @@ inline size_t fold_index(int slice, int m, int iv, int nk, int nivp) {
     const int k = (m - 1) & 15, ks = (m - 1) >> 4, q = (k & 7) >> 1;
     return (((size_t)slice * nk + ks) * nivp + iv) * 16 + q * 4 + (k >> 3) * 2 + (k & 1);
 }
+// index of the half s_j of (slice, iv, m) in RangeTables::unfold: per (slice, step of 16 intervals, m)
+// a row of 16 halves in the same order, over the intervals
+inline size_t unfold_index(int slice, int m, int iv, int nis, int nmp) {
+    const int k = iv & 15, q = (k & 7) >> 1;
+    return (((size_t)slice * nis + (iv >> 4)) * nmp + (m - 1)) * 16 + q * 4 + (k >> 3) * 2 + (k & 1);
+}
 // The plan's weight rule itself at each distance, Q[i * (m_max + 1) + m] (for checks).
 void local_weights_exact(const Params& P, const std::vector<double>& d, std::vector<double>& Q);
 // targets per block of the range-mode local sum (one per thread); cells of the distance lookup table
 constexpr int kRsTargets = 256;
 constexpr int kRsPairTargets = 128; // targets per block of its pair kernel
 constexpr int kRsRecord = 12;       // floats of an e-vector record in memory
-constexpr int kRsTTargets = 128;    // outputs per block of the transposed local sum (reverse march)
+constexpr int kRsTTargets = 128;    // outputs per block where a host check walks the transposed sum
 constexpr int kRsCells = 2048;
 
 struct HostPlan {
@@ -333,13 +343,18 @@ struct RangeDev {
     const double* cheb;         // [iv][m][8] Chebyshev coefficients in z (FP64)
     const int* cell;            // kRsCells: first interval of each cell of [0, delta)
     float cell_scale;           // kRsCells / delta
+    int fold_shift;             // RangeTables::fold_shift
     int nk, nivp;               // steps of 16 m, padded intervals of the fold's table
     const uint16_t* fold;       // coefficient slices (RangeTables::fold)
     const float* fold_scale;    // [nivp][8]
     uint16_t* slices;           // [M][kRsSlices][nk][16] halves: the step's density slices
     float* slice_scale;         // M: their scales
-    int slab;                   // intervals whose e-vectors are held at once (a multiple of 8)
-    float* evec;                // [M][slab][kRsRecord]: e-vector records of the slab
+    int nis, nmp;               // steps of 16 intervals and padded m of the transposed sum's table
+    const uint16_t* unfold;     // coefficient slices (RangeTables::unfold)
+    int slab;                   // intervals whose e-vectors are held at once (a multiple of 16)
+    int folded;                 // 1: the local sum comes from k_rs_pairs (csum), 0: from k_rs_local (clocal)
+    float* evec;                // [M][slab][kRsRecord]: e-vector records of the slab; the reverse march's
+                                //   moments
     int32_t* cursor;            // [2][M]: per side, each target's next source
     float* csum;                // [2][M]: per side, each target's sum so far as a pair
     const int32_t* blk_win;     // [block][4] (see HostPlan::blk_win)

@@ -1214,9 +1214,13 @@ static uint16_t half_bits(int v) {
 static void fold_slices(const std::vector<double>& a, RangeTables& rt) {
     const int n = rt.nint, nm = rt.nm;
     rt.nk = (nm - 1 + 15) / 16;
-    rt.nivp = n + 8;                                      // a tile of 8 intervals may start at the last one
+    rt.nivp = n + 16;                                     // tiles of 8 intervals (16, transposed) may pass the end
     rt.fold.assign((size_t)kRsAllSlices * rt.nk * rt.nivp * 16, 0);
     rt.fold_scale.assign((size_t)rt.nivp * kRsPowers, 0.0f);
+    rt.nis = (n + 15) / 16;
+    rt.nmp = (nm - 1 + 7) / 8 * 8;
+    rt.unfold.assign((size_t)kRsAllSlices * rt.nis * rt.nmp * 16, 0);
+    double most = 0.0;                                    // largest sum_m |s_0|
     for (int iv = 0; iv < n; iv++)
         for (int r = 0; r < kRsPowers; r++) {
             double mx = 0.0;
@@ -1225,15 +1229,21 @@ static void fold_slices(const std::vector<double>& a, RangeTables& rt) {
             int e;
             (void)std::frexp(mx, &e);                     // mx < 2^e
             rt.fold_scale[(size_t)iv * kRsPowers + r] = (float)std::ldexp(1.0, e - 10);
+            double sum = 0.0;
             for (int m = 1; m < nm; m++) {
                 double v = std::ldexp(a[((size_t)iv * nm + m) * kRsPowers + r], 10 - e);
+                sum += std::fabs(std::nearbyint(v));
                 for (int j = 0; j < kRsSlicesOf[r]; j++) {
                     const double s = std::nearbyint(v);
-                    rt.fold[fold_index(kRsFirstSlice[r] + j, m, iv, rt.nk, rt.nivp)] = half_bits((int)s);
+                    const uint16_t h = half_bits((int)s);
+                    rt.fold[fold_index(kRsFirstSlice[r] + j, m, iv, rt.nk, rt.nivp)] = h;
+                    rt.unfold[unfold_index(kRsFirstSlice[r] + j, m, iv, rt.nis, rt.nmp)] = h;
                     v = (v - s) * 2048.0;
                 }
             }
+            most = std::max(most, sum);
         }
+    while (most > std::ldexp(1.0, 14 + rt.fold_shift)) rt.fold_shift++;
 }
 
 void build_range_tables(const Params& P, RangeTables& rt) {

@@ -24,6 +24,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "internal.h"
 #include "phases.cuh"
@@ -34,7 +35,6 @@
 namespace wave1d {
 
 namespace {
-constexpr int kRsChunk = 32;      // inputs per chunk of the transposed local sum
 constexpr int kRsPosChunk = 1024; // source positions staged at once by a block of k_rs_pairs
 }  // namespace
 
@@ -75,8 +75,8 @@ __device__ __forceinline__ double rs_q0(const RangeDev& R, double d) {
 // slices of 11 bits, whole numbers of at most 1024 that halves hold exactly (sigma = 2^(e-10)
 // sum_i s_i 2^(-11 i), one exponent per source; coefficients likewise, one per (interval, r)).  The
 // product of slices i and j is a whole number, products of equal i + j share an accumulator, and
-// every partial sum stays below 2^24 (sum_m |a_m| is about 11 times the largest |a_m|), so FP32
-// accumulation is exact; what is dropped lies below 2^-43 of the largest |a sigma| of the source and
+// every partial sum stays below 2^24 (sum_m |a_m| is about 11 times the largest |a_m|; longer windows
+// take larger units, fold_shift), so FP32 accumulation is exact; what is dropped lies below 2^-43 of the largest |a sigma| of the source and
 // interval for e_0, and by as many bits less for the higher powers as their coefficients are smaller.
 // ---------------------------------------------------------------------------------------------
 
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(256) k_rs_slices(DevPlan P, RangeDev R) {
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
         // units of 2^(E-10); a non-finite density makes the scale NaN, so every sum it enters is NaN
-        const int E = rs::slice_exponent(mx);
+        const int E = min(127, rs::slice_exponent(mx) + R.fold_shift);
         const bool fin = mx < 0x7f800000u;
         if ((t & 3) == 0) {
             sInv[k] = __uint_as_float((unsigned)(127 + 10 - E) << 23);
@@ -388,9 +388,12 @@ __device__ __forceinline__ int rs_warp_first(int n, F&& pred) {
     return hi;
 }
 
-template <int S>
+// One side of one block's pairs of a slab: v.stage(k, e) is called for each of the block's sources as
+// their positions are staged (k: place in the chunk), v.pair(k, e, iv, zh, zl) for each pair of this
+// thread's target in the order of its sources (iv: interval in the slab).
+template <int S, typename Visitor>
 __device__ __forceinline__ void rs_pair_block(const DevPlan& P, const RangeDev& R, int s0, int s1, float* sIv, float2* sPos,
-                                              int* sRed) {
+                                              int* sRed, Visitor& v) {
     constexpr int side = S > 0 ? 1 : 0;
     const int64_t M = P.M;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -411,7 +414,6 @@ __device__ __forceinline__ void rs_pair_block(const DevPlan& P, const RangeDev& 
     }
     const int nbl = __ldg(R.nb_lo + j), nbc = __ldg(R.nb_cnt + j);
     int cur;
-    float ah = 0.f, al = 0.f;
     if (s0 == 0) {
         // lb_j: the first spring at x_j's position (sources below it are strictly left of x_j)
         int64_t lbj = j;
@@ -426,9 +428,6 @@ __device__ __forceinline__ void rs_pair_block(const DevPlan& P, const RangeDev& 
         cur = (int)(S > 0 ? lbj : lbj - 1);
     } else {
         cur = R.cursor[side * M + j];
-        const float2 a = ((const float2*)R.csum)[side * M + j];
-        ah = a.x;
-        al = a.y;
     }
     // the block's sources of the slab: from the nearest cursor (k = 0) to the first one beyond the
     // slab's far end of every target, inside the window of its 256-target block
@@ -463,6 +462,7 @@ __device__ __forceinline__ void rs_pair_block(const DevPlan& P, const RangeDev& 
             float h, l;
             rs::grid_split(rs_xext(P, start + S * k) - xa, G, h, l);
             sPos[k - base] = make_float2(h, l);
+            v.stage(k - base, start + S * k);
         }
         __syncthreads();
         int k = max(base, __reduce_min_sync(0xffffffffu, done ? count : kcur));
@@ -511,26 +511,41 @@ __device__ __forceinline__ void rs_pair_block(const DevPlan& P, const RangeDev& 
                     done = true;
                     kcur = k;
                 } else {
-                    const float4* rec = (const float4*)(R.evec + ((size_t)rs_spring(e, M) * R.slab + tr.iv) * kRsRecord);
-                    const float4 r0 = __ldg(rec), r1 = __ldg(rec + 1), r2 = __ldg(rec + 2);
-                    rs_eval(r0, r1, r2, zh, zl, ah, al);
+                    v.pair(k - base, e, tr.iv, zh, zl);
                     kcur = k + 1;
                 }
             }
             if (__all_sync(0xffffffffu, done)) break;
         }
     }
-    if (!valid) return;
-    if (s1 < R.nint) R.cursor[side * M + j] = start + S * kcur;
-    ((float2*)R.csum)[side * M + j] = make_float2(ah, al);
+    if (valid && s1 < R.nint) R.cursor[side * M + j] = start + S * kcur;
+    __syncthreads();                                      // the staged positions are free again
 }
+
+// the local sum of one side: each target's polynomials into its pair, carried from slab to slab
+struct RsSum {
+    const DevPlan& P;
+    const RangeDev& R;
+    float ah, al;
+    __device__ __forceinline__ void stage(int, int) {}
+    __device__ __forceinline__ void pair(int, int e, int iv, float zh, float zl) {
+        const float4* rec = (const float4*)(R.evec + ((size_t)rs_spring(e, P.M) * R.slab + iv) * kRsRecord);
+        const float4 r0 = __ldg(rec), r1 = __ldg(rec + 1), r2 = __ldg(rec + 2);
+        rs_eval(r0, r1, r2, zh, zl, ah, al);
+    }
+};
 
 __global__ void __launch_bounds__(kRsPairTargets, 8) k_rs_pairs(DevPlan P, RangeDev R, int s0, int s1) {
     extern __shared__ __align__(16) float pair_sm[];
     __shared__ float2 sPos[kRsPosChunk];
     __shared__ int sRed[kRsPairTargets / 32 + 1];
-    if (blockIdx.y == 0) rs_pair_block<-1>(P, R, s0, s1, pair_sm, sPos, sRed);
-    else rs_pair_block<1>(P, R, s0, s1, pair_sm, sPos, sRed);
+    const int64_t j = (int64_t)blockIdx.x * kRsPairTargets + threadIdx.x;
+    float2* acc = (float2*)R.csum + blockIdx.y * P.M + j;
+    const float2 a = j < P.M && s0 > 0 ? *acc : make_float2(0.f, 0.f);
+    RsSum v{P, R, a.x, a.y};
+    if (blockIdx.y == 0) rs_pair_block<-1>(P, R, s0, s1, pair_sm, sPos, sRed, v);
+    else rs_pair_block<1>(P, R, s0, s1, pair_sm, sPos, sRed, v);
+    if (j < P.M) *acc = make_float2(v.ah, v.al);
 }
 
 // plan time: the terms of the local sum, sum over pairs (j, l) closer than delta of the number of
@@ -594,7 +609,7 @@ __global__ void k_rs_solve_init(DevPlan P, RangeDev R) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P.M; j += (int64_t)gridDim.x * blockDim.x) {
         // the two sides of the local sum
         double c;
-        if (R.csum) {
+        if (R.folded) {
             const float2 cl = ((const float2*)R.csum)[j], cr = ((const float2*)R.csum)[P.M + j];
             c = ((double)cl.x + (double)cl.y) + ((double)cr.x + (double)cr.y);
             P.clocal[j] = c;
@@ -762,176 +777,237 @@ __global__ void k_rs_finish(DevPlan P, RangeDev R) {
 // ---------------------------------------------------------------------------------------------
 // Reverse march (wave1d_adjoint on a plan without pair lists): the transposed local sum,
 //   sigmabar_l^{n+1-m} += sum_j Q_m(d_jl) cbar_j,   m >= 1,
-// over the same pairs as k_rs_local (every j within delta of l, each once).  On interval iv,
+// over the same pairs as k_rs_pairs (every j within delta of l, each once).  On interval iv,
 // Q_m(d) = sum_r a_{iv,m,r} z^r, so the pairs of output l that fall in iv enter only through the
-// moments F_r = sum_{j in iv} z_jl^r cbar_j, and the interval adds sum_r a_{iv,m,r} F_r to
-// output m.  One block of kRsTTargets outputs (thread t: output j0 + t) walks the inputs of its
-// window as k_rs_local walks its sources (the same grid, index side test, interval walk and
-// near/far rule); a thread accumulates the moments of its current interval (F_0, F_1 as
-// compensated pairs, F_2 .. F_7 single) and flushes them into its per-m FP64 outputs in shared
-// memory when the interval changes.  No atomics: every output has one writer, in a fixed order.
+// moments F_{l,iv,r} = sum_{j in iv} z_jl^r cbar_j (k_rs_moments: F_0, F_1 as pairs, F_2 .. F_7 single),
+// and the rest is a contraction over intervals and powers with the same coefficients for every
+// output, sum_{iv,r} a_{iv,m,r} F_{l,iv,r}, on the tensor cores (k_rs_unfold).  Per output and interval
+// it was 26 m x (48 FP32 instructions and 4 on the FP64 pipe, 16 cycles of an SM each): 3e4 uniform
+// springs 7.1 -> 2.7 ms per reverse step (5 slabs of moments 0.19 and contraction 0.34).  No atomics:
+// every output has one writer, in a fixed order.
 // ---------------------------------------------------------------------------------------------
-size_t rs_local_T_smem(int nint, int nm) {
-    return (size_t)4 * nint * sizeof(float) + (size_t)kRsTTargets * nm * sizeof(double) +
-           (size_t)kRsChunk * sizeof(float2);
-}
-
 struct RsMoments {
+    const DevPlan& P;
+    const RangeDev& R;
+    const double* cbar;
+    float2* sC;               // cbar of the staged sources as pairs
+    float* rec;               // this output's records of the slab
+    bool add;                 // the second side adds to the first one's
+    int cur;                  // the interval whose moments are held, -1: none
     float f0h, f0l, f1h, f1l, f2, f3, f4, f5, f6, f7;
+    __device__ __forceinline__ void clear() { f0h = f0l = f1h = f1l = f2 = f3 = f4 = f5 = f6 = f7 = 0.f; }
+    __device__ __forceinline__ void flush() {
+        if (cur < 0) return;
+        float4* o = (float4*)(rec + (size_t)cur * kRsRecord);
+        if (add) {
+            const float4 a = o[0], b = o[1], c = o[2];
+            rs::acc_add(f0h, f0l, a.x, a.y);
+            rs::acc_add(f1h, f1l, a.z, a.w);
+            f2 = __fadd_rn(f2, b.x);
+            f3 = __fadd_rn(f3, b.y);
+            f4 = __fadd_rn(f4, b.z);
+            f5 = __fadd_rn(f5, b.w);
+            f6 = __fadd_rn(f6, c.x);
+            f7 = __fadd_rn(f7, c.y);
+        }
+        o[0] = make_float4(f0h, f0l, f1h, f1l);
+        o[1] = make_float4(f2, f3, f4, f5);
+        o[2] = make_float4(f6, f7, 0.f, 0.f);
+    }
+    __device__ __forceinline__ void stage(int k, int e) {
+        const double c = cbar[rs_spring(e, P.M)];
+        const float hi = (float)c;
+        sC[k] = make_float2(hi, (float)(c - (double)hi));
+    }
+    __device__ __forceinline__ void pair(int k, int, int iv, float zh, float zl) {
+        if (iv != cur) {
+            flush();
+            cur = iv;
+            clear();
+        }
+        const float2 c = sC[k];
+        rs::acc_add(f0h, f0l, c.x, c.y);
+        rs::acc_mac(f1h, f1l, zh, zl, c.x, c.y);
+        float p = __fmul_rn(__fmul_rn(zh, zh), c.x);
+        f2 = __fadd_rn(f2, p);
+        p = __fmul_rn(p, zh);
+        f3 = __fadd_rn(f3, p);
+        p = __fmul_rn(p, zh);
+        f4 = __fadd_rn(f4, p);
+        p = __fmul_rn(p, zh);
+        f5 = __fadd_rn(f5, p);
+        p = __fmul_rn(p, zh);
+        f6 = __fadd_rn(f6, p);
+        p = __fmul_rn(p, zh);
+        f7 = __fadd_rn(f7, p);
+    }
 };
 
-// out[m] += sum_r a_{iv,m,r} F_r for the interval's m >= 1 (out: this thread's column, stride kRsTTargets)
-__device__ __forceinline__ void rs_flush(const RangeDev& R, int iv, const RsMoments& F, double* out) {
-    const int m0 = max(1, __ldg(R.mr + 2 * iv)), m1 = __ldg(R.mr + 2 * iv + 1);
-    const float4* c = (const float4*)R.coef + (size_t)iv * R.nm * 3;
-    for (int m = m0; m <= m1; m++) {
-        const float4 c01 = __ldg(c + 3 * m), c23 = __ldg(c + 3 * m + 1), c47 = __ldg(c + 3 * m + 2);
-        float h = 0.f, l = 0.f;
-        rs::acc_mac(h, l, c01.x, c01.y, F.f0h, F.f0l);
-        rs::acc_mac(h, l, c01.z, c01.w, F.f1h, F.f1l);
-        float r = __fmaf_rn(c23.y, F.f2, __fmaf_rn(c23.x, F.f2, 0.f));
-        r = __fmaf_rn(c23.w, F.f3, __fmaf_rn(c23.z, F.f3, r));
-        r = __fmaf_rn(c47.x, F.f4, r);
-        r = __fmaf_rn(c47.y, F.f5, r);
-        r = __fmaf_rn(c47.z, F.f6, r);
-        r = __fmaf_rn(c47.w, F.f7, r);
-        rs::acc_add(h, l, r, 0.f);
-        out[(size_t)m * kRsTTargets] += (double)h + (double)l;
-    }
+// the moments of a slab, both sides (the records are zero on entry)
+__global__ void __launch_bounds__(kRsPairTargets) k_rs_moments(DevPlan P, RangeDev R, int s0, int s1,
+                                                              const double* __restrict__ cbar) {
+    extern __shared__ __align__(16) float pair_sm[];
+    __shared__ float2 sPos[kRsPosChunk], sC[kRsPosChunk];
+    __shared__ int sRed[kRsPairTargets / 32 + 1];
+    const int64_t j = min((int64_t)blockIdx.x * kRsPairTargets + threadIdx.x, P.M - 1);
+    RsMoments v{P, R, cbar, sC, R.evec + (size_t)j * R.slab * kRsRecord, false, -1};
+    v.clear();
+    rs_pair_block<-1>(P, R, s0, s1, pair_sm, sPos, sRed, v);
+    v.flush();
+    v.cur = -1;
+    v.add = true;
+    rs_pair_block<1>(P, R, s0, s1, pair_sm, sPos, sRed, v);
+    v.flush();
 }
 
-// F += cbar z^r for one pair (z = zh + zl normalised, cbar = (ch, cl))
-__device__ __forceinline__ void rs_moments_add(RsMoments& F, float zh, float zl, float ch, float cl) {
-    rs::acc_add(F.f0h, F.f0l, ch, cl);
-    rs::acc_mac(F.f1h, F.f1l, zh, zl, ch, cl);
-    const float z2 = __fmul_rn(zh, zh);
-    float p = __fmul_rn(z2, ch);
-    F.f2 = __fadd_rn(F.f2, p);
-    p = __fmul_rn(p, zh);
-    F.f3 = __fadd_rn(F.f3, p);
-    p = __fmul_rn(p, zh);
-    F.f4 = __fadd_rn(F.f4, p);
-    p = __fmul_rn(p, zh);
-    F.f5 = __fadd_rn(F.f5, p);
-    p = __fmul_rn(p, zh);
-    F.f6 = __fadd_rn(F.f6, p);
-    p = __fmul_rn(p, zh);
-    F.f7 = __fadd_rn(F.f7, p);
-}
-
-// the pairs of one side for one output, inputs [k0, k1) of the chunk (cf. rs_pairs)
-template <int S>
-__device__ __forceinline__ void rs_pairs_T(const RangeDev& R, const float4* sMeta, const float2* sC, const float* ivt,
-                                           float cscale, int k0, int k1, int lbj, int nbl, int nbc, float bh, float bl,
-                                           rs::Track& tr, int& cur, RsMoments& F, double* out) {
-    for (int kk = k0; kk < k1; kk++) {
-        const float4 mt = sMeta[kk];
-        const int e = __float_as_int(mt.z), lohi = __float_as_int(mt.w);
-        if ((lohi & 0x7fff) > (lohi >> 16) || (S < 0 ? e >= lbj : e < lbj)) continue;
-        float zh, zl;
-        rs::z_of<S>(tr, mt.x, mt.y, zh, zl);
-        if (fabsf(zh) > rs::kZTol) rs::walk<S>(ivt, R.cell, cscale, R.nint, bh, bl, mt.x, mt.y, tr, zh, zl);
-        if (lohi & 0x8000)
-            rs::near_side<S>(ivt, R.iv_dt, (unsigned)(e - nbl) < (unsigned)nbc, bh, bl, mt.x, mt.y, tr, zh, zl);
-        if (!(fabsf(zh) <= rs::kZTol)) continue;
-        if (tr.iv != cur) {
-            if (cur >= 0) rs_flush(R, cur, F, out);
-            cur = tr.iv;
-            F = RsMoments{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        }
-        const float2 cb = sC[kk];
-        rs_moments_add(F, zh, zl, cb.x, cb.y);
-    }
-}
-
-__global__ void __launch_bounds__(kRsTTargets) k_rs_local_T(DevPlan P, RangeDev R, int64_t n,
-                                                           const double* __restrict__ cbar, double* sb) {
-    extern __shared__ __align__(16) float rs_sm[];
-    float* sIv = rs_sm;
-    double* sOut = (double*)(sIv + 4 * R.nint);                  // [m][thread]
-    float2* sC = (float2*)(sOut + (size_t)R.nm * kRsTTargets);   // the chunk's cbar (pairs)
-    __shared__ float4 sMeta[kRsTTargets];
-
-    const int64_t M = P.M;
-    const int t = threadIdx.x;
-    const int64_t j0 = (int64_t)blockIdx.x * kRsTTargets;
-    const int nT = (int)min((int64_t)kRsTTargets, M - j0);
-    const int b = (int)(j0 / kRsTargets);                        // the forward block holding these outputs
-    const double xa = P.x[j0], span = P.x[j0 + nT - 1] - xa;
-    const rs::Grid G = rs::grid_of(span, R.delta);
-    for (int iv = t; iv < R.nint; iv += blockDim.x) rs::interval_on_grid(__ldg(R.mid + iv), __ldg(R.ih + iv), G, sIv + 4 * iv);
-    double* out = sOut + t;
-    for (int m = 0; m < R.nm; m++) out[(size_t)m * kRsTTargets] = 0.0;
-    const bool valid = t < nT;
-    const int64_t j = j0 + (valid ? t : 0);
-    const double xj = P.x[j];
-    float hj, lj;
-    rs::grid_split(xj - xa, G, hj, lj);
-    int64_t lbj = j;
-    if (j > 0 && P.x[j - 1] == xj) {
-        int64_t lo = 0;
-        while (lo < lbj) {
-            const int64_t mid = (lo + lbj) >> 1;
-            if (P.x[mid] < xj) lo = mid + 1;
-            else lbj = mid;
-        }
-    }
-    const int nbl = __ldg(R.nb_lo + j), nbc = __ldg(R.nb_cnt + j);
-    // the forward block's window holds every input within delta of these outputs
-    const int wlo = __ldg(R.blk_win + 4 * b), inlo = __ldg(R.blk_win + 4 * b + 1);
-    const int inhi = __ldg(R.blk_win + 4 * b + 2), whi = __ldg(R.blk_win + 4 * b + 3);
-    const int nL = max(0, inhi - wlo), total = nL + max(0, whi - inlo);
-    const float cscale = R.cell_scale;
-    __syncthreads();
-    rs::Track trL, trR;
-    rs::track_to(sIv, 0, hj, lj, trL);
-    rs::track_to(sIv, 0, -hj, -lj, trR);
-    int cur = -1;
-    RsMoments F{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int base = 0; base < total; base += kRsChunk) {
-        const int grp = base & (kRsTTargets - 1);                // the chunk's place in its group of 4
-        if (grp == 0) {
-            __syncthreads();
-            const int v = base + t;
-            int lohi = 1, e = 0;
-            float h = 0.f, l = 0.f;
-            if (v < total) {
-                const bool left = v < nL;
-                e = left ? wlo + v : inlo + (v - nL);
-                const double xr = rs_xext(P, e) - xa;
-                rs::grid_split(xr, G, h, l);
-                lohi = rs::source_range(xr, left, span, R.delta, P.dt, R.bp2, R.cell, cscale, R.nint);
+// The contraction of a slab's moments with the coefficients, a warp per 16 outputs: A = moments (16
+// outputs x 16 intervals, one power), B = coefficients (16 intervals x 8 m).  A lane holds the moments
+// of its 2 outputs and 4 intervals of a step, scales them by the coefficients' units and one power
+// of two per output and step (the largest of the step's moments), and cuts them into four slices of 11
+// bits (density_slices) in place as its part of A.  Products of slices i + j <= 4 of all powers share
+// accumulators, which are whole numbers below 2^24 within a step (16 intervals, 8 powers whose
+// coefficients fall by 10 or more from one to the next) and go into the output's pairs after it;
+// slices that are zero in the whole warp are skipped.  sums: [M][nmp] pairs carried from slab to slab;
+// the last slab adds them to the ring.
+constexpr int kRsUnfoldWarps = 4;
+constexpr int kRsUnfoldTiles = 5;                     // tiles of 8 m at a time (m_max up to 40 in one go)
+__global__ void __launch_bounds__(32 * kRsUnfoldWarps) k_rs_unfold(DevPlan P, RangeDev R, int s0, int s1, int64_t n,
+                                                                  float2* __restrict__ sums, double* __restrict__ sb) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    const int64_t l0 = ((int64_t)blockIdx.x * kRsUnfoldWarps + (threadIdx.x >> 5)) * 16;
+    if (l0 >= P.M) return;
+    const int mtiles = R.nmp >> 3, mt0 = blockIdx.y * kRsUnfoldTiles, mt1 = min(mtiles, mt0 + kRsUnfoldTiles);
+    const int64_t row[2] = {min(l0 + g, P.M - 1), min(l0 + g + 8, P.M - 1)};
+    float2 out[kRsUnfoldTiles][4];                    // (row c >> 1, m = 8 mt + 2 q + (c & 1) + 1)
+#pragma unroll
+    for (int mt = 0; mt < kRsUnfoldTiles; mt++)
+#pragma unroll
+        for (int c = 0; c < 4; c++)
+            out[mt][c] = s0 > 0 && mt0 + mt < mt1 ? sums[row[c >> 1] * R.nmp + 8 * (mt0 + mt) + 2 * q + (c & 1)]
+                                                  : make_float2(0.f, 0.f);
+    for (int i0 = s0; i0 < s1; i0 += 16) {
+        // first m of the step's intervals (all later ones are met)
+        const int m0 = __reduce_min_sync(0xffffffffu, __ldg(R.mr + 2 * min(i0 + (lane & 15), R.nint - 1)));
+        if (8 * mt1 < m0) continue;
+        // the lane's moments times 2^30 and the coefficients' units: element (w, u): output row[w],
+        // interval i0 + 2q + (u & 1) + 8 (u >> 1)
+        float hi[2][4][kRsPowers], lo[2][4][2];
+        float mx[2] = {0.f, 0.f};
+#pragma unroll
+        for (int w = 0; w < 2; w++)
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int iv = i0 + 2 * q + (u & 1) + 8 * (u >> 1);
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a, c = a;
+                if (iv < s1) {
+                    const float4* rec = (const float4*)(R.evec + ((size_t)row[w] * R.slab + (iv - s0)) * kRsRecord);
+                    a = __ldg(rec);
+                    b = __ldg(rec + 1);
+                    c = __ldg(rec + 2);
+                }
+                const float4* sc = (const float4*)(R.fold_scale + (size_t)iv * kRsPowers);
+                const float4 s03 = __ldg(sc), s47 = __ldg(sc + 1);
+                const float f[kRsPowers] = {a.x, a.z, b.x, b.y, b.z, b.w, c.x, c.y};
+                const float s[kRsPowers] = {s03.x, s03.y, s03.z, s03.w, s47.x, s47.y, s47.z, s47.w};
+#pragma unroll
+                for (int r = 0; r < kRsPowers; r++) {
+                    hi[w][u][r] = __fmul_rn(f[r], __fmul_rn(s[r], 0x1p30f));
+                    mx[w] = __uint_as_float(max(__float_as_uint(mx[w]), __float_as_uint(hi[w][u][r]) & 0x7fffffffu));
+                }
+                lo[w][u][0] = __fmul_rn(a.y, __fmul_rn(s[0], 0x1p30f));
+                lo[w][u][1] = __fmul_rn(a.w, __fmul_rn(s[1], 0x1p30f));
             }
-            sMeta[t] = make_float4(h, l, __int_as_float(e), __int_as_float(lohi));
+        float inv[2], unit[2];
+#pragma unroll
+        for (int w = 0; w < 2; w++) {
+            unsigned m = __float_as_uint(mx[w]);
+            m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+            m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+            const int E = rs::slice_exponent(m);
+            // units of 2^(E-9): 512 x 1024 x 16 intervals = 2^23, and the higher powers' tenth of it
+            inv[w] = __uint_as_float((unsigned)(127 + 9 - E) << 23);
+            unit[w] = m < 0x7f800000u ? __uint_as_float((unsigned)(127 + E - 9) << 23) : __uint_as_float(0x7fc00000u);
         }
-        __syncthreads();
-        if (t < kRsChunk) {
-            const int v = base + t;
-            float2 cb = make_float2(0.f, 0.f);
-            if (v < total) {
-                const double c = cbar[rs_spring(v < nL ? wlo + v : inlo + (v - nL), M)];
-                const float hi = (float)c;
-                cb = make_float2(hi, (float)(c - (double)hi));
+        float acc[kRsUnfoldTiles][5][4] = {};
+        auto power = [&](auto rc) {
+            constexpr int r = decltype(rc)::value, first = kRsFirstSlice[r], count = kRsSlicesOf[r];
+            unsigned a[kRsSlices][4];
+            unsigned any[kRsSlices] = {0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int w = 0; w < 2; w++) {
+                float sl[4][kRsSlices];
+#pragma unroll
+                for (int u = 0; u < 4; u++) rs::density_slices(hi[w][u][r], r < 2 ? lo[w][u][r & 1] : 0.f, inv[w], sl[u]);
+#pragma unroll
+                for (int i = 0; i < kRsSlices; i++) {
+                    const __half2 p0 = __floats2half2_rn(sl[0][i], sl[1][i]), p1 = __floats2half2_rn(sl[2][i], sl[3][i]);
+                    a[i][w] = __half_as_ushort(p0.x) | (unsigned)__half_as_ushort(p0.y) << 16;
+                    a[i][w + 2] = __half_as_ushort(p1.x) | (unsigned)__half_as_ushort(p1.y) << 16;
+                    any[i] |= (a[i][w] | a[i][w + 2]) & 0x7fff7fffu;
+                }
             }
-            sC[t] = cb;
+            bool use[kRsSlices];
+#pragma unroll
+            for (int i = 0; i < kRsSlices; i++) use[i] = __any_sync(0xffffffffu, any[i] != 0u);
+            const uint2* tab = (const uint2*)R.unfold + (((size_t)first * R.nis + (i0 >> 4)) * R.nmp + 8 * mt0) * 4 + lane;
+            const size_t stride = (size_t)R.nis * R.nmp * 4;
+#pragma unroll
+            for (int mt = 0; mt < kRsUnfoldTiles; mt++) {
+                if (mt0 + mt < mt1 && 8 * (mt0 + mt + 1) >= m0) {
+                    uint2 b[count];
+#pragma unroll
+                    for (int jj = 0; jj < count; jj++) b[jj] = __ldg(tab + jj * stride + 32 * mt);
+#pragma unroll
+                    for (int i = 0; i < kRsSlices; i++) {
+                        if (use[i]) {
+#pragma unroll
+                            for (int jj = 0; jj < count; jj++)
+                                if (i + jj <= 4) rs_mma(acc[mt][i + jj], a[i], b[jj]);
+                        }
+                    }
+                }
+            }
+        };
+        power(std::integral_constant<int, 0>{});
+        power(std::integral_constant<int, 1>{});
+        power(std::integral_constant<int, 2>{});
+        power(std::integral_constant<int, 3>{});
+        power(std::integral_constant<int, 4>{});
+        power(std::integral_constant<int, 5>{});
+        power(std::integral_constant<int, 6>{});
+        power(std::integral_constant<int, 7>{});
+#pragma unroll
+        for (int mt = 0; mt < kRsUnfoldTiles; mt++) {
+            if (mt0 + mt >= mt1 || 8 * (mt0 + mt + 1) < m0) continue;
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                const float(&v)[5][4] = acc[mt];
+                const float sc = unit[c >> 1];
+                float s, e;
+                rs::two_sum(v[0][c], __fmul_rn(v[1][c], 0x1p-11f), s, e);
+                const float t = __fmaf_rn(__fmaf_rn(v[4][c], 0x1p-11f, v[3][c]), 0x1p-11f, v[2][c]);
+                rs::acc_add(out[mt][c].x, out[mt][c].y, __fmul_rn(s, sc), __fmul_rn(__fmaf_rn(t, 0x1p-22f, e), sc));
+            }
         }
-        __syncthreads();
-        if (valid) {
-            const int kend = min(kRsChunk, total - base), kL = min(kend, max(0, nL - base));
-            const float4* meta = sMeta + grp;
-            rs_pairs_T<-1>(R, meta, sC, sIv, cscale, 0, kL, (int)lbj, nbl, nbc, hj, lj, trL, cur, F, out);
-            rs_pairs_T<1>(R, meta, sC, sIv, cscale, kL, kend, (int)lbj, nbl, nbc, -hj, -lj, trR, cur, F, out);
-        }
-        __syncthreads();
     }
-    if (!valid) return;
-    if (cur >= 0) rs_flush(R, cur, F, out);
-    for (int m = 1; m < R.nm; m++) {
-        const double v = out[(size_t)m * kRsTTargets];
-        if (v != 0.0) {
-            int64_t q = (n + 1 - m) % P.ring;
-            if (q < 0) q += P.ring;
-            sb[q * M + j] += v;
+#pragma unroll
+    for (int mt = 0; mt < kRsUnfoldTiles; mt++) {
+        if (mt0 + mt >= mt1) continue;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            const int64_t l = l0 + g + 8 * (c >> 1);
+            const int m = 8 * (mt0 + mt) + 2 * q + (c & 1) + 1;
+            if (l >= P.M) continue;
+            if (s1 < R.nint) {
+                sums[l * R.nmp + m - 1] = out[mt][c];
+            } else if (m < R.nm) {
+                const double v = ((double)out[mt][c].x + (double)out[mt][c].y) * 0x1p-30;
+                if (v != 0.0) {
+                    int64_t slot = (n + 1 - m) % P.ring;
+                    if (slot < 0) slot += P.ring;
+                    sb[slot * P.M + l] += v;
+                }
+            }
         }
     }
 }

@@ -31,6 +31,11 @@ int main() {
     if (build_host_plan(x, b, 2, 0, dt, 10, tol, p, 0.5, 0, 0, 32, 0, 0, 4096, 1ll << 30, hp, err, true)) return 2;
     const RangeTables& rt = hp.rt;
     const int nm = rt.nm;
+    // the transposed sum's table holds the same slices
+    for (int sl = 0; sl < kRsAllSlices; sl++)
+        for (int iv = 0; iv < rt.nint; iv++)
+            for (int m = 1; m < nm; m++)
+                if (rt.fold[fold_index(sl, m, iv, rt.nk, rt.nivp)] != rt.unfold[unfold_index(sl, m, iv, rt.nis, rt.nmp)]) return 3;
     std::mt19937_64 rng(7);
     std::uniform_real_distribution<double> U(-1.0, 1.0);
     double maxq = 0.0, worst = 0.0, most = 0.0;
