@@ -62,7 +62,8 @@ __global__ void k_rs_local(DevPlan P, RangeDev R);
 size_t rs_local_smem(int nint, int nm);
 __global__ void k_rs_slices(DevPlan P, RangeDev R);
 __global__ void k_rs_fold(DevPlan P, RangeDev R, int s0);
-__global__ void k_rs_pairs(DevPlan P, RangeDev R, int s0, int s1);
+__global__ void k_rs_pairs(DevPlan P, RangeDev R, int s0);
+size_t rs_pair_smem(int part, int fine_span);
 __global__ void k_rs_moments(DevPlan P, RangeDev R, int s0, int s1, const double* cbar);
 __global__ void k_rs_unfold(DevPlan P, RangeDev R, int s0, int s1, int64_t n, float2* sums, double* sb);
 __global__ void k_rs_adj_init(DevPlan P, RangeDev R, double* slot_vals, double* rhs);
@@ -318,17 +319,31 @@ int fold_tables(wave1d_plan_t p) {
     rd.fold_scale = f32;
     if ((rc = dalloc(p, &rd.slices, (size_t)P.M * kRsSlices * rt.nk * 16))) return rc;
     if ((rc = dalloc(p, &rd.slice_scale, (size_t)P.M))) return rc;
-    // e-vectors of a slab of intervals at a time: 8 KB a spring (some 170 intervals) up to 2 GiB,
-    // never more than an eighth of the memory that is free, so that many plans fit beside one
-    // another; the results do not depend on the slab
+    if ((rc = upload(p, rt.fine, &h16))) return rc;
+    rd.fine = h16;
+    rd.fine_span = rt.fine_span;
+    rd.fine_scale = (float)(kRsFineCells / P.delta);
+    // parts of the pair kernel: intervals that hold about 160 sources to a side on average (a warp's 32
+    // targets start and end up to 32 sources apart, which it waits for), 64 to 160 of them: a million
+    // clustered springs 80.7 ms per step with parts of 16, 74.5 of 32, 72.6 of 64; 1e5 uniform springs
+    // 3.46 ms with parts of 80, 3.33 of 160
+    const double side = std::max(1.0, 0.5 * (double)p->hp.range_pairs / (double)P.M);
+    const int padded = (rt.nint + 15) / 16 * 16;
+    rd.part = std::min(padded, std::max(64, std::min(160, (int)std::ceil(rt.nint * 160.0 / side / 16.0) * 16)));
+    // e-vectors of a slab of intervals at a time: 16 KB a spring (some 340 intervals; 8 KB below 16384
+    // springs, whose plans stay smaller than one with stored weights) up to 4 GiB, never more than an
+    // eighth of the memory that is free, so that many plans fit beside one another; the results do not
+    // depend on the slab (unless it has to be smaller than a part)
     size_t free_b = 0, all_b = 0;
     if (cudaMemGetInfo(&free_b, &all_b) != cudaSuccess) return fail(WAVE1D_ECUDA, "cudaMemGetInfo");
     const size_t per_iv = (size_t)P.M * kRsRecord * sizeof(float);
-    const size_t want = std::min({(size_t)8192 * P.M, (size_t)2 << 30, free_b / 8});
-    rd.slab = (int)std::min<size_t>((size_t)((rt.nint + 15) / 16) * 16, std::max<size_t>(16, want / per_iv / 16 * 16));
+    const size_t want = std::min({(size_t)(P.M < 16384 ? 8192 : 16384) * P.M, (size_t)4 << 30, free_b / 8});
+    const int most_iv = std::max(16, (int)std::min<size_t>((size_t)padded, want / per_iv / 16 * 16));
+    rd.part = std::min(rd.part, most_iv);
+    rd.slab = most_iv / rd.part * rd.part;
+    rd.nparts = (rt.nint + rd.part - 1) / rd.part;
     if ((rc = dalloc(p, &rd.evec, (size_t)P.M * rd.slab * kRsRecord))) return rc;
-    if ((rc = dalloc(p, &rd.cursor, (size_t)2 * P.M))) return rc;
-    if ((rc = dalloc(p, &rd.csum, (size_t)4 * P.M))) return rc;
+    if ((rc = dalloc(p, &rd.csum, (size_t)4 * rd.nparts * P.M))) return rc;
     p->rs_slice_smem = (size_t)(rt.nm - 1) * 64 * sizeof(float2);
     p->rs_fold_smem = rs_fold_smem(rt.nk);
     // all a block may have, for every plan: the attribute belongs to the kernel, not the plan
@@ -406,7 +421,8 @@ int enqueue_step(wave1d_plan_t p, int64_t n, const double* g_ext, double* sig_hi
             const int s1 = std::min(r.nint, s0 + r.slab), tiles = (s1 - s0 + 7) / 8;
             const unsigned gy = (unsigned)std::max(1, std::min(tiles / 2, (int)((6u * p->sms + gx - 1) / gx)));
             k_rs_fold<<<dim3(gx, gy), T, p->rs_fold_smem, s>>>(d, r, s0);
-            k_rs_pairs<<<dim3(blocks(P.M, kRsPairTargets), 2), kRsPairTargets, (size_t)16 * (s1 - s0), s>>>(d, r, s0, s1);
+            k_rs_pairs<<<dim3(blocks(P.M, kRsPairTargets), 2, (unsigned)((s1 - s0 + r.part - 1) / r.part)), kRsPairTargets,
+                         rs_pair_smem(r.part, r.fine_span), s>>>(d, r, s0);
         }
     } else {
         k_local_items<<<local_grid(p), T, 0, s>>>(d);
@@ -1453,7 +1469,7 @@ struct Reverse {
                 for (int s0 = 0; s0 < rd.nint; s0 += rd.slab) {
                     const int s1 = std::min(rd.nint, s0 + rd.slab);
                     CK(cudaMemsetAsync(rd.evec, 0, (size_t)M * rd.slab * kRsRecord * sizeof(float), s));
-                    k_rs_moments<<<gp, kRsPairTargets, (size_t)16 * (s1 - s0), s>>>(d, rd, s0, s1, cbar);
+                    k_rs_moments<<<gp, kRsPairTargets, rs_pair_smem(s1 - s0, rd.fine_span), s>>>(d, rd, s0, s1, cbar);
                     k_rs_unfold<<<dim3(blocks_for(M, 64, INT32_MAX), (unsigned)(rd.nmp / 8 + 4) / 5), 128, 0, s>>>(d, rd, s0, s1, n,
                                                                                                           usum, sb);
                 }

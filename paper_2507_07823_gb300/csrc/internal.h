@@ -88,6 +88,8 @@ struct RangeTables {
     std::vector<float> fold_scale;     // [nivp][8]: 2^(e - 10)
     int fold_shift = 0;                // the density slices' units are 2^shift larger, so that
                                        //   1024 sum_m |s_0| stays below 2^(24 + shift) (long windows)
+    std::vector<uint16_t> fine;        // kRsFineCells: interval of the left end of each cell of [0, delta)
+    int fine_span = 0;                 // breakpoints in one of those cells at most
     int nis = 0, nmp = 0;              // steps of 16 intervals, m = 1 .. nmp (a multiple of 8)
     std::vector<uint16_t> unfold;      // the same s_j as operands of the transposed sum (unfold_index)
     std::vector<int32_t> cell;         // kRsCells: interval of the left end of each cell of [0, delta)
@@ -120,6 +122,7 @@ void local_weights_exact(const Params& P, const std::vector<double>& d, std::vec
 // targets per block of the range-mode local sum (one per thread); cells of the distance lookup table
 constexpr int kRsTargets = 256;
 constexpr int kRsPairTargets = 128; // targets per block of its pair kernel
+constexpr int kRsFineCells = 8192;
 constexpr int kRsRecord = 12;       // floats of an e-vector record in memory
 constexpr int kRsTTargets = 128;    // outputs per block where a host check walks the transposed sum
 constexpr int kRsCells = 2048;
@@ -355,8 +358,11 @@ struct RangeDev {
     int folded;                 // 1: the local sum comes from k_rs_pairs (csum), 0: from k_rs_local (clocal)
     float* evec;                // [M][slab][kRsRecord]: e-vector records of the slab; the reverse march's
                                 //   moments
-    int32_t* cursor;            // [2][M]: per side, each target's next source
-    float* csum;                // [2][M]: per side, each target's sum so far as a pair
+    int part, nparts;           // intervals whose pairs are summed together (a multiple of 16), their number
+    const uint16_t* fine;       // RangeTables::fine
+    int fine_span;
+    float fine_scale;           // kRsFineCells / delta
+    float* csum;                // [nparts][2][M]: per part and side, each target's sum as a pair
     const int32_t* blk_win;     // [block][4] (see HostPlan::blk_win)
     const int32_t* nb_lo;       // M
     const int32_t* nb_cnt;      // M

@@ -1244,6 +1244,17 @@ static void fold_slices(const std::vector<double>& a, RangeTables& rt) {
             most = std::max(most, sum);
         }
     while (most > std::ldexp(1.0, 14 + rt.fold_shift)) rt.fold_shift++;
+    rt.fine.assign(kRsFineCells, 0);
+    int last = 0;
+    for (int c = 0; c < kRsFineCells; c++) {
+        const double d = rt.bp[n] * c / kRsFineCells;
+        int iv = (int)(std::upper_bound(rt.bp.begin(), rt.bp.end(), d) - rt.bp.begin()) - 1;
+        iv = std::max(0, std::min(n - 1, iv));
+        rt.fine[c] = (uint16_t)iv;
+        if (c > 0) rt.fine_span = std::max(rt.fine_span, iv - last);
+        last = iv;
+    }
+    rt.fine_span = std::max(rt.fine_span, n - 1 - last);
 }
 
 void build_range_tables(const Params& P, RangeTables& rt) {

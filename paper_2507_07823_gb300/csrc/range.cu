@@ -351,13 +351,15 @@ __global__ void __launch_bounds__(32 * kRsFoldWarps, 2) k_rs_fold(DevPlan P, Ran
 }
 
 // ---------------------------------------------------------------------------------------------
-// Pairs of one slab of intervals [s0, s1): one block per kRsPairTargets consecutive targets and side
-// (0: sources strictly left of the target, d = x_j - x_e; 1: at or right of it, d = x_e - x_j).  A
-// target meets its sources in order of distance, so those of the slab are a run that starts where the
-// last slab's ended (cursor); the warp takes the sources one by one for its 32 targets together,
-// whose records lie next to one another (same source, neighbouring intervals).  Positions on the
-// block grid (range.cuh) are staged kRsPosChunk at a time.  Each target's sum is carried from slab to
-// slab as a pair, in the order of its sources, so the result does not depend on the slabs.
+// Pairs whose distances lie in the intervals [p0, p1) of a slab: one block per kRsPairTargets
+// consecutive targets and side (0: sources strictly left of the target, d = x_j - x_e; 1: at or right
+// of it, d = x_e - x_j).  The block stages the positions of the sources that some target meets at such
+// a distance on the block grid (range.cuh), kRsPosChunk at a time; a warp takes its own run of them one
+// by one for its 32 targets together, whose records lie next to one another (same source,
+// neighbouring intervals).  The interval of a pair comes from a table of fine cells of the distance and
+// the next breakpoints, in FP32, and is checked by z, so it depends on the pair alone and each pair falls
+// in one part whatever the parts are.  Two sources are in flight at a time: the chain position - cell -
+// interval - record of a pair is four dependent loads.
 // Which side counts a source is decided by index: e < lb_j (the first spring at x_j's position) is
 // strictly left.  Q_m is continuous across the breakpoints other than dt, so a pair within
 // rounding of one takes either neighbouring interval's polynomial; at dt the spring's FP64 window
@@ -388,21 +390,31 @@ __device__ __forceinline__ int rs_warp_first(int n, F&& pred) {
     return hi;
 }
 
-// One side of one block's pairs of a slab: v.stage(k, e) is called for each of the block's sources as
-// their positions are staged (k: place in the chunk), v.pair(k, e, iv, zh, zl) for each pair of this
-// thread's target in the order of its sources (iv: interval in the slab).
+// an interval on the block grid, from its midpoint as a float pair: (mid_h, mid_l, ih, next breakpoint)
+__device__ __forceinline__ float4 rs_interval(const RangeDev& R, int iv, float g, float ig) {
+    const double mid = __ldg(R.mid + iv);              // exactly a float pair
+    const float mh = __double2float_rn(mid), ml = __double2float_rn(mid - (double)mh);
+    const float h = __fmul_rn(rintf(__fmul_rn(mh, ig)), g);
+    return make_float4(h, __fadd_rn(__fsub_rn(mh, h), ml), __ldg(R.ih + iv),
+                       iv + 1 < R.nint ? __ldg(R.bp2 + 2 * (iv + 1)) : __uint_as_float(0x7f800000u));
+}
+
+// One side of one block's pairs of the intervals [p0, p1): v.stage(k, e) is called for each of the
+// block's sources as their positions are staged (k: place in the chunk), v.pair(u, k, e, iv, zh, zl)
+// for each pair of this thread's target in the order of its sources (u: the source's parity).
 template <int S, typename Visitor>
-__device__ __forceinline__ void rs_pair_block(const DevPlan& P, const RangeDev& R, int s0, int s1, float* sIv, float2* sPos,
+__device__ __forceinline__ void rs_pair_block(const DevPlan& P, const RangeDev& R, int p0, int p1, float4* sIv, float2* sPos,
                                               int* sRed, Visitor& v) {
-    constexpr int side = S > 0 ? 1 : 0;
     const int64_t M = P.M;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int64_t j0 = (int64_t)blockIdx.x * kRsPairTargets;
     const int nT = (int)min((int64_t)kRsPairTargets, M - j0);
     const double xa = P.x[j0], xb = P.x[j0 + nT - 1];
     const rs::Grid G = rs::grid_of(xb - xa, R.delta);
-    for (int iv = s0 + t; iv < s1; iv += blockDim.x)
-        rs::interval_on_grid(__ldg(R.mid + iv), __ldg(R.ih + iv), G, sIv + 4 * (iv - s0));
+    const float gf = (float)G.g, igf = (float)G.ig;
+    // the part's intervals and those a pair of it may be looked up as first
+    const int v0 = max(0, p0 - R.fine_span - 2), v1 = min(R.nint, p1 + 2);
+    for (int iv = v0 + t; iv < v1; iv += blockDim.x) sIv[iv - v0] = rs_interval(R, iv, gf, igf);
     const bool valid = t < nT;
     const int64_t j = j0 + (valid ? t : nT - 1);
     const double xj = P.x[j];
@@ -413,140 +425,146 @@ __device__ __forceinline__ void rs_pair_block(const DevPlan& P, const RangeDev& 
         bl = -bl;
     }
     const int nbl = __ldg(R.nb_lo + j), nbc = __ldg(R.nb_cnt + j);
-    int cur;
-    if (s0 == 0) {
-        // lb_j: the first spring at x_j's position (sources below it are strictly left of x_j)
-        int64_t lbj = j;
-        if (j > 0 && P.x[j - 1] == xj) {
-            int64_t lo = 0;
-            while (lo < lbj) {
-                const int64_t mid = (lo + lbj) >> 1;
-                if (P.x[mid] < xj) lo = mid + 1;
-                else lbj = mid;
-            }
+    // lb_j: the first spring at x_j's position (sources below it are strictly left of x_j)
+    int64_t lbj = j;
+    if (j > 0 && P.x[j - 1] == xj) {
+        int64_t lo = 0;
+        while (lo < lbj) {
+            const int64_t mid = (lo + lbj) >> 1;
+            if (P.x[mid] < xj) lo = mid + 1;
+            else lbj = mid;
         }
-        cur = (int)(S > 0 ? lbj : lbj - 1);
-    } else {
-        cur = R.cursor[side * M + j];
     }
-    // the block's sources of the slab: from the nearest cursor (k = 0) to the first one beyond the
-    // slab's far end of every target, inside the window of its 256-target block
+    const int lb = (int)lbj;
+    // the block's sources in the order of their distance: from the first one that may lie at the
+    // part's near end from some target to the first one beyond its far end from all of them, inside
+    // the window of its 256-target block
     const int* win = R.blk_win + 4 * (j0 / kRsTargets);
-    const int e0 = S > 0 ? __reduce_min_sync(0xffffffffu, cur) : __reduce_max_sync(0xffffffffu, cur);
-    if (lane == 0) sRed[warp] = e0;
-    __syncthreads();
-    int start = sRed[0];
-#pragma unroll
-    for (int w = 1; w < kRsPairTargets / 32; w++) start = S > 0 ? min(start, sRed[w]) : max(start, sRed[w]);
-    const int bound = max(0, S > 0 ? __ldg(win + 3) - start : start - __ldg(win) + 1);
-    const double reach = __ldg(R.bp + s1) + R.delta * rs::kRangeMargin;
-    if (warp == 0) {
-        const int c = rs_warp_first(bound, [&](int k) {
-            const double x = rs_xext(P, start + S * k);
-            return !((S > 0 ? x - xb : xa - x) < reach);
+    const int top = S > 0 ? __ldg(win) : (int)(j0 + nT - 1), all = max(0, S > 0 ? __ldg(win + 3) - top : top - __ldg(win) + 1);
+    const double marg = 2e-6 * R.delta + 8.0 * G.g, d0 = __ldg(R.bp + p0) - marg, d1 = __ldg(R.bp + p1) + marg;
+    if (warp < 2) {
+        const int c = rs_warp_first(all, [&](int k) {
+            const double x = rs_xext(P, top + S * k);
+            return warp == 0 ? (S > 0 ? x - xa : xb - x) >= d0 : !((S > 0 ? x - xb : xa - x) < d1);
         });
-        if (lane == 0) sRed[kRsPairTargets / 32] = c;
+        if (lane == 0) sRed[warp] = c;
     }
     __syncthreads();
-    const int count = sRed[kRsPairTargets / 32];
-    int kcur = valid ? S * (cur - start) : count;         // the lane's next source
-    bool done = !valid;
-    const bool at_dt = s0 <= R.iv_dt && R.iv_dt <= s1;    // the slab touches the breakpoint dt
-    rs::Track tr;
-    rs::track_to(sIv, 0, bh, bl, tr);
-    const int ns = s1 - s0, ivd = R.iv_dt - s0;
+    const int start = top + S * sRed[0], count = sRed[1] - sRed[0];
+    const bool at_dt = p0 <= R.iv_dt && R.iv_dt <= p1;    // the part touches the breakpoint dt
+    const float bfar = __shfl_sync(0xffffffffu, bh, S > 0 ? 0 : 31), bnear = __shfl_sync(0xffffffffu, bh, S > 0 ? 31 : 0);
+    const float df0 = (float)d0, df1 = (float)d1;
+    const int ns = v1 - v0, ivd = R.iv_dt - v0;
     for (int base = 0; base < count; base += kRsPosChunk) {
-        const int lim = min(count, base + kRsPosChunk);
+        const int lim = min(count - base, kRsPosChunk), e0 = start + S * base;
         if (base > 0) __syncthreads();
-        for (int k = base + t; k < lim; k += blockDim.x) {
+        for (int k = t; k < lim; k += blockDim.x) {
             float h, l;
-            rs::grid_split(rs_xext(P, start + S * k) - xa, G, h, l);
-            sPos[k - base] = make_float2(h, l);
-            v.stage(k - base, start + S * k);
+            rs::grid_split(rs_xext(P, e0 + S * k) - xa, G, h, l);
+            sPos[k] = make_float2(h, l);
+            v.stage(k, e0 + S * k);
         }
         __syncthreads();
-        int k = max(base, __reduce_min_sync(0xffffffffu, done ? count : kcur));
-        for (; k < lim; k++) {
-            const float2 ps = sPos[k - base];
-            const int e = start + S * k;
-            if (!done && k >= kcur) {
-                float zh, zl;
-                rs::z_of<S>(tr, ps.x, ps.y, zh, zl);
-                bool beyond = false;
-                if (zh > rs::kZTol) {
-                    if (zh > 4.f) {
-                        // far off: the interval of the cell of the distance, if that is farther
-                        const float d = __fadd_rn(S < 0 ? __fsub_rn(bh, ps.x) : __fadd_rn(bh, ps.x),
-                                                  S < 0 ? __fsub_rn(bl, ps.y) : __fadd_rn(bl, ps.y));
-                        const int c = min(kRsCells - 1, max(0, (int)__fmul_rn(d, R.cell_scale)));
-                        const int iv = min(__ldg(R.cell + c) - s0, ns - 1);
-                        if (iv > tr.iv) {
-                            rs::track_to(sIv, iv, bh, bl, tr);
-                            rs::z_of<S>(tr, ps.x, ps.y, zh, zl);
-                        }
-                    }
-                    while (zh > rs::kZTol) {
-                        if (tr.iv + 1 >= ns) {
-                            beyond = true;
-                            break;
-                        }
-                        rs::track_to(sIv, tr.iv + 1, bh, bl, tr);
-                        rs::z_of<S>(tr, ps.x, ps.y, zh, zl);
+        // the warp's run of the chunk
+        const int klo = rs_warp_first(lim, [&](int k) { return (S < 0 ? bfar - sPos[k].x : bfar + sPos[k].x) >= df0; });
+        const int khi = rs_warp_first(lim, [&](int k) { return (S < 0 ? bnear - sPos[k].x : bnear + sPos[k].x) >= df1; });
+        for (int k0 = klo; k0 < khi; k0 += 2) {
+            float zh[2], zl[2];
+            int iv[2];
+            bool in[2];
+#pragma unroll
+            for (int u = 0; u < 2; u++) {
+                const int k = k0 + u, e = e0 + S * k;
+                const float2 ps = sPos[min(k, lim - 1)];
+                // distance = dh + dl (dh exact on the block grid)
+                const float dh = S < 0 ? __fsub_rn(bh, ps.x) : __fadd_rn(bh, ps.x);
+                const float dl = S < 0 ? __fsub_rn(bl, ps.y) : __fadd_rn(bl, ps.y);
+                const float d = __fadd_rn(dh, dl);
+                const int c = min(kRsFineCells - 1, max(0, (int)__fmul_rn(d, R.fine_scale)));
+                int i = (int)__ldg(R.fine + c) - v0;
+                bool ok = valid && k < khi && (S > 0 ? e >= lb : e < lb) && i >= 0 && i < ns;
+                float4 q = sIv[ok ? i : 0];
+                while (ok && d >= q.w) {
+                    if (++i < ns) q = sIv[i];
+                    else ok = false;
+                }
+                auto place = [&]() {
+                    const float A = __fsub_rn(dh, q.x), B = __fsub_rn(dl, q.y);
+                    const float p = __fmul_rn(A, q.z);
+                    rs::two_sum(p, __fmaf_rn(B, q.z, __fmaf_rn(A, q.z, -p)), zh[u], zl[u]);
+                };
+                place();
+                // within FP32 rounding of a breakpoint, or past the last one: one way only, so it ends
+                for (int dir = 0; ok && fabsf(zh[u]) > rs::kZTol;) {
+                    const int want = zh[u] > 0.f ? 1 : -1;
+                    if (dir != 0 && want != dir) break;
+                    dir = want;
+                    i += want;
+                    ok = i >= 0 && i < ns;
+                    if (ok) {
+                        q = sIv[i];
+                        place();
                     }
                 }
                 if (at_dt) {
                     const bool near = (unsigned)(e - nbl) < (unsigned)nbc;
-                    int to = -1;
-                    if (near && (beyond || tr.iv >= ivd) && ivd - 1 < ns) to = max(0, ivd - 1);
-                    else if (!near && !beyond && tr.iv < ivd) to = ivd;
-                    if (to >= ns) {
-                        beyond = true;
-                    } else if (to >= 0) {
-                        beyond = false;
-                        rs::track_to(sIv, to, bh, bl, tr);
-                        rs::z_of<S>(tr, ps.x, ps.y, zh, zl);
+                    if (ok && near != (i < ivd)) {
+                        i = near ? ivd - 1 : ivd;
+                        ok = i >= 0 && i < ns;
+                        if (ok) {
+                            q = sIv[i];
+                            place();
+                        }
                     }
                 }
-                if (beyond) {
-                    done = true;
-                    kcur = k;
-                } else {
-                    v.pair(k - base, e, tr.iv, zh, zl);
-                    kcur = k + 1;
-                }
+                iv[u] = i + v0;
+                in[u] = ok && iv[u] >= p0 && iv[u] < p1;
             }
-            if (__all_sync(0xffffffffu, done)) break;
+            v.pairs(in, k0, e0 + S * k0, S, iv, zh, zl);
         }
     }
-    if (valid && s1 < R.nint) R.cursor[side * M + j] = start + S * kcur;
     __syncthreads();                                      // the staged positions are free again
 }
 
-// the local sum of one side: each target's polynomials into its pair, carried from slab to slab
+// the local sum of one side and part: each target's polynomials, two sources at a time into two pairs
 struct RsSum {
     const DevPlan& P;
     const RangeDev& R;
-    float ah, al;
+    int s0;                   // the slab's first interval
+    float ah[2], al[2];
     __device__ __forceinline__ void stage(int, int) {}
-    __device__ __forceinline__ void pair(int, int e, int iv, float zh, float zl) {
-        const float4* rec = (const float4*)(R.evec + ((size_t)rs_spring(e, P.M) * R.slab + iv) * kRsRecord);
-        const float4 r0 = __ldg(rec), r1 = __ldg(rec + 1), r2 = __ldg(rec + 2);
-        rs_eval(r0, r1, r2, zh, zl, ah, al);
+    __device__ __forceinline__ void pairs(const bool (&in)[2], int, int e, int step, const int (&iv)[2], const float (&zh)[2],
+                                          const float (&zl)[2]) {
+        float4 r[2][3];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const float4* rec = (const float4*)(R.evec + ((size_t)rs_spring(e + u * step, P.M) * R.slab + (iv[u] - s0)) * kRsRecord);
+            if (in[u]) {
+#pragma unroll
+                for (int i = 0; i < 3; i++) r[u][i] = __ldg(rec + i);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; u++)
+            if (in[u]) rs_eval(r[u][0], r[u][1], r[u][2], zh[u], zl[u], ah[u], al[u]);
     }
 };
 
-__global__ void __launch_bounds__(kRsPairTargets, 8) k_rs_pairs(DevPlan P, RangeDev R, int s0, int s1) {
-    extern __shared__ __align__(16) float pair_sm[];
+__global__ void __launch_bounds__(kRsPairTargets, 6) k_rs_pairs(DevPlan P, RangeDev R, int s0) {
+    extern __shared__ __align__(16) float4 pair_sm[];
     __shared__ float2 sPos[kRsPosChunk];
-    __shared__ int sRed[kRsPairTargets / 32 + 1];
+    __shared__ int sRed[2];
+    const int p0 = s0 + blockIdx.z * R.part, p1 = min(R.nint, p0 + R.part);
+    RsSum v{P, R, s0, {0.f, 0.f}, {0.f, 0.f}};
+    if (blockIdx.y == 0) rs_pair_block<-1>(P, R, p0, p1, pair_sm, sPos, sRed, v);
+    else rs_pair_block<1>(P, R, p0, p1, pair_sm, sPos, sRed, v);
+    rs::acc_add(v.ah[0], v.al[0], v.ah[1], v.al[1]);
     const int64_t j = (int64_t)blockIdx.x * kRsPairTargets + threadIdx.x;
-    float2* acc = (float2*)R.csum + blockIdx.y * P.M + j;
-    const float2 a = j < P.M && s0 > 0 ? *acc : make_float2(0.f, 0.f);
-    RsSum v{P, R, a.x, a.y};
-    if (blockIdx.y == 0) rs_pair_block<-1>(P, R, s0, s1, pair_sm, sPos, sRed, v);
-    else rs_pair_block<1>(P, R, s0, s1, pair_sm, sPos, sRed, v);
-    if (j < P.M) *acc = make_float2(v.ah, v.al);
+    if (j < P.M) ((float2*)R.csum)[((size_t)(p0 / R.part) * 2 + blockIdx.y) * P.M + j] = make_float2(v.ah[0], v.al[0]);
 }
+
+// shared memory of a pair block's interval table
+size_t rs_pair_smem(int part, int fine_span) { return (size_t)(part + fine_span + 4) * sizeof(float4); }
 
 // plan time: the terms of the local sum, sum over pairs (j, l) closer than delta of the number of
 // m >= 1 with a non-zero weight on the pair's interval (the multiply-adds sum_m Q_m sigma_l^{n+1-m}
@@ -610,8 +628,13 @@ __global__ void k_rs_solve_init(DevPlan P, RangeDev R) {
         // the two sides of the local sum
         double c;
         if (R.folded) {
-            const float2 cl = ((const float2*)R.csum)[j], cr = ((const float2*)R.csum)[P.M + j];
-            c = ((double)cl.x + (double)cl.y) + ((double)cr.x + (double)cr.y);
+            // the parts and sides of the local sum, in order
+            float h = 0.f, l = 0.f;
+            for (int q = 0; q < 2 * R.nparts; q++) {
+                const float2 a = ((const float2*)R.csum)[(size_t)q * P.M + j];
+                rs::acc_add(h, l, a.x, a.y);
+            }
+            c = (double)h + (double)l;
             P.clocal[j] = c;
         } else {
             c = P.clocal[j];                            // the mixed form's k_rs_local
@@ -792,24 +815,22 @@ struct RsMoments {
     const double* cbar;
     float2* sC;               // cbar of the staged sources as pairs
     float* rec;               // this output's records of the slab
-    bool add;                 // the second side adds to the first one's
+    int s0;                   // the slab's first interval
     int cur;                  // the interval whose moments are held, -1: none
     float f0h, f0l, f1h, f1l, f2, f3, f4, f5, f6, f7;
     __device__ __forceinline__ void clear() { f0h = f0l = f1h = f1l = f2 = f3 = f4 = f5 = f6 = f7 = 0.f; }
     __device__ __forceinline__ void flush() {
         if (cur < 0) return;
         float4* o = (float4*)(rec + (size_t)cur * kRsRecord);
-        if (add) {
-            const float4 a = o[0], b = o[1], c = o[2];
-            rs::acc_add(f0h, f0l, a.x, a.y);
-            rs::acc_add(f1h, f1l, a.z, a.w);
-            f2 = __fadd_rn(f2, b.x);
-            f3 = __fadd_rn(f3, b.y);
-            f4 = __fadd_rn(f4, b.z);
-            f5 = __fadd_rn(f5, b.w);
-            f6 = __fadd_rn(f6, c.x);
-            f7 = __fadd_rn(f7, c.y);
-        }
+        const float4 a = o[0], b = o[1], c = o[2];        // (the records start as zeros)
+        rs::acc_add(f0h, f0l, a.x, a.y);
+        rs::acc_add(f1h, f1l, a.z, a.w);
+        f2 = __fadd_rn(f2, b.x);
+        f3 = __fadd_rn(f3, b.y);
+        f4 = __fadd_rn(f4, b.z);
+        f5 = __fadd_rn(f5, b.w);
+        f6 = __fadd_rn(f6, c.x);
+        f7 = __fadd_rn(f7, c.y);
         o[0] = make_float4(f0h, f0l, f1h, f1l);
         o[1] = make_float4(f2, f3, f4, f5);
         o[2] = make_float4(f6, f7, 0.f, 0.f);
@@ -819,7 +840,13 @@ struct RsMoments {
         const float hi = (float)c;
         sC[k] = make_float2(hi, (float)(c - (double)hi));
     }
-    __device__ __forceinline__ void pair(int k, int, int iv, float zh, float zl) {
+    __device__ __forceinline__ void pairs(const bool (&in)[2], int k, int, int, const int (&iv)[2], const float (&zh)[2],
+                                          const float (&zl)[2]) {
+#pragma unroll
+        for (int u = 0; u < 2; u++)
+            if (in[u]) pair(k + u, iv[u] - s0, zh[u], zl[u]);
+    }
+    __device__ __forceinline__ void pair(int k, int iv, float zh, float zl) {
         if (iv != cur) {
             flush();
             cur = iv;
@@ -846,16 +873,13 @@ struct RsMoments {
 // the moments of a slab, both sides (the records are zero on entry)
 __global__ void __launch_bounds__(kRsPairTargets) k_rs_moments(DevPlan P, RangeDev R, int s0, int s1,
                                                               const double* __restrict__ cbar) {
-    extern __shared__ __align__(16) float pair_sm[];
+    extern __shared__ __align__(16) float4 pair_sm[];
     __shared__ float2 sPos[kRsPosChunk], sC[kRsPosChunk];
-    __shared__ int sRed[kRsPairTargets / 32 + 1];
+    __shared__ int sRed[2];
     const int64_t j = min((int64_t)blockIdx.x * kRsPairTargets + threadIdx.x, P.M - 1);
-    RsMoments v{P, R, cbar, sC, R.evec + (size_t)j * R.slab * kRsRecord, false, -1};
+    RsMoments v{P, R, cbar, sC, R.evec + (size_t)j * R.slab * kRsRecord, s0, -1};
     v.clear();
     rs_pair_block<-1>(P, R, s0, s1, pair_sm, sPos, sRed, v);
-    v.flush();
-    v.cur = -1;
-    v.add = true;
     rs_pair_block<1>(P, R, s0, s1, pair_sm, sPos, sRed, v);
     v.flush();
 }
