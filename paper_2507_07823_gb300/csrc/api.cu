@@ -482,7 +482,7 @@ int enqueue_step(wave1d_plan_t p, int64_t n, const double* g_ext, double* sig_hi
     mark(WAVE1D_STAGE_SOLVE);
     if (fork) cudaStreamWaitEvent(s, p->ev_join, 0);
     if (p->range) {
-        const unsigned rows = blocks(P.M, T), sweeps = (unsigned)std::min<int64_t>(blocks(P.M * 32, T), 16 * (int64_t)p->sms);
+        const unsigned rows = blocks(P.M, T), sweeps = (unsigned)std::min<int64_t>(blocks(P.M, 64), 16 * (int64_t)p->sms);
         k_rs_solve_init<<<rows, T, 0, s>>>(d, p->rd);
         for (int it = 1; it <= kRsMaxIter; it++) k_rs_jacobi<<<sweeps, T, 0, s>>>(d, p->rd, it);
         k_rs_store<<<rows, T, 0, s>>>(d, p->rd);
@@ -1460,7 +1460,7 @@ struct Reverse {
                 k_rs_adj_init<<<gM, 256, 0, s>>>(d, rd, sb + (int64_t)((n + 1) % ring) * M, rrhs);
                 DevPlan dj = d;
                 dj.rhs = rrhs;
-                const unsigned sweeps = (unsigned)std::min<int64_t>(blocks_for(M * 32, 256, INT32_MAX), 16 * (int64_t)p->sms);
+                const unsigned sweeps = (unsigned)std::min<int64_t>(blocks_for(M, 64, INT32_MAX), 16 * (int64_t)p->sms);
                 for (int it = 1; it <= kRsMaxIter; it++) k_rs_jacobi<<<sweeps, 256, 0, s>>>(dj, rd, it);
                 k_rs_adj_post<<<gM, 256, 0, s>>>(d, rd, sig_rows + (n - row0) * M, g ? g + n * M : nullptr,
                                                  want_beta ? gsum : nullptr, grad_g ? grad_g + n * M : nullptr, cbar, uHbar);

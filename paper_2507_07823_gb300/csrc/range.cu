@@ -655,8 +655,12 @@ __global__ void k_rs_solve_init(DevPlan P, RangeDev R) {
     }
 }
 
-// sweep `it` (1 .. kRsMaxIter): iterate it from iterate it - 1, unless sweep it - 1 converged.
-// Warp per spring; the row sum sum_{l != j} S_jl sigma_l in compensated pairs.
+// sweep `it` (1 .. kRsMaxIter): iterate it from iterate it - 1, unless sweep it - 1 converged.  A warp
+// takes kRsRows consecutive springs: each row's sum sum_{l != j} S_jl sigma_l in compensated pairs over
+// the lanes, then one lane per row does the row's FP64 work (the division above all: some 20
+// instructions of 16 cycles of an SM each, whether one lane or 32 take part; with one row at a time it
+// bound the sweep, 120 us at 1e5 springs and 0.9 ms at a million).
+constexpr int kRsRows = 8;
 __global__ void __launch_bounds__(256) k_rs_jacobi(DevPlan P, RangeDev R, int it) {
     if (it >= 2) {
         const double dmax = rs_from_bits(__ldcg(R.stats + 2 * (it - 1)));
@@ -670,44 +674,63 @@ __global__ void __launch_bounds__(256) k_rs_jacobi(DevPlan P, RangeDev R, int it
     double* dst = R.it64[it & 1];
     float* dst2 = R.it2[it & 1];
     double dmax = 0.0, smax = 0.0;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < P.M; j += nw) {
-        const int lo = __ldg(R.nb_lo + j), cnt = __ldg(R.nb_cnt + j);
-        const int64_t off = __ldg(R.nb_off + j);
-        // four entries per lane in flight (their weight and iterate loads issued together), two
-        // accumulators; the row's entries are streamed once per sweep
-        float ah = 0.f, al = 0.f, bh = 0.f, bl = 0.f;
-        int k = lane;
-        for (; k + 96 < cnt; k += 128) {
-            float2 w[4], sv[4];
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5, groups = (P.M + kRsRows - 1) / kRsRows;
+    for (int64_t gr = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; gr < groups; gr += nw) {
+        const int64_t j0 = gr * kRsRows, mine = j0 + lane;
+        const bool own = lane < kRsRows && mine < P.M;
+        // the rows' windows, one per lane, and what their FP64 work reads
+        const int lo_r = own ? __ldg(R.nb_lo + mine) : 0, cnt_r = own ? __ldg(R.nb_cnt + mine) : 0;
+        const int64_t off_r = own ? __ldg(R.nb_off + mine) : 0;
+        const double rhs = own ? __ldcg(P.rhs + mine) : 0.0, diag = own ? R.diag[mine] : 1.0, prev = own ? __ldcg(src + mine) : 0.0;
+        float sh = 0.f, sl = 0.f;
+#pragma unroll 2
+        for (int r = 0; r < kRsRows; r++) {
+            const int lo = __shfl_sync(0xffffffffu, lo_r, r), cnt = __shfl_sync(0xffffffffu, cnt_r, r);
+            const int64_t off = __shfl_sync(0xffffffffu, off_r, r);
+            // four entries per lane in flight (their weight and iterate loads issued together), two
+            // accumulators; the row's entries are streamed once per sweep
+            float ah = 0.f, al = 0.f, bh = 0.f, bl = 0.f;
+            int k = lane;
+            for (; k + 96 < cnt; k += 128) {
+                float2 w[4], sv[4];
 #pragma unroll
-            for (int u = 0; u < 4; u++) w[u] = __ldcs((const float2*)R.nb_w + off + k + 32 * u);
+                for (int u = 0; u < 4; u++) w[u] = __ldcs((const float2*)R.nb_w + off + k + 32 * u);
 #pragma unroll
-            for (int u = 0; u < 4; u++) sv[u] = __ldcg((const float2*)src2 + rs_spring((int64_t)lo + k + 32 * u, P.M));
-            rs::acc_mac(ah, al, w[0].x, w[0].y, sv[0].x, sv[0].y);
-            rs::acc_mac(bh, bl, w[1].x, w[1].y, sv[1].x, sv[1].y);
-            rs::acc_mac(ah, al, w[2].x, w[2].y, sv[2].x, sv[2].y);
-            rs::acc_mac(bh, bl, w[3].x, w[3].y, sv[3].x, sv[3].y);
+                for (int u = 0; u < 4; u++) sv[u] = __ldcg((const float2*)src2 + rs_spring((int64_t)lo + k + 32 * u, P.M));
+                rs::acc_mac(ah, al, w[0].x, w[0].y, sv[0].x, sv[0].y);
+                rs::acc_mac(bh, bl, w[1].x, w[1].y, sv[1].x, sv[1].y);
+                rs::acc_mac(ah, al, w[2].x, w[2].y, sv[2].x, sv[2].y);
+                rs::acc_mac(bh, bl, w[3].x, w[3].y, sv[3].x, sv[3].y);
+            }
+            for (; k < cnt; k += 32) {
+                const float2 w = __ldcs((const float2*)R.nb_w + off + k);
+                const float2 s = __ldcg((const float2*)src2 + rs_spring((int64_t)lo + k, P.M));
+                rs::acc_mac(ah, al, w.x, w.y, s.x, s.y);
+            }
+            rs::acc_add(ah, al, bh, bl);
+            for (int o = 16; o > 0; o >>= 1) {
+                const float oh = __shfl_xor_sync(0xffffffffu, ah, o), ol = __shfl_xor_sync(0xffffffffu, al, o);
+                rs::acc_add(ah, al, oh, ol);
+            }
+            // lane 0's sum (the tree's order differs from lane to lane) goes to the row's lane
+            const float th = __shfl_sync(0xffffffffu, ah, 0), tl = __shfl_sync(0xffffffffu, al, 0);
+            if (lane == r) {
+                sh = th;
+                sl = tl;
+            }
         }
-        for (; k < cnt; k += 32) {
-            const float2 w = __ldcs((const float2*)R.nb_w + off + k);
-            const float2 s = __ldcg((const float2*)src2 + rs_spring((int64_t)lo + k, P.M));
-            rs::acc_mac(ah, al, w.x, w.y, s.x, s.y);
-        }
-        rs::acc_add(ah, al, bh, bl);
-        for (int o = 16; o > 0; o >>= 1) {
-            const float oh = __shfl_xor_sync(0xffffffffu, ah, o), ol = __shfl_xor_sync(0xffffffffu, al, o);
-            rs::acc_add(ah, al, oh, ol);
-        }
-        if (lane == 0) {
-            const double x = (__ldcg(P.rhs + j) - ((double)ah + (double)al)) / R.diag[j];
-            dmax = fmax(dmax, fabs(x - __ldcg(src + j)));
+        if (own) {
+            const double x = (rhs - ((double)sh + (double)sl)) / diag;
+            dmax = fmax(dmax, fabs(x - prev));
             smax = fmax(smax, fabs(x));
-            dst[j] = x;
+            dst[mine] = x;
             const rs::Pair p2 = rs::split(x);
-            dst2[2 * j] = p2.hi;
-            dst2[2 * j + 1] = p2.lo;
+            ((float2*)dst2)[mine] = make_float2(p2.hi, p2.lo);
         }
+    }
+    for (int o = kRsRows / 2; o > 0; o >>= 1) {
+        dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+        smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
     }
     if (lane == 0) {
         red[0][wid] = dmax;
