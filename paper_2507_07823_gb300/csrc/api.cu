@@ -76,6 +76,7 @@ __global__ void k_rs_jacobi(DevPlan P, RangeDev R, int it);
 __global__ void k_rs_store(DevPlan P, RangeDev R);
 __global__ void k_rs_receivers(DevPlan P, RangeDev R);
 __global__ void k_rs_finish(DevPlan P, RangeDev R);
+int rs_receiver_chunks(int64_t window);
 __global__ void k_rs_count_terms(DevPlan P, RangeDev R, unsigned long long* total);
 size_t rs_fold_smem(int nk);
 }  // namespace wave1d
@@ -251,7 +252,7 @@ int upload_receivers(wave1d_plan_t p) {
         p->rd.r_win = i32;
         int64_t most = 1;
         for (int64_t r = 0; r < d.R; r++) most = std::max<int64_t>(most, hp.r_win[2 * r + 1] - hp.r_win[2 * r]);
-        p->rd.rchunks = (int)((most + 255) / 256);
+        p->rd.rchunks = rs_receiver_chunks(most);
         if ((rc = zeros(p, &p->rd.r_part, (size_t)p->rd.rchunks * std::max<int64_t>(1, d.R)))) return rc;
         if ((rc = zeros(p, &d.uHr, (size_t)std::max<int64_t>(1, d.R)))) return rc;
         if ((rc = zeros(p, &d.rec_hist, (size_t)p->chunk * std::max<int64_t>(1, d.R)))) return rc;
@@ -488,7 +489,7 @@ int enqueue_step(wave1d_plan_t p, int64_t n, const double* g_ext, double* sig_hi
         k_rs_store<<<rows, T, 0, s>>>(d, p->rd);
         mark(WAVE1D_STAGE_RECEIVERS);
         if (P.R > 0) k_rs_receivers<<<dim3((unsigned)p->rd.rchunks, (unsigned)P.R), T, 0, s>>>(d, p->rd);
-        k_rs_finish<<<1, 32, 0, s>>>(d, p->rd);
+        k_rs_finish<<<1, 256, 0, s>>>(d, p->rd);
         mark(WAVE1D_NSTAGE);
         CK(cudaGetLastError());
         return WAVE1D_OK;
@@ -1456,7 +1457,7 @@ struct Reverse {
                 // plan without pair lists: receivers, solve and local sum transposed on the
                 // range tables; the solve is the forward Jacobi sweeps on beta-scaled data
                 const RangeDev& rd = p->rd;
-                if (R > 0) k_rs_adj_receivers<<<gM, 256, 0, s>>>(d, rd, n, ub, sb);
+                if (R > 0) k_rs_adj_receivers<<<dim3(gM, 8), 256, 0, s>>>(d, rd, n, ub, sb);
                 k_rs_adj_init<<<gM, 256, 0, s>>>(d, rd, sb + (int64_t)((n + 1) % ring) * M, rrhs);
                 DevPlan dj = d;
                 dj.rhs = rrhs;

@@ -771,26 +771,45 @@ __global__ void k_rs_store(DevPlan P, RangeDev R) {
     }
 }
 
-// receivers' local part (eq. localSol2), block (chunk c of 256 sources, receiver r): every m of
-// the pair's interval, m = 0 with sigma^{n+1} (already stored), FP64; block sums in a fixed order
-__global__ void __launch_bounds__(256) k_rs_receivers(DevPlan P, RangeDev R) {
-    __shared__ double red[8];
+// T_0(z) .. T_7(z); a series is then 7 FMAs (a Clenshaw sum per m would be 15)
+__device__ __forceinline__ void rs_cheb_basis(double z, double (&T)[8]) {
+    T[0] = 1.0;
+    T[1] = z;
+#pragma unroll
+    for (int r = 2; r < 8; r++) T[r] = fma(2.0 * z, T[r - 1], -T[r - 2]);
+}
+__device__ __forceinline__ double rs_cheb_sum(const double* c, const double (&T)[8]) {
+    double v = __ldg(c);
+#pragma unroll
+    for (int r = 1; r < 8; r++) v = fma(__ldg(c + r), T[r], v);
+    return v;
+}
+
+// receivers' local part (eq. localSol2), block (chunk c of kRsRecvChunk sources, receiver r): every m of
+// the pair's interval, m = 0 with sigma^{n+1} (already stored), FP64; block sums in a fixed order.  Four
+// threads share a source, each every fourth m: with one thread each the 25 to 40 series in a row took
+// 73 us whatever the number of receivers.
+constexpr int kRsRecvChunk = 64;
+int rs_receiver_chunks(int64_t window) { return (int)((window + kRsRecvChunk - 1) / kRsRecvChunk); }
+__global__ void __launch_bounds__(4 * kRsRecvChunk) k_rs_receivers(DevPlan P, RangeDev R) {
+    __shared__ double red[kRsRecvChunk / 8];
     const int64_t n = load_step(P);
     const int r = blockIdx.y, c = blockIdx.x;
     const int lo = R.r_win[2 * r], hi = R.r_win[2 * r + 1];
-    const int64_t e = (int64_t)lo + (int64_t)c * blockDim.x + threadIdx.x;
+    const int64_t e = (int64_t)lo + (int64_t)c * kRsRecvChunk + (threadIdx.x & (kRsRecvChunk - 1));
+    const int q = threadIdx.x / kRsRecvChunk;
     double v = 0.0;
     if (e < hi) {
         const int64_t l = rs_spring(e, P.M);
         const double d = fabs(rs_xext(P, e) - P.xr[r]);
         if (d < R.delta) {
             const int iv = rs_locate64(R, d);
-            const double z = (d - __ldg(R.mid + iv)) * (double)__ldg(R.ih + iv);
+            double T[8];
+            rs_cheb_basis((d - __ldg(R.mid + iv)) * (double)__ldg(R.ih + iv), T);
             const int m0 = __ldg(R.mr0 + 2 * iv), m1 = __ldg(R.mr0 + 2 * iv + 1);
-            for (int m = m0; m <= m1; m++) {
-                const double q = rs_cheb(R.cheb + ((size_t)iv * R.nm + m) * 8, z);
-                v = fma(q, __ldcg(P.sig + (int64_t)ring_slot(n + 1 - m, P.ring) * P.M + l), v);
-            }
+            for (int m = m0 + q; m <= m1; m += 4)
+                v = fma(rs_cheb_sum(R.cheb + ((size_t)iv * R.nm + m) * 8, T),
+                        __ldcg(P.sig + (int64_t)ring_slot(n + 1 - m, P.ring) * P.M + l), v);
         }
     }
     v = warp_sum(v);
@@ -803,13 +822,15 @@ __global__ void __launch_bounds__(256) k_rs_receivers(DevPlan P, RangeDev R) {
     }
 }
 
-// u = u_L + u_H at the receivers (chunk partials in order), then the step counter
+// u = u_L + u_H at the receivers (a warp per receiver over its chunks' partials), then the step counter
 __global__ void k_rs_finish(DevPlan P, RangeDev R) {
     const int64_t n = load_step(P);
-    for (int64_t r = threadIdx.x; r < P.R; r += blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t r = threadIdx.x >> 5; r < P.R; r += blockDim.x >> 5) {
         double s = 0.0;
-        for (int c = 0; c < R.rchunks; c++) s += __ldcg(R.r_part + r * R.rchunks + c);
-        P.rec_hist[(n % P.chunk) * P.R + r] = 0.5 * s + __ldcg(P.uHr + r);
+        for (int c = lane; c < R.rchunks; c += 32) s += __ldcg(R.r_part + r * R.rchunks + c);
+        s = warp_sum(s);
+        if (lane == 0) P.rec_hist[(n % P.chunk) * P.R + r] = 0.5 * s + __ldcg(P.uHr + r);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1110,7 +1131,8 @@ __global__ void k_rs_adj_post(DevPlan P, RangeDev R, const double* __restrict__ 
 
 // Transposed receiver read-out (eq. localSol2, every m including m = 0, FP64): for spring l and
 // each receiver r in order, the extended indices of l inside r's window (those of the forward
-// read-out), sigmabar_l^{n+1-m} += (1/2) Q_m(d) ubar_r.  One thread per spring, no atomics.
+// read-out), sigmabar_l^{n+1-m} += (1/2) Q_m(d) ubar_r.  One thread per spring and eighth of the m
+// (blockIdx.y: m = y, y + 8, ..), so each output has one writer; no atomics.
 __global__ void k_rs_adj_receivers(DevPlan P, RangeDev R, int64_t n, const double* __restrict__ ubar, double* sb) {
     const int64_t M = P.M;
     for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < M; l += (int64_t)gridDim.x * blockDim.x) {
@@ -1122,13 +1144,13 @@ __global__ void k_rs_adj_receivers(DevPlan P, RangeDev R, int64_t n, const doubl
                 const double d = fabs(rs_xext(P, e) - P.xr[r]);
                 if (!(d < R.delta)) continue;
                 const int iv = rs_locate64(R, d);
-                const double z = (d - __ldg(R.mid + iv)) * (double)__ldg(R.ih + iv);
+                double T[8];
+                rs_cheb_basis((d - __ldg(R.mid + iv)) * (double)__ldg(R.ih + iv), T);
                 const int m0 = __ldg(R.mr0 + 2 * iv), m1 = __ldg(R.mr0 + 2 * iv + 1);
-                for (int m = m0; m <= m1; m++) {
-                    const double q = rs_cheb(R.cheb + ((size_t)iv * R.nm + m) * 8, z);
+                for (int m = m0 + ((blockIdx.y - m0) & 7); m <= m1; m += 8) {
                     int64_t s = (n + 1 - m) % P.ring;
                     if (s < 0) s += P.ring;
-                    sb[s * M + l] += 0.5 * q * ubar[r];
+                    sb[s * M + l] += 0.5 * rs_cheb_sum(R.cheb + ((size_t)iv * R.nm + m) * 8, T) * ubar[r];
                 }
             }
         }
