@@ -64,7 +64,9 @@ __global__ void k_rs_slices(DevPlan P, RangeDev R);
 __global__ void k_rs_fold(DevPlan P, RangeDev R, int s0);
 __global__ void k_rs_pairs(DevPlan P, RangeDev R, int s0);
 size_t rs_pair_smem(int part, int fine_span);
-__global__ void k_rs_moments(DevPlan P, RangeDev R, int s0, int s1, const double* cbar);
+__global__ void k_rs_moments(DevPlan P, RangeDev R, int s0, const double* cbar);
+__global__ void k_rs_sweeps(DevPlan P, RangeDev R);
+size_t rs_unfold_smem();
 __global__ void k_rs_unfold(DevPlan P, RangeDev R, int s0, int s1, int64_t n, float2* sums, double* sb);
 __global__ void k_rs_adj_init(DevPlan P, RangeDev R, double* slot_vals, double* rhs);
 __global__ void k_rs_adj_post(DevPlan P, RangeDev R, const double* sigma_next, const double* g_next, double* grad,
@@ -370,6 +372,19 @@ bool is_rbc_step(const wave1d_plan_t p, int64_t n) {
     return p->hp.P.bc == WAVE1D_FREE && ((n + 1) % p->hp.P.rbc_period) == 0;
 }
 
+// the Jacobi sweeps of a plan without pair lists (d.rhs: their right-hand side).  Up to 2^19 pairs
+// closer than dt and 65536 springs one cluster takes all of them in one launch; larger plans need the
+// whole chip for a sweep, and mixed plans keep the order of their sums (range_fp32.cu)
+void enqueue_sweeps(wave1d_plan_t p, const DevPlan& d) {
+    const int64_t M = p->hp.P.M;
+    if (!p->mixed && M <= 65536 && p->hp.nb_off[M] <= (1 << 19)) {
+        k_rs_sweeps<<<8, 1024, 0, p->s>>>(d, p->rd);
+        return;
+    }
+    const unsigned sweeps = (unsigned)std::min<int64_t>((M + 63) / 64, 16 * (int64_t)p->sms);
+    for (int it = 1; it <= kRsMaxIter; it++) k_rs_jacobi<<<sweeps, 256, 0, p->s>>>(d, p->rd, it);
+}
+
 // queue one step n -> n+1 on the private stream; ev (optional) gets WAVE1D_NSTAGE + 1 events
 // recorded between the stages
 int enqueue_step(wave1d_plan_t p, int64_t n, const double* g_ext, double* sig_hist,
@@ -483,9 +498,9 @@ int enqueue_step(wave1d_plan_t p, int64_t n, const double* g_ext, double* sig_hi
     mark(WAVE1D_STAGE_SOLVE);
     if (fork) cudaStreamWaitEvent(s, p->ev_join, 0);
     if (p->range) {
-        const unsigned rows = blocks(P.M, T), sweeps = (unsigned)std::min<int64_t>(blocks(P.M, 64), 16 * (int64_t)p->sms);
+        const unsigned rows = blocks(P.M, T);
         k_rs_solve_init<<<rows, T, 0, s>>>(d, p->rd);
-        for (int it = 1; it <= kRsMaxIter; it++) k_rs_jacobi<<<sweeps, T, 0, s>>>(d, p->rd, it);
+        enqueue_sweeps(p, d);
         k_rs_store<<<rows, T, 0, s>>>(d, p->rd);
         mark(WAVE1D_STAGE_RECEIVERS);
         if (P.R > 0) k_rs_receivers<<<dim3((unsigned)p->rd.rchunks, (unsigned)P.R), T, 0, s>>>(d, p->rd);
@@ -1429,6 +1444,7 @@ struct Reverse {
                 p->rd.nis = hp.rt.nis;
                 p->rd.nmp = hp.rt.nmp;
                 p->rd.unfold = h16;
+                CK(cudaFuncSetAttribute(k_rs_unfold, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs_unfold_smem()));
             }
             return wk.zeros(&usum, (size_t)M * p->rd.nmp);
         }
@@ -1461,8 +1477,7 @@ struct Reverse {
                 k_rs_adj_init<<<gM, 256, 0, s>>>(d, rd, sb + (int64_t)((n + 1) % ring) * M, rrhs);
                 DevPlan dj = d;
                 dj.rhs = rrhs;
-                const unsigned sweeps = (unsigned)std::min<int64_t>(blocks_for(M, 64, INT32_MAX), 16 * (int64_t)p->sms);
-                for (int it = 1; it <= kRsMaxIter; it++) k_rs_jacobi<<<sweeps, 256, 0, s>>>(dj, rd, it);
+                enqueue_sweeps(p, dj);
                 k_rs_adj_post<<<gM, 256, 0, s>>>(d, rd, sig_rows + (n - row0) * M, g ? g + n * M : nullptr,
                                                  want_beta ? gsum : nullptr, grad_g ? grad_g + n * M : nullptr, cbar, uHbar);
                 if (n == 0) break;
@@ -1470,9 +1485,10 @@ struct Reverse {
                 for (int s0 = 0; s0 < rd.nint; s0 += rd.slab) {
                     const int s1 = std::min(rd.nint, s0 + rd.slab);
                     CK(cudaMemsetAsync(rd.evec, 0, (size_t)M * rd.slab * kRsRecord * sizeof(float), s));
-                    k_rs_moments<<<gp, kRsPairTargets, rs_pair_smem(s1 - s0, rd.fine_span), s>>>(d, rd, s0, s1, cbar);
-                    k_rs_unfold<<<dim3(blocks_for(M, 64, INT32_MAX), (unsigned)(rd.nmp / 8 + 4) / 5), 128, 0, s>>>(d, rd, s0, s1, n,
-                                                                                                          usum, sb);
+                    k_rs_moments<<<dim3(gp, 1, (unsigned)((s1 - s0 + rd.part - 1) / rd.part)), kRsPairTargets,
+                                   rs_pair_smem(rd.part, rd.fine_span), s>>>(d, rd, s0, cbar);
+                    k_rs_unfold<<<dim3(blocks_for(M, 128, INT32_MAX), (unsigned)(rd.nmp / 8 + 4) / 5), 256, rs_unfold_smem(), s>>>(
+                        d, rd, s0, s1, n, usum, sb);
                 }
             } else {
                 if (have_rcv) k_adj_receivers<<<gM, 256, 0, s>>>(M, ring, n, rptr, rrcv, rmr, rwoff, rw, ub, sb);

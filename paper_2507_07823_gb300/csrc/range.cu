@@ -748,6 +748,75 @@ __global__ void __launch_bounds__(256) k_rs_jacobi(DevPlan P, RangeDev R, int it
     }
 }
 
+// All sweeps of a small plan in one launch: a cluster of kRsCluster blocks, a thread per row (rows of
+// these plans hold a few tens of sources), the cluster's barrier between sweeps, until the stopping rule
+// is met.  Forty launches, of which 7 to 10 do work, cost a plan of 3e4 springs more than its sweeps, and
+// a batch runs many such plans side by side.
+constexpr int kRsCluster = 8;
+__global__ void __cluster_dims__(kRsCluster, 1, 1) __launch_bounds__(1024) k_rs_sweeps(DevPlan P, RangeDev R) {
+    __shared__ double red[2][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int it = 1; it <= kRsMaxIter; it++) {
+        const float2* src2 = (const float2*)R.it2[(it - 1) & 1];
+        const double* src = R.it64[(it - 1) & 1];
+        double* dst = R.it64[it & 1];
+        float2* dst2 = (float2*)R.it2[it & 1];
+        double dmax = 0.0, smax = 0.0;
+        for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P.M; j += (int64_t)gridDim.x * blockDim.x) {
+            const int lo = __ldg(R.nb_lo + j), cnt = __ldg(R.nb_cnt + j);
+            const float2* w = (const float2*)R.nb_w + __ldg(R.nb_off + j);
+            float ah = 0.f, al = 0.f, bh = 0.f, bl = 0.f;
+            int k = 0;
+            for (; k + 4 <= cnt; k += 4) {
+                float2 wv[4], sv[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    wv[u] = __ldg(w + k + u);
+                    sv[u] = __ldcg(src2 + rs_spring((int64_t)lo + k + u, P.M));
+                }
+                rs::acc_mac(ah, al, wv[0].x, wv[0].y, sv[0].x, sv[0].y);
+                rs::acc_mac(bh, bl, wv[1].x, wv[1].y, sv[1].x, sv[1].y);
+                rs::acc_mac(ah, al, wv[2].x, wv[2].y, sv[2].x, sv[2].y);
+                rs::acc_mac(bh, bl, wv[3].x, wv[3].y, sv[3].x, sv[3].y);
+            }
+            for (; k < cnt; k++) {
+                const float2 wv = __ldg(w + k), sv = __ldcg(src2 + rs_spring((int64_t)lo + k, P.M));
+                rs::acc_mac(ah, al, wv.x, wv.y, sv.x, sv.y);
+            }
+            rs::acc_add(ah, al, bh, bl);
+            const double x = (__ldcg(P.rhs + j) - ((double)ah + (double)al)) / R.diag[j];
+            dmax = fmax(dmax, fabs(x - __ldcg(src + j)));
+            smax = fmax(smax, fabs(x));
+            dst[j] = x;
+            const rs::Pair p2 = rs::split(x);
+            dst2[j] = make_float2(p2.hi, p2.lo);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+            smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+        }
+        if (lane == 0) {
+            red[0][wid] = dmax;
+            red[1][wid] = smax;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < (int)(blockDim.x >> 5); w++) {
+                dmax = fmax(dmax, red[0][w]);
+                smax = fmax(smax, red[1][w]);
+            }
+            atomicMax(R.stats + 2 * it, (unsigned long long)__double_as_longlong(dmax));
+            atomicMax(R.stats + 2 * it + 1, (unsigned long long)__double_as_longlong(smax));
+            __threadfence();
+        }
+        __syncthreads();
+        // every block's rows and its part of the record are in place for the whole cluster
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (rs_from_bits(__ldcg(R.stats + 2 * it)) <= kRsTol * rs_from_bits(__ldcg(R.stats + 2 * it + 1))) break;
+    }
+}
+
 // the converged iterate into the rings: the first sweep whose record meets the stopping rule
 // (sweeps after it did not run and left zero records)
 __global__ void k_rs_store(DevPlan P, RangeDev R) {
@@ -914,8 +983,8 @@ struct RsMoments {
     }
 };
 
-// the moments of a slab, both sides (the records are zero on entry)
-__global__ void __launch_bounds__(kRsPairTargets) k_rs_moments(DevPlan P, RangeDev R, int s0, int s1,
+// the moments of a slab, both sides (the records are zero on entry), parts in blocks of their own
+__global__ void __launch_bounds__(kRsPairTargets) k_rs_moments(DevPlan P, RangeDev R, int s0,
                                                               const double* __restrict__ cbar) {
     extern __shared__ __align__(16) float4 pair_sm[];
     __shared__ float2 sPos[kRsPosChunk], sC[kRsPosChunk];
@@ -923,8 +992,9 @@ __global__ void __launch_bounds__(kRsPairTargets) k_rs_moments(DevPlan P, RangeD
     const int64_t j = min((int64_t)blockIdx.x * kRsPairTargets + threadIdx.x, P.M - 1);
     RsMoments v{P, R, cbar, sC, R.evec + (size_t)j * R.slab * kRsRecord, s0, -1};
     v.clear();
-    rs_pair_block<-1>(P, R, s0, s1, pair_sm, sPos, sRed, v);
-    rs_pair_block<1>(P, R, s0, s1, pair_sm, sPos, sRed, v);
+    const int p0 = s0 + blockIdx.z * R.part, p1 = min(R.nint, p0 + R.part);
+    rs_pair_block<-1>(P, R, p0, p1, pair_sm, sPos, sRed, v);
+    rs_pair_block<1>(P, R, p0, p1, pair_sm, sPos, sRed, v);
     v.flush();
 }
 
@@ -937,13 +1007,17 @@ __global__ void __launch_bounds__(kRsPairTargets) k_rs_moments(DevPlan P, RangeD
 // coefficients fall by 10 or more from one to the next) and go into the output's pairs after it;
 // slices that are zero in the whole warp are skipped.  sums: [M][nmp] pairs carried from slab to slab;
 // the last slab adds them to the ring.
-constexpr int kRsUnfoldWarps = 4;
+// The block stages a step's coefficients in shared memory (two buffers, asynchronous copies): read from
+// L2 by each warp they held it up 40 times a step (576 us a slab of 336 intervals at 3e4 outputs).
+constexpr int kRsUnfoldWarps = 8;
 constexpr int kRsUnfoldTiles = 5;                     // tiles of 8 m at a time (m_max up to 40 in one go)
+constexpr int kRsUnfoldStep = kRsAllSlices * kRsUnfoldTiles * 8 * 32;     // bytes of a step's coefficients
+size_t rs_unfold_smem() { return 2 * (size_t)kRsUnfoldStep; }
 __global__ void __launch_bounds__(32 * kRsUnfoldWarps) k_rs_unfold(DevPlan P, RangeDev R, int s0, int s1, int64_t n,
                                                                   float2* __restrict__ sums, double* __restrict__ sb) {
     const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    extern __shared__ __align__(16) unsigned char unfold_sm[];
     const int64_t l0 = ((int64_t)blockIdx.x * kRsUnfoldWarps + (threadIdx.x >> 5)) * 16;
-    if (l0 >= P.M) return;
     const int mtiles = R.nmp >> 3, mt0 = blockIdx.y * kRsUnfoldTiles, mt1 = min(mtiles, mt0 + kRsUnfoldTiles);
     const int64_t row[2] = {min(l0 + g, P.M - 1), min(l0 + g + 8, P.M - 1)};
     float2 out[kRsUnfoldTiles][4];                    // (row c >> 1, m = 8 mt + 2 q + (c & 1) + 1)
@@ -953,7 +1027,23 @@ __global__ void __launch_bounds__(32 * kRsUnfoldWarps) k_rs_unfold(DevPlan P, Ra
         for (int c = 0; c < 4; c++)
             out[mt][c] = s0 > 0 && mt0 + mt < mt1 ? sums[row[c >> 1] * R.nmp + 8 * (mt0 + mt) + 2 * q + (c & 1)]
                                                   : make_float2(0.f, 0.f);
+    const int rows = 8 * (mt1 - mt0);
+    auto fetch = [&](int i0, int buf) {
+        const unsigned char* src = (const unsigned char*)R.unfold + ((size_t)(i0 >> 4) * R.nmp + 8 * mt0) * 32;
+        for (int i = threadIdx.x; i < kRsAllSlices * rows * 2; i += blockDim.x) {
+            const int sl = i / (rows * 2), o = i - sl * rows * 2;
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(unfold_sm + buf * kRsUnfoldStep + (sl * kRsUnfoldTiles * 16 + o) * 16);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
+                         "l"(src + (size_t)sl * R.nis * R.nmp * 32 + (size_t)o * 16));
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    fetch(s0, 0);
     for (int i0 = s0; i0 < s1; i0 += 16) {
+        const int buf = ((i0 - s0) >> 4) & 1;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();                              // this step has arrived, the other buffer is free
+        if (i0 + 16 < s1) fetch(i0 + 16, buf ^ 1);
         // first m of the step's intervals (all later ones are met)
         const int m0 = __reduce_min_sync(0xffffffffu, __ldg(R.mr + 2 * min(i0 + (lane & 15), R.nint - 1)));
         if (8 * mt1 < m0) continue;
@@ -1017,14 +1107,14 @@ __global__ void __launch_bounds__(32 * kRsUnfoldWarps) k_rs_unfold(DevPlan P, Ra
             bool use[kRsSlices];
 #pragma unroll
             for (int i = 0; i < kRsSlices; i++) use[i] = __any_sync(0xffffffffu, any[i] != 0u);
-            const uint2* tab = (const uint2*)R.unfold + (((size_t)first * R.nis + (i0 >> 4)) * R.nmp + 8 * mt0) * 4 + lane;
-            const size_t stride = (size_t)R.nis * R.nmp * 4;
+            const uint2* tab = (const uint2*)(unfold_sm + buf * kRsUnfoldStep) + first * kRsUnfoldTiles * 32 + lane;
+            constexpr int stride = kRsUnfoldTiles * 32;
 #pragma unroll
             for (int mt = 0; mt < kRsUnfoldTiles; mt++) {
                 if (mt0 + mt < mt1 && 8 * (mt0 + mt + 1) >= m0) {
                     uint2 b[count];
 #pragma unroll
-                    for (int jj = 0; jj < count; jj++) b[jj] = __ldg(tab + jj * stride + 32 * mt);
+                    for (int jj = 0; jj < count; jj++) b[jj] = tab[jj * stride + 32 * mt];
 #pragma unroll
                     for (int i = 0; i < kRsSlices; i++) {
                         if (use[i]) {
