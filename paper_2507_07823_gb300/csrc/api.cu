@@ -402,7 +402,12 @@ int enqueue_step(wave1d_plan_t p, int64_t n, const double* g_ext, double* sig_hi
     bool rbc = is_rbc_step(p, n);
     if (p->step_kernel && !rbc && !ev) {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(p->step_grid);
+        // as many blocks as the step has work for: the history group and the widest of the other parts
+        // (local-sum items and solve tasks a warp each, FIR tails two warps to a block); every block
+        // more is one more arrival at the grid barrier and one more count at the end
+        const int64_t rest = std::max({(d.l_nitems + d.r_nitems + 7) / 8, (int64_t)(P.K + 8) / 8,
+                                       (d.n_sgroups + d.n_big + 7) / 8, (P.M + 255) / 256});
+        cfg.gridDim = dim3((unsigned)std::min<int64_t>(p->step_grid, d.hist_blocks + rest));
         cfg.blockDim = dim3(kStepThreads);
         cfg.dynamicSmemBytes = p->step_smem;
         cfg.stream = s;

@@ -525,25 +525,40 @@ __device__ __forceinline__ void solve_tasks(const DevPlan& P, int64_t n, int64_t
 }
 
 // receivers, after every density of the step is stored: u = 1/2 (sum of the receiver row's item
-// partials (m >= 1) + sum over sources closer than dt of Q_0 sigma^{n+1}) + u_H; one warp per
-// receiver, the m = 0 terms padded to r0_stride lanes (zero weight on padding), run by the block
-// that finishes the step last.
+// partials (m >= 1) + sum over sources closer than dt of Q_0 sigma^{n+1}) + u_H, run by the block that
+// finishes the step last.  Eight lanes per receiver, so a block reads out 32 at a time: each round is a
+// chain of three loads, and with a warp per receiver the 100 receivers of the disordered medium took
+// thirteen rounds (25 us of a 56 us step).  The m = 0 terms are padded to r0_stride entries (zero
+// weight on padding).
 __device__ __forceinline__ void receivers_readout(const DevPlan& P, int64_t n) {
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int q = threadIdx.x & 7, ngroups = blockDim.x >> 3;
     const double* s1 = P.sig + (int64_t)ring_slot(n + 1, P.ring) * P.M;
-    for (int64_t r = wid; r < P.R; r += nwarps) {
-        const double uh = __ldcg(P.uHr + r);
-        double cr = 0.0;
-        for (int64_t it = __ldg(P.r_item_ptr + r) + lane; it < __ldg(P.r_item_ptr + r + 1); it += 32)
-            cr += __ldcg(P.r_part + it);
-        double acc = 0.0;
-        for (int e = lane; e < P.r0_stride; e += 32) {
-            const int64_t idx = r * P.r0_stride + e;
-            acc = fma(__ldg(P.r0p_w + idx), __ldcg(s1 + __ldg(P.r0p_src + idx)), acc);
+    for (int64_t r0 = 0; r0 < P.R; r0 += ngroups) {
+        const int64_t r = r0 + (threadIdx.x >> 3);
+        const bool in = r < P.R;
+        const double uh = in ? __ldcg(P.uHr + r) : 0.0;
+        double cr = 0.0, acc = 0.0;
+        if (in) {
+            const int64_t e1 = __ldg(P.r_item_ptr + r + 1);
+            for (int64_t it = __ldg(P.r_item_ptr + r) + q; it < e1; it += 8) cr += __ldcg(P.r_part + it);
+            for (int e = q; e < P.r0_stride; e += 32) {       // r0_stride is a multiple of 32
+                double w[4], v[4];
+                int src[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const int64_t idx = r * P.r0_stride + e + 8 * u;
+                    w[u] = __ldg(P.r0p_w + idx);
+                    src[u] = __ldg(P.r0p_src + idx);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; u++) v[u] = __ldcg(s1 + src[u]);
+#pragma unroll
+                for (int u = 0; u < 4; u++) acc = fma(w[u], v[u], acc);
+            }
         }
-        cr = warp_sum(cr);
-        acc = warp_sum(acc);
-        if (lane == 0) P.rec_hist[(n % P.chunk) * P.R + r] = 0.5 * (cr + acc) + uh;
+        cr += acc;
+        for (int o = 4; o > 0; o >>= 1) cr += __shfl_xor_sync(0xffffffffu, cr, o);
+        if (in && q == 0) P.rec_hist[(n % P.chunk) * P.R + r] = 0.5 * cr + uh;
     }
 }
 
