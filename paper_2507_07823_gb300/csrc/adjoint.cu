@@ -17,23 +17,22 @@
 
 namespace wave1d {
 
-// receivers' transposed readout, one thread per source over the receiver weights regrouped by
-// source (m >= 0: the m = 0 terms of sources closer than dt included)
+// receivers' transposed readout over the receiver weights regrouped by source (m >= 0: the m = 0 terms
+// of sources closer than dt included): one thread per source and eighth of the m (blockIdx.y: m = y,
+// y + 8, ..), so each ring entry has one writer, which meets the receivers in order
+constexpr int kAdjParts = 8;
 __global__ void k_adj_receivers(int64_t M, int ring, int64_t n, const int64_t* __restrict__ ptr,
                                 const int32_t* __restrict__ rcv, const int32_t* __restrict__ mrange,
                                 const int64_t* __restrict__ woff, const double* __restrict__ w,
                                 const double* __restrict__ ubar, double* sb) {
     for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < M; l += (int64_t)gridDim.x * blockDim.x)
-        adj::receivers_T_source(l, ptr, rcv, mrange, woff, w, ubar, n + 1, ring,
-                                [&](int s, double v) { sb[(int64_t)s * M + l] += v; });
-}
-
-// sigmabar^{n+1} is complete: move it out of its ring slot (which becomes sigma^{n-m_max}'s)
-__global__ void k_adj_take(int64_t M, double* __restrict__ slot_vals, double* __restrict__ out) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < M; j += (int64_t)gridDim.x * blockDim.x) {
-        out[j] = slot_vals[j];
-        slot_vals[j] = 0.0;
-    }
+        for (int64_t e = ptr[l]; e < ptr[l + 1]; e++) {
+            const double coef = 0.5 * ubar[rcv[e]];
+            if (coef == 0.0) continue;
+            const int mlo = mrange[e] & 0xffff, cnt = mrange[e] >> 16;
+            for (int c = ((int)blockIdx.y - mlo) & (kAdjParts - 1); c < cnt; c += kAdjParts)
+                sb[(int64_t)adj::slot(n + 1 - mlo - c, ring) * M + l] += w[woff[e] + c] * coef;
+        }
 }
 
 // transposed block solve, one thread per member position e of blk_members (blk_of[e] = its
@@ -43,6 +42,7 @@ __global__ void k_adj_take(int64_t M, double* __restrict__ slot_vals, double* __
 //             rhsbar_j sigma_j^{n+1} / beta_j),
 //   gbar_j^{n+1} = -rhsbar_j,  cbar_j = -beta_j rhsbar_j / 2,  u_Hbar_j = -beta_j rhsbar_j.
 // sigma_next, g_next and gbar_next are rows in caller order; g_next, grad and gbar_next may be null.
+// sigbar: the ring slot of sigmabar^{n+1} itself (k_adj_gather clears it afterwards).
 __global__ void k_adj_solve(DevPlan P, const int32_t* __restrict__ blk_of, const double* __restrict__ sigbar,
                             const double* __restrict__ sigma_next, const double* __restrict__ g_next, double* grad,
                             double* __restrict__ gbar_next, double* cbar, double* uHbar) {
@@ -64,9 +64,10 @@ __global__ void k_adj_solve(DevPlan P, const int32_t* __restrict__ blk_of, const
 // transposed local sum of the springs, one warp per row l (the row's items read in the transposed
 // direction, Q_m being symmetric in the pair), in the compensated FP32 arithmetic of the forward
 // local sum: each lane accumulates its slices into the warp's shared pairs acc[m][lane] (row
-// stride kAdjAccStride), then lane i adds m = i, i + 32, ... over the 32 lanes in lane order (in
-// FP64) and adds the result to sigmabar^{n+1-m}[l].  Dynamic shared memory: warps per block x
-// (m_max + 1) x kAdjAccStride float pairs.
+// stride kAdjAccStride), eight slices' weights in flight, then lane i adds m = i, i + 32, ... over the
+// 32 lanes in lane order, as pairs, and adds the result to sigmabar^{n+1-m}[l].  Dynamic shared memory:
+// warps per block x (m_max + 1) x kAdjAccStride float pairs.  With the lanes' sums in FP64 (4 x 32
+// instructions a row and m of the FP64 pipe) and one slice in flight it took 137 us for 1.1e7 weights.
 constexpr int kAdjAccStride = 33;
 
 __global__ void k_adj_local(DevPlan P, int64_t n, const double* __restrict__ cbar, double* sb) {
@@ -80,27 +81,55 @@ __global__ void k_adj_local(DevPlan P, int64_t n, const double* __restrict__ cba
     for (int64_t it = P.l_item_ptr[l]; it < P.l_item_ptr[l + 1]; it++) {
         float ch, cl;
         adj::split_pair(cbar[P.l_src[it * 32 + lane]], ch, cl);
-        adj::item_lane_gather(P.l_w, P.l_wbase[it], P.l_s0[it], P.l_len[it], lane, P.l_mfirst, ch, cl,
-                              [&](int m) { return (float*)(acc + m * kAdjAccStride + lane); });
+        const float4* w = (const float4*)(P.l_w + 2 * P.l_wbase[it]) + lane;     // slices 2i, 2i + 1
+        float2* a = acc + (P.l_mfirst + P.l_s0[it]) * kAdjAccStride + lane;
+        const int len = P.l_len[it];
+        auto mac = [&](int t, float wh, float wl) {
+            if (wh != 0.0f) {                              // zero: padding, maybe past the last m
+                float2 v = a[t * kAdjAccStride];
+                adj::pair_mac(v.x, v.y, wh, wl, ch, cl);
+                a[t * kAdjAccStride] = v;
+            }
+        };
+        int t = 0;
+        for (; t + 8 <= len; t += 8) {
+            float4 q[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) q[u] = __ldcs(w + 32 * ((t >> 1) + u));
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                mac(t + 2 * u, q[u].x, q[u].y);
+                mac(t + 2 * u + 1, q[u].z, q[u].w);
+            }
+        }
+        for (; t < len; t += 2) {
+            const float4 q = __ldcs(w + 32 * (t >> 1));
+            mac(t, q.x, q.y);
+            mac(t + 1, q.z, q.w);
+        }
     }
     __syncwarp();
     for (int m = lane; m < nm; m += 32) {
-        double s = 0.0;
+        float sh = 0.f, sl = 0.f;
         for (int i = 0; i < 32; i++) {
             const float2 a = acc[m * kAdjAccStride + i];
-            s += (double)a.x + (double)a.y;
+            adj::pair_mac(sh, sl, 1.f, 0.f, a.x, a.y);
         }
+        const double s = (double)sh + (double)sl;
         if (s != 0.0) sb[(int64_t)adj::slot(n + 1 - m, P.ring) * P.M + l] += s;
     }
 }
 
 size_t adj_local_smem(int m_max, int warps) { return (size_t)warps * (m_max + 1) * kAdjAccStride * sizeof(float2); }
 
-// out[i] = in[perm[i]] (spring order -> NUFFT point order)
+// out[i] = in[perm[i]] (spring order -> NUFFT point order); clear: the ring slot of sigmabar^{n+1}, read by
+// the solve, becomes sigma^{n-m_max}'s
 __global__ void k_adj_gather(int64_t M, const int64_t* __restrict__ perm, const double* __restrict__ in,
-                             double* __restrict__ out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < M; i += (int64_t)gridDim.x * blockDim.x)
+                             double* __restrict__ out, double* __restrict__ clear) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < M; i += (int64_t)gridDim.x * blockDim.x) {
         out[i] = in[perm[i]];
+        if (clear) clear[i] = 0.0;
+    }
 }
 
 // acc[perm[i]] += in[i] (NUFFT point order -> spring order; perm is a permutation)
@@ -110,30 +139,153 @@ __global__ void k_adj_scatter_add(int64_t M, const int64_t* __restrict__ perm, c
         acc[perm[i]] += in[i];
 }
 
+// e^{i k x_r} of the receivers, [r][k], once per call (a sine and cosine of FP64 are some 200 instructions of
+// the FP64 pipe: 26 us a step for eight receivers)
+__global__ void k_adj_receiver_waves(int K, const double* __restrict__ xr, int64_t R, double2* __restrict__ out) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k > K) return;
+    for (int64_t r = blockIdx.y; r < R; r += gridDim.y) {
+        const double a = (double)k * xr[r];
+        out[r * (K + 1) + k] = make_double2(cos(a), sin(a));
+    }
+}
+
+// alphabar_k += w_k (2 pi S1_k + sum_r ubar_r e^{i k x_r}) (adj::modes_in); waves may be null (too many
+// receivers for the table): the waves are then formed here
 __global__ void k_adj_modes_in(int K, const double* __restrict__ S1, const double* __restrict__ xr,
-                               const double* __restrict__ ubar, int64_t R, double* ab) {
+                               const double2* __restrict__ waves, const double* __restrict__ ubar, int64_t R,
+                               double* ab) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k <= K) adj::modes_in(k, S1, xr, ubar, R, ab);
+    if (k > K) return;
+    if (!waves) {
+        adj::modes_in(k, S1, xr, ubar, R, ab);
+        return;
+    }
+    const double two_pi = 6.283185307179586476925286766559, wk = k == 0 ? 1.0 : 2.0;
+    double re = two_pi * S1[2 * k], im = two_pi * S1[2 * k + 1];
+#pragma unroll 4
+    for (int64_t r = 0; r < R; r++) {
+        const double2 e = __ldg(waves + r * (K + 1) + k);
+        const double u = __ldg(ubar + r);
+        re = fma(u, e.x, re);
+        im = fma(u, e.y, im);
+    }
+    ab[2 * k] = fma(wk, re, ab[2 * k]);
+    ab[2 * k + 1] = fma(wk, im, ab[2 * k + 1]);
 }
 
-__global__ void k_adj_rbc_grid(int K, int npts, const int32_t* __restrict__ idx, const double* __restrict__ tw2K,
-                               const double* __restrict__ phi, const double* __restrict__ dphi,
-                               const double* __restrict__ ab, const double* __restrict__ apb,
-                               double* __restrict__ uvbar) {
-    const int pt = blockIdx.x * blockDim.x + threadIdx.x;
-    if (pt < npts) adj::rbc_grid_T(idx[pt], K, tw2K, ab, apb, phi[pt], dphi[pt], uvbar + 2 * pt, uvbar + 2 * pt + 1);
+// transposed projection, grid part: a block per rolled-off point (cf. adj::rbc_grid_T; the block's sum
+// in a fixed order)
+__global__ void __launch_bounds__(256) k_adj_rbc_grid(int K, int npts, const int32_t* __restrict__ idx,
+                                                      const double* __restrict__ tw2K, const double* __restrict__ phi,
+                                                      const double* __restrict__ dphi, const double* __restrict__ ab,
+                                                      const double* __restrict__ apb, double* __restrict__ uvbar) {
+    __shared__ double red[2][8];
+    const int pt = blockIdx.x;
+    const int64_t twoK = 2 * (int64_t)K, ig = idx[pt], inc = ((int64_t)blockDim.x * ig) % twoK;
+    double su = 0.0, sv = 0.0;
+    int64_t a = ((int64_t)(1 + threadIdx.x) * ig) % twoK;
+    for (int k = 1 + threadIdx.x; k < K; k += blockDim.x) {
+        const double2 e = __ldg((const double2*)tw2K + a);               // e^{+i k x}
+        const double2 u = ((const double2*)ab)[k], v = ((const double2*)apb)[k];
+        su += u.x * e.x + u.y * e.y;
+        sv += v.x * e.x + v.y * e.y;
+        a += inc;
+        if (a >= twoK) a -= twoK;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        su += __shfl_xor_sync(0xffffffffu, su, o);
+        sv += __shfl_xor_sync(0xffffffffu, sv, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        red[0][threadIdx.x >> 5] = su;
+        red[1][threadIdx.x >> 5] = sv;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        su = ab[0];
+        sv = apb[0];
+        for (int w = 0; w < 8; w++) {
+            su += red[0][w];
+            sv += red[1][w];
+        }
+        const double Du = su / (double)twoK, Dv = sv / (double)twoK;
+        uvbar[2 * pt] = fma(phi[pt] - 1.0, Du, dphi[pt] * Dv);
+        uvbar[2 * pt + 1] = (phi[pt] - 1.0) * Dv;
+    }
 }
 
-__global__ void k_adj_rbc_update(int K, int npts, const int32_t* __restrict__ idx, const double* __restrict__ tw2K,
-                                 const double* __restrict__ uvbar, double* ab, double* apb) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k <= K) adj::rbc_update_T(k, K, npts, idx, tw2K, uvbar, ab, apb);
+// mode part (cf. adj::rbc_update_T): eight lanes per mode, each every eighth point, a fixed tree
+__global__ void __launch_bounds__(256) k_adj_rbc_update(int K, int npts, const int32_t* __restrict__ idx,
+                                                        const double* __restrict__ tw2K,
+                                                        const double* __restrict__ uvbar, double* ab, double* apb) {
+    const int k = blockIdx.x * 32 + (threadIdx.x >> 3), q = threadIdx.x & 7;
+    const int64_t twoK = 2 * (int64_t)K;
+    double ur = 0.0, ui = 0.0, vr = 0.0, vi = 0.0;
+    if (k < K) {
+        for (int pt = q; pt < npts; pt += 8) {
+            const double2 e = __ldg((const double2*)tw2K + ((int64_t)k * idx[pt]) % twoK), w = __ldg((const double2*)uvbar + pt);
+            ur = fma(w.x, e.x, ur);
+            ui = fma(w.x, e.y, ui);
+            vr = fma(w.y, e.x, vr);
+            vi = fma(w.y, e.y, vi);
+        }
+    }
+    for (int o = 4; o > 0; o >>= 1) {
+        ur += __shfl_xor_sync(0xffffffffu, ur, o);
+        ui += __shfl_xor_sync(0xffffffffu, ui, o);
+        vr += __shfl_xor_sync(0xffffffffu, vr, o);
+        vi += __shfl_xor_sync(0xffffffffu, vi, o);
+    }
+    if (q != 0 || k > K) return;
+    if (k == K) {
+        ab[2 * k] = ab[2 * k + 1] = 0.0;
+        apb[2 * k] = apb[2 * k + 1] = 0.0;
+    } else if (k == 0) {                 // Re alpha_0 only
+        ab[0] += ur;
+        apb[0] += vr;
+    } else {
+        ab[2 * k] = fma(2.0, ur, ab[2 * k]);
+        ab[2 * k + 1] = fma(2.0, ui, ab[2 * k + 1]);
+        apb[2 * k] = fma(2.0, vr, apb[2 * k]);
+        apb[2 * k + 1] = fma(2.0, vi, apb[2 * k + 1]);
+    }
 }
 
+// rotation and FIR transposed (adj::modes_T), one thread per mode and kAdjTaps of the W taps
+// (blockIdx.y): every part reads the old (ab, apb) and updates its own ring slots, part 0 also writes
+// the rotated modes to (ab_out, apb_out) and takes Sbar^n out of its slot.  One thread per mode took 33
+// us for 36 taps, a chain of ring reads and writes.
+constexpr int kAdjTaps = 4;
 __global__ void k_adj_modes(int K, int W, int64_t n, const double* __restrict__ rot, const double* __restrict__ pq,
-                            double* ab, double* apb, double* Sb, double* __restrict__ a2) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k <= K) adj::modes_T(k, K + 1, W, n, rot, pq, ab, apb, Sb, a2);
+                            const double* __restrict__ ab, const double* __restrict__ apb, double* __restrict__ ab_out,
+                            double* __restrict__ apb_out, double* Sb, double* __restrict__ a2) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, K1 = K + 1, ma = blockIdx.y * kAdjTaps;
+    if (k > K) return;
+    const double2 h = ((const double2*)ab)[k], g = ((const double2*)apb)[k];
+    double2 w[kAdjTaps], s[kAdjTaps];
+    double2* at[kAdjTaps];
+#pragma unroll
+    for (int u = 0; u < kAdjTaps; u++) {
+        const int m = min(ma + u, W - 1);
+        at[u] = (double2*)Sb + (int64_t)adj::slot(n - m, W) * K1 + k;
+        w[u] = __ldg((const double2*)pq + (int64_t)m * K1 + k);
+        s[u] = *at[u];
+    }
+#pragma unroll
+    for (int u = 0; u < kAdjTaps; u++) {
+        s[u].x = fma(w[u].x, h.x, fma(w[u].y, g.x, s[u].x));
+        s[u].y = fma(w[u].x, h.y, fma(w[u].y, g.y, s[u].y));
+        if (ma + u > 0 && ma + u < W) *at[u] = s[u];
+    }
+    if (ma > 0) return;
+    const double cs = rot[3 * k], so = rot[3 * k + 1], ks = rot[3 * k + 2];
+    ((double2*)ab_out)[k] = make_double2(fma(cs, h.x, -ks * g.x), fma(cs, h.y, -ks * g.y));
+    ((double2*)apb_out)[k] = make_double2(fma(so, h.x, cs * g.x), fma(so, h.y, cs * g.y));
+    const double scale = (k == 0 ? 1.0 : 0.5) / 6.283185307179586476925286766559;
+    a2[2 * k] = s[0].x * scale;
+    a2[2 * k + 1] = k == 0 ? 0.0 : s[0].y * scale;
+    *at[0] = make_double2(0.0, 0.0);
 }
 
 // Checkpoint restore (wave1d_adjoint_checkpointed): the float-pair copy of the density ring

@@ -40,19 +40,20 @@ __global__ void k_adj_receivers(int64_t M, int ring, int64_t n, const int64_t* p
                                 const int32_t* mrange, const int64_t* woff, const double* w, const double* ubar,
                                 double* sb);
 size_t adj_local_smem(int m_max, int warps);
-__global__ void k_adj_take(int64_t M, double* slot_vals, double* out);
 __global__ void k_adj_solve(DevPlan P, const int32_t* blk_of, const double* sigbar, const double* sigma_next,
                             const double* g_next, double* grad, double* gbar_next, double* cbar, double* uHbar);
 __global__ void k_adj_local(DevPlan P, int64_t n, const double* cbar, double* sb);
-__global__ void k_adj_gather(int64_t M, const int64_t* perm, const double* in, double* out);
+__global__ void k_adj_gather(int64_t M, const int64_t* perm, const double* in, double* out, double* clear);
+__global__ void k_adj_receiver_waves(int K, const double* xr, int64_t R, double2* out);
 __global__ void k_adj_scatter_add(int64_t M, const int64_t* perm, const double* in, double* acc);
-__global__ void k_adj_modes_in(int K, const double* S1, const double* xr, const double* ubar, int64_t R, double* ab);
+__global__ void k_adj_modes_in(int K, const double* S1, const double* xr, const double2* waves, const double* ubar,
+                               int64_t R, double* ab);
 __global__ void k_adj_rbc_grid(int K, int npts, const int32_t* idx, const double* tw2K, const double* phi,
                                const double* dphi, const double* ab, const double* apb, double* uvbar);
 __global__ void k_adj_rbc_update(int K, int npts, const int32_t* idx, const double* tw2K, const double* uvbar,
                                  double* ab, double* apb);
-__global__ void k_adj_modes(int K, int W, int64_t n, const double* rot, const double* pq, double* ab, double* apb,
-                            double* Sb, double* a2);
+__global__ void k_adj_modes(int K, int W, int64_t n, const double* rot, const double* pq, const double* ab,
+                            const double* apb, double* ab_out, double* apb_out, double* Sb, double* a2);
 __global__ void k_ck_sig2(int64_t n, const double* sig, float2* sig2);
 __global__ void k_ck_step(int64_t* step, int64_t n);
 __global__ void k_mx_gather(DevPlan P, const int64_t* perm, double* c);
@@ -474,7 +475,7 @@ int enqueue_step(wave1d_plan_t p, int64_t n, const double* g_ext, double* sig_hi
     if (rbc) {
         int npts = (int)p->hp.rbc_idx.size();
         k_rbc_grid<<<npts, T, 0, s>>>(d);
-        k_rbc_update<<<blocks(P.K + 1, 128), 128, 0, s>>>(d, npts);
+        k_rbc_update<<<blocks(P.K + 1, 32), 256, 0, s>>>(d, npts);
     }
     mark(WAVE1D_STAGE_FFT_INV);
     if (rbc) {
@@ -1400,12 +1401,13 @@ namespace {
 struct Reverse {
     AdjointWork wk;
     wave1d_plan_t p = nullptr;
-    double *sb, *Sb, *ab, *apb, *a2, *S1, *tmp, *cbar, *uHbar, *gsum, *cnu, *unu, *xr, *uvbar, *rw;
+    double *sb, *Sb, *ab, *apb, *ab2, *apb2, *a2, *S1, *cbar, *uHbar, *gsum, *cnu, *unu, *xr, *uvbar, *rw;
     int32_t *dblk, *rrcv, *rmr;
     int64_t *dperm, *rptr, *rwoff;
     bool have_rcv = false;
     int npts = 0;
     size_t lsmem = 0;
+    double2* waves = nullptr;
     double* rrhs = nullptr;   // plans without pair lists: the transposed solve's right-hand side
     float2* usum = nullptr;   // the transposed local sum's pairs between slabs
     static constexpr int kLocalWarps = 4;     // the transposed local sum: one warp per spring row
@@ -1432,7 +1434,7 @@ struct Reverse {
         if ((rc = wk.zeros(&sb, (size_t)P.ring * M)) || (rc = wk.zeros(&Sb, (size_t)P.W * K1 * 2)) ||
             (rc = wk.zeros(&ab, 2 * (size_t)K1)) || (rc = wk.zeros(&apb, 2 * (size_t)K1)) ||
             (rc = wk.zeros(&a2, 2 * (size_t)K1)) || (rc = wk.zeros(&S1, 2 * (size_t)K1)) ||
-            (rc = wk.zeros(&tmp, (size_t)M)) || (rc = wk.zeros(&cbar, (size_t)M)) || (rc = wk.zeros(&uHbar, (size_t)M)) ||
+            (rc = wk.zeros(&ab2, 2 * (size_t)K1)) || (rc = wk.zeros(&apb2, 2 * (size_t)K1)) || (rc = wk.zeros(&cbar, (size_t)M)) || (rc = wk.zeros(&uHbar, (size_t)M)) ||
             (rc = wk.zeros(&gsum, (size_t)M)) || (rc = wk.zeros(&cnu, (size_t)M)) || (rc = wk.zeros(&unu, (size_t)M)) ||
             (rc = wk.zeros(&uvbar, 2 * (size_t)std::max(npts, 1))) || (rc = wk.upload(hp.xr, &xr)) ||
             (rc = wk.upload(blk_of, &dblk)) || (rc = wk.upload(nperm, &dperm)) ||
@@ -1440,6 +1442,13 @@ struct Reverse {
             (rc = wk.upload(rcol.mrange, &rmr)) || (rc = wk.upload(rcol.woff, &rwoff)) ||
             (rc = wk.upload(hp.rloc.w, &rw)))
             return rc;
+        // the receivers' waves e^{i k x_r}, unless there are so many that the table passes 64 MB
+        if (P.R > 0 && (size_t)P.R * K1 * sizeof(double2) <= ((size_t)64 << 20)) {
+            if ((rc = wk.zeros(&waves, (size_t)P.R * K1))) return rc;
+            k_adj_receiver_waves<<<dim3(blocks_for(K1, 64, INT32_MAX), (unsigned)std::min<int64_t>(P.R, 1024)), 64, 0, p->s>>>(
+                P.K, xr, P.R, waves);
+            CK(cudaGetLastError());
+        }
         if (p->range) {
             if ((rc = wk.zeros(&rrhs, (size_t)M))) return rc;
             if (!p->rd.fold && (rc = fold_tables(p))) return rc;        // a mixed plan's first reverse march
@@ -1469,7 +1478,7 @@ struct Reverse {
         const int K = P.K, K1 = P.K + 1, ring = P.ring;
         const DevPlan& d = p->dp;
         const int64_t cap = (int64_t)p->sms * 8;
-        const unsigned gM = blocks_for(M, 256, cap), gK = blocks_for(K1, 256, INT32_MAX);
+        const unsigned gM = blocks_for(M, 256, cap);
         cudaStream_t s = p->s;
         int rc;
         for (int64_t n = n_hi - 1; n >= n_lo; n--) {
@@ -1496,23 +1505,24 @@ struct Reverse {
                         d, rd, s0, s1, n, usum, sb);
                 }
             } else {
-                if (have_rcv) k_adj_receivers<<<gM, 256, 0, s>>>(M, ring, n, rptr, rrcv, rmr, rwoff, rw, ub, sb);
-                k_adj_take<<<gM, 256, 0, s>>>(M, sb + (int64_t)(((n + 1) % ring)) * M, tmp);
-                k_adj_solve<<<gM, 256, 0, s>>>(d, dblk, tmp, sig_rows + (n - row0) * M, g ? g + n * M : nullptr,
+                if (have_rcv) k_adj_receivers<<<dim3(gM, 8), 256, 0, s>>>(M, ring, n, rptr, rrcv, rmr, rwoff, rw, ub, sb);
+                k_adj_solve<<<gM, 256, 0, s>>>(d, dblk, sb + (int64_t)((n + 1) % ring) * M, sig_rows + (n - row0) * M, g ? g + n * M : nullptr,
                                                want_beta ? gsum : nullptr, grad_g ? grad_g + n * M : nullptr, cbar, uHbar);
                 if (n == 0) break;
                 if (d.l_nitems > 0)
                     k_adj_local<<<blocks_for(M * 32, 32 * kLocalWarps, INT32_MAX), 32 * kLocalWarps, lsmem, s>>>(d, n, cbar, sb);
             }
-            k_adj_gather<<<gM, 256, 0, s>>>(M, dperm, uHbar, cnu);
+            k_adj_gather<<<gM, 256, 0, s>>>(M, dperm, uHbar, cnu, p->range ? nullptr : sb + (int64_t)((n + 1) % ring) * M);
             if ((rc = wave1d_nufft_type1(wk.nu, cnu, S1))) return fail(rc, wave1d_nufft_strerror());
-            k_adj_modes_in<<<gK, 256, 0, s>>>(K, S1, xr, ub, R, ab);
+            k_adj_modes_in<<<blocks_for(K1, 64, INT32_MAX), 64, 0, s>>>(K, S1, xr, waves, ub, R, ab);
             if (P.bc == WAVE1D_FREE && (n + 1) % P.rbc_period == 0 && npts > 0) {
-                k_adj_rbc_grid<<<blocks_for(npts, 64, INT32_MAX), 64, 0, s>>>(K, npts, d.rbc_idx, d.tw2K, d.rbc_phi,
-                                                                             d.rbc_dphi, ab, apb, uvbar);
-                k_adj_rbc_update<<<gK, 256, 0, s>>>(K, npts, d.rbc_idx, d.tw2K, uvbar, ab, apb);
+                k_adj_rbc_grid<<<npts, 256, 0, s>>>(K, npts, d.rbc_idx, d.tw2K, d.rbc_phi, d.rbc_dphi, ab, apb, uvbar);
+                k_adj_rbc_update<<<blocks_for(K1, 32, INT32_MAX), 256, 0, s>>>(K, npts, d.rbc_idx, d.tw2K, uvbar, ab, apb);
             }
-            k_adj_modes<<<gK, 256, 0, s>>>(K, P.W, n, d.rot, d.pq, ab, apb, Sb, a2);
+            k_adj_modes<<<dim3(blocks_for(K1, 128, INT32_MAX), (unsigned)(P.W + 3) / 4), 128, 0, s>>>(K, P.W, n, d.rot, d.pq, ab, apb,
+                                                                                                ab2, apb2, Sb, a2);
+            std::swap(ab, ab2);
+            std::swap(apb, apb2);
             if ((rc = wave1d_nufft_type2(wk.nu, a2, unu))) return fail(rc, wave1d_nufft_strerror());
             k_adj_scatter_add<<<gM, 256, 0, s>>>(M, dperm, unu, sb + (int64_t)(n % ring) * M);
             CK(cudaGetLastError());

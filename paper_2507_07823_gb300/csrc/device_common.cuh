@@ -17,6 +17,7 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
 
 __device__ __forceinline__ int ring_slot(int64_t q, int ring) {
+    if ((uint64_t)q < 0x80000000ull) return (int)((unsigned)q % (unsigned)ring);     // (64-bit division is slow)
     int64_t r = q % ring;
     return (int)(r < 0 ? r + ring : r);
 }

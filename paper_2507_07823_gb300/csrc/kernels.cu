@@ -109,28 +109,35 @@ __global__ void k_rbc_grid(DevPlan P) {
     }
 }
 
-__global__ void k_rbc_update(DevPlan P, int npts) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > P.K) return;
-    double2* al = (double2*)P.alpha;
-    double2* alp = (double2*)P.alpha_p;
+// eight lanes per mode, each every eighth point, then a fixed tree (one thread per mode was a chain of 4W
+// loads and 64-bit remainders: 66 us)
+__global__ void __launch_bounds__(256) k_rbc_update(DevPlan P, int npts) {
+    const int k = blockIdx.x * 32 + (threadIdx.x >> 3), q = threadIdx.x & 7;
     const double2* t2 = (const double2*)P.tw2K;
-    double2 a, ap;
-    if (k == P.K) {
-        a = make_double2(0.0, 0.0);
-        ap = a;
-    } else {
-        double2 du = make_double2(0.0, 0.0), dv = make_double2(0.0, 0.0);
-        int64_t twoK = 2 * (int64_t)P.K;
-        for (int pt = 0; pt < npts; pt++) {
-            double2 e = t2[((int64_t)k * P.rbc_idx[pt]) % twoK];
-            double xu = P.rbc_uv[4 * pt + 2], xv = P.rbc_uv[4 * pt + 3];
+    double2 du = make_double2(0.0, 0.0), dv = make_double2(0.0, 0.0);
+    const int64_t twoK = 2 * (int64_t)P.K;
+    if (k < P.K) {
+        for (int pt = q; pt < npts; pt += 8) {
+            const double2 e = __ldg(t2 + ((int64_t)k * __ldg(P.rbc_idx + pt)) % twoK);
+            const double xu = P.rbc_uv[4 * pt + 2], xv = P.rbc_uv[4 * pt + 3];
             du.x = fma(xu, e.x, du.x);
             du.y = fma(xu, e.y, du.y);
             dv.x = fma(xv, e.x, dv.x);
             dv.y = fma(xv, e.y, dv.y);
         }
-        double inv = 1.0 / (double)twoK;
+    }
+    for (int o = 4; o > 0; o >>= 1) {
+        du.x += __shfl_xor_sync(0xffffffffu, du.x, o);
+        du.y += __shfl_xor_sync(0xffffffffu, du.y, o);
+        dv.x += __shfl_xor_sync(0xffffffffu, dv.x, o);
+        dv.y += __shfl_xor_sync(0xffffffffu, dv.y, o);
+    }
+    if (q != 0 || k > P.K) return;
+    double2* al = (double2*)P.alpha;
+    double2* alp = (double2*)P.alpha_p;
+    double2 a = make_double2(0.0, 0.0), ap = a;            // alpha_K = 0
+    if (k < P.K) {
+        const double inv = 1.0 / (double)twoK;
         a = al[k];
         ap = alp[k];
         a = make_double2(fma(du.x, inv, a.x), fma(du.y, inv, a.y));
