@@ -105,6 +105,7 @@ struct wave1d_plan_s {
     int device = 0;
     int sms = 1;                      // multiprocessors of the device
     int64_t n = 0;                    // host mirror of the device step counter
+    int* h_status = nullptr;          // pinned: where the device's status word is read
     std::vector<void*> allocs;
     int64_t bytes = 0;
     bool started = false;
@@ -523,9 +524,9 @@ int enqueue_step(wave1d_plan_t p, int64_t n, const double* g_ext, double* sig_hi
 }
 
 int check_status(wave1d_plan_t p) {
-    int st = 0;
-    CK(cudaMemcpyAsync(&st, p->dp.status, sizeof(int), cudaMemcpyDeviceToHost, p->s));
+    CK(cudaMemcpyAsync(p->h_status, p->dp.status, sizeof(int), cudaMemcpyDeviceToHost, p->s));
     CK(cudaStreamSynchronize(p->s));
+    const int st = *p->h_status;
     if (st == WAVE1D_ETIMEOUT) return fail(st, "a bounded wait between the blocks of the step kernel ran out");
     if (st == WAVE1D_ENOTCONV)
         return fail(st, "the Jacobi sweeps of the implicit solve did not converge (local_weights = 1)");
@@ -690,6 +691,7 @@ int wave1d_plan(const double* x, const double* beta, int64_t M, int bc, double d
         cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming) != cudaSuccess)
         return cleanup(fail(WAVE1D_ECUDA, "stream/event creation failed"));
+    if (cudaMallocHost(&p->h_status, sizeof(int)) != cudaSuccess) return cleanup(fail(WAVE1D_ENOMEM, "pinned status word"));
     if ((rc = enter(p))) return cleanup(rc);
     if (cudaFuncSetAttribute(k_hist_cols, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)cols_phase_smem(P.L1)) != cudaSuccess)
@@ -1734,6 +1736,7 @@ int wave1d_destroy(wave1d_plan_t p) {
     if (p->nu_s) wave1d_nufft_destroy(p->nu_s);
     if (p->nu_r) wave1d_nufft_destroy(p->nu_r);
     for (void* a : p->allocs) cudaFree(a);
+    if (p->h_status) cudaFreeHost(p->h_status);
     if (p->ev_in) cudaEventDestroy(p->ev_in);
     if (p->ev_out) cudaEventDestroy(p->ev_out);
     if (p->ev_fork) cudaEventDestroy(p->ev_fork);
