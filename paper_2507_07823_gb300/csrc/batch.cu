@@ -190,13 +190,13 @@ __global__ void __launch_bounds__(kBStepThreads, 4) k_batch_step(BatchStep A) {
         const int64_t ts = (A.ns.M + kInterpTile - 1) / kInterpTile, tr = (A.nr.M + kInterpTile - 1) / kInterpTile;
         for (int64_t t = b; t < ts + tr; t += H) {
             if (t < ts) {
-                interp64_unit(t, (const double*)V[0].grid, A.u, A.ns.i0, A.ns.ker, A.ns.M, A.ns.w, A.ns.nf,
+                interp64_unit<W>(t, (const double*)V[0].grid, A.u, A.ns.i0, A.ns.ker, A.ns.M, A.ns.nf,
                               (double*)smraw);
                 const int64_t i = t * kInterpTile + threadIdx.x;
                 if (threadIdx.x < kInterpTile && i < A.ns.M) b_rhs_point(P, n, i, A.perm_s, A.u, A.inst_of, A.pulse);
             } else {
                 const int64_t tt = t - ts;
-                interp64_unit(tt, (const double*)V[0].grid, A.ur, A.nr.i0, A.nr.ker, A.nr.M, A.nr.w, A.nr.nf,
+                interp64_unit<W>(tt, (const double*)V[0].grid, A.ur, A.nr.i0, A.nr.ker, A.nr.M, A.nr.nf,
                               (double*)smraw);
                 const int64_t i = tt * kInterpTile + threadIdx.x;
                 if (threadIdx.x < kInterpTile && i < A.nr.M) P.uHr[A.perm_r[i]] = A.ur[i];
@@ -571,7 +571,7 @@ int enqueue_batch_step(wave1d_batch_t p, double* sig_hist) {
     // history part: batched FP64 spreading, per-instance FFT columns, FIR tails, rows + modes,
     // inverse columns, batched interpolation
     k_mx_gather<<<blocks(P.M, T), T, 0, s>>>(d, p->perm_s, p->c);
-    int rc = wave1d_nufft_spread(p->nu_s, p->c, p->grids);
+    int rc = nufft_spread_ranges(p->nu_s, p->c, p->grids);      // the one-launch step's units
     if (rc) return bfail(rc, std::string("batched spreading: ") + wave1d_nufft_strerror());
     const int l1 = 31 - __builtin_clz((unsigned)P.L1);
     const int t1 = std::max(32, std::min(P.L1 / 2, 512));

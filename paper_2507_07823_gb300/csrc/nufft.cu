@@ -262,6 +262,75 @@ __global__ void __launch_bounds__(kUnitThreads) k_nu_spread64(const NuRange* __r
 }
 
 // ---------------------------------------------------------------------------------------------
+// FP64 spreading of a standalone plan, in two launches over all instances.  k_nu_tap_sums: each cell's points
+// are cut into segments of at most kSegPoints, a half-warp per segment with a lane per tap, so the
+// weights (w doubles a point, the pass's stream) are read in order; the partial sums S_t of every
+// segment go to memory.  k_nu_assemble: grid real g = sum_t S_t(g - t) over the segments of w cells.
+// Bound by the FP64 pipe (90 % busy): 44 us and 9 us at 1e6 clustered points and w = 11.  The form by
+// cell ranges (spread64_unit) recomputes its halos, rounds cells up to whole groups of lanes and reads the
+// weights lane by lane, 88 bytes apart: 67 us there.  (Compensated FP32 pairs in place of FP64 here: 43 us
+// with unequal segments, as splitting each weight costs what they save.)
+// ---------------------------------------------------------------------------------------------
+constexpr int kSegPoints = 64;      // points of a segment at most
+
+template <int W>
+__global__ void __launch_bounds__(256) k_nu_tap_sums(const int32_t* __restrict__ seg, int64_t nseg,
+                                                     const double* __restrict__ c, const double* __restrict__ ker,
+                                                     double* __restrict__ S) {
+    const int64_t sg = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+    const int t = threadIdx.x & 15;
+    if (sg >= nseg || t >= W) return;
+    const int j0 = __ldg(seg + sg), np = __ldg(seg + sg + 1) - j0;
+    const double* kr = ker + (int64_t)j0 * W + t;
+    const double* cr = c + j0;
+    double out = 0.0;
+    int i = 0;
+    for (; i + 8 <= np; i += 8) {
+        double k[8], v[8];
+#pragma unroll
+        for (int p = 0; p < 8; p++) {
+            k[p] = __ldcs(kr + (i + p) * W);
+            v[p] = __ldg(cr + i + p);
+        }
+#pragma unroll
+        for (int p = 0; p < 8; p++) out = fma(k[p], v[p], out);
+    }
+    {
+        double k[7], v[7];
+#pragma unroll
+        for (int p = 0; p < 7; p++) {
+            k[p] = i + p < np ? __ldcs(kr + (i + p) * W) : 0.0;
+            v[p] = i + p < np ? __ldg(cr + i + p) : 0.0;
+        }
+#pragma unroll
+        for (int p = 0; p < 7; p++)
+            if (i + p < np) out = fma(k[p], v[p], out);
+    }
+    S[sg * W + t] = out;
+}
+
+// cseg: first segment of each cell (instance x nf + cell), one more at the end
+template <int W>
+__global__ void __launch_bounds__(256) k_nu_assemble(const int32_t* __restrict__ cseg, const double* __restrict__ S,
+                                                     double* __restrict__ grid, int64_t cells, int nf) {
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= cells) return;
+    const int64_t gb = g & ~(int64_t)(nf - 1);
+    int s0[W], s1[W];
+#pragma unroll
+    for (int t = 0; t < W; t++) {
+        const int64_t f = gb | ((g - t) & (nf - 1));
+        s0[t] = __ldg(cseg + f);
+        s1[t] = __ldg(cseg + f + 1);
+    }
+    double a = 0.0;
+#pragma unroll
+    for (int t = 0; t < W; t++)
+        for (int s = s0[t]; s < s1[t]; s++) a += __ldg(S + (int64_t)s * W + t);
+    grid[g] = a;
+}
+
+// ---------------------------------------------------------------------------------------------
 // The FFTs of the transforms (L = L1 L2 complex points per instance, z[i2 + L2 i1] -> X[k1 + L1 k2]),
 // blockIdx.y = instance: one launch per pass covers all instances.  A block takes two lines at a time
 // (two adjacent columns or rows: 32-byte pieces, and two threads per butterfly of both lines,
@@ -386,12 +455,12 @@ __global__ void __launch_bounds__(kFftThreads) k_nu_rows2(const double2* __restr
 }
 
 // FP64 interpolation, tiles of kInterpTile consecutive points (interp64_unit, nufft_units.cuh).
+template <int W>
 __global__ void __launch_bounds__(kInterpTile) k_nu_interp64(const double* __restrict__ grid, double* __restrict__ u,
                                                              const int32_t* __restrict__ i0,
-                                                             const double* __restrict__ ker, int64_t M, int w, int nf) {
-    __shared__ double ks[kInterpTile * 16];
-    const int64_t tiles = (M + kInterpTile - 1) / kInterpTile;
-    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) interp64_unit(t, grid, u, i0, ker, M, w, nf, ks);
+                                                             const double* __restrict__ ker, int64_t M, int nf) {
+    __shared__ __align__(16) double ks[kInterpTile * W];
+    interp64_unit<W>(blockIdx.x, grid, u, i0, ker, M, nf, ks);
 }
 
 // mixed interpolation (A6).  With psi_t(y) = sum_d a[t][d] T_d(y),
@@ -530,6 +599,10 @@ struct wave1d_nufft_s {
     int64_t nunits = 0;              // ranges
     int32_t* runs = nullptr;
     int range_cells = 0, range_points = 0;   // the caps the ranges were cut with
+    // FP64: segments of points (kSegPoints of one cell at most), the first one of every cell, tap sums
+    int32_t *seg = nullptr, *cseg = nullptr;
+    int64_t nseg = 0;
+    double* tap_sums = nullptr;
     std::vector<int32_t> i0_host;    // points' first cells (sorted within each instance), for re-cutting
     std::vector<int64_t> off_host;   // instance offsets
     // FFT and deconvolution
@@ -575,6 +648,15 @@ int nufft_dev64(wave1d_nufft_t h, NuDev64& out) {
     out.w = h->P.nufft_w;
     out.nf = h->P.nf;
     return WAVE1D_OK;
+}
+int nufft_spread_ranges(wave1d_nufft_t h, const double* c, double* grid) {
+    if (!h || h->precision != 0) return WAVE1D_EINVAL;
+    if (!nu_with_w(h->P.nufft_w, [&](auto wc) {
+            k_nu_spread64<decltype(wc)::value><<<(unsigned)h->nunits, kUnitThreads, 0, h->stream>>>(h->ranges, h->runs, c, h->ker,
+                                                                                             grid);
+        }))
+        return nfail(WAVE1D_EUNSUPPORTED, "kernel width not built");
+    return cudaGetLastError() == cudaSuccess ? WAVE1D_OK : nfail(WAVE1D_ECUDA, "spread launch failed");
 }
 }  // namespace wave1d
 
@@ -719,6 +801,24 @@ int wave1d_nufft_plan_many(const double* x, const int64_t* offsets, int n_inst, 
         std::vector<int32_t> runs;
         nufft_ranges(i0, offsets, n_inst, nf, w, precision == 1 ? kRangeCells : kRangeCells64,
                      precision == 1 ? kRangePoints : kRangePoints64, kEmptyCells, kUnitThreads, ranges, runs);
+        if (precision == 0) {
+            std::vector<int32_t> seg, cseg((size_t)n_inst * nf + 1, 0);
+            int64_t cell = 0;                        // cells below it know their first segment
+            for (int64_t i = 0; i < M;) {
+                int64_t e = i;
+                while (e < M && gfirst[e] == gfirst[i]) e++;
+                for (; cell <= gfirst[i]; cell++) cseg[cell] = (int32_t)seg.size();
+                const int64_t parts = (e - i + kSegPoints - 1) / kSegPoints;      // equal, as a warp takes two
+                for (int64_t q = 0; q < parts; q++) seg.push_back((int32_t)(i + (e - i) * q / parts));
+                i = e;
+            }
+            for (; cell <= (int64_t)n_inst * nf; cell++) cseg[cell] = (int32_t)seg.size();
+            h->nseg = (int64_t)seg.size();
+            seg.push_back((int32_t)M);
+            if ((rc = nu_upload(h, seg, &h->seg)) || (rc = nu_upload(h, cseg, &h->cseg)) ||
+                (rc = nu_alloc(h, (size_t)h->nseg * w, &h->tap_sums)))
+                return cleanup(rc);
+        }
         h->nunits = (int64_t)ranges.size();
         h->range_cells = precision == 1 ? kRangeCells : kRangeCells64;
         h->range_points = precision == 1 ? kRangePoints : kRangePoints64;
@@ -773,9 +873,11 @@ int wave1d_nufft_spread(wave1d_nufft_t h, const double* c, double* grid) {
     const unsigned nu = (unsigned)h->nunits;
     bool ok;
     if (h->precision == 0) {
+        const int64_t cells = (int64_t)h->B * h->P.nf;
         ok = nu_with_w(w, [&](auto wc) {
-            k_nu_spread64<decltype(wc)::value><<<nu, kUnitThreads, 0, h->stream>>>(h->ranges, h->runs, c, h->ker,
-                                                                                    grid);
+            constexpr int W = decltype(wc)::value;
+            k_nu_tap_sums<W><<<(unsigned)((h->nseg * 16 + 255) / 256), 256, 0, h->stream>>>(h->seg, h->nseg, c, h->ker, h->tap_sums);
+            k_nu_assemble<W><<<(unsigned)((cells + 255) / 256), 256, 0, h->stream>>>(h->cseg, h->tap_sums, grid, cells, h->P.nf);
         });
     } else {
         ok = nu_with_mixed(w, h->D, [&](auto wc, auto dc) {
@@ -791,8 +893,11 @@ int wave1d_nufft_interp(wave1d_nufft_t h, const double* grid, double* u) {
     if (!h || !grid || !u) return nfail(WAVE1D_EINVAL, "bad arguments");
     if (cudaSetDevice(h->device) != cudaSuccess) return nfail(WAVE1D_ECUDA, "cudaSetDevice");
     if (h->precision == 0) {
-        k_nu_interp64<<<(unsigned)((h->M + kInterpTile - 1) / kInterpTile), kInterpTile, 0, h->stream>>>(
-            grid, u, h->first, h->ker, h->M, h->P.nufft_w, h->P.nf);
+        if (!nu_with_w(h->P.nufft_w, [&](auto wc) {
+                k_nu_interp64<decltype(wc)::value><<<(unsigned)((h->M + kInterpTile - 1) / kInterpTile), kInterpTile, 0,
+                                                     h->stream>>>(grid, u, h->first, h->ker, h->M, h->P.nf);
+            }))
+            return nfail(WAVE1D_EUNSUPPORTED, "kernel width not built");
     } else if (!nu_with_mixed(h->P.nufft_w, h->D, [&](auto wc, auto dc) {
                    const unsigned nb = (unsigned)((h->M + 256 * kInterpPer - 1) / (256 * kInterpPer));
                    k_nu_interp_mixed<decltype(wc)::value, decltype(dc)::value><<<nb, 256, 0, h->stream>>>(

@@ -87,29 +87,40 @@ __device__ __forceinline__ void spread64_unit(const NuRange& u, const int32_t* _
 }
 
 // FP64 interpolation of tile t (points t kInterpTile ..): u_j = sum_u G[(i0_j + u) mod nf] ker[j][u]
-// (i0_j: instance x nf + cell).  The tile's weights (one contiguous run of np w doubles) are staged
-// through ks (kInterpTile x 16 doubles) with coalesced streaming loads, and all w grid loads of a
-// point are issued before any is used.  The block synchronises on entry and after staging.
+// (i0_j: instance x nf + cell).  The tile's weights (one contiguous run of np W doubles) are staged
+// through ks (kInterpTile x W doubles) with asynchronous copies; the points' cells and grid values are
+// loaded while they travel.  Blocks of at least kInterpTile threads, one point each.  The block
+// synchronises on entry and after staging.
+template <int W>
 __device__ __forceinline__ void interp64_unit(int64_t t, const double* __restrict__ grid, double* __restrict__ u,
                                               const int32_t* __restrict__ i0, const double* __restrict__ ker,
-                                              int64_t M, int w, int nf, double* ks) {
+                                              int64_t M, int nf, double* ks) {
     const int64_t base = t * kInterpTile;
     const int np = (int)(M - base < kInterpTile ? M - base : kInterpTile);
     __syncthreads();
-    const double* kr = ker + base * w;
-    for (int e = threadIdx.x; e < np * w; e += blockDim.x) ks[e] = __ldcs(kr + e);
-    __syncthreads();
-    for (int p = threadIdx.x; p < np; p += blockDim.x) {
-        const int64_t j = base + p;
-        const int a = __ldg(i0 + j), gb = a & ~(nf - 1);   // instance x nf + cell
-        double g[16];
+    const double* kr = ker + base * W;                  // 16-byte aligned: kInterpTile is even
+    for (int e = threadIdx.x; 2 * e < np * W; e += blockDim.x) {
+        const unsigned dst = (unsigned)__cvta_generic_to_shared(ks + 2 * e);
+        if (2 * e + 1 < np * W)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(kr + 2 * e));
+        else
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(kr + 2 * e));
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const int p = threadIdx.x;
+    double g[W];
+    if (p < np) {
+        const int a = __ldg(i0 + base + p), gb = a & ~(nf - 1);   // instance x nf + cell
 #pragma unroll
-        for (int q = 0; q < 16; q++) g[q] = q < w ? __ldg(grid + (gb | ((a + q) & (nf - 1)))) : 0.0;
+        for (int q = 0; q < W; q++) g[q] = __ldg(grid + (gb | ((a + q) & (nf - 1))));
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (p < np) {
         double acc = 0.0;
 #pragma unroll
-        for (int q = 0; q < 16; q++)
-            if (q < w) acc = fma(g[q], ks[p * w + q], acc);
-        u[j] = acc;
+        for (int q = 0; q < W; q++) acc = fma(g[q], ks[p * W + q], acc);
+        u[base + p] = acc;
     }
 }
 
@@ -125,5 +136,8 @@ struct NuDev64 {
 };
 // WAVE1D_EINVAL for a plan that is not FP64 (defined in nufft.cu)
 int nufft_dev64(wave1d_nufft_t h, NuDev64& out);
+// the spreading of an FP64 plan by its cell ranges (spread64_unit), whose sums a batch's one-launch step
+// repeats; wave1d_nufft_spread takes segments of points instead (defined in nufft.cu)
+int nufft_spread_ranges(wave1d_nufft_t h, const double* c, double* grid);
 
 }  // namespace wave1d
