@@ -237,13 +237,16 @@ struct RsDensities {
 constexpr int kRsFoldWarps = 8;
 constexpr int kRsStageRow = 8 * kRsRecord + 4;       // floats of a spring's staged records (8 intervals)
 __host__ __device__ constexpr size_t rs_fold_tile(int nk) { return (size_t)kRsAllSlices * nk * 256; }
-size_t rs_fold_smem(int nk) { return 2 * rs_fold_tile(nk) + (size_t)kRsFoldWarps * 16 * kRsStageRow * sizeof(float); }
+constexpr int kRsTileScales = 8 * kRsPowers * sizeof(float);
+size_t rs_fold_smem(int nk) {
+    return 2 * (rs_fold_tile(nk) + kRsTileScales) + (size_t)kRsFoldWarps * 16 * kRsStageRow * sizeof(float);
+}
 
 template <int NK>
 __device__ __forceinline__ void rs_fold_block(const DevPlan& P, const RangeDev& R, int s0, unsigned char* sm) {
     const int nk = NK > 0 ? NK : R.nk;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
-    const size_t tile_bytes = rs_fold_tile(nk);
+    const size_t tile_bytes = rs_fold_tile(nk) + kRsTileScales;       // slices, then the units
     float* stage = (float*)(sm + 2 * tile_bytes) + warp * 16 * kRsStageRow;
     const int64_t l0 = ((int64_t)blockIdx.x * kRsFoldWarps + warp) * 16;
     const int64_t la = min(l0 + g, P.M - 1), lb = min(l0 + g + 8, P.M - 1);
@@ -260,24 +263,32 @@ __device__ __forceinline__ void rs_fold_block(const DevPlan& P, const RangeDev& 
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
                          "l"(src + (size_t)(i >> 4) * R.nivp * 32 + (i & 15) * 16));
         }
+        if (threadIdx.x < kRsTileScales / 16) {
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(sm + buf * tile_bytes + rs_fold_tile(nk) + 16 * threadIdx.x);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
+                         "l"(R.fold_scale + (size_t)(s0 + 8 * tile) * kRsPowers + 4 * threadIdx.x));
+        }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
+    // the first m of a tile's interval of this lane
+    auto first_m = [&](int tile) { return __ldg(R.mr + 2 * min(s0 + 8 * tile + (lane & 7), R.nint - 1)); };
+    int mnext = first_m(t0);
     if (t0 < t1) fetch(t0, 0);
     for (int tile = t0; tile < t1; tile++) {
         const int buf = (tile - t0) & 1;
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();                                  // this tile has arrived, the other buffer is free
         if (tile + 1 < t1) fetch(tile + 1, buf ^ 1);
-        const int iv0 = s0 + 8 * tile;
-        const int m0 = __reduce_min_sync(0xffffffffu, __ldg(R.mr + 2 * min(iv0 + (lane & 7), R.nint - 1)));
+        const int m0 = __reduce_min_sync(0xffffffffu, mnext);
+        mnext = first_m(tile + 1);
         const int ks0 = min(nk - 1, max(0, (m0 - 1) >> 4));
         const uint2* tab = (const uint2*)(sm + buf * tile_bytes) + lane;
         const int stride = nk * 32;
-        const float* scale = R.fold_scale + (size_t)(iv0 + 2 * q) * kRsPowers;      // intervals 2q, 2q + 1
+        const float* scale = (const float*)(sm + buf * tile_bytes + rs_fold_tile(nk)) + 2 * q * kRsPowers;   // intervals 2q, 2q + 1
         // element c of a fragment: spring g + 8 (c >> 1), interval 2q + (c & 1)
         float* out = stage + g * kRsStageRow + 2 * q * kRsRecord;
         auto at = [&](int c) { return out + (c & 1) * kRsRecord + (c >> 1) * 8 * kRsStageRow; };
-        auto sc = [&](int c, int r) { return __fmul_rn(c & 2 ? sb : sa, __ldg(scale + (c & 1) * kRsPowers + r)); };
+        auto sc = [&](int c, int r) { return __fmul_rn(c & 2 ? sb : sa, scale[(c & 1) * kRsPowers + r]); };
         {
             RsAcc<0> x;
             RsAcc<5> y;
@@ -550,7 +561,10 @@ struct RsSum {
     }
 };
 
-__global__ void __launch_bounds__(kRsPairTargets, 6) k_rs_pairs(DevPlan P, RangeDev R, int s0) {
+// ten blocks to an SM (48 registers): the loads' latency is what a warp waits for.  A million clustered
+// springs 72.2 ms per step with six blocks (66 registers), 69.8 with eight, 66.2 with ten
+constexpr int kRsPairBlocks = 10;
+__global__ void __launch_bounds__(kRsPairTargets, kRsPairBlocks) k_rs_pairs(DevPlan P, RangeDev R, int s0) {
     extern __shared__ __align__(16) float4 pair_sm[];
     __shared__ float2 sPos[kRsPosChunk];
     __shared__ int sRed[2];
