@@ -133,6 +133,7 @@ struct wave1d_plan_s {
     bool range = false;
     RangeDev rd{};
     size_t rs_smem = 0, rs_slice_smem = 0, rs_fold_smem = 0;
+    int sweep_blocks = 8;                                       // cluster of the implicit sweeps (k_rs_sweeps)
     int64_t info_range_pairs = 0;
     int64_t info_terms = 0;           // (pair, m) terms of the local sum per step
     bool mixed = false;
@@ -374,13 +375,44 @@ bool is_rbc_step(const wave1d_plan_t p, int64_t n) {
     return p->hp.P.bc == WAVE1D_FREE && ((n + 1) % p->hp.P.rbc_period) == 0;
 }
 
+// blocks of the sweeps' cluster: 16 where the device takes that size, from 8192 springs (a row a thread
+// of eight blocks), else 8
+int sweep_cluster(int64_t M) {
+    if (M <= 8192) return 8;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(16);
+    cfg.blockDim = dim3(1024);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 16;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaFuncSetAttribute(k_rs_sweeps, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, k_rs_sweeps, &cfg) != cudaSuccess)
+        clusters = 0;
+    cudaGetLastError();
+    return clusters > 0 ? 16 : 8;
+}
+
 // the Jacobi sweeps of a plan without pair lists (d.rhs: their right-hand side).  Up to 2^19 pairs
 // closer than dt and 65536 springs one cluster takes all of them in one launch; larger plans need the
 // whole chip for a sweep, and mixed plans keep the order of their sums (range_fp32.cu)
 void enqueue_sweeps(wave1d_plan_t p, const DevPlan& d) {
     const int64_t M = p->hp.P.M;
     if (!p->mixed && M <= 65536 && p->hp.nb_off[M] <= (1 << 19)) {
-        k_rs_sweeps<<<8, 1024, 0, p->s>>>(d, p->rd);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)p->sweep_blocks);
+        cfg.blockDim = dim3(1024);
+        cfg.stream = p->s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)p->sweep_blocks;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        cudaLaunchKernelEx(&cfg, k_rs_sweeps, d, p->rd);      // read with the step's cudaGetLastError
         return;
     }
     const unsigned sweeps = (unsigned)std::min<int64_t>((M + 63) / 64, 16 * (int64_t)p->sms);
@@ -821,7 +853,7 @@ int wave1d_plan(const double* x, const double* beta, int64_t M, int bc, double d
         if ((rc = upload(p, hp.nb_off, &r64))) return cleanup(rc);
         rd.nb_off = r64;
         if ((rc = dalloc(p, &rd.nb_w, 2 * (size_t)std::max<int64_t>(1, hp.nb_off[P.M])))) return cleanup(rc);
-        if ((rc = dalloc(p, &rd.diag, (size_t)P.M))) return cleanup(rc);
+        if ((rc = dalloc(p, &rd.diag, (size_t)P.M)) || (rc = dalloc(p, &rd.idiag, (size_t)P.M))) return cleanup(rc);
         for (int i = 0; i < 2; i++) {
             if ((rc = zeros(p, &rd.it64[i], (size_t)P.M))) return cleanup(rc);
             if ((rc = zeros(p, &rd.it2[i], 2 * (size_t)P.M))) return cleanup(rc);
@@ -908,6 +940,7 @@ int wave1d_plan(const double* x, const double* beta, int64_t M, int bc, double d
     }
 #undef UP
     if (p->range) {
+        p->sweep_blocks = sweep_cluster(P.M);
         // the implicit part's weights (beta_j / 2) Q_0(d_jl) of every spring's dt-window
         k_rs_nearby_weights<<<(unsigned)std::min<int64_t>((P.M + 7) / 8, 64 * (int64_t)p->sms), 256, 0, p->s>>>(d, p->rd);
         // the local sum's terms per step (reported by wave1d_get_info)

@@ -369,6 +369,7 @@ struct RangeDev {
     const int64_t* nb_off;      // M + 1
     float* nb_w;                // (beta_j / 2) Q_0(d_jl) as (hi, lo), the entry l = j zero
     double* diag;               // M: 1 + (beta_j / 2) Q_0(0)
+    double* idiag;              // M: its reciprocal
     double* it64[2];            // Jacobi iterates (FP64) and the same as (hi, lo) pairs
     float* it2[2];
     unsigned long long* stats;  // [kRsMaxIter + 1][2]: max |change|, max |sigma| of each iterate (bits)

@@ -625,7 +625,11 @@ __global__ void k_rs_nearby_weights(DevPlan P, RangeDev R) {
             R.nb_w[2 * (off + k)] = pw.hi;
             R.nb_w[2 * (off + k) + 1] = pw.lo;
         }
-        if (lane == 0) R.diag[j] = 1.0 + hb * rs_q0(R, 0.0);
+        if (lane == 0) {
+            const double diag = 1.0 + hb * rs_q0(R, 0.0);
+            R.diag[j] = diag;
+            R.idiag[j] = 1.0 / diag;
+        }
     }
 }
 
@@ -762,52 +766,81 @@ __global__ void __launch_bounds__(256) k_rs_jacobi(DevPlan P, RangeDev R, int it
     }
 }
 
-// All sweeps of a small plan in one launch: a cluster of kRsCluster blocks, a thread per row (rows of
-// these plans hold a few tens of sources), the cluster's barrier between sweeps, until the stopping rule
+// All sweeps of a small plan in one launch: one cluster (8 or 16 blocks, api.cu), four lanes to a
+// row (rows of these plans hold a few tens of sources), the cluster's barrier between sweeps, until the stopping rule
 // is met.  Forty launches, of which 7 to 10 do work, cost a plan of 3e4 springs more than its sweeps, and
-// a batch runs many such plans side by side.
-constexpr int kRsCluster = 8;
-__global__ void __cluster_dims__(kRsCluster, 1, 1) __launch_bounds__(1024) k_rs_sweeps(DevPlan P, RangeDev R) {
-    __shared__ double red[2][32];
+// a batch runs many such plans side by side.  Four lanes to a row: the weights of a row lie together, and a
+// lane per row fetched 32 lines an instruction.  The FP64 epilogue (16 cycles of the SM an instruction)
+// takes 32 rows at once: the quotient by the stored reciprocal with one residual correction, the two
+// largest moduli as bit patterns on the integer pipe.  A reverse march of 3e4 springs (30 solves) 46.1 ms
+// with eight blocks, a lane per row, the division and FP64 maxima; 40.8 with sixteen blocks and the new
+// epilogue; 39.5 with four lanes to a row.
+__device__ __forceinline__ unsigned long long rs_modulus_bits(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    return b > 0x7ff0000000000000ull ? 0ull : b;       // a NaN does not count, as with fmax
+}
+__global__ void __launch_bounds__(1024) k_rs_sweeps(DevPlan P, RangeDev R) {
+    __shared__ unsigned long long red[2][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int it = 1; it <= kRsMaxIter; it++) {
         const float2* src2 = (const float2*)R.it2[(it - 1) & 1];
         const double* src = R.it64[(it - 1) & 1];
         double* dst = R.it64[it & 1];
         float2* dst2 = (float2*)R.it2[it & 1];
-        double dmax = 0.0, smax = 0.0;
-        for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P.M; j += (int64_t)gridDim.x * blockDim.x) {
-            const int lo = __ldg(R.nb_lo + j), cnt = __ldg(R.nb_cnt + j);
-            const float2* w = (const float2*)R.nb_w + __ldg(R.nb_off + j);
-            float ah = 0.f, al = 0.f, bh = 0.f, bl = 0.f;
-            int k = 0;
-            for (; k + 4 <= cnt; k += 4) {
-                float2 wv[4], sv[4];
+        unsigned long long dmax = 0, smax = 0;
+        for (int64_t j0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ll; j0 < P.M; j0 += (int64_t)gridDim.x * blockDim.x) {
+            const bool own = j0 + lane < P.M;
+            const int64_t j = own ? j0 + lane : P.M - 1;
+            const int lo = __ldg(R.nb_lo + j), cnt = own ? __ldg(R.nb_cnt + j) : 0;
+            const long long off = __ldg(R.nb_off + j);
+            const double rhs = __ldcg(P.rhs + j), prev = __ldcg(src + j), diag = __ldg(R.diag + j), inv = __ldg(R.idiag + j);
+            float sh = 0.f, sl = 0.f;
+            // four lanes a row, eight rows at a time; each row's sum goes to the row's lane
+#pragma unroll 1
+            for (int g = 0; g < 4; g++) {
+                const int r = 8 * g + (lane >> 2);
+                const int rlo = __shfl_sync(0xffffffffu, lo, r), rcnt = __shfl_sync(0xffffffffu, cnt, r);
+                const float2* w = (const float2*)R.nb_w + __shfl_sync(0xffffffffu, off, r);
+                float ah = 0.f, al = 0.f, bh = 0.f, bl = 0.f;
+                for (int k = lane & 3; k < rcnt; k += 16) {
+                    float2 wv[4], sv[4];
 #pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    wv[u] = __ldg(w + k + u);
-                    sv[u] = __ldcg(src2 + rs_spring((int64_t)lo + k + u, P.M));
+                    for (int u = 0; u < 4; u++) {
+                        const bool in = k + 4 * u < rcnt;
+                        wv[u] = in ? __ldg(w + k + 4 * u) : make_float2(0.f, 0.f);
+                        sv[u] = in ? __ldcg(src2 + rs_spring((int64_t)rlo + k + 4 * u, P.M)) : make_float2(0.f, 0.f);
+                    }
+                    rs::acc_mac(ah, al, wv[0].x, wv[0].y, sv[0].x, sv[0].y);
+                    rs::acc_mac(bh, bl, wv[1].x, wv[1].y, sv[1].x, sv[1].y);
+                    rs::acc_mac(ah, al, wv[2].x, wv[2].y, sv[2].x, sv[2].y);
+                    rs::acc_mac(bh, bl, wv[3].x, wv[3].y, sv[3].x, sv[3].y);
                 }
-                rs::acc_mac(ah, al, wv[0].x, wv[0].y, sv[0].x, sv[0].y);
-                rs::acc_mac(bh, bl, wv[1].x, wv[1].y, sv[1].x, sv[1].y);
-                rs::acc_mac(ah, al, wv[2].x, wv[2].y, sv[2].x, sv[2].y);
-                rs::acc_mac(bh, bl, wv[3].x, wv[3].y, sv[3].x, sv[3].y);
+                __syncwarp();
+                rs::acc_add(ah, al, bh, bl);
+#pragma unroll
+                for (int o = 2; o > 0; o >>= 1) {
+                    const float oh = __shfl_xor_sync(0xffffffffu, ah, o), ol = __shfl_xor_sync(0xffffffffu, al, o);
+                    rs::acc_add(ah, al, oh, ol);
+                }
+                const float th = __shfl_sync(0xffffffffu, ah, 4 * (lane & 7)), tl = __shfl_sync(0xffffffffu, al, 4 * (lane & 7));
+                if (lane >> 3 == g) {
+                    sh = th;
+                    sl = tl;
+                }
             }
-            for (; k < cnt; k++) {
-                const float2 wv = __ldg(w + k), sv = __ldcg(src2 + rs_spring((int64_t)lo + k, P.M));
-                rs::acc_mac(ah, al, wv.x, wv.y, sv.x, sv.y);
-            }
-            rs::acc_add(ah, al, bh, bl);
-            const double x = (__ldcg(P.rhs + j) - ((double)ah + (double)al)) / R.diag[j];
-            dmax = fmax(dmax, fabs(x - __ldcg(src + j)));
-            smax = fmax(smax, fabs(x));
+            if (!own) continue;
+            const double t = rhs - ((double)sh + (double)sl);
+            const double q = t * inv, x = fma(fma(-diag, q, t), inv, q);
+            dmax = max(dmax, rs_modulus_bits(x - prev));
+            smax = max(smax, rs_modulus_bits(x));
             dst[j] = x;
             const rs::Pair p2 = rs::split(x);
             dst2[j] = make_float2(p2.hi, p2.lo);
         }
+        __syncwarp();
         for (int o = 16; o > 0; o >>= 1) {
-            dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-            smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+            dmax = max(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+            smax = max(smax, __shfl_xor_sync(0xffffffffu, smax, o));
         }
         if (lane == 0) {
             red[0][wid] = dmax;
@@ -816,11 +849,11 @@ __global__ void __cluster_dims__(kRsCluster, 1, 1) __launch_bounds__(1024) k_rs_
         __syncthreads();
         if (threadIdx.x == 0) {
             for (int w = 1; w < (int)(blockDim.x >> 5); w++) {
-                dmax = fmax(dmax, red[0][w]);
-                smax = fmax(smax, red[1][w]);
+                dmax = max(dmax, red[0][w]);
+                smax = max(smax, red[1][w]);
             }
-            atomicMax(R.stats + 2 * it, (unsigned long long)__double_as_longlong(dmax));
-            atomicMax(R.stats + 2 * it + 1, (unsigned long long)__double_as_longlong(smax));
+            atomicMax(R.stats + 2 * it, dmax);
+            atomicMax(R.stats + 2 * it + 1, smax);
             __threadfence();
         }
         __syncthreads();
