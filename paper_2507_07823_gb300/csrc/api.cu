@@ -1516,6 +1516,18 @@ struct Reverse {
         const unsigned gM = blocks_for(M, 256, cap);
         cudaStream_t s = p->s;
         int rc;
+        // The transposed local sum (cbar into the slots of steps <= n) and the history part's chain (uHbar to
+        // the modes and back) share nothing until the chain's result joins slot n: the local sum runs on the
+        // plan's side stream meanwhile.  The chain's kernels leave most of the chip idle.
+        auto fork = [&] {
+            cudaEventRecord(p->ev_fork, s);
+            cudaStreamWaitEvent(p->s2, p->ev_fork, 0);
+            return p->s2;
+        };
+        auto nufft_fail = [&](int code) {
+            cudaStreamSynchronize(p->s2);              // the local sum's arrays go with this call
+            return fail(code, wave1d_nufft_strerror());
+        };
         for (int64_t n = n_hi - 1; n >= n_lo; n--) {
             const double* ub = R > 0 ? ubar + n * R : nullptr;
             if (p->range) {
@@ -1531,12 +1543,13 @@ struct Reverse {
                                                  want_beta ? gsum : nullptr, grad_g ? grad_g + n * M : nullptr, cbar, uHbar);
                 if (n == 0) break;
                 const unsigned gp = blocks_for(M, kRsPairTargets, INT32_MAX);
+                const cudaStream_t sl = fork();
                 for (int s0 = 0; s0 < rd.nint; s0 += rd.slab) {
                     const int s1 = std::min(rd.nint, s0 + rd.slab);
-                    CK(cudaMemsetAsync(rd.evec, 0, (size_t)M * rd.slab * kRsRecord * sizeof(float), s));
+                    CK(cudaMemsetAsync(rd.evec, 0, (size_t)M * rd.slab * kRsRecord * sizeof(float), sl));
                     k_rs_moments<<<dim3(gp, 1, (unsigned)((s1 - s0 + rd.part - 1) / rd.part)), kRsPairTargets,
-                                   rs_pair_smem(rd.part, rd.fine_span), s>>>(d, rd, s0, cbar);
-                    k_rs_unfold<<<dim3(blocks_for(M, 128, INT32_MAX), (unsigned)(rd.nmp / 8 + 4) / 5), 256, rs_unfold_smem(), s>>>(
+                                   rs_pair_smem(rd.part, rd.fine_span), sl>>>(d, rd, s0, cbar);
+                    k_rs_unfold<<<dim3(blocks_for(M, 128, INT32_MAX), (unsigned)(rd.nmp / 8 + 4) / 5), 256, rs_unfold_smem(), sl>>>(
                         d, rd, s0, s1, n, usum, sb);
                 }
             } else {
@@ -1544,11 +1557,13 @@ struct Reverse {
                 k_adj_solve<<<gM, 256, 0, s>>>(d, dblk, sb + (int64_t)((n + 1) % ring) * M, sig_rows + (n - row0) * M, g ? g + n * M : nullptr,
                                                want_beta ? gsum : nullptr, grad_g ? grad_g + n * M : nullptr, cbar, uHbar);
                 if (n == 0) break;
+                const cudaStream_t sl = fork();
                 if (d.l_nitems > 0)
-                    k_adj_local<<<blocks_for(M * 32, 32 * kLocalWarps, INT32_MAX), 32 * kLocalWarps, lsmem, s>>>(d, n, cbar, sb);
+                    k_adj_local<<<blocks_for(M * 32, 32 * kLocalWarps, INT32_MAX), 32 * kLocalWarps, lsmem, sl>>>(d, n, cbar, sb);
             }
+            cudaEventRecord(p->ev_join, p->s2);
             k_adj_gather<<<gM, 256, 0, s>>>(M, dperm, uHbar, cnu, p->range ? nullptr : sb + (int64_t)((n + 1) % ring) * M);
-            if ((rc = wave1d_nufft_type1(wk.nu, cnu, S1))) return fail(rc, wave1d_nufft_strerror());
+            if ((rc = wave1d_nufft_type1(wk.nu, cnu, S1))) return nufft_fail(rc);
             k_adj_modes_in<<<blocks_for(K1, 64, INT32_MAX), 64, 0, s>>>(K, S1, xr, waves, ub, R, ab);
             if (P.bc == WAVE1D_FREE && (n + 1) % P.rbc_period == 0 && npts > 0) {
                 k_adj_rbc_grid<<<npts, 256, 0, s>>>(K, npts, d.rbc_idx, d.tw2K, d.rbc_phi, d.rbc_dphi, ab, apb, uvbar);
@@ -1558,7 +1573,8 @@ struct Reverse {
                                                                                                 ab2, apb2, Sb, a2);
             std::swap(ab, ab2);
             std::swap(apb, apb2);
-            if ((rc = wave1d_nufft_type2(wk.nu, a2, unu))) return fail(rc, wave1d_nufft_strerror());
+            if ((rc = wave1d_nufft_type2(wk.nu, a2, unu))) return nufft_fail(rc);
+            cudaStreamWaitEvent(s, p->ev_join, 0);
             k_adj_scatter_add<<<gM, 256, 0, s>>>(M, dperm, unu, sb + (int64_t)(n % ring) * M);
             CK(cudaGetLastError());
         }
