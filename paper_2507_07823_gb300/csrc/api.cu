@@ -453,35 +453,37 @@ int enqueue_step(wave1d_plan_t p, int64_t n, const double* g_ext, double* sig_hi
         CK(cudaLaunchKernelEx(&cfg, k_step, d));
         return WAVE1D_OK;
     }
-    // The local sum needs only sigma^{<= n} and could overlap the history pipeline on the side
-    // stream, but on GB300 the two slow each other down (the latency-bound history kernels wait
-    // longer on an HBM the local sum keeps busy): measured 169 us per step concurrently against
-    // 143 us back to back at M = 1e4, so they run back to back.
-    bool fork = false;
+    // The local sum needs only sigma^{<= n}, the history pipeline none of it.  Plans without pair lists run
+    // the local sum on the side stream meanwhile, unless the stages are timed.  With stored weights the
+    // two slow each other down (the latency-bound history kernels wait longer on an HBM the local sum keeps
+    // busy): 169 us per step concurrently against 143 us back to back at M = 1e4, so they run back to back.
+    const bool fork = p->range && !ev;
+    cudaStream_t sl = s;
     mark(WAVE1D_STAGE_LOCAL);
     if (fork) {
         cudaEventRecord(p->ev_fork, s);
         cudaStreamWaitEvent(p->s2, p->ev_fork, 0);
-        k_local_items<<<local_grid(p), T, 0, p->s2>>>(d);
-        cudaEventRecord(p->ev_join, p->s2);
-    } else if (p->range && p->mixed) {
-        k_rs_local<<<p->rd.nblk, kRsTargets, p->rs_smem, s>>>(d, p->rd);
+        sl = p->s2;
+    }
+    if (p->range && p->mixed) {
+        k_rs_local<<<p->rd.nblk, kRsTargets, p->rs_smem, sl>>>(d, p->rd);
     } else if (p->range) {
         // local sum: the step's density slices, then per slab of intervals the e-vectors of every
         // spring and the pairs whose distances lie in the slab
         const RangeDev& r = p->rd;
-        k_rs_slices<<<blocks(P.M, 64), T, p->rs_slice_smem, s>>>(d, r);
+        k_rs_slices<<<blocks(P.M, 64), T, p->rs_slice_smem, sl>>>(d, r);
         const unsigned gx = blocks(P.M, 128);
         for (int s0 = 0; s0 < r.nint; s0 += r.slab) {
             const int s1 = std::min(r.nint, s0 + r.slab), tiles = (s1 - s0 + 7) / 8;
             const unsigned gy = (unsigned)std::max(1, std::min(tiles / 2, (int)((6u * p->sms + gx - 1) / gx)));
-            k_rs_fold<<<dim3(gx, gy), T, p->rs_fold_smem, s>>>(d, r, s0);
+            k_rs_fold<<<dim3(gx, gy), T, p->rs_fold_smem, sl>>>(d, r, s0);
             k_rs_pairs<<<dim3(blocks(P.M, kRsPairTargets), 2, (unsigned)((s1 - s0 + r.part - 1) / r.part)), kRsPairTargets,
-                         rs_pair_smem(r.part, r.fine_span), s>>>(d, r, s0);
+                         rs_pair_smem(r.part, r.fine_span), sl>>>(d, r, s0);
         }
     } else {
         k_local_items<<<local_grid(p), T, 0, s>>>(d);
     }
+    if (fork) cudaEventRecord(p->ev_join, p->s2);
     // history pipeline: spreading + forward columns | forward rows + modes (+ inverse rows) |
     // [projection] | inverse columns
     double2* Y = (double2*)d.work;
