@@ -43,12 +43,13 @@ L2_FLUSH_BYTES = 512 << 20
 # (dram__bytes_read.sum + dram__bytes_write.sum), valid only for the kernel sources it was taken
 # with: reported as roofline.traffic while their SHA-256 matches, else null
 STEP_KERNEL_SOURCES = ["step.cu", "grid_sync.cuh", "phases.cuh", "device_common.cuh", "internal.h"]
-STEP_TRAFFIC = {"sources_sha256": "0453b92af3711282c1935bfbfe99074ca9290f375d132ba9ff09e97526413ac9", "bytes_per_launch": 316612437 + 4545109}
+STEP_TRAFFIC = {"sources_sha256": "7eb459635b849cfa2fd0795fbb4a3f1fbf3ae75954968e7d6afb630d826588d3", "bytes_per_launch": 317395712 + 5562880}
 L2_CLEAN_BYTES = 256 << 20
-# DRAM bytes of one k_rs_local launch from one ncu capture of the clustered layout at M = 2e5 (its
-# pairs below), for the kernel sources it was taken with (null once they change)
-RS_LOCAL_SOURCES = ["range.cu", "range.cuh", "phases.cuh", "device_common.cuh", "internal.h"]
-RS_LOCAL_TRAFFIC = {"sources_sha256": "3b8b29ccbe01c9db3548bd9b08fc635e68d5ec064449b29392f4d5ef30967b2e", "bytes_per_launch": 71751168.0, "pairs": 2935880666}
+# DRAM bytes of one step's local sum (k_rs_slices, k_rs_fold and k_rs_pairs over all slabs) from one ncu
+# capture of the clustered layout at the springs below, for the kernel sources it was taken with (null
+# once they change)
+RS_LOCAL_SOURCES = ["range.cu", "range_dev.cuh", "range.cuh", "phases.cuh", "device_common.cuh", "internal.h"]
+RS_LOCAL_TRAFFIC = {"sources_sha256": "f7562d31d9278ed433cd5cb38c168481561408eebb2cb7704229d2cdd66d0671", "bytes_per_step": 18108773120.0, "springs": 250000}
 
 
 def _peaks():
@@ -194,7 +195,7 @@ def run_ours(args):
     launches = K * range_launches_per_step(w)
 
     # --- per-stage device times (CUDA events between the stages, K steps): the local-sum stage is
-    # exactly one launch of k_rs_local, which gives its per-launch time for the roofline ---------
+    # the density slices and, per slab of intervals, the fold and the pair kernel ------------------
     wave1d.wave1d_profile(plan.h, 1)
     for i in range(K):
         wave1d._check(wave1d.wave1d_step(plan.h), "wave1d_step")
@@ -219,20 +220,21 @@ def run_ours(args):
     e2e_value = w.M * K * world / e2e_s
     plan.close()
 
-    # --- roofline of the dominant kernel, k_rs_local: bound by FP32 issue, not by HBM.  Algorithmic
-    # work per launch: the local sum's multiply-adds Q_m(d) sigma (info.local_terms, 2 flops each),
+    # --- roofline of the local sum (k_rs_fold on the tensor cores, k_rs_pairs in FP32, the larger part):
+    # bound by FP32 issue, not by HBM.  Algorithmic work per step: the local sum's multiply-adds
+    # Q_m(d) sigma (info.local_terms, 2 flops each),
     # the work the method does whatever the arithmetic; peak: 152 SMs x 128 FP32 lanes x 2 flops x
     # the maximum SM clock.
     fp32_peak, clk_src = _fp32_peak()
     ms_local = per_step["local"]
     achieved = 2.0 * info.local_terms / (ms_local * 1e-3) / 1e12
-    roof = {"kernel": "k_rs_local", "bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
+    roof = {"kernel": "k_rs_slices + k_rs_fold + k_rs_pairs (one step)", "bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
             "frac": achieved / fp32_peak, "traffic": rs_local_traffic(info),
             "peak_source": f"derived: 152 SMs x 128 FP32 lanes x 2 flops x {clk_src}",
             "algorithmic_flops_per_launch": 2.0 * info.local_terms, "launch_ms": ms_local,
             "local_pairs": info.local_pairs, "local_terms": info.local_terms,
             "pairs_per_s": info.local_pairs / (ms_local * 1e-3),
-            "timing": "CUDA events around the local-sum stage (one k_rs_local launch) of K profiled steps",
+            "timing": "CUDA events around the local-sum stage (all its launches of a step) of K profiled steps",
             "arithmetic": "compensated FP32 pairs (about 48 significant bits); 2 flops per term counts only the "
                           "multiply-add of the method, not the compensation or the weights' polynomials"}
 
@@ -245,7 +247,8 @@ def run_ours(args):
                    "local_pairs": info.local_pairs, "nearby_pairs": info.nearby_pairs,
                    "plan": "local_weights = 1: no pair lists (local sum over sorted index windows with "
                            "weights from distance polynomials, implicit part by Jacobi sweeps)",
-                   "arithmetic": "local sum in compensated FP32 pairs (k_rs_local); history part (NUFFTs, "
+                   "arithmetic": "local sum in compensated FP32 pairs (k_rs_pairs) on e-vectors folded exactly on the "
+                                 "tensor cores (k_rs_fold, 11-bit integer slices); history part (NUFFTs, "
                                  "FFTs, mode recurrence), implicit solve and receivers in FP64",
                    "parallelism": f"replicas x{world}",
                    "l2": "not flushed: every step reads the 3.6 GB of implicit-part weights and the 0.84 GB "
@@ -291,12 +294,17 @@ def run_ours(args):
         dist.destroy_process_group()
 
 
-def range_launches_per_step(w):
-    """Kernel launches of one step of a plan without pair lists: the local sum, five history-part
-    launches (spreading + FFT columns, FIR tail, FFT rows + mode update, inverse FFT columns,
-    interpolation), the solve's set-up, its 40 Jacobi sweep launches (those after convergence return
-    at once), the store, the receivers' local part (with receivers) and the finishing launch."""
-    return 1 + 5 + 1 + 40 + 1 + (1 if len(w.xr) else 0) + 1
+def range_launches_per_step(w, intervals=484):
+    """Kernel launches of one step of the clustered plan without pair lists: the density slices, a fold
+    and a pair launch per slab of intervals, five history-part launches (spreading + FFT columns, FIR
+    tail, FFT rows + mode update, inverse FFT columns, interpolation), the solve's set-up, its 40 Jacobi
+    sweep launches (those after convergence return at once), the store, the receivers' local part (with
+    receivers) and the finishing launch.  Slabs: 64 intervals at a time (one part) of the 484 at dt =
+    5e-4, tol 1e-10, p = 4, as many parts as 4 GiB of 48-byte records (16 KB a spring) hold."""
+    part = 64
+    slab = max(1, int(min(16384 * w.M, 4 << 30) / (48 * w.M)) // 16 * 16 // part) * part
+    slabs = -(-intervals // slab)
+    return 1 + 2 * slabs + 5 + 1 + 40 + 1 + (1 if len(w.xr) else 0) + 1
 
 
 def periodic_gaussians(w, tt):
@@ -377,10 +385,10 @@ def free_space_secondary(torch, stream):
 
 
 def rs_local_traffic(info):
-    """DRAM bytes per k_rs_local launch at this workload, scaled by pairs from one ncu capture of a
-    smaller clustered case (M = 2.5e5 in 4 clusters, the million-spring cluster density; the
-    kernel's DRAM bytes are the window densities and positions it reads, which grow with the pairs),
-    while the kernel sources match the ones it was taken with."""
+    """DRAM bytes of the local sum of one step at this workload, scaled by springs from one ncu capture
+    of a smaller clustered case (M = 2.5e5 in 4 clusters, the million-spring cluster density; the bytes
+    are the e-vector records, a fixed number per spring), while the kernel sources match the ones it was
+    taken with."""
     import hashlib
     h = hashlib.sha256()
     src = os.path.join(ROOT, "paper_2507_07823_gb300", "csrc")
@@ -389,7 +397,7 @@ def rs_local_traffic(info):
             h.update(fh.read())
     if h.hexdigest() != RS_LOCAL_TRAFFIC["sources_sha256"]:
         return None
-    return RS_LOCAL_TRAFFIC["bytes_per_launch"] * info.local_pairs / RS_LOCAL_TRAFFIC["pairs"]
+    return RS_LOCAL_TRAFFIC["bytes_per_step"] * info.M / RS_LOCAL_TRAFFIC["springs"]
 
 
 def spread_interp_million(torch, stream, flush_l2, hbm, reps=20):
@@ -940,7 +948,7 @@ def run_free_only(args):
 
 
 def run_local_only(args):
-    """The local sum of the plan without pair lists alone (k_rs_local) on the clustered recipe at
+    """The local sum of the plan without pair lists alone (k_rs_slices, k_rs_fold, k_rs_pairs) on the clustered recipe at
     --local-M springs in --local-clusters clusters (50,000 springs per cluster keeps the million-
     spring workload's cluster density), or with --local-uniform on a uniform instance of the
     batched workload's recipe: 2 steps, then 3 profiled steps.  The small cases the kernel's full

@@ -14,7 +14,8 @@
 //   k_rs_jacobi     Jacobi sweeps of (I + S) sigma^{n+1} = rhs (eq. linearSystem), S_jl =
 //                   (beta_j / 2) Q_0(d_jl) over the sources closer than dt, until the largest
 //                   change is below kRsTol of the largest density (launches after that return at
-//                   once, so the step is a fixed sequence of launches and can be captured)
+//                   once, so the step is a fixed sequence of launches and can be captured);
+//                   k_rs_sweeps: all of them in one launch, for small plans
 //   k_rs_store      sigma^{n+1} into the rings (status WAVE1D_ENOTCONV if no sweep converged)
 //   k_rs_receivers  u_L at the receivers (eq. localSol2, all m including m = 0), FP64
 //   k_rs_finish     u = u_L + u_H at the receivers, step counter
