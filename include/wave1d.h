@@ -314,7 +314,7 @@ int wave1d_adjoint_checkpointed(wave1d_plan_t plan, int64_t nsteps, int64_t inte
  *       Allocates the plan's device arrays.
  *   Point arrays (c, u) are device arrays of M FP64 in the plan's point order: point i is the
  *   caller's point perm[i] (wave1d_nufft_perm, host array of M).  S and alpha: device, K + 1
- *   complex (re, im interleaved).  grid: device, nf reals (wave1d_nufft_info).  Calls are queued on
+ *   complex (re, im interleaved), aligned to 8 bytes like every array.  grid: device, nf reals (wave1d_nufft_info).  Calls are queued on
  *   the plan's stream and do not synchronise; the plan owns its work arrays, so calls on one plan
  *   must not overlap.
  * Returns WAVE1D_EINVAL for bad arguments, WAVE1D_ENOMEM / WAVE1D_ECUDA on CUDA failures

@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(kFftThreads) k_nu_rows1(const double2* __restr
     extern __shared__ __align__(16) double2 nu_sm[];
     double2 *a = nu_sm, *b = nu_sm + L2, *twN = nu_sm + 2 * L2;
     const double2* Y = works + (int64_t)blockIdx.y * L;
-    double2* S = (double2*)Ss + (int64_t)blockIdx.y * (K + 1);
+    double* S = Ss + (int64_t)blockIdx.y * 2 * (K + 1);
     const int logL2 = 31 - __clz(L2), k1 = blockIdx.x, k1p = (L1 - k1) % L1;
     const bool pair = k1p != k1;
     nu_line_twiddles(twN, tw, L, L2, 1);
@@ -432,7 +432,9 @@ __global__ void __launch_bounds__(kFftThreads) k_nu_rows1(const double2* __restr
         const double2 E = make_double2(0.5 * (zk.x + zm.x), 0.5 * (zk.y - zm.y));
         const double2 D = make_double2(0.5 * (zk.x - zm.x), 0.5 * (zk.y + zm.y));
         const double2 O = make_double2(D.y, -D.x);
-        S[k] = cadd(make_double2(f0 * E.x, f0 * E.y), cmul(make_double2(__ldg(f + 1), __ldg(f + 2)), O));
+        const double2 s = cadd(make_double2(f0 * E.x, f0 * E.y), cmul(make_double2(__ldg(f + 1), __ldg(f + 2)), O));
+        S[2 * k] = s.x;                       // the caller's array: aligned to a double, no more
+        S[2 * k + 1] = s.y;
     }
 }
 
