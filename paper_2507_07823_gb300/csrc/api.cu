@@ -352,11 +352,7 @@ int fold_tables(wave1d_plan_t p) {
     if ((rc = dalloc(p, &rd.csum, (size_t)4 * rd.nparts * P.M))) return rc;
     p->rs_slice_smem = (size_t)(rt.nm - 1) * 64 * sizeof(float2);
     p->rs_fold_smem = rs_fold_smem(rt.nk);
-    // all a block may have, for every plan: the attribute belongs to the kernel, not the plan
-    const int most = 227 * 1024;
-    if (p->rs_fold_smem > (size_t)most || p->rs_slice_smem > (size_t)most - 1024 ||
-        cudaFuncSetAttribute(k_rs_fold, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
-        cudaFuncSetAttribute(k_rs_slices, cudaFuncAttributeMaxDynamicSharedMemorySize, most - 1024) != cudaSuccess)
+    if (!allow_smem((const void*)k_rs_fold, p->rs_fold_smem) || !allow_smem((const void*)k_rs_slices, p->rs_slice_smem))
         return fail(WAVE1D_ECUDA, "cannot size the shared memory of the range-mode local sum");
     return WAVE1D_OK;
 }
@@ -727,8 +723,7 @@ int wave1d_plan(const double* x, const double* beta, int64_t M, int bc, double d
         return cleanup(fail(WAVE1D_ECUDA, "stream/event creation failed"));
     if (cudaMallocHost(&p->h_status, sizeof(int)) != cudaSuccess) return cleanup(fail(WAVE1D_ENOMEM, "pinned status word"));
     if ((rc = enter(p))) return cleanup(rc);
-    if (cudaFuncSetAttribute(k_hist_cols, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)cols_phase_smem(P.L1)) != cudaSuccess)
+    if (!allow_smem((const void*)k_hist_cols, cols_phase_smem(P.L1)))
         return cleanup(fail(WAVE1D_ECUDA, "cannot size the shared memory of the column pass"));
     // one-launch step kernel: as many blocks as are resident at once, the history group one block
     // per column / row pair
@@ -736,7 +731,7 @@ int wave1d_plan(const double* x, const double* beta, int64_t M, int bc, double d
         size_t sm = std::max({cols_phase_smem(P.L1), rows_phase_smem(P.L2), icols_phase_smem(P.L1),
                               (size_t)kSolveStage * sizeof(double) * (kStepThreads / 32)});
         int occ = 0;
-        if (cudaFuncSetAttribute(k_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
+        if (!allow_smem((const void*)k_step, sm) ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step, kStepThreads, sm) != cudaSuccess)
             return cleanup(fail(WAVE1D_ECUDA, "cannot configure the step kernel"));
         int coop = 0;
@@ -864,8 +859,7 @@ int wave1d_plan(const double* x, const double* beta, int64_t M, int bc, double d
         if ((rc = zeros(p, &rd.iters, 1))) return cleanup(rc);
         if (o.precision == 1) {
             p->rs_smem = rs_local_smem(rt.nint, rt.nm);
-            if (cudaFuncSetAttribute(k_rs_local, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->rs_smem) !=
-                cudaSuccess)
+            if (!allow_smem((const void*)k_rs_local, p->rs_smem))
                 return cleanup(fail(WAVE1D_ECUDA, "cannot size the shared memory of the range-mode local sum"));
         } else {
             if ((rc = fold_tables(p))) return cleanup(rc);
@@ -1495,14 +1489,14 @@ struct Reverse {
                 p->rd.nis = hp.rt.nis;
                 p->rd.nmp = hp.rt.nmp;
                 p->rd.unfold = h16;
-                CK(cudaFuncSetAttribute(k_rs_unfold, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs_unfold_smem()));
+                if (!allow_smem((const void*)k_rs_unfold, rs_unfold_smem()))
+                    return fail(WAVE1D_ECUDA, "cannot size the shared memory of the transposed local sum");
             }
             return wk.zeros(&usum, (size_t)M * p->rd.nmp);
         }
         lsmem = adj_local_smem(P.m_max, kLocalWarps);
-        if (lsmem > 227 * 1024) return fail(WAVE1D_EUNSUPPORTED, "window too long for the adjoint's local-sum accumulators");
-        if (lsmem > 48 * 1024)
-            CK(cudaFuncSetAttribute(k_adj_local, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsmem));
+        if (!allow_smem((const void*)k_adj_local, lsmem))
+            return fail(WAVE1D_EUNSUPPORTED, "window too long for the adjoint's local-sum accumulators");
         return WAVE1D_OK;
     }
 

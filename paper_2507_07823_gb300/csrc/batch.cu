@@ -503,7 +503,7 @@ int setup_batch_step(wave1d_batch_t p, const wave1d_opts& o) {
     const size_t sm = std::max({spread, kInterp64Smem, fft_smem_bytes(P.L1), rows_phase_smem(P.L2),
                                 icols_phase_smem(P.L1), (size_t)kSolveStage * sizeof(double) * (kBStepThreads / 32)});
     int occ = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
+    if (!allow_smem(fn, sm) ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kBStepThreads, sm) != cudaSuccess)
         return bfail(WAVE1D_ECUDA, "cannot configure the batched step kernel");
     if (occ < 1) return WAVE1D_OK;
@@ -624,12 +624,9 @@ int upload_joined_part(wave1d_batch_t p, const std::vector<int>& joined, const d
         if ((rc = wave1d_nufft_perm(p->nu_r, permr.data()))) return bfail(rc, wave1d_nufft_strerror());
         if ((rc = bupload(p, permr, &p->perm_r)) || (rc = balloc(p, &p->ur, (size_t)P.R))) return rc;
     }
-    if (cudaFuncSetAttribute(k_bhist_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_phase_smem(P.L2)) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(k_bfft_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fft_smem_bytes(P.L1)) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(k_bhist_icols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)icols_phase_smem(P.L1)) !=
-            cudaSuccess)
+    if (!allow_smem((const void*)k_bhist_rows, rows_phase_smem(P.L2)) ||
+        !allow_smem((const void*)k_bfft_cols, fft_smem_bytes(P.L1)) ||
+        !allow_smem((const void*)k_bhist_icols, icols_phase_smem(P.L1)))
         return bfail(WAVE1D_ECUDA, "cannot size the shared memory of the history passes");
     p->g.spin_limit = o.spin_limit > 0 ? (unsigned)o.spin_limit : (1u << 22);
     return setup_batch_step(p, o);

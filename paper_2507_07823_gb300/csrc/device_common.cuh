@@ -9,6 +9,20 @@
 
 namespace wave1d {
 
+// Lets the launches of a kernel take all the dynamic shared memory that a block may have beside the
+// kernel's own arrays; false where that is less than `need`.  The limit belongs to the kernel and the device,
+// not to a plan: set to one plan's need, it would refuse the launches of an open plan that needs more.
+inline bool allow_smem(const void* kernel, size_t need) {
+    int dev = 0, most = 0;
+    cudaFuncAttributes a;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaFuncGetAttributes(&a, kernel) != cudaSuccess ||
+        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+        return false;
+    most -= (int)a.sharedSizeBytes;
+    return need <= (size_t)most &&
+           cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess;
+}
+
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {

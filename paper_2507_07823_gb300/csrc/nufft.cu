@@ -841,13 +841,9 @@ int wave1d_nufft_plan_many(const double* x, const int64_t* offsets, int n_inst, 
     if ((rc = nu_upload(h, mf, &h->modefac)) || (rc = nu_upload(h, tw, &h->twiddle)) ||
         (rc = nu_alloc(h, (size_t)n_inst * nf, &h->grid)) || (rc = nu_alloc(h, (size_t)h->group * nf, &h->work)))
         return cleanup(rc);
-    // the largest line (2048 points) for every plan: the attribute belongs to the kernel, not the plan
-    const int most = (int)nu_fft_smem(2048);
-    if (cudaFuncSetAttribute(k_nu_cols1, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
-        cudaFuncSetAttribute(k_nu_cols2, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
-        cudaFuncSetAttribute(k_nu_rows1, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
-        cudaFuncSetAttribute(k_nu_rows2, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess)
-        return cleanup(nfail(WAVE1D_ECUDA, "cannot size the shared memory of the FFT passes"));
+    for (const void* k : {(const void*)k_nu_cols1, (const void*)k_nu_cols2, (const void*)k_nu_rows1, (const void*)k_nu_rows2})
+        if (!allow_smem(k, nu_fft_smem(std::max(P.L1, P.L2))))
+            return cleanup(nfail(WAVE1D_ECUDA, "cannot size the shared memory of the FFT passes"));
     if (cudaDeviceSynchronize() != cudaSuccess) return cleanup(nfail(WAVE1D_ECUDA, "upload failed"));
     *out = h;
     return WAVE1D_OK;
