@@ -61,8 +61,8 @@ __global__ void k_mx_rhs(DevPlan P, const int64_t* perm, const double* u);
 __global__ void k_mx_receivers(int64_t R, const int64_t* perm, const double* u, double* uHr);
 __global__ void k_rs_local(DevPlan P, RangeDev R);
 size_t rs_local_smem(int nint, int nm);
-__global__ void k_rs_slices(DevPlan P, RangeDev R);
 __global__ void k_rs_fold(DevPlan P, RangeDev R, int s0);
+__global__ void k_rs_fold_long(DevPlan P, RangeDev R, int s0);
 __global__ void k_rs_pairs(DevPlan P, RangeDev R, int s0);
 size_t rs_pair_smem(int part, int fine_span);
 __global__ void k_rs_moments(DevPlan P, RangeDev R, int s0, const double* cbar);
@@ -81,7 +81,11 @@ __global__ void k_rs_receivers(DevPlan P, RangeDev R);
 __global__ void k_rs_finish(DevPlan P, RangeDev R);
 int rs_receiver_chunks(int64_t window);
 __global__ void k_rs_count_terms(DevPlan P, RangeDev R, unsigned long long* total);
-size_t rs_fold_smem(int nk);
+size_t rs_fold_smem(int nm, bool copied);
+__global__ void k_rs_fold_used(DevPlan P, RangeDev R, int s0);
+__global__ void k_rs_mark_used(DevPlan P, RangeDev R);
+size_t rs_used_smem(int nm);
+int rs_used_blocks(int intervals);
 }  // namespace wave1d
 
 using namespace wave1d;
@@ -132,7 +136,8 @@ struct wave1d_plan_s {
     // from their polynomials in the distance, implicit part solved by Jacobi sweeps (range.cu)
     bool range = false;
     RangeDev rd{};
-    size_t rs_smem = 0, rs_slice_smem = 0, rs_fold_smem = 0;
+    size_t rs_smem = 0, rs_fold_smem = 0;
+    bool fold_copied = true;                                    // the fold's coefficients fit its shared memory
     int sweep_blocks = 8;                                       // cluster of the implicit sweeps (k_rs_sweeps)
     int64_t info_range_pairs = 0;
     int64_t info_terms = 0;           // (pair, m) terms of the local sum per step
@@ -308,7 +313,7 @@ int upload_receivers(wave1d_plan_t p) {
     return WAVE1D_OK;
 }
 
-// the tables and work arrays of the range-mode local sum on the tensor cores (range.cu)
+// the tables and work arrays of the range-mode local sum (range.cu)
 int fold_tables(wave1d_plan_t p) {
     const RangeTables& rt = p->hp.rt;
     const Params& P = p->hp.P;
@@ -316,15 +321,8 @@ int fold_tables(wave1d_plan_t p) {
     int rc;
     float* f32;
     uint16_t* h16;
-    rd.nk = rt.nk;
-    rd.nivp = rt.nivp;
-    rd.fold_shift = rt.fold_shift;
-    if ((rc = upload(p, rt.fold, &h16))) return rc;
-    rd.fold = h16;
     if ((rc = upload(p, rt.fold_scale, &f32))) return rc;
     rd.fold_scale = f32;
-    if ((rc = dalloc(p, &rd.slices, (size_t)P.M * kRsSlices * rt.nk * 16))) return rc;
-    if ((rc = dalloc(p, &rd.slice_scale, (size_t)P.M))) return rc;
     if ((rc = upload(p, rt.fine, &h16))) return rc;
     rd.fine = h16;
     rd.fine_span = rt.fine_span;
@@ -350,9 +348,19 @@ int fold_tables(wave1d_plan_t p) {
     rd.nparts = (rt.nint + rd.part - 1) / rd.part;
     if ((rc = dalloc(p, &rd.evec, (size_t)P.M * rd.slab * kRsRecord))) return rc;
     if ((rc = dalloc(p, &rd.csum, (size_t)4 * rd.nparts * P.M))) return rc;
-    p->rs_slice_smem = (size_t)(rt.nm - 1) * 64 * sizeof(float2);
-    p->rs_fold_smem = rs_fold_smem(rt.nk);
-    if (!allow_smem((const void*)k_rs_fold, p->rs_fold_smem) || !allow_smem((const void*)k_rs_slices, p->rs_slice_smem))
+    // where there is less than a pair to a record, only the records that some pair reads are made
+    if ((double)p->hp.range_pairs < (double)P.M * rt.nint) {
+        rd.used_words = (rt.nint + 31) / 32;
+        if ((rc = zeros(p, &rd.used, (size_t)P.M * rd.used_words))) return rc;
+        p->rs_fold_smem = rs_used_smem(rt.nm);
+        if (!allow_smem((const void*)k_rs_fold_used, p->rs_fold_smem))
+            return fail(WAVE1D_ECUDA, "cannot size the shared memory of the range-mode local sum");
+        return WAVE1D_OK;
+    }
+    p->rs_fold_smem = rs_fold_smem(rt.nm, true);
+    p->fold_copied = allow_smem((const void*)k_rs_fold, p->rs_fold_smem);
+    if (!p->fold_copied) p->rs_fold_smem = rs_fold_smem(rt.nm, false);
+    if (!p->fold_copied && !allow_smem((const void*)k_rs_fold_long, p->rs_fold_smem))
         return fail(WAVE1D_ECUDA, "cannot size the shared memory of the range-mode local sum");
     return WAVE1D_OK;
 }
@@ -464,15 +472,15 @@ int enqueue_step(wave1d_plan_t p, int64_t n, const double* g_ext, double* sig_hi
     if (p->range && p->mixed) {
         k_rs_local<<<p->rd.nblk, kRsTargets, p->rs_smem, sl>>>(d, p->rd);
     } else if (p->range) {
-        // local sum: the step's density slices, then per slab of intervals the e-vectors of every
-        // spring and the pairs whose distances lie in the slab
+        // local sum, per slab of intervals: the e-vectors of every spring and the pairs whose distances
+        // lie in the slab
         const RangeDev& r = p->rd;
-        k_rs_slices<<<blocks(P.M, 64), T, p->rs_slice_smem, sl>>>(d, r);
-        const unsigned gx = blocks(P.M, 128);
+        const unsigned gx = blocks(P.M, 32);
         for (int s0 = 0; s0 < r.nint; s0 += r.slab) {
             const int s1 = std::min(r.nint, s0 + r.slab), tiles = (s1 - s0 + 7) / 8;
-            const unsigned gy = (unsigned)std::max(1, std::min(tiles / 2, (int)((6u * p->sms + gx - 1) / gx)));
-            k_rs_fold<<<dim3(gx, gy), T, p->rs_fold_smem, sl>>>(d, r, s0);
+            const unsigned gy = (unsigned)std::max(1, std::min(tiles / 2, (int)((24u * p->sms + gx - 1) / gx)));
+            if (r.used) k_rs_fold_used<<<dim3(gx, (unsigned)rs_used_blocks(s1 - s0)), T, p->rs_fold_smem, sl>>>(d, r, s0);
+            else (p->fold_copied ? k_rs_fold : k_rs_fold_long)<<<dim3(gx, gy), T, p->rs_fold_smem, sl>>>(d, r, s0);
             k_rs_pairs<<<dim3(blocks(P.M, kRsPairTargets), 2, (unsigned)((s1 - s0 + r.part - 1) / r.part)), kRsPairTargets,
                          rs_pair_smem(r.part, r.fine_span), sl>>>(d, r, s0);
         }
@@ -824,10 +832,8 @@ int wave1d_plan(const double* x, const double* beta, int64_t M, int bc, double d
         rd.bp2 = f32;
         if ((rc = upload(p, rt.ih, &f32))) return cleanup(rc);
         rd.ih = f32;
-        if (o.precision == 1) {
-            if ((rc = upload(p, rt.coef, &f32))) return cleanup(rc);
-            rd.coef = f32;
-        }
+        if ((rc = upload(p, rt.coef, &f32))) return cleanup(rc);
+        rd.coef = f32;
         if ((rc = upload(p, mr, &r32))) return cleanup(rc);
         rd.mr = r32;
         if ((rc = upload(p, mr0, &r32))) return cleanup(rc);
@@ -939,6 +945,9 @@ int wave1d_plan(const double* x, const double* beta, int64_t M, int bc, double d
         p->sweep_blocks = sweep_cluster(P.M);
         // the implicit part's weights (beta_j / 2) Q_0(d_jl) of every spring's dt-window
         k_rs_nearby_weights<<<(unsigned)std::min<int64_t>((P.M + 7) / 8, 64 * (int64_t)p->sms), 256, 0, p->s>>>(d, p->rd);
+        if (p->rd.used)
+            k_rs_mark_used<<<dim3((unsigned)((P.M + kRsPairTargets - 1) / kRsPairTargets), 2, (unsigned)p->rd.nparts), kRsPairTargets,
+                             rs_pair_smem(p->rd.part, p->rd.fine_span), p->s>>>(d, p->rd);
         // the local sum's terms per step (reported by wave1d_get_info)
         unsigned long long* cnt;
         if ((rc = zeros(p, &cnt, 1))) return cleanup(rc);
@@ -1482,7 +1491,7 @@ struct Reverse {
         }
         if (p->range) {
             if ((rc = wk.zeros(&rrhs, (size_t)M))) return rc;
-            if (!p->rd.fold && (rc = fold_tables(p))) return rc;        // a mixed plan's first reverse march
+            if (!p->rd.evec && (rc = fold_tables(p))) return rc;        // a mixed plan's first reverse march
             if (!p->rd.unfold) {
                 uint16_t* h16;
                 if ((rc = upload(p, hp.rt.unfold, &h16))) return rc;

@@ -346,12 +346,7 @@ struct RangeDev {
     const double* cheb;         // [iv][m][8] Chebyshev coefficients in z (FP64)
     const int* cell;            // kRsCells: first interval of each cell of [0, delta)
     float cell_scale;           // kRsCells / delta
-    int fold_shift;             // RangeTables::fold_shift
-    int nk, nivp;               // steps of 16 m, padded intervals of the fold's table
-    const uint16_t* fold;       // coefficient slices (RangeTables::fold)
     const float* fold_scale;    // [nivp][8]
-    uint16_t* slices;           // [M][kRsSlices][nk][16] halves: the step's density slices
-    float* slice_scale;         // M: their scales
     int nis, nmp;               // steps of 16 intervals and padded m of the transposed sum's table
     const uint16_t* unfold;     // coefficient slices (RangeTables::unfold)
     int slab;                   // intervals whose e-vectors are held at once (a multiple of 16)
@@ -363,6 +358,8 @@ struct RangeDev {
     int fine_span;
     float fine_scale;           // kRsFineCells / delta
     float* csum;                // [nparts][2][M]: per part and side, each target's sum as a pair
+    unsigned* used;             // [M][used_words] bits: the records that some pair reads; null: all are made
+    int used_words;
     const int32_t* blk_win;     // [block][4] (see HostPlan::blk_win)
     const int32_t* nb_lo;       // M
     const int32_t* nb_cnt;      // M

@@ -3,9 +3,8 @@
 // weights Q_m(d) (Sec. 4.1) come from their polynomials in the distance (range.cuh).  One step:
 //
 //   local explicit sum c_j over m >= 1 (Sec. 4.1), compensated FP32 pairs:
-//     k_rs_slices   the step's densities as 11-bit slices (operands of the fold)
 //     per slab of intervals of the distance:
-//     k_rs_fold     e-vectors of every spring and interval on the tensor cores
+//     k_rs_fold     e-vectors of every spring and interval (k_rs_fold_used: those that some pair reads)
 //     k_rs_pairs    the polynomials of all pairs whose distance lies in the slab
 //   (k_rs_local, range_fp32.cu, with FP32 spreading and interpolation)
 //   history pipeline (type-1 NUFFT, mode update, [projection], type-2 NUFFT): the per-stage
@@ -70,295 +69,174 @@ __device__ __forceinline__ double rs_q0(const RangeDev& R, double d) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// The fold e_{l,iv,r} = sum_m a_{iv,m,r} sigma_l^{n+1-m} is a contraction over m with the same
-// coefficients for every source, so it runs on the tensor cores: A = densities (16 sources x 16 m),
-// B = coefficients (16 m x 8 intervals).  To keep the pairs' precision both operands are split into
-// slices of 11 bits, whole numbers of at most 1024 that halves hold exactly (sigma = 2^(e-10)
-// sum_i s_i 2^(-11 i), one exponent per source; coefficients likewise, one per (interval, r)).  The
-// product of slices i and j is a whole number, products of equal i + j share an accumulator, and
-// every partial sum stays below 2^24 (sum_m |a_m| is about 11 times the largest |a_m|; longer windows
-// take larger units, fold_shift), so FP32 accumulation is exact; what is dropped lies below 2^-43 of the largest |a sigma| of the source and
-// interval for e_0, and by as many bits less for the higher powers as their coefficients are smaller.
-// ---------------------------------------------------------------------------------------------
-
-// the step's density slices of every spring: sigma^{n+1-m}, m = 1 .. 16 nk (zero past m_max), a row
-// of [slice][step of 16 m][16] halves in the order of RangeTables::fold.  A block takes 64 springs:
-// the ring rows are read coalesced into shared memory, then a thread makes the slices of eight m.
-constexpr int kRsSliceSprings = 64;
-__global__ void __launch_bounds__(256) k_rs_slices(DevPlan P, RangeDev R) {
-    extern __shared__ __align__(16) float2 sl_sm[];          // [m_max][kRsSliceSprings]
-    __shared__ float sUnit[kRsSliceSprings], sInv[kRsSliceSprings];
-    const int64_t n = load_step(P), l0 = (int64_t)blockIdx.x * kRsSliceSprings;
-    const int t = threadIdx.x, mm = R.nm - 1;
-    for (int i = t; i < mm * kRsSliceSprings; i += blockDim.x) {
-        const int k = i & (kRsSliceSprings - 1), m = 1 + i / kRsSliceSprings;
-        float2 v = make_float2(0.f, 0.f);
-        if (l0 + k < P.M) v = __ldg((const float2*)P.sig2 + (int64_t)ring_slot(n + 1 - m, P.ring) * P.M + l0 + k);
-        sl_sm[i] = v;
-    }
-    __syncthreads();
-    {
-        // the largest magnitude of the spring's history (as bits: a NaN sorts above every number),
-        // four threads per spring
-        const int k = t >> 2;
-        unsigned mx = 0;
-        for (int m = t & 3; m < mm; m += 4) mx = max(mx, __float_as_uint(sl_sm[m * kRsSliceSprings + k].x) & 0x7fffffffu);
-        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        // units of 2^(E-10); a non-finite density makes the scale NaN, so every sum it enters is NaN
-        const int E = min(127, rs::slice_exponent(mx) + R.fold_shift);
-        const bool fin = mx < 0x7f800000u;
-        if ((t & 3) == 0) {
-            sInv[k] = __uint_as_float((unsigned)(127 + 10 - E) << 23);
-            sUnit[k] = fin ? __uint_as_float((unsigned)(127 + E - 10) << 23) : __uint_as_float(0x7fc00000u);
-            if (l0 + k < P.M) R.slice_scale[l0 + k] = sUnit[k];
-        }
-    }
-    __syncthreads();
-    const int per = 2 * R.nk;                                  // groups of 8 halves of a row's slice
-    for (int i = t; i < kRsSliceSprings * per; i += blockDim.x) {
-        const int k = i / per, c = i - k * per, ks = c >> 1, q0 = 2 * (c & 1);
-        if (l0 + k >= P.M) break;
-        const float inv = sInv[k];
-        const bool fin = sUnit[k] == sUnit[k];
-        unsigned short h[kRsSlices][8];
-#pragma unroll
-        for (int u = 0; u < 8; u++) {
-            const int m = ks * 16 + 2 * (q0 + (u >> 2)) + 8 * ((u >> 1) & 1) + (u & 1);      // m - 1
-            float2 v = make_float2(0.f, 0.f);
-            if (m < mm && fin) v = sl_sm[m * kRsSliceSprings + k];
-            float sl[kRsSlices];
-            rs::density_slices(v.x, v.y, inv, sl);
-#pragma unroll
-            for (int j = 0; j < kRsSlices; j++) h[j][u] = __half_as_ushort(__float2half_rn(sl[j]));
-        }
-        uint4* row = (uint4*)(R.slices + (size_t)(l0 + k) * kRsSlices * R.nk * 16);
-#pragma unroll
-        for (int j = 0; j < kRsSlices; j++)
-            row[(j * R.nk + ks) * 2 + (c & 1)] =
-                make_uint4(h[j][0] | (unsigned)h[j][1] << 16, h[j][2] | (unsigned)h[j][3] << 16,
-                           h[j][4] | (unsigned)h[j][5] << 16, h[j][6] | (unsigned)h[j][7] << 16);
-    }
-}
-
-__device__ __forceinline__ void rs_mma(float (&d)[4], const unsigned (&a)[4], uint2 b) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
-}
-
-// accumulators of power R by the weight of its products: acc[g] += sum_{i+j=g} A_i B_j
-template <int R>
-struct RsAcc {
-    float v[kRsDiagonals[R]][4] = {};
-    // tab: this lane's operand of slice 0 at the step of 16 m, slice_stride apart
-    __device__ __forceinline__ void add(const unsigned (&a)[kRsSlices][4], const uint2* tab, int slice_stride) {
-        constexpr int S = kRsSlicesOf[R], first = kRsFirstSlice[R], D = kRsDiagonals[R];
-        uint2 b[S];
-#pragma unroll
-        for (int j = 0; j < S; j++) b[j] = tab[(first + j) * slice_stride];
-#pragma unroll
-        for (int g = 0; g < D; g++)
-#pragma unroll
-            for (int i = 0; i <= g; i++)
-                if (i < kRsSlices && g - i < S) rs_mma(v[g], a[i], b[g - i]);
-    }
-    // element c as a pair or a single float, times the scale
-    __device__ __forceinline__ float2 pair(int c, float sc) const {
-        float s, e;
-        rs::two_sum(v[0][c], __fmul_rn(v[1][c], 0x1p-11f), s, e);
-        constexpr int D = kRsDiagonals[R];
-        float u = v[D - 1][c];
-#pragma unroll
-        for (int g = D - 2; g >= 2; g--) u = __fmaf_rn(u, 0x1p-11f, v[g][c]);
-        return make_float2(__fmul_rn(s, sc), __fmul_rn(__fmaf_rn(u, 0x1p-22f, e), sc));
-    }
-    __device__ __forceinline__ float single(int c, float sc) const {
-        constexpr int D = kRsDiagonals[R];
-        float u = v[D - 1][c];
-#pragma unroll
-        for (int g = D - 2; g >= 0; g--) u = __fmaf_rn(u, 0x1p-11f, v[g][c]);
-        return __fmul_rn(u, sc);
-    }
-};
-
-// The A operand of a warp: the four slices of 16 sources.  NK > 0: all steps of 16 m in registers;
-// NK = 0 (windows of more than 64 steps): read again from memory at every use.
-template <int NK>
-struct RsDensities {
-    unsigned a[NK > 0 ? NK : 1][kRsSlices][4];
-    const uint2 *r0, *r1;
-    int nk;
-    __device__ __forceinline__ void load(int slot, int ks) {
-#pragma unroll
-        for (int i = 0; i < kRsSlices; i++) {
-            const uint2 u = __ldg(r0 + (i * nk + ks) * 4), v = __ldg(r1 + (i * nk + ks) * 4);
-            a[slot][i][0] = u.x;
-            a[slot][i][1] = v.x;
-            a[slot][i][2] = u.y;
-            a[slot][i][3] = v.y;
-        }
-    }
-    // rows: the slices of the lane's two sources (g, g + 8), offset by its quarter of a row
-    __device__ __forceinline__ RsDensities(const uint2* row0, const uint2* row1, int nk_) : r0(row0), r1(row1), nk(nk_) {
-        if constexpr (NK > 0) {
-#pragma unroll
-            for (int ks = 0; ks < NK; ks++) load(ks, ks);
-        }
-    }
-    // f(operand of step ks, ks) for the steps ks0 .. nk - 1
-    template <typename F>
-    __device__ __forceinline__ void each(int ks0, F&& f) {
-        if constexpr (NK > 0) {
-#pragma unroll
-            for (int ks = 0; ks < NK; ks++)
-                if (ks >= ks0) f(a[ks], ks);
-        } else {
-            for (int ks = ks0; ks < nk; ks++) {
-                load(0, ks);
-                f(a[0], ks);
-            }
-        }
-    }
-};
-
-// What this costs, against folding in FP32 pairs inside the pair kernel (36 instructions per m, paid
-// again for each side and block of targets; range_fp32.cu): free space, 1e5 uniform springs, 676
-// intervals, 41 m: local sum 16.9 -> 3.2 ms per step (fold 1.3, bound by the tensor pipe's m16n8k16
-// rate of one per 2 cycles; pairs 1.9); a million clustered springs, 484 intervals, 33 m: 103 -> 66 ms
-// (fold 7, pairs 47-55).  Slabs hold 2 GiB of records at most, so memory grows by 8 KB a spring.
+// The fold: e-vectors e_{l,iv,r} = sum_m a_{iv,m,r} sigma_l^{n+1-m} for the intervals [s0, s0 + slab), in the
+// compensated FP32 pairs of range.cuh, m ascending; records (e0h e0l e1h e1l | e2 e3 e4 e5 | e6 e7 - -).
+// Bound by FP32 issue: 32 instructions per record and m (evec_mac).
+// Every product is one of float pairs.  A contraction of 11-bit slices on the tensor cores took 1.2 ms for
+// 1e5 springs (2.7 here), but a slice's unit is that of the largest density of the window and the largest
+// coefficient of the interval: where an interval is reached by small coefficients or old densities alone
+// (a march from rest, a growing history) e_0 kept 1e-8 of sum_m |a_m sigma_m| or nothing, against 1e-13.
 //
-// The e-vectors of every spring for the intervals [s0, s0 + slab): a warp holds the densities of 16
-// springs and goes over tiles of 8 intervals, whose coefficient slices the block stages in shared
-// memory (two buffers, asynchronous copies).  Per tile and step of 16 m 61 products m16n8k16, in four
-// groups of powers (0, 5 | 1, 6 | 2, 7 | 3, 4) so that their accumulators fit the registers beside the
-// densities; steps of m before the tile's first m are skipped.  Records
-// (e0h e0l e5 - | e1h e1l e6 - | e2 e7 e3 e4) are staged per warp and written as whole rows.
-constexpr int kRsFoldWarps = 8;
-constexpr int kRsStageRow = 8 * kRsRecord + 4;       // floats of a spring's staged records (8 intervals)
-__host__ __device__ constexpr size_t rs_fold_tile(int nk) { return (size_t)kRsAllSlices * nk * 256; }
-constexpr int kRsTileScales = 8 * kRsPowers * sizeof(float);
-size_t rs_fold_smem(int nk) {
-    return 2 * (rs_fold_tile(nk) + kRsTileScales) + (size_t)kRsFoldWarps * 16 * kRsStageRow * sizeof(float);
+// k_rs_fold makes every record, where springs are dense.  A block takes 32 springs, one to a lane, whose
+// densities of the window it holds in shared memory, and tiles of 8 intervals, one to a warp, whose
+// coefficient rows (read by all lanes alike) each warp copies ahead of the tile that needs them.  Records
+// are staged and written as whole rows, two buffers, one barrier a tile.  1e5 springs, 676 intervals, 26 m on
+// average: 2.7 ms, of which the FP32 pipe needs 1.5; two springs to a lane the same; coefficients by loads
+// from L2 3.5; a lane to an interval 2.7 to 3.3.
+// ---------------------------------------------------------------------------------------------
+constexpr int kRsFoldSprings = 32;
+constexpr int kRsFoldTile = 8;
+constexpr int kRsFoldRow = kRsFoldTile * kRsRecord + 4;      // floats of a spring's staged records
+size_t rs_fold_smem(int nm, bool copied) {
+    return (size_t)2 * kRsFoldSprings * kRsFoldRow * sizeof(float) + (size_t)(nm - 1) * kRsFoldSprings * sizeof(float2) +
+           (copied ? (size_t)2 * kRsFoldTile * nm * 3 * sizeof(float4) : 0);
 }
 
-template <int NK>
-__device__ __forceinline__ void rs_fold_block(const DevPlan& P, const RangeDev& R, int s0, unsigned char* sm) {
-    const int nk = NK > 0 ? NK : R.nk;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
-    const size_t tile_bytes = rs_fold_tile(nk) + kRsTileScales;       // slices, then the units
-    float* stage = (float*)(sm + 2 * tile_bytes) + warp * 16 * kRsStageRow;
-    const int64_t l0 = ((int64_t)blockIdx.x * kRsFoldWarps + warp) * 16;
-    const int64_t la = min(l0 + g, P.M - 1), lb = min(l0 + g + 8, P.M - 1);
-    const size_t row = (size_t)kRsSlices * nk * 4;                     // uint2 of a spring's slices
-    RsDensities<NK> A((const uint2*)R.slices + la * row + q, (const uint2*)R.slices + lb * row + q, nk);
-    const float sa = __ldg(R.slice_scale + la), sb = __ldg(R.slice_scale + lb);
+// COPIED: the tile's coefficients come through shared memory; windows too long for that read them in place
+template <bool COPIED>
+__device__ __forceinline__ void rs_fold_block(const DevPlan& P, const RangeDev& R, int s0) {
+    extern __shared__ __align__(16) float fold_sm[];         // staged records, densities [m - 1][spring], coefficients
+    float2* sSig = (float2*)(fold_sm + 2 * kRsFoldSprings * kRsFoldRow);
+    float4* sCoef = (float4*)(sSig + (R.nm - 1) * kRsFoldSprings);
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int64_t n = load_step(P), l0 = (int64_t)blockIdx.x * kRsFoldSprings;
     // this block's tiles of the slab
-    const int ntile = (min(R.slab, R.nint - s0) + 7) >> 3;
+    const int s1 = min(R.nint, s0 + R.slab), ntile = (s1 - s0 + kRsFoldTile - 1) / kRsFoldTile;
     const int t0 = (int)((int64_t)ntile * blockIdx.y / gridDim.y), t1 = (int)((int64_t)ntile * (blockIdx.y + 1) / gridDim.y);
-    auto fetch = [&](int tile, int buf) {
-        const unsigned char* src = (const unsigned char*)R.fold + (size_t)(s0 + 8 * tile) * 32;
-        for (int i = threadIdx.x; i < kRsAllSlices * nk * 16; i += blockDim.x) {
-            const unsigned dst = (unsigned)__cvta_generic_to_shared(sm + buf * tile_bytes + 16 * i);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
-                         "l"(src + (size_t)(i >> 4) * R.nivp * 32 + (i & 15) * 16));
-        }
-        if (threadIdx.x < kRsTileScales / 16) {
-            const unsigned dst = (unsigned)__cvta_generic_to_shared(sm + buf * tile_bytes + rs_fold_tile(nk) + 16 * threadIdx.x);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
-                         "l"(R.fold_scale + (size_t)(s0 + 8 * tile) * kRsPowers + 4 * threadIdx.x));
+    auto fetch = [&](int tile) {
+        const int iv = s0 + kRsFoldTile * tile + warp;
+        if (iv < s1) {
+            const int m0 = __ldg(R.mr + 2 * iv), rows = 3 * (__ldg(R.mr + 2 * iv + 1) - m0 + 1);
+            const float4* src = (const float4*)R.coef + ((size_t)iv * R.nm + m0) * 3;
+            float4* dst = sCoef + ((tile & 1) * kRsFoldTile + warp) * R.nm * 3;
+            for (int i = lane; i < rows; i += 32)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst + i)),
+                             "l"(src + i));
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    // the first m of a tile's interval of this lane
-    auto first_m = [&](int tile) { return __ldg(R.mr + 2 * min(s0 + 8 * tile + (lane & 7), R.nint - 1)); };
-    int mnext = first_m(t0);
-    if (t0 < t1) fetch(t0, 0);
+    if (COPIED && t0 < t1) fetch(t0);
+    for (int i = t; i < (R.nm - 1) * kRsFoldSprings; i += blockDim.x) {
+        const int k = i & (kRsFoldSprings - 1), m = 1 + i / kRsFoldSprings;
+        float2 v = make_float2(0.f, 0.f);
+        if (l0 + k < P.M) v = __ldg((const float2*)P.sig2 + (int64_t)ring_slot(n + 1 - m, P.ring) * P.M + l0 + k);
+        sSig[i] = v;
+    }
+    __syncthreads();
     for (int tile = t0; tile < t1; tile++) {
-        const int buf = (tile - t0) & 1;
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();                                  // this tile has arrived, the other buffer is free
-        if (tile + 1 < t1) fetch(tile + 1, buf ^ 1);
-        const int m0 = __reduce_min_sync(0xffffffffu, mnext);
-        mnext = first_m(tile + 1);
-        const int ks0 = min(nk - 1, max(0, (m0 - 1) >> 4));
-        const uint2* tab = (const uint2*)(sm + buf * tile_bytes) + lane;
-        const int stride = nk * 32;
-        const float* scale = (const float*)(sm + buf * tile_bytes + rs_fold_tile(nk)) + 2 * q * kRsPowers;   // intervals 2q, 2q + 1
-        // element c of a fragment: spring g + 8 (c >> 1), interval 2q + (c & 1)
-        float* out = stage + g * kRsStageRow + 2 * q * kRsRecord;
-        auto at = [&](int c) { return out + (c & 1) * kRsRecord + (c >> 1) * 8 * kRsStageRow; };
-        auto sc = [&](int c, int r) { return __fmul_rn(c & 2 ? sb : sa, scale[(c & 1) * kRsPowers + r]); };
-        {
-            RsAcc<0> x;
-            RsAcc<5> y;
-            A.each(ks0, [&](const unsigned (&a)[kRsSlices][4], int ks) {
-                x.add(a, tab + ks * 32, stride);
-                y.add(a, tab + ks * 32, stride);
-            });
-#pragma unroll
-            for (int c = 0; c < 4; c++) {
-                const float2 e = x.pair(c, sc(c, 0));
-                *(float4*)at(c) = make_float4(e.x, e.y, y.single(c, sc(c, 5)), 0.f);
+        float* stage = fold_sm + (tile & 1) * kRsFoldSprings * kRsFoldRow;
+        const int iv0 = s0 + kRsFoldTile * tile, iv = iv0 + warp;
+        if (COPIED) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncwarp();                                     // the warp's rows have arrived, its other buffer is free
+            if (tile + 1 < t1) fetch(tile + 1);
+        }
+        if (iv < s1) {
+            rs::EVec ev;
+            rs::evec_zero(ev);
+            const int m0 = __ldg(R.mr + 2 * iv), m1 = __ldg(R.mr + 2 * iv + 1);
+            const float2* sg = sSig + (m0 - 1) * kRsFoldSprings + lane;
+            const float4* c = COPIED ? sCoef + ((tile & 1) * kRsFoldTile + warp) * R.nm * 3
+                                     : (const float4*)R.coef + ((size_t)iv * R.nm + m0) * 3;
+#pragma unroll 2
+            for (int m = m0; m <= m1; m++, sg += kRsFoldSprings, c += 3) {
+                const float4 a = c[0], b = c[1], d = c[2];
+                const float2 s = *sg;
+                const float c01[4] = {a.x, a.y, a.z, a.w}, c23[4] = {b.x, b.y, b.z, b.w}, c47[4] = {d.x, d.y, d.z, d.w};
+                rs::evec_mac(ev, c01, c23, c47, s.x, s.y);
             }
+            float4* rec = (float4*)(stage + lane * kRsFoldRow + warp * kRsRecord);
+            rec[0] = make_float4(ev.e0h, ev.e0l, ev.e1h, ev.e1l);
+            rec[1] = make_float4(ev.e2, ev.e3, ev.e4, ev.e5);
+            rec[2] = make_float4(ev.e6, ev.e7, 0.f, 0.f);
         }
-        {
-            RsAcc<1> x;
-            RsAcc<6> y;
-            A.each(ks0, [&](const unsigned (&a)[kRsSlices][4], int ks) {
-                x.add(a, tab + ks * 32, stride);
-                y.add(a, tab + ks * 32, stride);
-            });
+        __syncthreads();                                      // the tile is staged; the other buffer has been written out
+        constexpr int rowq = kRsFoldTile * kRsRecord / 4;
+        const int per = min(kRsFoldTile, s1 - iv0) * (kRsRecord / 4);
+        float* dst = R.evec + ((size_t)l0 * R.slab + (iv0 - s0)) * kRsRecord;
 #pragma unroll
-            for (int c = 0; c < 4; c++) {
-                const float2 e = x.pair(c, sc(c, 1));
-                *(float4*)(at(c) + 4) = make_float4(e.x, e.y, y.single(c, sc(c, 6)), 0.f);
-            }
+        for (int i = t; i < kRsFoldSprings * rowq; i += 32 * kRsFoldTile) {
+            const int r = i / rowq, o = i - r * rowq;
+            if (o < per && l0 + r < P.M)
+                *(float4*)(dst + (size_t)r * R.slab * kRsRecord + 4 * o) = *(const float4*)(stage + r * kRsFoldRow + 4 * o);
         }
-        float2 e27[4];
-        {
-            RsAcc<2> x;
-            RsAcc<7> y;
-            A.each(ks0, [&](const unsigned (&a)[kRsSlices][4], int ks) {
-                x.add(a, tab + ks * 32, stride);
-                y.add(a, tab + ks * 32, stride);
-            });
-#pragma unroll
-            for (int c = 0; c < 4; c++) e27[c] = make_float2(x.single(c, sc(c, 2)), y.single(c, sc(c, 7)));
-        }
-        {
-            RsAcc<3> x;
-            RsAcc<4> y;
-            A.each(ks0, [&](const unsigned (&a)[kRsSlices][4], int ks) {
-                x.add(a, tab + ks * 32, stride);
-                y.add(a, tab + ks * 32, stride);
-            });
-#pragma unroll
-            for (int c = 0; c < 4; c++)
-                *(float4*)(at(c) + 8) = make_float4(e27[c].x, e27[c].y, x.single(c, sc(c, 3)), y.single(c, sc(c, 4)));
-        }
-        __syncwarp();
-        // 16 springs x 384 bytes
-        float* dst = R.evec + ((size_t)l0 * R.slab + 8 * tile) * kRsRecord;
-#pragma unroll
-        for (int i = 0; i < 12; i++) {
-            const int c = 32 * i + lane, r = c / 24, o = c - 24 * r;
-            if (l0 + r < P.M)
-                *(float4*)(dst + (size_t)r * R.slab * kRsRecord + 4 * o) = *(const float4*)(stage + r * kRsStageRow + 4 * o);
-        }
-        __syncwarp();
     }
 }
+__global__ void __launch_bounds__(32 * kRsFoldTile, 3) k_rs_fold(DevPlan P, RangeDev R, int s0) {
+    rs_fold_block<true>(P, R, s0);
+}
+__global__ void __launch_bounds__(32 * kRsFoldTile, 3) k_rs_fold_long(DevPlan P, RangeDev R, int s0) {
+    rs_fold_block<false>(P, R, s0);
+}
 
-__global__ void __launch_bounds__(32 * kRsFoldWarps, 2) k_rs_fold(DevPlan P, RangeDev R, int s0) {
-    extern __shared__ __align__(16) unsigned char fold_sm[];
-    switch (R.nk) {
-        case 1: rs_fold_block<1>(P, R, s0, fold_sm); break;
-        case 2: rs_fold_block<2>(P, R, s0, fold_sm); break;
-        case 3: rs_fold_block<3>(P, R, s0, fold_sm); break;
-        case 4: rs_fold_block<4>(P, R, s0, fold_sm); break;
-        default: rs_fold_block<0>(P, R, s0, fold_sm); break;
+// k_rs_fold_used makes the records that some pair reads (R.used), where there is less than a pair to a
+// record: a block lists the used records of 32 springs and kRsUsedIntervals intervals, interval by
+// interval, and its threads take one each, so a warp reads the coefficients of one or two intervals.  A step
+// of uniform springs in free space, every record against the used ones, by pairs per record: 0.11 (6,000
+// springs) 0.55 and 0.42 ms, 0.27 0.97 and 0.73, 0.54 1.33 and 1.12, 0.9 2.43 and 2.35, 1.1 2.81 and 2.84,
+// 1.8 (100,000) 4.62 and 5.17.
+constexpr int kRsUsedIntervals = 64;
+size_t rs_used_smem(int nm) { return (size_t)(nm - 1) * kRsFoldSprings * sizeof(float2); }
+int rs_used_blocks(int intervals) { return (intervals + kRsUsedIntervals - 1) / kRsUsedIntervals; }
+__global__ void __launch_bounds__(256, 3) k_rs_fold_used(DevPlan P, RangeDev R, int s0) {
+    extern __shared__ __align__(16) float2 used_sm[];        // densities [m - 1][spring]
+    __shared__ unsigned sWord[kRsUsedIntervals];             // per interval: the springs that use it
+    __shared__ int sFirst[kRsUsedIntervals + 1];
+    __shared__ uint16_t sItem[kRsUsedIntervals * kRsFoldSprings];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nwarps = blockDim.x >> 5;
+    const int64_t n = load_step(P), l0 = (int64_t)blockIdx.x * kRsFoldSprings;
+    const int b0 = s0 + kRsUsedIntervals * blockIdx.y, nb = min(kRsUsedIntervals, min(R.nint, s0 + R.slab) - b0);
+    for (int k = warp; k < nb; k += nwarps) {
+        const int iv = b0 + k;
+        const bool u = l0 + lane < P.M && (__ldg(R.used + (size_t)(l0 + lane) * R.used_words + (iv >> 5)) >> (iv & 31) & 1u);
+        const unsigned w = __ballot_sync(0xffffffffu, u);
+        if (lane == 0) sWord[k] = w;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        static_assert(kRsUsedIntervals == 64, "two intervals a lane");
+        const int a = 2 * lane < nb ? __popc(sWord[2 * lane]) : 0, b = 2 * lane + 1 < nb ? __popc(sWord[2 * lane + 1]) : 0;
+        int sum = a + b;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, sum, o);
+            if (lane >= o) sum += v;
+        }
+        sFirst[2 * lane + 1] = sum - b;
+        sFirst[2 * lane + 2] = sum;
+        if (lane == 0) sFirst[0] = 0;
+    }
+    __syncthreads();
+    const int total = sFirst[kRsUsedIntervals];
+    if (total == 0) return;
+    for (int k = warp; k < nb; k += nwarps) {
+        const unsigned w = sWord[k];
+        if (w >> lane & 1u) sItem[sFirst[k] + __popc(w & ((1u << lane) - 1u))] = (uint16_t)(k * kRsFoldSprings + lane);
+    }
+    for (int i = t; i < (R.nm - 1) * kRsFoldSprings; i += blockDim.x) {
+        const int k = i & (kRsFoldSprings - 1), m = 1 + i / kRsFoldSprings;
+        float2 v = make_float2(0.f, 0.f);
+        if (l0 + k < P.M) v = __ldg((const float2*)P.sig2 + (int64_t)ring_slot(n + 1 - m, P.ring) * P.M + l0 + k);
+        used_sm[i] = v;
+    }
+    __syncthreads();
+    for (int i = t; i < total; i += blockDim.x) {
+        const int item = sItem[i], iv = b0 + item / kRsFoldSprings, sp = item & (kRsFoldSprings - 1);
+        rs::EVec ev;
+        rs::evec_zero(ev);
+        const int m0 = __ldg(R.mr + 2 * iv), m1 = __ldg(R.mr + 2 * iv + 1);
+        const float4* c = (const float4*)R.coef + ((size_t)iv * R.nm + m0) * 3;
+        const float2* sg = used_sm + (m0 - 1) * kRsFoldSprings + sp;
+#pragma unroll 2
+        for (int m = m0; m <= m1; m++, sg += kRsFoldSprings, c += 3) {
+            const float4 a = __ldg(c), b = __ldg(c + 1), d = __ldg(c + 2);
+            const float2 s = *sg;
+            const float c01[4] = {a.x, a.y, a.z, a.w}, c23[4] = {b.x, b.y, b.z, b.w}, c47[4] = {d.x, d.y, d.z, d.w};
+            rs::evec_mac(ev, c01, c23, c47, s.x, s.y);
+        }
+        float4* rec = (float4*)(R.evec + ((size_t)(l0 + sp) * R.slab + (iv - s0)) * kRsRecord);
+        rec[0] = make_float4(ev.e0h, ev.e0l, ev.e1h, ev.e1l);
+        rec[1] = make_float4(ev.e2, ev.e3, ev.e4, ev.e5);
+        rec[2] = make_float4(ev.e6, ev.e7, 0.f, 0.f);
     }
 }
 
@@ -377,10 +255,10 @@ __global__ void __launch_bounds__(32 * kRsFoldWarps, 2) k_rs_fold(DevPlan P, Ran
 // rounding of one takes either neighbouring interval's polynomial; at dt the spring's FP64 window
 // of near sources decides.
 // ---------------------------------------------------------------------------------------------
-// acc += the polynomial of a record at z (record: e0h e0l e5 - | e1h e1l e6 - | e2 e7 e3 e4)
-__device__ __forceinline__ void rs_eval(const float4& a, const float4& b, const float4& c, float zh, float zl, float& ah,
+// acc += the polynomial of a record at z
+__device__ __forceinline__ void rs_eval(const float4& a, const float4& b, const float2& c, float zh, float zl, float& ah,
                                         float& al) {
-    rs::evec_eval4(rs::F4{a.x, a.y, b.x, b.y}, rs::F4{c.x, c.z, c.w, a.z}, rs::F4{b.z, c.y, 0.f, 0.f}, zh, zl, ah, al);
+    rs::evec_eval4(rs::F4{a.x, a.y, a.z, a.w}, rs::F4{b.x, b.y, b.z, b.w}, rs::F4{c.x, c.y, 0.f, 0.f}, zh, zl, ah, al);
 }
 
 // the first k in [0, n) with pred(k), or n (pred monotone), by a warp: 32 probes a round
@@ -547,18 +425,20 @@ struct RsSum {
     __device__ __forceinline__ void stage(int, int) {}
     __device__ __forceinline__ void pairs(const bool (&in)[2], int, int e, int step, const int (&iv)[2], const float (&zh)[2],
                                           const float (&zl)[2]) {
-        float4 r[2][3];
+        float4 r[2][2];
+        float2 q[2];
 #pragma unroll
         for (int u = 0; u < 2; u++) {
             const float4* rec = (const float4*)(R.evec + ((size_t)rs_spring(e + u * step, P.M) * R.slab + (iv[u] - s0)) * kRsRecord);
             if (in[u]) {
-#pragma unroll
-                for (int i = 0; i < 3; i++) r[u][i] = __ldg(rec + i);
+                r[u][0] = __ldg(rec);
+                r[u][1] = __ldg(rec + 1);
+                q[u] = __ldg((const float2*)(rec + 2));
             }
         }
 #pragma unroll
         for (int u = 0; u < 2; u++)
-            if (in[u]) rs_eval(r[u][0], r[u][1], r[u][2], zh[u], zl[u], ah[u], al[u]);
+            if (in[u]) rs_eval(r[u][0], r[u][1], q[u], zh[u], zl[u], ah[u], al[u]);
     }
 };
 
@@ -576,6 +456,32 @@ __global__ void __launch_bounds__(kRsPairTargets, kRsPairBlocks) k_rs_pairs(DevP
     rs::acc_add(v.ah[0], v.al[0], v.ah[1], v.al[1]);
     const int64_t j = (int64_t)blockIdx.x * kRsPairTargets + threadIdx.x;
     if (j < P.M) ((float2*)R.csum)[((size_t)(p0 / R.part) * 2 + blockIdx.y) * P.M + j] = make_float2(v.ah[0], v.al[0]);
+}
+
+// plan time: the records that k_rs_pairs reads, by its own walk (R.used zero on entry)
+struct RsUse {
+    const DevPlan& P;
+    const RangeDev& R;
+    __device__ __forceinline__ void stage(int, int) {}
+    __device__ __forceinline__ void pairs(const bool (&in)[2], int, int e, int step, const int (&iv)[2], const float (&)[2],
+                                          const float (&)[2]) {
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            if (!in[u]) continue;
+            unsigned* w = R.used + (size_t)rs_spring(e + u * step, P.M) * R.used_words + (iv[u] >> 5);
+            const unsigned bit = 1u << (iv[u] & 31);
+            if (!(__ldcg(w) & bit)) atomicOr(w, bit);
+        }
+    }
+};
+__global__ void __launch_bounds__(kRsPairTargets) k_rs_mark_used(DevPlan P, RangeDev R) {
+    extern __shared__ __align__(16) float4 pair_sm[];
+    __shared__ float2 sPos[kRsPosChunk];
+    __shared__ int sRed[2];
+    const int p0 = blockIdx.z * R.part, p1 = min(R.nint, p0 + R.part);
+    RsUse v{P, R};
+    if (blockIdx.y == 0) rs_pair_block<-1>(P, R, p0, p1, pair_sm, sPos, sRed, v);
+    else rs_pair_block<1>(P, R, p0, p1, pair_sm, sPos, sRed, v);
 }
 
 // shared memory of a pair block's interval table
@@ -1044,6 +950,13 @@ __global__ void __launch_bounds__(kRsPairTargets) k_rs_moments(DevPlan P, RangeD
     rs_pair_block<-1>(P, R, p0, p1, pair_sm, sPos, sRed, v);
     rs_pair_block<1>(P, R, p0, p1, pair_sm, sPos, sRed, v);
     v.flush();
+}
+
+__device__ __forceinline__ void rs_mma(float (&d)[4], const unsigned (&a)[4], uint2 b) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
 }
 
 // The contraction of a slab's moments with the coefficients, a warp per 16 outputs: A = moments (16

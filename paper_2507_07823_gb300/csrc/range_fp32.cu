@@ -1,9 +1,8 @@
-// Local sum of plans without pair lists with FP32 spreading and interpolation (opts.precision = 1):
-// the fold of the densities in compensated FP32 pairs, chunk by chunk in shared memory.  The FP64 form
-// folds on the tensor cores instead (range.cu), which is 1.5 to 4 times faster and differs in the
-// last bits; here those bits count: the FP32 passes round every grid value and u_H to 2^-24, so a
-// density that differs by 1e-12 flips roundings and moves results by 1e-7 of the field.  So a mixed
-// march keeps this order of sums, and its results stay the same bit for bit.
+// Local sum of plans without pair lists with FP32 spreading and interpolation (opts.precision = 1): the
+// fold and the pairs chunk by chunk in shared memory.  The FP64 form (range.cu) makes the same e-vectors
+// bit for bit but sums the pairs in another order, and here the order counts: the FP32 passes round every
+// grid value and u_H to 2^-24, so a density that differs by 1e-12 flips roundings and moves results by 1e-7
+// of the field.  A mixed march keeps this order of sums, and its results stay the same bit for bit.
 #include <cuda_runtime.h>
 
 #include <cstdint>
