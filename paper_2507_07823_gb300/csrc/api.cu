@@ -68,7 +68,11 @@ size_t rs_pair_smem(int part, int fine_span);
 __global__ void k_rs_moments(DevPlan P, RangeDev R, int s0, const double* cbar);
 __global__ void k_rs_sweeps(DevPlan P, RangeDev R);
 size_t rs_unfold_smem();
-__global__ void k_rs_unfold(DevPlan P, RangeDev R, int s0, int s1, int64_t n, float2* sums, double* sb);
+int rs_unfold_warps(int m_max);
+int rs_unfold_groups(int m_max);
+int rs_unfold_runs(int64_t M, int slab, int sms);
+__global__ void k_rs_unfold(DevPlan P, RangeDev R, int s0, int s1, double* sums);
+__global__ void k_rs_unfold_add(DevPlan P, RangeDev R, int runs, int64_t n, const double* sums, double* sb);
 __global__ void k_rs_adj_init(DevPlan P, RangeDev R, double* slot_vals, double* rhs);
 __global__ void k_rs_adj_post(DevPlan P, RangeDev R, const double* sigma_next, const double* g_next, double* grad,
                               double* gbar_next, double* cbar, double* uHbar);
@@ -319,10 +323,7 @@ int fold_tables(wave1d_plan_t p) {
     const Params& P = p->hp.P;
     RangeDev& rd = p->rd;
     int rc;
-    float* f32;
     uint16_t* h16;
-    if ((rc = upload(p, rt.fold_scale, &f32))) return rc;
-    rd.fold_scale = f32;
     if ((rc = upload(p, rt.fine, &h16))) return rc;
     rd.fine = h16;
     rd.fine_span = rt.fine_span;
@@ -1449,7 +1450,8 @@ struct Reverse {
     size_t lsmem = 0;
     double2* waves = nullptr;
     double* rrhs = nullptr;   // plans without pair lists: the transposed solve's right-hand side
-    float2* usum = nullptr;   // the transposed local sum's pairs between slabs
+    double* usum = nullptr;   // the transposed local sum's runs between slabs
+    int runs = 1;
     static constexpr int kLocalWarps = 4;     // the transposed local sum: one warp per spring row
 
     int init(wave1d_plan_t pl) {
@@ -1492,16 +1494,10 @@ struct Reverse {
         if (p->range) {
             if ((rc = wk.zeros(&rrhs, (size_t)M))) return rc;
             if (!p->rd.evec && (rc = fold_tables(p))) return rc;        // a mixed plan's first reverse march
-            if (!p->rd.unfold) {
-                uint16_t* h16;
-                if ((rc = upload(p, hp.rt.unfold, &h16))) return rc;
-                p->rd.nis = hp.rt.nis;
-                p->rd.nmp = hp.rt.nmp;
-                p->rd.unfold = h16;
-                if (!allow_smem((const void*)k_rs_unfold, rs_unfold_smem()))
-                    return fail(WAVE1D_ECUDA, "cannot size the shared memory of the transposed local sum");
-            }
-            return wk.zeros(&usum, (size_t)M * p->rd.nmp);
+            if (!allow_smem((const void*)k_rs_unfold, rs_unfold_smem()))
+                return fail(WAVE1D_ECUDA, "cannot size the shared memory of the transposed local sum");
+            runs = rs_unfold_runs(M, p->rd.slab, p->sms);
+            return wk.zeros(&usum, (size_t)runs * M * P.m_max);
         }
         lsmem = adj_local_smem(P.m_max, kLocalWarps);
         if (!allow_smem((const void*)k_adj_local, lsmem))
@@ -1547,16 +1543,17 @@ struct Reverse {
                 k_rs_adj_post<<<gM, 256, 0, s>>>(d, rd, sig_rows + (n - row0) * M, g ? g + n * M : nullptr,
                                                  want_beta ? gsum : nullptr, grad_g ? grad_g + n * M : nullptr, cbar, uHbar);
                 if (n == 0) break;
-                const unsigned gp = blocks_for(M, kRsPairTargets, INT32_MAX);
+                const unsigned gp = blocks_for(M, kRsPairTargets, INT32_MAX), uw = (unsigned)rs_unfold_warps(P.m_max);
                 const cudaStream_t sl = fork();
                 for (int s0 = 0; s0 < rd.nint; s0 += rd.slab) {
                     const int s1 = std::min(rd.nint, s0 + rd.slab);
                     CK(cudaMemsetAsync(rd.evec, 0, (size_t)M * rd.slab * kRsRecord * sizeof(float), sl));
                     k_rs_moments<<<dim3(gp, 1, (unsigned)((s1 - s0 + rd.part - 1) / rd.part)), kRsPairTargets,
                                    rs_pair_smem(rd.part, rd.fine_span), sl>>>(d, rd, s0, cbar);
-                    k_rs_unfold<<<dim3(blocks_for(M, 128, INT32_MAX), (unsigned)(rd.nmp / 8 + 4) / 5), 256, rs_unfold_smem(), sl>>>(
-                        d, rd, s0, s1, n, usum, sb);
+                    k_rs_unfold<<<dim3(blocks_for(M, 64, INT32_MAX), (unsigned)rs_unfold_groups(P.m_max), (unsigned)runs), 32 * uw,
+                                  rs_unfold_smem(), sl>>>(d, rd, s0, s1, usum);
                 }
+                k_rs_unfold_add<<<dim3(gM, (unsigned)P.m_max), 256, 0, sl>>>(d, rd, runs, n, usum, sb);
             } else {
                 if (have_rcv) k_adj_receivers<<<dim3(gM, 8), 256, 0, s>>>(M, ring, n, rptr, rrcv, rmr, rwoff, rw, ub, sb);
                 k_adj_solve<<<gM, 256, 0, s>>>(d, dblk, sb + (int64_t)((n + 1) % ring) * M, sig_rows + (n - row0) * M, g ? g + n * M : nullptr,

@@ -346,9 +346,6 @@ struct RangeDev {
     const double* cheb;         // [iv][m][8] Chebyshev coefficients in z (FP64)
     const int* cell;            // kRsCells: first interval of each cell of [0, delta)
     float cell_scale;           // kRsCells / delta
-    const float* fold_scale;    // [nivp][8]
-    int nis, nmp;               // steps of 16 intervals and padded m of the transposed sum's table
-    const uint16_t* unfold;     // coefficient slices (RangeTables::unfold)
     int slab;                   // intervals whose e-vectors are held at once (a multiple of 16)
     int folded;                 // 1: the local sum comes from k_rs_pairs (csum), 0: from k_rs_local (clocal)
     float* evec;                // [M][slab][kRsRecord]: e-vector records of the slab; the reverse march's

@@ -20,11 +20,10 @@
 //   k_rs_finish     u = u_L + u_H at the receivers, step counter
 //
 // Every kernel reads the step index from the device counter (graphs of steps are replayed).
-#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
-#include <type_traits>
 
 #include "internal.h"
 #include "phases.cuh"
@@ -870,11 +869,8 @@ __global__ void k_rs_finish(DevPlan P, RangeDev R) {
 // over the same pairs as k_rs_pairs (every j within delta of l, each once).  On interval iv,
 // Q_m(d) = sum_r a_{iv,m,r} z^r, so the pairs of output l that fall in iv enter only through the
 // moments F_{l,iv,r} = sum_{j in iv} z_jl^r cbar_j (k_rs_moments: F_0, F_1 as pairs, F_2 .. F_7 single),
-// and the rest is a contraction over intervals and powers with the same coefficients for every
-// output, sum_{iv,r} a_{iv,m,r} F_{l,iv,r}, on the tensor cores (k_rs_unfold).  Per output and interval
-// it was 26 m x (48 FP32 instructions and 4 on the FP64 pipe, 16 cycles of an SM each): 3e4 uniform
-// springs 7.1 -> 2.7 ms per reverse step (5 slabs of moments 0.19 and contraction 0.34).  No atomics:
-// every output has one writer, in a fixed order.
+// and the rest is a sum over intervals and powers with the same coefficients for every output,
+// sum_{iv,r} a_{iv,m,r} F_{l,iv,r} (k_rs_unfold).  No atomics: every output has one writer, in a fixed order.
 // ---------------------------------------------------------------------------------------------
 struct RsMoments {
     const DevPlan& P;
@@ -952,182 +948,129 @@ __global__ void __launch_bounds__(kRsPairTargets) k_rs_moments(DevPlan P, RangeD
     v.flush();
 }
 
-__device__ __forceinline__ void rs_mma(float (&d)[4], const unsigned (&a)[4], uint2 b) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
+// The sums over a slab's intervals: out_{l,m} = sum_{iv} sum_r a_{iv,m,r} F_{l,iv,r}, in float pairs per interval
+// (r = 0, 1 as pairs, the rest single, as the fold's e-vectors), added up over the intervals in three floats (acc3_add), which
+// hold more than FP64's bits.  A block takes 64 outputs, two to a lane, a run of the slab's intervals
+// (blockIdx.z) and a group of steps (blockIdx.y); it stages records and coefficients of 8 intervals at a time (two
+// buffers, asynchronous copies).  Warp w takes the group's steps w, w + nwarps, .., four at most, so that the warps'
+// work is even.  sums: [blockIdx.z][m][M], carried from slab to slab; k_rs_unfold_add puts them into the ring.
+// Bound by FP32 issue, 52 instructions per output, interval and m: 30,000 outputs and 676 intervals about 1.1 ms,
+// of which the FP32 pipe needs 0.7 (one run of intervals with four warps' steps of eight: 3.3 ms, 469 blocks in two
+// uneven rounds).  11-bit slices on the tensor cores took 0.84 ms, held moments and coefficients in common
+// units and the sums as pairs, and gave NaN at p = 16.
+constexpr int kRsOutputs = 64;
+constexpr int kRsOutPer = 4;
+constexpr int kRsOutWarps = 10;                       // 40 steps to a group at most: one group for windows of 36 steps
+constexpr int kRsOutTile = 8;
+constexpr int kRsOutRow = kRsOutTile * kRsRecord + 4;
+constexpr int kRsOutRows = kRsOutputs * kRsOutRow;    // floats of a tile's records
+int rs_unfold_groups(int m_max) { return (m_max + kRsOutPer * kRsOutWarps - 1) / (kRsOutPer * kRsOutWarps); }
+int rs_unfold_warps(int m_max) {
+    const int g = rs_unfold_groups(m_max) * kRsOutPer;
+    return (m_max + g - 1) / g;
 }
-
-// The contraction of a slab's moments with the coefficients, a warp per 16 outputs: A = moments (16
-// outputs x 16 intervals, one power), B = coefficients (16 intervals x 8 m).  A lane holds the moments
-// of its 2 outputs and 4 intervals of a step, scales them by the coefficients' units and one power
-// of two per output and step (the largest of the step's moments), and cuts them into four slices of 11
-// bits (density_slices) in place as its part of A.  Products of slices i + j <= 4 of all powers share
-// accumulators, which are whole numbers below 2^24 within a step (16 intervals, 8 powers whose
-// coefficients fall by 10 or more from one to the next) and go into the output's pairs after it;
-// slices that are zero in the whole warp are skipped.  sums: [M][nmp] pairs carried from slab to slab;
-// the last slab adds them to the ring.
-// The block stages a step's coefficients in shared memory (two buffers, asynchronous copies): read from
-// L2 by each warp they held it up 40 times a step (576 us a slab of 336 intervals at 3e4 outputs).
-constexpr int kRsUnfoldWarps = 8;
-constexpr int kRsUnfoldTiles = 5;                     // tiles of 8 m at a time (m_max up to 40 in one go)
-constexpr int kRsUnfoldStep = kRsAllSlices * kRsUnfoldTiles * 8 * 32;     // bytes of a step's coefficients
-size_t rs_unfold_smem() { return 2 * (size_t)kRsUnfoldStep; }
-__global__ void __launch_bounds__(32 * kRsUnfoldWarps) k_rs_unfold(DevPlan P, RangeDev R, int s0, int s1, int64_t n,
-                                                                  float2* __restrict__ sums, double* __restrict__ sb) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
-    extern __shared__ __align__(16) unsigned char unfold_sm[];
-    const int64_t l0 = ((int64_t)blockIdx.x * kRsUnfoldWarps + (threadIdx.x >> 5)) * 16;
-    const int mtiles = R.nmp >> 3, mt0 = blockIdx.y * kRsUnfoldTiles, mt1 = min(mtiles, mt0 + kRsUnfoldTiles);
-    const int64_t row[2] = {min(l0 + g, P.M - 1), min(l0 + g + 8, P.M - 1)};
-    float2 out[kRsUnfoldTiles][4];                    // (row c >> 1, m = 8 mt + 2 q + (c & 1) + 1)
+size_t rs_unfold_smem() {
+    return (size_t)2 * (kRsOutRows * sizeof(float) + kRsOutTile * kRsOutPer * kRsOutWarps * 3 * sizeof(float4));
+}
+// runs of a slab's intervals: enough blocks for the chip (six resident rounds) where there are few outputs
+int rs_unfold_runs(int64_t M, int slab, int sms) {
+    const int64_t gx = (M + kRsOutputs - 1) / kRsOutputs;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(slab / (2 * kRsOutTile), (12 * (int64_t)sms + gx - 1) / gx));
+}
+__global__ void __launch_bounds__(32 * kRsOutWarps, 2) k_rs_unfold(DevPlan P, RangeDev R, int s0, int s1,
+                                                                  double* __restrict__ sums) {
+    extern __shared__ __align__(16) float unfold_sm[];       // 2 x records, 2 x coefficients [interval][step][3]
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nwarps = blockDim.x >> 5, steps = nwarps * kRsOutPer;
+    const int64_t l0 = (int64_t)blockIdx.x * kRsOutputs;
+    const int mg = 1 + blockIdx.y * steps, mfirst = mg + warp;               // the group's and the warp's first step
+    float4* const sCoef = (float4*)(unfold_sm + 2 * kRsOutRows);
+    sums += (int64_t)blockIdx.z * (R.nm - 1) * P.M;
+    // this block's tiles of the slab
+    const int ntile = (s1 - s0 + kRsOutTile - 1) / kRsOutTile;
+    const int t0 = (int)((int64_t)ntile * blockIdx.z / gridDim.z), t1 = (int)((int64_t)ntile * (blockIdx.z + 1) / gridDim.z);
+    float acc[kRsOutPer][2][3];
 #pragma unroll
-    for (int mt = 0; mt < kRsUnfoldTiles; mt++)
+    for (int i = 0; i < kRsOutPer; i++)
 #pragma unroll
-        for (int c = 0; c < 4; c++)
-            out[mt][c] = s0 > 0 && mt0 + mt < mt1 ? sums[row[c >> 1] * R.nmp + 8 * (mt0 + mt) + 2 * q + (c & 1)]
-                                                  : make_float2(0.f, 0.f);
-    const int rows = 8 * (mt1 - mt0);
-    auto fetch = [&](int i0, int buf) {
-        const unsigned char* src = (const unsigned char*)R.unfold + ((size_t)(i0 >> 4) * R.nmp + 8 * mt0) * 32;
-        for (int i = threadIdx.x; i < kRsAllSlices * rows * 2; i += blockDim.x) {
-            const int sl = i / (rows * 2), o = i - sl * rows * 2;
-            const unsigned dst = (unsigned)__cvta_generic_to_shared(unfold_sm + buf * kRsUnfoldStep + (sl * kRsUnfoldTiles * 16 + o) * 16);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
-                         "l"(src + (size_t)sl * R.nis * R.nmp * 32 + (size_t)o * 16));
+        for (int u = 0; u < 2; u++) {
+            const int m = mfirst + i * nwarps;
+            const int64_t l = l0 + lane + 32 * u;
+            rs::acc3_set(s0 > 0 && m < R.nm && l < P.M ? sums[(int64_t)(m - 1) * P.M + l] : 0.0, acc[i][u][0], acc[i][u][1],
+                         acc[i][u][2]);
+        }
+    auto copy = [&](void* dst, const void* src) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+    };
+    auto fetch = [&](int tile) {
+        const int i0 = s0 + kRsOutTile * tile, n = min(kRsOutTile, s1 - i0), buf = tile & 1;
+        constexpr int rowq = kRsOutTile * kRsRecord / 4;
+        const float* src = R.evec + ((size_t)l0 * R.slab + (i0 - s0)) * kRsRecord;
+        for (int i = t; i < kRsOutputs * rowq; i += blockDim.x) {
+            const int r = i / rowq, o = i - r * rowq;
+            if (o < n * (kRsRecord / 4) && l0 + r < P.M)
+                copy(unfold_sm + buf * kRsOutRows + r * kRsOutRow + 4 * o, src + (size_t)r * R.slab * kRsRecord + 4 * o);
+        }
+        const int rows = 3 * min(steps, R.nm - mg);          // (the steps of an interval lie together)
+        for (int k = warp; k < n; k += nwarps) {
+            const float4* c = (const float4*)R.coef + ((size_t)(i0 + k) * R.nm + mg) * 3;
+            for (int i = lane; i < rows; i += 32) copy(sCoef + (buf * kRsOutTile + k) * steps * 3 + i, c + i);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    fetch(s0, 0);
-    for (int i0 = s0; i0 < s1; i0 += 16) {
-        const int buf = ((i0 - s0) >> 4) & 1;
+    if (t0 < t1) fetch(t0);
+    for (int tile = t0; tile < t1; tile++) {
         asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();                              // this step has arrived, the other buffer is free
-        if (i0 + 16 < s1) fetch(i0 + 16, buf ^ 1);
-        // first m of the step's intervals (all later ones are met)
-        const int m0 = __reduce_min_sync(0xffffffffu, __ldg(R.mr + 2 * min(i0 + (lane & 15), R.nint - 1)));
-        if (8 * mt1 < m0) continue;
-        // the lane's moments times 2^30 and the coefficients' units: element (w, u): output row[w],
-        // interval i0 + 2q + (u & 1) + 8 (u >> 1)
-        float hi[2][4][kRsPowers], lo[2][4][2];
-        float mx[2] = {0.f, 0.f};
+        __syncthreads();                              // this tile has arrived, the other buffers are free
+        if (tile + 1 < t1) fetch(tile + 1);
+        const int i0 = s0 + kRsOutTile * tile, buf = tile & 1;
+        const float* rec0 = unfold_sm + buf * kRsOutRows + lane * kRsOutRow;
+        for (int k = 0; k < min(kRsOutTile, s1 - i0); k++) {
+            const int m0 = __ldg(R.mr + 2 * (i0 + k)), m1 = __ldg(R.mr + 2 * (i0 + k) + 1);
+            if (mfirst + (kRsOutPer - 1) * nwarps < m0) continue;
+            float4 a[2], b[2];
+            float2 c[2];
 #pragma unroll
-        for (int w = 0; w < 2; w++)
-#pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const int iv = i0 + 2 * q + (u & 1) + 8 * (u >> 1);
-                float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a, c = a;
-                if (iv < s1) {
-                    const float4* rec = (const float4*)(R.evec + ((size_t)row[w] * R.slab + (iv - s0)) * kRsRecord);
-                    a = __ldg(rec);
-                    b = __ldg(rec + 1);
-                    c = __ldg(rec + 2);
-                }
-                const float4* sc = (const float4*)(R.fold_scale + (size_t)iv * kRsPowers);
-                const float4 s03 = __ldg(sc), s47 = __ldg(sc + 1);
-                const float f[kRsPowers] = {a.x, a.z, b.x, b.y, b.z, b.w, c.x, c.y};
-                const float s[kRsPowers] = {s03.x, s03.y, s03.z, s03.w, s47.x, s47.y, s47.z, s47.w};
-#pragma unroll
-                for (int r = 0; r < kRsPowers; r++) {
-                    hi[w][u][r] = __fmul_rn(f[r], __fmul_rn(s[r], 0x1p30f));
-                    mx[w] = __uint_as_float(max(__float_as_uint(mx[w]), __float_as_uint(hi[w][u][r]) & 0x7fffffffu));
-                }
-                lo[w][u][0] = __fmul_rn(a.y, __fmul_rn(s[0], 0x1p30f));
-                lo[w][u][1] = __fmul_rn(a.w, __fmul_rn(s[1], 0x1p30f));
+            for (int u = 0; u < 2; u++) {
+                const float* rec = rec0 + 32 * u * kRsOutRow + k * kRsRecord;
+                a[u] = *(const float4*)rec;
+                b[u] = *(const float4*)(rec + 4);
+                c[u] = *(const float2*)(rec + 8);
             }
-        float inv[2], unit[2];
+            const float4* cf = sCoef + ((buf * kRsOutTile + k) * steps + warp) * 3;
 #pragma unroll
-        for (int w = 0; w < 2; w++) {
-            unsigned m = __float_as_uint(mx[w]);
-            m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
-            m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
-            const int E = rs::slice_exponent(m);
-            // units of 2^(E-9): 512 x 1024 x 16 intervals = 2^23, and the higher powers' tenth of it
-            inv[w] = __uint_as_float((unsigned)(127 + 9 - E) << 23);
-            unit[w] = m < 0x7f800000u ? __uint_as_float((unsigned)(127 + E - 9) << 23) : __uint_as_float(0x7fc00000u);
-        }
-        float acc[kRsUnfoldTiles][5][4] = {};
-        auto power = [&](auto rc) {
-            constexpr int r = decltype(rc)::value, first = kRsFirstSlice[r], count = kRsSlicesOf[r];
-            unsigned a[kRsSlices][4];
-            unsigned any[kRsSlices] = {0u, 0u, 0u, 0u};
+            for (int i = 0; i < kRsOutPer; i++) {
+                const int m = mfirst + i * nwarps;
+                if (m < m0 || m > m1) continue;
+                const float4 c01 = cf[3 * i * nwarps], c23 = cf[3 * i * nwarps + 1], c47 = cf[3 * i * nwarps + 2];
 #pragma unroll
-            for (int w = 0; w < 2; w++) {
-                float sl[4][kRsSlices];
-#pragma unroll
-                for (int u = 0; u < 4; u++) rs::density_slices(hi[w][u][r], r < 2 ? lo[w][u][r & 1] : 0.f, inv[w], sl[u]);
-#pragma unroll
-                for (int i = 0; i < kRsSlices; i++) {
-                    const __half2 p0 = __floats2half2_rn(sl[0][i], sl[1][i]), p1 = __floats2half2_rn(sl[2][i], sl[3][i]);
-                    a[i][w] = __half_as_ushort(p0.x) | (unsigned)__half_as_ushort(p0.y) << 16;
-                    a[i][w + 2] = __half_as_ushort(p1.x) | (unsigned)__half_as_ushort(p1.y) << 16;
-                    any[i] |= (a[i][w] | a[i][w + 2]) & 0x7fff7fffu;
+                for (int u = 0; u < 2; u++) {
+                    float h, l;
+                    rs::moments_sum(h, l, rs::F4{c01.x, c01.y, c01.z, c01.w}, rs::F4{c23.x, c23.y, c23.z, c23.w},
+                                    rs::F4{c47.x, c47.y, c47.z, c47.w}, rs::F4{a[u].x, a[u].y, a[u].z, a[u].w},
+                                    rs::F4{b[u].x, b[u].y, b[u].z, b[u].w}, c[u].x, c[u].y);
+                    rs::acc3_add(acc[i][u][0], acc[i][u][1], acc[i][u][2], h, l);
                 }
-            }
-            bool use[kRsSlices];
-#pragma unroll
-            for (int i = 0; i < kRsSlices; i++) use[i] = __any_sync(0xffffffffu, any[i] != 0u);
-            const uint2* tab = (const uint2*)(unfold_sm + buf * kRsUnfoldStep) + first * kRsUnfoldTiles * 32 + lane;
-            constexpr int stride = kRsUnfoldTiles * 32;
-#pragma unroll
-            for (int mt = 0; mt < kRsUnfoldTiles; mt++) {
-                if (mt0 + mt < mt1 && 8 * (mt0 + mt + 1) >= m0) {
-                    uint2 b[count];
-#pragma unroll
-                    for (int jj = 0; jj < count; jj++) b[jj] = tab[jj * stride + 32 * mt];
-#pragma unroll
-                    for (int i = 0; i < kRsSlices; i++) {
-                        if (use[i]) {
-#pragma unroll
-                            for (int jj = 0; jj < count; jj++)
-                                if (i + jj <= 4) rs_mma(acc[mt][i + jj], a[i], b[jj]);
-                        }
-                    }
-                }
-            }
-        };
-        power(std::integral_constant<int, 0>{});
-        power(std::integral_constant<int, 1>{});
-        power(std::integral_constant<int, 2>{});
-        power(std::integral_constant<int, 3>{});
-        power(std::integral_constant<int, 4>{});
-        power(std::integral_constant<int, 5>{});
-        power(std::integral_constant<int, 6>{});
-        power(std::integral_constant<int, 7>{});
-#pragma unroll
-        for (int mt = 0; mt < kRsUnfoldTiles; mt++) {
-            if (mt0 + mt >= mt1 || 8 * (mt0 + mt + 1) < m0) continue;
-#pragma unroll
-            for (int c = 0; c < 4; c++) {
-                const float(&v)[5][4] = acc[mt];
-                const float sc = unit[c >> 1];
-                float s, e;
-                rs::two_sum(v[0][c], __fmul_rn(v[1][c], 0x1p-11f), s, e);
-                const float t = __fmaf_rn(__fmaf_rn(v[4][c], 0x1p-11f, v[3][c]), 0x1p-11f, v[2][c]);
-                rs::acc_add(out[mt][c].x, out[mt][c].y, __fmul_rn(s, sc), __fmul_rn(__fmaf_rn(t, 0x1p-22f, e), sc));
             }
         }
     }
 #pragma unroll
-    for (int mt = 0; mt < kRsUnfoldTiles; mt++) {
-        if (mt0 + mt >= mt1) continue;
+    for (int i = 0; i < kRsOutPer; i++)
 #pragma unroll
-        for (int c = 0; c < 4; c++) {
-            const int64_t l = l0 + g + 8 * (c >> 1);
-            const int m = 8 * (mt0 + mt) + 2 * q + (c & 1) + 1;
-            if (l >= P.M) continue;
-            if (s1 < R.nint) {
-                sums[l * R.nmp + m - 1] = out[mt][c];
-            } else if (m < R.nm) {
-                const double v = ((double)out[mt][c].x + (double)out[mt][c].y) * 0x1p-30;
-                if (v != 0.0) {
-                    int64_t slot = (n + 1 - m) % P.ring;
-                    if (slot < 0) slot += P.ring;
-                    sb[slot * P.M + l] += v;
-                }
-            }
+        for (int u = 0; u < 2; u++) {
+            const int m = mfirst + i * nwarps;
+            const int64_t l = l0 + lane + 32 * u;
+            if (m < R.nm && l < P.M) sums[(int64_t)(m - 1) * P.M + l] = rs::acc3_value(acc[i][u][0], acc[i][u][1], acc[i][u][2]);
         }
+}
+
+// the runs' sums in order into the ring: sigmabar_l^{n+1-m} += sum_z sums[z][m][l] (blockIdx.y: m - 1)
+__global__ void k_rs_unfold_add(DevPlan P, RangeDev R, int runs, int64_t n, const double* __restrict__ sums, double* __restrict__ sb) {
+    const int m = 1 + blockIdx.y;
+    double* out = sb + (int64_t)ring_slot(n + 1 - m, P.ring) * P.M;
+    for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < P.M; l += (int64_t)gridDim.x * blockDim.x) {
+        double v = 0.0;
+        for (int z = 0; z < runs; z++) v += __ldg(sums + ((int64_t)z * (R.nm - 1) + m - 1) * P.M + l);
+        if (v != 0.0) out[l] += v;
     }
 }
 

@@ -94,6 +94,25 @@ WAVE1D_RS_HD void acc_mac(float& ah, float& al, float wh, float wl, float vh, fl
     acc_add(ah, al, p, e);
 }
 
+// A sum of pairs in three floats h + m + l: the residuals of the pairs' high and low parts are kept, l's own
+// rounding is 2^-24 of what is below 2^-47 of the sum, so the sum of thousands of pairs is good to more than
+// FP64's 53 bits.
+WAVE1D_RS_HD void acc3_add(float& h, float& m, float& l, float vh, float vl) {
+    float s, e1, e2, e3;
+    two_sum(h, vh, s, e1);
+    h = s;
+    two_sum(m, vl, s, e2);
+    two_sum(s, e1, m, e3);
+    l = add(l, add(e2, e3));
+}
+WAVE1D_RS_HD double acc3_value(float h, float m, float l) { return (double)h + ((double)m + (double)l); }
+WAVE1D_RS_HD void acc3_set(double v, float& h, float& m, float& l) {
+    h = (float)v;
+    v -= (double)h;
+    m = (float)v;
+    l = (float)(v - (double)m);
+}
+
 // the pair of a double: hi = fl(v), lo = fl(v - hi)
 WAVE1D_RS_HD Pair split(double v) {
     const float h = (float)v;
@@ -200,6 +219,24 @@ WAVE1D_RS_HD void evec_eval(const float* e, float zh, float zl, float& ah, float
 // the same from an e-vector held in registers
 WAVE1D_RS_HD void evec_eval_v(const EVec& v, float zh, float zl, float& ah, float& al) {
     evec_eval4(F4{v.e0h, v.e0l, v.e1h, v.e1l}, F4{v.e2, v.e3, v.e4, v.e5}, F4{v.e6, v.e7, 0.f, 0.f}, zh, zl, ah, al);
+}
+
+// (h, l) = sum_r a_r F_r, one interval's part of a transposed sum: coefficients as in evec_mac, moments f01 =
+// (F0h F0l F1h F1l), f25 = (F2 .. F5), f6, f7
+WAVE1D_RS_HD void moments_sum(float& h, float& l, const F4& c01, const F4& c23, const F4& c47, const F4& f01,
+                              const F4& f25, float f6, float f7) {
+    h = mul(c01.x, f01.x);                          // acc_mac into zeros
+    l = fma_(c01.x, f01.x, -h);
+    l = fma_(c01.x, f01.y, l);
+    l = fma_(c01.y, f01.x, l);
+    acc_mac(h, l, c01.z, c01.w, f01.z, f01.w);
+    float r = fma_(c23.y, f25.x, mul(c23.x, f25.x));
+    r = fma_(c23.w, f25.y, fma_(c23.z, f25.y, r));
+    r = fma_(c47.x, f25.z, r);
+    r = fma_(c47.y, f25.w, r);
+    r = fma_(c47.z, f6, r);
+    r = fma_(c47.w, f7, r);
+    acc_add(h, l, r, 0.f);
 }
 
 // ---------------------------------------------------------------------------------------------
