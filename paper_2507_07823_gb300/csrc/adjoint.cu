@@ -14,6 +14,7 @@
 
 #include "adjoint.cuh"
 #include "internal.h"
+#include "range.cuh"
 
 namespace wave1d {
 
@@ -65,9 +66,10 @@ __global__ void k_adj_solve(DevPlan P, const int32_t* __restrict__ blk_of, const
 // direction, Q_m being symmetric in the pair), in the compensated FP32 arithmetic of the forward
 // local sum: each lane accumulates its slices into the warp's shared pairs acc[m][lane] (row
 // stride kAdjAccStride), eight slices' weights in flight, then lane i adds m = i, i + 32, ... over the
-// 32 lanes in lane order, as pairs, and adds the result to sigmabar^{n+1-m}[l].  Dynamic shared memory:
-// warps per block x (m_max + 1) x kAdjAccStride float pairs.  With the lanes' sums in FP64 (4 x 32
-// instructions a row and m of the FP64 pipe) and one slice in flight it took 137 us for 1.1e7 weights.
+// 32 lanes in lane order, in three floats (acc3_add, more than FP64's bits), and adds the result to
+// sigmabar^{n+1-m}[l].  Dynamic shared memory: warps per block x (m_max + 1) x kAdjAccStride float pairs.
+// With the lanes' sums in FP64 (4 x 32 instructions a row and m of the FP64 pipe) and one slice in flight
+// it took 137 us for 1.1e7 weights; now 48 (45 with the sums as one pair, which holds less).
 constexpr int kAdjAccStride = 33;
 
 __global__ void k_adj_local(DevPlan P, int64_t n, const double* __restrict__ cbar, double* sb) {
@@ -110,12 +112,12 @@ __global__ void k_adj_local(DevPlan P, int64_t n, const double* __restrict__ cba
     }
     __syncwarp();
     for (int m = lane; m < nm; m += 32) {
-        float sh = 0.f, sl = 0.f;
+        float sh = 0.f, sm = 0.f, sl = 0.f;
         for (int i = 0; i < 32; i++) {
             const float2 a = acc[m * kAdjAccStride + i];
-            adj::pair_mac(sh, sl, 1.f, 0.f, a.x, a.y);
+            rs::acc3_add(sh, sm, sl, a.x, a.y);
         }
-        const double s = (double)sh + (double)sl;
+        const double s = rs::acc3_value(sh, sm, sl);
         if (s != 0.0) sb[(int64_t)adj::slot(n + 1 - m, P.ring) * P.M + l] += s;
     }
 }
