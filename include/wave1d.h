@@ -90,6 +90,13 @@ typedef struct {
                            (WAVE1D_ENOTCONV after 40).  For layouts whose weights or blocks do
                            not fit (a million clustered springs: 1.3e10 pairs); steps run as
                            per-stage launches; wave1d_adjoint needs every stiffness > 0.
+                           Device memory beside the density rings: 48 bytes per spring and interval
+                           of distance (some 15 to 20 intervals to a step of the window) for as many
+                           intervals as fit 16 KB a spring (8 KB below 16384 springs), 4 GiB and an
+                           eighth of what is free, but 64 to 160 of them at least (3 to 8 KB a spring,
+                           4 GiB at most, above 5.6e6 springs 16 intervals); 8 bytes per pair closer than
+                           dt; a bit per spring and interval where pairs are few.  Results do not
+                           depend on how much memory is free.
                            Batched plans also take 2: each instance's form chosen from its layout
                            (see wave1d_batch_plan)                                             */
     int spin_limit;     /* polls of a counter before a wait between the blocks of the one-launch

@@ -328,25 +328,12 @@ int fold_tables(wave1d_plan_t p) {
     rd.fine = h16;
     rd.fine_span = rt.fine_span;
     rd.fine_scale = (float)(kRsFineCells / P.delta);
-    // parts of the pair kernel: intervals that hold about 160 sources to a side on average (a warp's 32
-    // targets start and end up to 32 sources apart, which it waits for), 64 to 160 of them: a million
-    // clustered springs 80.7 ms per step with parts of 16, 74.5 of 32, 72.6 of 64; 1e5 uniform springs
-    // 3.46 ms with parts of 80, 3.33 of 160
-    const double side = std::max(1.0, 0.5 * (double)p->hp.range_pairs / (double)P.M);
-    const int padded = (rt.nint + 15) / 16 * 16;
-    rd.part = std::min(padded, std::max(64, std::min(160, (int)std::ceil(rt.nint * 160.0 / side / 16.0) * 16)));
-    // e-vectors of a slab of intervals at a time: 16 KB a spring (some 340 intervals; 8 KB below 16384
-    // springs, whose plans stay smaller than one with stored weights) up to 4 GiB, never more than an
-    // eighth of the memory that is free, so that many plans fit beside one another; the results do not
-    // depend on the slab (unless it has to be smaller than a part)
     size_t free_b = 0, all_b = 0;
     if (cudaMemGetInfo(&free_b, &all_b) != cudaSuccess) return fail(WAVE1D_ECUDA, "cudaMemGetInfo");
-    const size_t per_iv = (size_t)P.M * kRsRecord * sizeof(float);
-    const size_t want = std::min({(size_t)(P.M < 16384 ? 8192 : 16384) * P.M, (size_t)4 << 30, free_b / 8});
-    const int most_iv = std::max(16, (int)std::min<size_t>((size_t)padded, want / per_iv / 16 * 16));
-    rd.part = std::min(rd.part, most_iv);
-    rd.slab = most_iv / rd.part * rd.part;
-    rd.nparts = (rt.nint + rd.part - 1) / rd.part;
+    const RangeSplit split = range_split(rt.nint, P.M, p->hp.range_pairs, free_b);
+    rd.part = split.part;
+    rd.nparts = split.nparts;
+    rd.slab = split.slab;
     if ((rc = dalloc(p, &rd.evec, (size_t)P.M * rd.slab * kRsRecord))) return rc;
     if ((rc = dalloc(p, &rd.csum, (size_t)4 * rd.nparts * P.M))) return rc;
     // where there is less than a pair to a record, only the records that some pair reads are made

@@ -127,6 +127,14 @@ constexpr int kRsRecord = 12;       // floats of an e-vector record in memory
 constexpr int kRsTTargets = 128;    // outputs per block where a host check walks the transposed sum
 constexpr int kRsCells = 2048;
 
+// How the intervals of a plan without pair lists are cut: parts, whose pairs are summed together (so they
+// set the order of every sum, and follow from the layout alone), and slabs, whose records are held at once (whole
+// parts, one at least; the results do not depend on them).
+struct RangeSplit {
+    int part, nparts, slab;
+};
+RangeSplit range_split(int nint, int64_t M, int64_t pairs, size_t free_bytes);
+
 struct HostPlan {
     Params P;
     std::vector<int32_t> perm;         // internal index -> caller index

@@ -1257,6 +1257,29 @@ static void fold_slices(const std::vector<double>& a, RangeTables& rt) {
     rt.fine_span = std::max(rt.fine_span, n - 1 - last);
 }
 
+// Parts hold about 160 sources to a side on average (a warp's 32 targets start and end up to 32 sources apart,
+// which it waits for), 64 to 160 intervals: a million clustered springs 80.7 ms per step with parts of 16,
+// 74.5 of 32, 72.6 of 64; 1e5 uniform springs 3.46 ms with parts of 80, 3.33 of 160.  No more than 4 GiB of
+// records to a part, 16 intervals at least.
+// Slabs: 16 KB of records a spring (some 340 intervals; 8 KB below 16384 springs, whose plans stay smaller
+// than one with stored weights) up to 4 GiB, and no more than an eighth of the memory that is free where
+// that is more than a part, so that many plans fit beside one another.
+RangeSplit range_split(int nint, int64_t M, int64_t pairs, size_t free_bytes) {
+    const int padded = (nint + 15) / 16 * 16;
+    const size_t per_iv = (size_t)M * kRsRecord * sizeof(float), cap = (size_t)4 << 30;
+    auto intervals = [&](size_t bytes) {
+        return std::max(16, (int)std::min<size_t>((size_t)padded, bytes / per_iv / 16 * 16));
+    };
+    const double side = std::max(1.0, 0.5 * (double)pairs / (double)M);
+    RangeSplit r;
+    r.part = std::min(padded, std::max(64, (int)std::min(160.0, std::ceil(nint * 160.0 / side / 16.0) * 16)));
+    r.part = std::min(r.part, intervals(std::min((size_t)(M < 16384 ? 8192 : 16384) * M, cap)));
+    r.nparts = (nint + r.part - 1) / r.part;
+    const int most = intervals(std::min({(size_t)(M < 16384 ? 8192 : 16384) * M, cap, free_bytes / 8}));
+    r.slab = std::max(1, most / r.part) * r.part;
+    return r;
+}
+
 void build_range_tables(const Params& P, RangeTables& rt) {
     rt = RangeTables();
     rt.nm = P.m_max + 1;
