@@ -317,23 +317,24 @@ int upload_receivers(wave1d_plan_t p) {
     return WAVE1D_OK;
 }
 
-// the tables and work arrays of the range-mode local sum (range.cu)
-int fold_tables(wave1d_plan_t p) {
+// the cut of the intervals for the memory that is free now
+int split_intervals(wave1d_plan_t p, RangeDev& rd) {
+    size_t free_b = 0, all_b = 0;
+    if (cudaMemGetInfo(&free_b, &all_b) != cudaSuccess) return fail(WAVE1D_ECUDA, "cudaMemGetInfo");
+    const RangeSplit split = range_split(p->hp.rt.nint, p->hp.P.M, p->hp.range_pairs, free_b);
+    rd.part = split.part;
+    rd.nparts = split.nparts;
+    rd.slab = split.slab;
+    return WAVE1D_OK;
+}
+
+// the work arrays of the range-mode local sum (range.cu)
+int fold_arrays(wave1d_plan_t p) {
     const RangeTables& rt = p->hp.rt;
     const Params& P = p->hp.P;
     RangeDev& rd = p->rd;
     int rc;
-    uint16_t* h16;
-    if ((rc = upload(p, rt.fine, &h16))) return rc;
-    rd.fine = h16;
-    rd.fine_span = rt.fine_span;
-    rd.fine_scale = (float)(kRsFineCells / P.delta);
-    size_t free_b = 0, all_b = 0;
-    if (cudaMemGetInfo(&free_b, &all_b) != cudaSuccess) return fail(WAVE1D_ECUDA, "cudaMemGetInfo");
-    const RangeSplit split = range_split(rt.nint, P.M, p->hp.range_pairs, free_b);
-    rd.part = split.part;
-    rd.nparts = split.nparts;
-    rd.slab = split.slab;
+    if ((rc = split_intervals(p, rd))) return rc;
     if ((rc = dalloc(p, &rd.evec, (size_t)P.M * rd.slab * kRsRecord))) return rc;
     if ((rc = dalloc(p, &rd.csum, (size_t)4 * rd.nparts * P.M))) return rc;
     // where there is less than a pair to a record, only the records that some pair reads are made
@@ -835,6 +836,11 @@ int wave1d_plan(const double* x, const double* beta, int64_t M, int bc, double d
         if ((rc = upload(p, rt.cell, &r32))) return cleanup(rc);
         rd.cell = r32;
         rd.cell_scale = rt.cell_scale;
+        uint16_t* r16;
+        if ((rc = upload(p, rt.fine, &r16))) return cleanup(rc);
+        rd.fine = r16;
+        rd.fine_span = rt.fine_span;
+        rd.fine_scale = (float)(kRsFineCells / P.delta);
         if ((rc = upload(p, hp.blk_win, &r32))) return cleanup(rc);
         rd.blk_win = r32;
         if ((rc = upload(p, hp.nb_lo, &r32))) return cleanup(rc);
@@ -856,7 +862,7 @@ int wave1d_plan(const double* x, const double* beta, int64_t M, int bc, double d
             if (!allow_smem((const void*)k_rs_local, p->rs_smem))
                 return cleanup(fail(WAVE1D_ECUDA, "cannot size the shared memory of the range-mode local sum"));
         } else {
-            if ((rc = fold_tables(p))) return cleanup(rc);
+            if ((rc = fold_arrays(p))) return cleanup(rc);
             rd.folded = 1;
         }
         p->info_range_pairs = hp.range_pairs;
@@ -1436,7 +1442,8 @@ struct Reverse {
     int npts = 0;
     size_t lsmem = 0;
     double2* waves = nullptr;
-    double* rrhs = nullptr;   // plans without pair lists: the transposed solve's right-hand side
+    RangeDev rd{};            // plans without pair lists: the plan's tables, and for a mixed plan this call's records
+    double* rrhs = nullptr;   // the transposed solve's right-hand side
     double* usum = nullptr;   // the transposed local sum's runs between slabs
     int runs = 1;
     static constexpr int kLocalWarps = 4;     // the transposed local sum: one warp per spring row
@@ -1480,10 +1487,14 @@ struct Reverse {
         }
         if (p->range) {
             if ((rc = wk.zeros(&rrhs, (size_t)M))) return rc;
-            if (!p->rd.evec && (rc = fold_tables(p))) return rc;        // a mixed plan's first reverse march
+            rd = p->rd;
+            if (p->mixed) {              // its forward march keeps no records: the moments' are this call's
+                if ((rc = split_intervals(p, rd))) return rc;
+                if ((rc = wk.zeros(&rd.evec, (size_t)M * rd.slab * kRsRecord))) return rc;
+            }
             if (!allow_smem((const void*)k_rs_unfold, rs_unfold_smem()))
                 return fail(WAVE1D_ECUDA, "cannot size the shared memory of the transposed local sum");
-            runs = rs_unfold_runs(M, p->rd.slab, p->sms);
+            runs = rs_unfold_runs(M, rd.slab, p->sms);
             return wk.zeros(&usum, (size_t)runs * M * P.m_max);
         }
         lsmem = adj_local_smem(P.m_max, kLocalWarps);
@@ -1521,7 +1532,6 @@ struct Reverse {
             if (p->range) {
                 // plan without pair lists: receivers, solve and local sum transposed on the
                 // range tables; the solve is the forward Jacobi sweeps on beta-scaled data
-                const RangeDev& rd = p->rd;
                 if (R > 0) k_rs_adj_receivers<<<dim3(gM, 8), 256, 0, s>>>(d, rd, n, ub, sb);
                 k_rs_adj_init<<<gM, 256, 0, s>>>(d, rd, sb + (int64_t)((n + 1) % ring) * M, rrhs);
                 DevPlan dj = d;

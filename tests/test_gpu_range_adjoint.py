@@ -41,3 +41,33 @@ def test_gradients_match_the_stored_weight_plan(bc, M, tol, p, opt):
             plan.close()
     for a, b in zip(*out):
         assert np.max(np.abs(a)) > 0 and np.max(np.abs(b - a)) <= 1e-9 * np.max(np.abs(a))
+
+
+def test_reverse_march_of_a_mixed_plan():
+    """Mixed plans march back in FP64 through the same kernels: the gradients of the FP64 plan without pair lists from
+    the same densities (bar: 1e-10, the sweeps' stopping rule and order), the same bits from call to call, and no
+    memory kept by the plan; from checkpoints the same bits as from stored densities."""
+    rng = np.random.default_rng(5)
+    M = 900
+    x = np.sort(rng.uniform(-0.6, 0.6, M))
+    w = W.Workload(name="mixed", bc=W.FREE, x=x, beta=rng.uniform(0.5, 2.0, M), amp=np.array([1.0]), center=np.array([-0.2]),
+                   width=np.array([0.3]), dt=1e-3, Nt=40, tol=1e-6, p=4, xr=np.array([-0.7, x[11], 0.65]), seed=5)
+    ubar = torch.from_numpy(rng.standard_normal((w.Nt, 3))).cuda()
+    f64 = wave1d.Plan.from_workload(w, local_weights=1)
+    mixed = wave1d.Plan.from_workload(w, local_weights=1, precision=1)
+    ck = wave1d.Plan.from_workload(w, local_weights=1, precision=1)
+    try:
+        sigma, _ = mixed.solve_device(w.Nt)
+        a = f64.adjoint(sigma, ubar, forcing_gradient=True)
+        before = wave1d.wave1d_get_info(mixed.h).device_bytes
+        b = mixed.adjoint(sigma, ubar, forcing_gradient=True)
+        c = mixed.adjoint(sigma, ubar, forcing_gradient=True)
+        assert wave1d.wave1d_get_info(mixed.h).device_bytes == before
+        _, buf = ck.solve_checkpointed(w.Nt, 7)
+        d = ck.adjoint_checkpointed(buf, w.Nt, 7, ubar, forcing_gradient=True)
+        for u, v, s, t in zip(a, b, c, d):
+            assert float((v - u).abs().max()) <= 1e-10 * float(u.abs().max()) and float(u.abs().max()) > 0
+            assert torch.equal(v, s) and torch.equal(v, t)
+    finally:
+        for plan in (f64, mixed, ck):
+            plan.close()
