@@ -613,7 +613,7 @@ int upload_joined_part(wave1d_batch_t p, const std::vector<int>& joined, const d
     // batched NUFFT plans of the springs and of the receivers: the instances' fine grids, kernel
     // (width from tol, as each instance's plan) and deconvolution
     rc = wave1d_nufft_plan_many(p->bt.g.x.data(), p->bt.moff.data(), p->B, P.K, tol, 0, (void*)p->s, &p->nu_s);
-    if (rc) return bfail(rc, std::string("batched NUFFT plan: ") + wave1d_nufft_strerror());
+    if (rc || (rc = nufft_build_ranges(p->nu_s))) return bfail(rc, std::string("batched NUFFT plan: ") + wave1d_nufft_strerror());
     std::vector<int64_t> perm((size_t)P.M);
     if ((rc = wave1d_nufft_perm(p->nu_s, perm.data()))) return bfail(rc, wave1d_nufft_strerror());
     if ((rc = bupload(p, perm, &p->perm_s))) return rc;

@@ -28,6 +28,7 @@
 #include <numeric>
 #include <string>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "internal.h"
@@ -271,7 +272,7 @@ __global__ void __launch_bounds__(kUnitThreads) k_nu_spread64(const NuRange* __r
 // weights lane by lane, 88 bytes apart: 67 us there.  (Compensated FP32 pairs in place of FP64 here: 43 us
 // with unequal segments, as splitting each weight costs what they save.)
 // ---------------------------------------------------------------------------------------------
-constexpr int kSegPoints = 64;      // points of a segment at most
+constexpr int kSegPoints = 64;      // points of a segment at most, unless the autotuner finds better
 
 template <int W>
 __global__ void __launch_bounds__(256) k_nu_tap_sums(const int32_t* __restrict__ seg, int64_t nseg,
@@ -580,6 +581,19 @@ bool nu_with_mixed(int w, int D, F&& f) {
 
 }  // namespace
 
+// How a plan's spreading is cut.  Ranges (mixed plans; FP64 plans of a batch, whose one-launch step spreads by
+// them): cell ranges tiling every instance's grid, with their run tables.  Segments (FP64): `points` points of one
+// cell at most, the first segment of every cell, tap sums.
+struct NuSplit {
+    int cells = 0, points = 0;       // the caps it was cut with (segments: one cell)
+    NuRange* ranges = nullptr;
+    int64_t nunits = 0;
+    int32_t* runs = nullptr;
+    int32_t *seg = nullptr, *cseg = nullptr;
+    int64_t nseg = 0;
+    double* tap_sums = nullptr;
+};
+
 struct wave1d_nufft_s {
     int device = 0;
     int precision = 0;
@@ -596,15 +610,7 @@ struct wave1d_nufft_s {
     float* soff = nullptr;
     NuPoly poly{};                   // tap polynomials (mixed), passed to the kernels by value
     double* ker = nullptr;
-    // spreading ranges (cell ranges tiling every instance's grid) and their run tables
-    NuRange* ranges = nullptr;
-    int64_t nunits = 0;              // ranges
-    int32_t* runs = nullptr;
-    int range_cells = 0, range_points = 0;   // the caps the ranges were cut with
-    // FP64: segments of points (kSegPoints of one cell at most), the first one of every cell, tap sums
-    int32_t *seg = nullptr, *cseg = nullptr;
-    int64_t nseg = 0;
-    double* tap_sums = nullptr;
+    NuSplit split;                   // the work split of the spreading
     std::vector<int32_t> i0_host;    // points' first cells (sorted within each instance), for re-cutting
     std::vector<int64_t> off_host;   // instance offsets
     // FFT and deconvolution
@@ -636,14 +642,76 @@ int nu_alloc(wave1d_nufft_t h, size_t count, T** out) {
     return WAVE1D_OK;
 }
 
+void nu_free(wave1d_nufft_t h, void* p) {
+    if (!p) return;
+    h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), p));
+    cudaFree(p);
+}
+
+void nu_drop(wave1d_nufft_t h, NuSplit& s) {
+    for (void* p : {(void*)s.ranges, (void*)s.runs, (void*)s.seg, (void*)s.cseg, (void*)s.tap_sums}) nu_free(h, p);
+    s = NuSplit();
+}
+
+// ranges of at most `cells` cells and `points` points
+int nu_cut_ranges(wave1d_nufft_t h, int cells, int points, NuSplit& s) {
+    std::vector<NuRange> ranges;
+    std::vector<int32_t> runs;
+    nufft_ranges(h->i0_host, h->off_host.data(), h->B, h->P.nf, h->P.nufft_w, cells, points, kEmptyCells, kUnitThreads, ranges,
+                 runs);
+    s.cells = cells;
+    s.points = points;
+    s.nunits = (int64_t)ranges.size();
+    int rc = nu_upload(h, ranges, &s.ranges);
+    return rc ? rc : nu_upload(h, runs, &s.runs);
+}
+
+// segments of at most `points` points of one cell
+int nu_cut_segments(wave1d_nufft_t h, int points, NuSplit& s) {
+    const int64_t cells = (int64_t)h->B * h->P.nf;
+    std::vector<int32_t> seg, cseg((size_t)cells + 1, 0);
+    int64_t cell = 0;                                // cells below it know their first segment
+    for (int b = 0; b < h->B; b++)
+        for (int64_t i = h->off_host[b]; i < h->off_host[b + 1];) {
+            int64_t e = i;
+            while (e < h->off_host[b + 1] && h->i0_host[e] == h->i0_host[i]) e++;
+            for (const int64_t at = (int64_t)b * h->P.nf + h->i0_host[i]; cell <= at; cell++) cseg[cell] = (int32_t)seg.size();
+            const int64_t parts = (e - i + points - 1) / points;              // equal, as a warp takes two
+            for (int64_t q = 0; q < parts; q++) seg.push_back((int32_t)(i + (e - i) * q / parts));
+            i = e;
+        }
+    for (; cell <= cells; cell++) cseg[cell] = (int32_t)seg.size();
+    s.cells = 1;
+    s.points = points;
+    s.nseg = (int64_t)seg.size();
+    seg.push_back((int32_t)h->M);
+    int rc;
+    if ((rc = nu_upload(h, seg, &s.seg)) || (rc = nu_upload(h, cseg, &s.cseg))) return rc;
+    return nu_alloc(h, (size_t)s.nseg * h->P.nufft_w, &s.tap_sums);
+}
+
 }  // namespace
 
 namespace wave1d {
+int nufft_build_ranges(wave1d_nufft_t h) {
+    if (!h || h->precision != 0) return WAVE1D_EINVAL;
+    if (h->split.ranges) return WAVE1D_OK;
+    NuSplit s;
+    const int rc = nu_cut_ranges(h, kRangeCells64, kRangePoints64, s);
+    if (rc) {
+        nu_drop(h, s);
+        return rc;
+    }
+    h->split.ranges = s.ranges;
+    h->split.runs = s.runs;
+    h->split.nunits = s.nunits;
+    return WAVE1D_OK;
+}
 int nufft_dev64(wave1d_nufft_t h, NuDev64& out) {
     if (!h || h->precision != 0) return WAVE1D_EINVAL;
-    out.ranges = h->ranges;
-    out.runs = h->runs;
-    out.nunits = h->nunits;
+    out.ranges = h->split.ranges;
+    out.runs = h->split.runs;
+    out.nunits = h->split.nunits;
     out.ker = h->ker;
     out.i0 = h->first;
     out.M = h->M;
@@ -652,10 +720,10 @@ int nufft_dev64(wave1d_nufft_t h, NuDev64& out) {
     return WAVE1D_OK;
 }
 int nufft_spread_ranges(wave1d_nufft_t h, const double* c, double* grid) {
-    if (!h || h->precision != 0) return WAVE1D_EINVAL;
+    if (!h || h->precision != 0 || !h->split.ranges) return WAVE1D_EINVAL;
     if (!nu_with_w(h->P.nufft_w, [&](auto wc) {
-            k_nu_spread64<decltype(wc)::value><<<(unsigned)h->nunits, kUnitThreads, 0, h->stream>>>(h->ranges, h->runs, c, h->ker,
-                                                                                             grid);
+            k_nu_spread64<decltype(wc)::value><<<(unsigned)h->split.nunits, kUnitThreads, 0, h->stream>>>(h->split.ranges, h->split.runs,
+                                                                                                   c, h->ker, grid);
         }))
         return nfail(WAVE1D_EUNSUPPORTED, "kernel width not built");
     return cudaGetLastError() == cudaSuccess ? WAVE1D_OK : nfail(WAVE1D_ECUDA, "spread launch failed");
@@ -798,38 +866,10 @@ int wave1d_nufft_plan_many(const double* x, const int64_t* offsets, int n_inst, 
         h->kernel_err = err;
         if ((rc = nu_upload(h, soff, &h->soff))) return cleanup(rc);
     }
-    {
-        std::vector<NuRange> ranges;
-        std::vector<int32_t> runs;
-        nufft_ranges(i0, offsets, n_inst, nf, w, precision == 1 ? kRangeCells : kRangeCells64,
-                     precision == 1 ? kRangePoints : kRangePoints64, kEmptyCells, kUnitThreads, ranges, runs);
-        if (precision == 0) {
-            std::vector<int32_t> seg, cseg((size_t)n_inst * nf + 1, 0);
-            int64_t cell = 0;                        // cells below it know their first segment
-            for (int64_t i = 0; i < M;) {
-                int64_t e = i;
-                while (e < M && gfirst[e] == gfirst[i]) e++;
-                for (; cell <= gfirst[i]; cell++) cseg[cell] = (int32_t)seg.size();
-                const int64_t parts = (e - i + kSegPoints - 1) / kSegPoints;      // equal, as a warp takes two
-                for (int64_t q = 0; q < parts; q++) seg.push_back((int32_t)(i + (e - i) * q / parts));
-                i = e;
-            }
-            for (; cell <= (int64_t)n_inst * nf; cell++) cseg[cell] = (int32_t)seg.size();
-            h->nseg = (int64_t)seg.size();
-            seg.push_back((int32_t)M);
-            if ((rc = nu_upload(h, seg, &h->seg)) || (rc = nu_upload(h, cseg, &h->cseg)) ||
-                (rc = nu_alloc(h, (size_t)h->nseg * w, &h->tap_sums)))
-                return cleanup(rc);
-        }
-        h->nunits = (int64_t)ranges.size();
-        h->range_cells = precision == 1 ? kRangeCells : kRangeCells64;
-        h->range_points = precision == 1 ? kRangePoints : kRangePoints64;
-        h->i0_host = i0;
-        h->off_host.assign(offsets, offsets + n_inst + 1);
-        if ((rc = nu_upload(h, ranges, &h->ranges)) || (rc = nu_upload(h, runs, &h->runs)) ||
-            (rc = nu_upload(h, gfirst, &h->first)))
-            return cleanup(rc);
-    }
+    h->i0_host = i0;
+    h->off_host.assign(offsets, offsets + n_inst + 1);
+    rc = precision == 1 ? nu_cut_ranges(h, kRangeCells, kRangePoints, h->split) : nu_cut_segments(h, kSegPoints, h->split);
+    if (rc || (rc = nu_upload(h, gfirst, &h->first))) return cleanup(rc);
     std::vector<double> d1, d2, mf, tw((size_t)P.L * 2);
     nufft_factors(P, d1, d2, mf);
     for (int j = 0; j < P.L; j++) {
@@ -868,19 +908,19 @@ int wave1d_nufft_spread(wave1d_nufft_t h, const double* c, double* grid) {
     if (!h || !c || !grid) return nfail(WAVE1D_EINVAL, "bad arguments");
     if (cudaSetDevice(h->device) != cudaSuccess) return nfail(WAVE1D_ECUDA, "cudaSetDevice");
     const int w = h->P.nufft_w;
-    const unsigned nu = (unsigned)h->nunits;
+    const NuSplit& sp = h->split;
     bool ok;
     if (h->precision == 0) {
         const int64_t cells = (int64_t)h->B * h->P.nf;
         ok = nu_with_w(w, [&](auto wc) {
             constexpr int W = decltype(wc)::value;
-            k_nu_tap_sums<W><<<(unsigned)((h->nseg * 16 + 255) / 256), 256, 0, h->stream>>>(h->seg, h->nseg, c, h->ker, h->tap_sums);
-            k_nu_assemble<W><<<(unsigned)((cells + 255) / 256), 256, 0, h->stream>>>(h->cseg, h->tap_sums, grid, cells, h->P.nf);
+            k_nu_tap_sums<W><<<(unsigned)((sp.nseg * 16 + 255) / 256), 256, 0, h->stream>>>(sp.seg, sp.nseg, c, h->ker, sp.tap_sums);
+            k_nu_assemble<W><<<(unsigned)((cells + 255) / 256), 256, 0, h->stream>>>(sp.cseg, sp.tap_sums, grid, cells, h->P.nf);
         });
     } else {
         ok = nu_with_mixed(w, h->D, [&](auto wc, auto dc) {
-            k_nu_spread_mixed<decltype(wc)::value, decltype(dc)::value><<<nu, kUnitThreads, 0, h->stream>>>(
-                h->ranges, h->runs, c, h->soff, h->poly, grid);
+            k_nu_spread_mixed<decltype(wc)::value, decltype(dc)::value><<<(unsigned)sp.nunits, kUnitThreads, 0, h->stream>>>(
+                sp.ranges, sp.runs, c, h->soff, h->poly, grid);
         });
     }
     if (!ok) return nfail(WAVE1D_EUNSUPPORTED, "kernel width / degree not built");
@@ -949,70 +989,64 @@ int wave1d_nufft_destroy(wave1d_nufft_t h) {
     return WAVE1D_OK;
 }
 
-// Picks the spreading work split (its tile width and bin size: the cells and points a range is cut
-// at) for this plan's points by timing: each candidate pair of caps, at or below the kernels'
-// shared-memory capacities, re-cuts the ranges from the points' first cells and is timed over
-// `reps` spreads of c (after one untimed spread) with CUDA events on the plan's stream; the fastest
-// stays.  The grid is overwritten.  Every candidate tiles the grids completely (the range builder
-// is the plan's own), so results change only in rounding (the lanes per cell follow the ranges).
+// Picks the work split of the spreading for this plan's points by timing: each candidate is cut from the
+// points' first cells and timed over `reps` spreads of c (after one untimed spread) with CUDA events on the
+// plan's stream; the fastest stays, the others' tables go.  Mixed: cells and points a range is cut at, at or below the
+// kernel's shared-memory capacities.  FP64: points of one cell to a segment.  The grid is overwritten.  Every
+// candidate takes every point once, so results change only in rounding.
 int wave1d_nufft_autotune(wave1d_nufft_t h, const double* c, double* grid, int reps, int* cells, int* points) {
     if (!h || !c || !grid || reps < 1) return nfail(WAVE1D_EINVAL, "bad arguments");
     if (cudaSetDevice(h->device) != cudaSuccess) return nfail(WAVE1D_ECUDA, "cudaSetDevice");
-    const bool mixed = h->precision == 1;
-    const int cmax = mixed ? kRangeCells : kRangeCells64, pmax = mixed ? kRangePoints : kRangePoints64;
-    const int cand_c[3] = {cmax / 4, cmax / 2, cmax}, cand_p[3] = {pmax / 4, pmax / 2, pmax};
+    std::vector<std::pair<int, int>> candidates;
+    if (h->precision == 1)
+        for (int cc : {kRangeCells / 4, kRangeCells / 2, kRangeCells})
+            for (int pp : {kRangePoints / 4, kRangePoints / 2, kRangePoints}) candidates.push_back({cc, pp});
+    else
+        for (int pp : {kSegPoints / 4, kSegPoints / 2, kSegPoints, 2 * kSegPoints, 4 * kSegPoints}) candidates.push_back({1, pp});
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
+    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
+        if (e0) cudaEventDestroy(e0);
         return nfail(WAVE1D_ECUDA, "cudaEventCreate");
-    float best = 0.f;
-    NuRange* best_r = h->ranges;
-    int32_t* best_runs = h->runs;
-    int64_t best_n = h->nunits;
-    int best_c = h->range_cells, best_p = h->range_points;
+    }
+    NuSplit before = h->split, best;
+    float best_ms = 0.f;
     int rc = WAVE1D_OK;
-    bool first = true;
-    for (int ci = 0; ci < 3 && rc == WAVE1D_OK; ci++)
-        for (int pi = 0; pi < 3 && rc == WAVE1D_OK; pi++) {
-            std::vector<NuRange> ranges;
-            std::vector<int32_t> runs;
-            nufft_ranges(h->i0_host, h->off_host.data(), h->B, h->P.nf, h->P.nufft_w, cand_c[ci], cand_p[pi],
-                         kEmptyCells, kUnitThreads, ranges, runs);
-            NuRange* r_dev;
-            int32_t* runs_dev;
-            if ((rc = nu_upload(h, ranges, &r_dev)) || (rc = nu_upload(h, runs, &runs_dev))) break;
-            h->ranges = r_dev;
-            h->runs = runs_dev;
-            h->nunits = (int64_t)ranges.size();
-            if ((rc = wave1d_nufft_spread(h, c, grid))) break;
-            cudaEventRecord(e0, h->stream);
-            for (int r = 0; r < reps && rc == WAVE1D_OK; r++) rc = wave1d_nufft_spread(h, c, grid);
-            cudaEventRecord(e1, h->stream);
-            if (rc || cudaEventSynchronize(e1) != cudaSuccess) {
-                if (!rc) rc = nfail(WAVE1D_ECUDA, "timing the spreading failed");
-                break;
-            }
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (first || ms < best) {
-                first = false;
-                best = ms;
-                best_r = r_dev;
-                best_runs = runs_dev;
-                best_n = h->nunits;
-                best_c = cand_c[ci];
-                best_p = cand_p[pi];
-            }
+    for (const auto& cand : candidates) {
+        NuSplit s;
+        rc = h->precision == 1 ? nu_cut_ranges(h, cand.first, cand.second, s) : nu_cut_segments(h, cand.second, s);
+        h->split = s;
+        if (!rc) rc = wave1d_nufft_spread(h, c, grid);
+        cudaEventRecord(e0, h->stream);
+        for (int r = 0; r < reps && rc == WAVE1D_OK; r++) rc = wave1d_nufft_spread(h, c, grid);
+        cudaEventRecord(e1, h->stream);
+        if (cudaEventSynchronize(e1) != cudaSuccess && !rc) rc = nfail(WAVE1D_ECUDA, "timing the spreading failed");
+        float ms = 0.f;
+        if (!rc) cudaEventElapsedTime(&ms, e0, e1);
+        if (!rc && (best.points == 0 || ms < best_ms)) {
+            nu_drop(h, best);
+            best = s;
+            best_ms = ms;
+        } else {
+            nu_drop(h, s);
         }
-    h->ranges = best_r;
-    h->runs = best_runs;
-    h->nunits = best_n;
-    h->range_cells = best_c;
-    h->range_points = best_p;
+        if (rc) break;
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (rc) return rc;
-    if (cells) *cells = best_c;
-    if (points) *points = best_p;
+    h->split = before;
+    if (rc) {
+        nu_drop(h, best);
+        return rc;
+    }
+    if (h->precision == 0) {                         // a batch's ranges stay
+        std::swap(best.ranges, before.ranges);
+        std::swap(best.runs, before.runs);
+        best.nunits = before.nunits;
+    }
+    nu_drop(h, before);
+    h->split = best;
+    if (cells) *cells = best.cells;
+    if (points) *points = best.points;
     return WAVE1D_OK;
 }
 

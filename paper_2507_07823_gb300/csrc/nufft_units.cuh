@@ -139,5 +139,7 @@ int nufft_dev64(wave1d_nufft_t h, NuDev64& out);
 // the spreading of an FP64 plan by its cell ranges (spread64_unit), whose sums a batch's one-launch step
 // repeats; wave1d_nufft_spread takes segments of points instead (defined in nufft.cu)
 int nufft_spread_ranges(wave1d_nufft_t h, const double* c, double* grid);
+// cuts and uploads those ranges (WAVE1D_EINVAL for a plan that is not FP64); nufft_dev64 and nufft_spread_ranges need them
+int nufft_build_ranges(wave1d_nufft_t h);
 
 }  // namespace wave1d

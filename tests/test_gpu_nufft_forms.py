@@ -42,3 +42,30 @@ def test_arrays_at_odd_offsets(precision, tol, instances):
         assert all(float(b[0]) == -7.0 and float(b[-1]) == -7.0 for b in bufs.values())
     finally:
         nu.close()
+
+
+@pytest.mark.parametrize("precision,tol,rel", [(0, 1e-10, 1e-12), (1, 1e-6, 1e-6)])
+def test_autotuner_cuts_what_the_spreading_runs(precision, tol, rel):
+    """Its caps are those of the spreading in use (FP64: one cell, points of a segment), the spread through them is the
+    default split's to rounding, and the tables of the candidates that lost are given back."""
+    import torch
+    rng = np.random.default_rng(3)
+    x = np.concatenate([1.234 + 1e-9 * rng.standard_normal(6000), rng.uniform(-np.pi, np.pi, 500_000)])
+    nu = wave1d.Nufft(x, 6283, tol, precision)
+    try:
+        c = torch.from_numpy(rng.standard_normal(nu.M)).cuda()
+        grids = [torch.zeros(nu.nf, dtype=torch.float64, device="cuda") for _ in range(2)]
+        nu.spread(c, grids[0])
+        caps = {nu.autotune(c, grids[1], reps=2)}
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        for _ in range(6):
+            caps.add(nu.autotune(c, grids[1], reps=2))
+            nu.spread(c, grids[1])
+            assert float((grids[1] - grids[0]).abs().max()) <= rel * float(grids[0].abs().max())
+        torch.cuda.synchronize()
+        assert abs(torch.cuda.mem_get_info()[0] - free) <= 8 << 20
+        assert all((cells == 1 and points in (16, 32, 64, 128, 256)) if precision == 0 else
+                   (cells in (60, 120, 240) and points in (512, 1024, 2048)) for cells, points in caps), caps
+    finally:
+        nu.close()
