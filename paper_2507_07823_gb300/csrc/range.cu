@@ -279,15 +279,6 @@ __device__ __forceinline__ int rs_warp_first(int n, F&& pred) {
     return hi;
 }
 
-// an interval on the block grid, from its midpoint as a float pair: (mid_h, mid_l, ih, next breakpoint)
-__device__ __forceinline__ float4 rs_interval(const RangeDev& R, int iv, float g, float ig) {
-    const double mid = __ldg(R.mid + iv);              // exactly a float pair
-    const float mh = __double2float_rn(mid), ml = __double2float_rn(mid - (double)mh);
-    const float h = __fmul_rn(rintf(__fmul_rn(mh, ig)), g);
-    return make_float4(h, __fadd_rn(__fsub_rn(mh, h), ml), __ldg(R.ih + iv),
-                       iv + 1 < R.nint ? __ldg(R.bp2 + 2 * (iv + 1)) : __uint_as_float(0x7f800000u));
-}
-
 // One side of one block's pairs of the intervals [p0, p1): v.stage(k, e) is called for each of the
 // block's sources as their positions are staged (k: place in the chunk), v.pair(u, k, e, iv, zh, zl)
 // for each pair of this thread's target in the order of its sources (u: the source's parity).
@@ -303,7 +294,11 @@ __device__ __forceinline__ void rs_pair_block(const DevPlan& P, const RangeDev& 
     const float gf = (float)G.g, igf = (float)G.ig;
     // the part's intervals and those a pair of it may be looked up as first
     const int v0 = max(0, p0 - R.fine_span - 2), v1 = min(R.nint, p1 + 2);
-    for (int iv = v0 + t; iv < v1; iv += blockDim.x) sIv[iv - v0] = rs_interval(R, iv, gf, igf);
+    for (int iv = v0 + t; iv < v1; iv += blockDim.x) {
+        const rs::F4 q = rs::interval_entry(__ldg(R.mid + iv), __ldg(R.ih + iv),
+                                            iv + 1 < R.nint ? __ldg(R.bp2 + 2 * (iv + 1)) : __uint_as_float(0x7f800000u), gf, igf);
+        sIv[iv - v0] = make_float4(q.x, q.y, q.z, q.w);
+    }
     const bool valid = t < nT;
     const int64_t j = j0 + (valid ? t : nT - 1);
     const double xj = P.x[j];
@@ -330,7 +325,7 @@ __device__ __forceinline__ void rs_pair_block(const DevPlan& P, const RangeDev& 
     // the window of its 256-target block
     const int* win = R.blk_win + 4 * (j0 / kRsTargets);
     const int top = S > 0 ? __ldg(win) : (int)(j0 + nT - 1), all = max(0, S > 0 ? __ldg(win + 3) - top : top - __ldg(win) + 1);
-    const double marg = 2e-6 * R.delta + 8.0 * G.g, d0 = __ldg(R.bp + p0) - marg, d1 = __ldg(R.bp + p1) + marg;
+    const double marg = rs::part_margin(R.delta, G.g), d0 = __ldg(R.bp + p0) - marg, d1 = __ldg(R.bp + p1) + marg;
     if (warp < 2) {
         const int c = rs_warp_first(all, [&](int k) {
             const double x = rs_xext(P, top + S * k);
@@ -365,49 +360,12 @@ __device__ __forceinline__ void rs_pair_block(const DevPlan& P, const RangeDev& 
             for (int u = 0; u < 2; u++) {
                 const int k = k0 + u, e = e0 + S * k;
                 const float2 ps = sPos[min(k, lim - 1)];
-                // distance = dh + dl (dh exact on the block grid)
-                const float dh = S < 0 ? __fsub_rn(bh, ps.x) : __fadd_rn(bh, ps.x);
-                const float dl = S < 0 ? __fsub_rn(bl, ps.y) : __fadd_rn(bl, ps.y);
-                const float d = __fadd_rn(dh, dl);
-                const int c = min(kRsFineCells - 1, max(0, (int)__fmul_rn(d, R.fine_scale)));
-                int i = (int)__ldg(R.fine + c) - v0;
-                bool ok = valid && k < khi && (S > 0 ? e >= lb : e < lb) && i >= 0 && i < ns;
-                float4 q = sIv[ok ? i : 0];
-                while (ok && d >= q.w) {
-                    if (++i < ns) q = sIv[i];
-                    else ok = false;
-                }
-                auto place = [&]() {
-                    const float A = __fsub_rn(dh, q.x), B = __fsub_rn(dl, q.y);
-                    const float p = __fmul_rn(A, q.z);
-                    rs::two_sum(p, __fmaf_rn(B, q.z, __fmaf_rn(A, q.z, -p)), zh[u], zl[u]);
-                };
-                place();
-                // within FP32 rounding of a breakpoint, or past the last one: one way only, so it ends
-                for (int dir = 0; ok && fabsf(zh[u]) > rs::kZTol;) {
-                    const int want = zh[u] > 0.f ? 1 : -1;
-                    if (dir != 0 && want != dir) break;
-                    dir = want;
-                    i += want;
-                    ok = i >= 0 && i < ns;
-                    if (ok) {
-                        q = sIv[i];
-                        place();
-                    }
-                }
-                if (at_dt) {
-                    const bool near = (unsigned)(e - nbl) < (unsigned)nbc;
-                    if (ok && near != (i < ivd)) {
-                        i = near ? ivd - 1 : ivd;
-                        ok = i >= 0 && i < ns;
-                        if (ok) {
-                            q = sIv[i];
-                            place();
-                        }
-                    }
-                }
+                const int i = rs::place_pair<S>([&](int k2) { return rs::load4((const float*)(sIv + k2)); },
+                                                [&](int c) { return (int)__ldg(R.fine + c); }, R.fine_scale, v0, ns, at_dt, ivd,
+                                                (unsigned)(e - nbl) < (unsigned)nbc, valid && k < khi && (S > 0 ? e >= lb : e < lb), bh,
+                                                bl, ps.x, ps.y, zh[u], zl[u]);
                 iv[u] = i + v0;
-                in[u] = ok && iv[u] >= p0 && iv[u] < p1;
+                in[u] = i >= 0 && iv[u] >= p0 && iv[u] < p1;
             }
             v.pairs(in, k0, e0 + S * k0, S, iv, zh, zl);
         }

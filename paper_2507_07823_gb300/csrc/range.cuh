@@ -273,6 +273,14 @@ WAVE1D_RS_HD void interval_on_grid(double mid, float ih, Grid G, float* out4) {
     out4[3] = 0.f;
 }
 
+// The same for the pair kernel, in FP32 from the midpoint as a float pair (mid is exactly one): (mid_h, mid_l, ih,
+// next breakpoint).
+WAVE1D_RS_HD F4 interval_entry(double mid, float ih, float next, float g, float ig) {
+    const float mh = (float)mid, ml = (float)(mid - (double)mh);
+    const float h = mul(rintf(mul(mh, ig)), g);
+    return {h, add(sub(mh, h), ml), ih, next};
+}
+
 // |z| above which a distance lies outside the tracked interval (z carries about 3e-11; the slack
 // lets the walk end where rounding puts a distance on a breakpoint)
 constexpr float kZTol = 1.000001f;
@@ -375,6 +383,60 @@ WAVE1D_RS_HD void near_side(const float* ivt, int iv_dt, bool near, float bh, fl
         z_of<S>(t, h, l, zh, zl);
     }
 }
+
+// The pair kernel's way to a pair's interval (rs_pair_block, range.cu), which depends on the pair alone: from the
+// fine cell of the FP32 distance on to the breakpoint above it, then by z within rounding of a breakpoint (one way
+// only, so it ends), and at dt by the spring's FP64 window of near sources.  (bh, bl): the target, negated for
+// right sources; (h, l): the source; entry(i), i in [0, ns): interval_entry of interval v0 + i; fine(c): first
+// interval of fine cell c; ivd: the interval at dt less v0; ok: the pair takes part.  Returns the interval less v0
+// with its z, or -1 where it is none of the ns.
+template <int S, typename Entry, typename Fine>
+WAVE1D_RS_HD int place_pair(const Entry& entry, const Fine& fine, float fine_scale, int v0, int ns, bool at_dt, int ivd, bool near,
+                            bool ok, float bh, float bl, float h, float l, float& zh, float& zl) {
+    // distance = dh + dl (dh exact on the block grid)
+    const float dh = S < 0 ? sub(bh, h) : add(bh, h);
+    const float dl = S < 0 ? sub(bl, l) : add(bl, l);
+    const float d = add(dh, dl);
+    int c = (int)mul(d, fine_scale);
+    c = c < 0 ? 0 : (c >= kRsFineCells ? kRsFineCells - 1 : c);
+    int i = fine(c) - v0;
+    ok = ok && i >= 0 && i < ns;
+    F4 q = entry(ok ? i : 0);
+    while (ok && d >= q.w) {
+        if (++i < ns) q = entry(i);
+        else ok = false;
+    }
+    auto place = [&]() {
+        const float A = sub(dh, q.x), B = sub(dl, q.y);
+        const float p = mul(A, q.z);
+        two_sum(p, fma_(B, q.z, fma_(A, q.z, -p)), zh, zl);
+    };
+    place();
+    for (int dir = 0; ok && fabsf(zh) > kZTol;) {
+        const int want = zh > 0.f ? 1 : -1;
+        if (dir != 0 && want != dir) break;
+        dir = want;
+        i += want;
+        ok = i >= 0 && i < ns;
+        if (ok) {
+            q = entry(i);
+            place();
+        }
+    }
+    if (at_dt && ok && near != (i < ivd)) {
+        i = near ? ivd - 1 : ivd;
+        ok = i >= 0 && i < ns;
+        if (ok) {
+            q = entry(i);
+            place();
+        }
+    }
+    return ok ? i : -1;
+}
+
+// How far beyond a part's ends (of the distance) a block looks for its sources: the FP32 rounding of positions on
+// the block grid
+WAVE1D_RS_HD double part_margin(double delta, double g) { return 2e-6 * delta + 8.0 * g; }
 
 }  // namespace rs
 }  // namespace wave1d
