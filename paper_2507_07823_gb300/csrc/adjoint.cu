@@ -21,19 +21,13 @@ namespace wave1d {
 // receivers' transposed readout over the receiver weights regrouped by source (m >= 0: the m = 0 terms
 // of sources closer than dt included): one thread per source and eighth of the m (blockIdx.y: m = y,
 // y + 8, ..), so each ring entry has one writer, which meets the receivers in order
-constexpr int kAdjParts = 8;
 __global__ void k_adj_receivers(int64_t M, int ring, int64_t n, const int64_t* __restrict__ ptr,
                                 const int32_t* __restrict__ rcv, const int32_t* __restrict__ mrange,
                                 const int64_t* __restrict__ woff, const double* __restrict__ w,
                                 const double* __restrict__ ubar, double* sb) {
     for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < M; l += (int64_t)gridDim.x * blockDim.x)
-        for (int64_t e = ptr[l]; e < ptr[l + 1]; e++) {
-            const double coef = 0.5 * ubar[rcv[e]];
-            if (coef == 0.0) continue;
-            const int mlo = mrange[e] & 0xffff, cnt = mrange[e] >> 16;
-            for (int c = ((int)blockIdx.y - mlo) & (kAdjParts - 1); c < cnt; c += kAdjParts)
-                sb[(int64_t)adj::slot(n + 1 - mlo - c, ring) * M + l] += w[woff[e] + c] * coef;
-        }
+        adj::receivers_T_part(l, (int)blockIdx.y, ptr, rcv, mrange, woff, w, ubar, n + 1, ring,
+                              [&](int s, double v) { sb[(int64_t)s * M + l] += v; });
 }
 
 // transposed block solve, one thread per member position e of blk_members (blk_of[e] = its
@@ -184,17 +178,8 @@ __global__ void __launch_bounds__(256) k_adj_rbc_grid(int K, int npts, const int
                                                       const double* __restrict__ apb, double* __restrict__ uvbar) {
     __shared__ double red[2][8];
     const int pt = blockIdx.x;
-    const int64_t twoK = 2 * (int64_t)K, ig = idx[pt], inc = ((int64_t)blockDim.x * ig) % twoK;
     double su = 0.0, sv = 0.0;
-    int64_t a = ((int64_t)(1 + threadIdx.x) * ig) % twoK;
-    for (int k = 1 + threadIdx.x; k < K; k += blockDim.x) {
-        const double2 e = __ldg((const double2*)tw2K + a);               // e^{+i k x}
-        const double2 u = ((const double2*)ab)[k], v = ((const double2*)apb)[k];
-        su += u.x * e.x + u.y * e.y;
-        sv += v.x * e.x + v.y * e.y;
-        a += inc;
-        if (a >= twoK) a -= twoK;
-    }
+    adj::rbc_grid_sum(idx[pt], K, 1 + threadIdx.x, blockDim.x, tw2K, ab, apb, su, sv);
     for (int o = 16; o > 0; o >>= 1) {
         su += __shfl_xor_sync(0xffffffffu, su, o);
         sv += __shfl_xor_sync(0xffffffffu, sv, o);
@@ -211,9 +196,7 @@ __global__ void __launch_bounds__(256) k_adj_rbc_grid(int K, int npts, const int
             su += red[0][w];
             sv += red[1][w];
         }
-        const double Du = su / (double)twoK, Dv = sv / (double)twoK;
-        uvbar[2 * pt] = fma(phi[pt] - 1.0, Du, dphi[pt] * Dv);
-        uvbar[2 * pt + 1] = (phi[pt] - 1.0) * Dv;
+        adj::rbc_grid_values(K, su, sv, phi[pt], dphi[pt], uvbar + 2 * pt);
     }
 }
 
@@ -222,72 +205,24 @@ __global__ void __launch_bounds__(256) k_adj_rbc_update(int K, int npts, const i
                                                         const double* __restrict__ tw2K,
                                                         const double* __restrict__ uvbar, double* ab, double* apb) {
     const int k = blockIdx.x * 32 + (threadIdx.x >> 3), q = threadIdx.x & 7;
-    const int64_t twoK = 2 * (int64_t)K;
-    double ur = 0.0, ui = 0.0, vr = 0.0, vi = 0.0;
-    if (k < K) {
-        for (int pt = q; pt < npts; pt += 8) {
-            const double2 e = __ldg((const double2*)tw2K + ((int64_t)k * idx[pt]) % twoK), w = __ldg((const double2*)uvbar + pt);
-            ur = fma(w.x, e.x, ur);
-            ui = fma(w.x, e.y, ui);
-            vr = fma(w.y, e.x, vr);
-            vi = fma(w.y, e.y, vi);
-        }
-    }
+    adj::Complex u = {0.0, 0.0}, v = {0.0, 0.0};
+    if (k < K) adj::rbc_update_sum(k, K, q, 8, npts, idx, tw2K, uvbar, u, v);
     for (int o = 4; o > 0; o >>= 1) {
-        ur += __shfl_xor_sync(0xffffffffu, ur, o);
-        ui += __shfl_xor_sync(0xffffffffu, ui, o);
-        vr += __shfl_xor_sync(0xffffffffu, vr, o);
-        vi += __shfl_xor_sync(0xffffffffu, vi, o);
+        u.x += __shfl_xor_sync(0xffffffffu, u.x, o);
+        u.y += __shfl_xor_sync(0xffffffffu, u.y, o);
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
     }
-    if (q != 0 || k > K) return;
-    if (k == K) {
-        ab[2 * k] = ab[2 * k + 1] = 0.0;
-        apb[2 * k] = apb[2 * k + 1] = 0.0;
-    } else if (k == 0) {                 // Re alpha_0 only
-        ab[0] += ur;
-        apb[0] += vr;
-    } else {
-        ab[2 * k] = fma(2.0, ur, ab[2 * k]);
-        ab[2 * k + 1] = fma(2.0, ui, ab[2 * k + 1]);
-        apb[2 * k] = fma(2.0, vr, apb[2 * k]);
-        apb[2 * k + 1] = fma(2.0, vi, apb[2 * k + 1]);
-    }
+    if (q == 0 && k <= K) adj::rbc_update_values(k, K, u, v, ab, apb);
 }
 
-// rotation and FIR transposed (adj::modes_T), one thread per mode and kAdjTaps of the W taps
-// (blockIdx.y): every part reads the old (ab, apb) and updates its own ring slots, part 0 also writes
-// the rotated modes to (ab_out, apb_out) and takes Sbar^n out of its slot.  One thread per mode took 33
-// us for 36 taps, a chain of ring reads and writes.
-constexpr int kAdjTaps = 4;
+// rotation and FIR transposed, one thread per mode and kModeTaps of the W taps (blockIdx.y; adj::modes_T_taps).
+// One thread per mode took 33 us for 36 taps, a chain of ring reads and writes.
 __global__ void k_adj_modes(int K, int W, int64_t n, const double* __restrict__ rot, const double* __restrict__ pq,
                             const double* __restrict__ ab, const double* __restrict__ apb, double* __restrict__ ab_out,
                             double* __restrict__ apb_out, double* Sb, double* __restrict__ a2) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x, K1 = K + 1, ma = blockIdx.y * kAdjTaps;
-    if (k > K) return;
-    const double2 h = ((const double2*)ab)[k], g = ((const double2*)apb)[k];
-    double2 w[kAdjTaps], s[kAdjTaps];
-    double2* at[kAdjTaps];
-#pragma unroll
-    for (int u = 0; u < kAdjTaps; u++) {
-        const int m = min(ma + u, W - 1);
-        at[u] = (double2*)Sb + (int64_t)adj::slot(n - m, W) * K1 + k;
-        w[u] = __ldg((const double2*)pq + (int64_t)m * K1 + k);
-        s[u] = *at[u];
-    }
-#pragma unroll
-    for (int u = 0; u < kAdjTaps; u++) {
-        s[u].x = fma(w[u].x, h.x, fma(w[u].y, g.x, s[u].x));
-        s[u].y = fma(w[u].x, h.y, fma(w[u].y, g.y, s[u].y));
-        if (ma + u > 0 && ma + u < W) *at[u] = s[u];
-    }
-    if (ma > 0) return;
-    const double cs = rot[3 * k], so = rot[3 * k + 1], ks = rot[3 * k + 2];
-    ((double2*)ab_out)[k] = make_double2(fma(cs, h.x, -ks * g.x), fma(cs, h.y, -ks * g.y));
-    ((double2*)apb_out)[k] = make_double2(fma(so, h.x, cs * g.x), fma(so, h.y, cs * g.y));
-    const double scale = (k == 0 ? 1.0 : 0.5) / 6.283185307179586476925286766559;
-    a2[2 * k] = s[0].x * scale;
-    a2[2 * k + 1] = k == 0 ? 0.0 : s[0].y * scale;
-    *at[0] = make_double2(0.0, 0.0);
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k <= K) adj::modes_T_taps(k, K + 1, W, n, blockIdx.y * adj::kModeTaps, rot, pq, ab, apb, ab_out, apb_out, Sb, a2);
 }
 
 // Checkpoint restore (wave1d_adjoint_checkpointed): the float-pair copy of the density ring

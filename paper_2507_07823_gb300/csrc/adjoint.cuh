@@ -1,6 +1,8 @@
-// Bodies of the reverse-time (adjoint) step of the discrete scheme, one output element each,
-// written for both the GPU kernels (adjoint.cu) and a host check that runs them over the same
-// tables.  Complex values are interleaved (re, im) doubles.
+// Bodies of the reverse-time (adjoint) step of the discrete scheme, written for both the GPU kernels
+// (adjoint.cu) and host checks that run them over the same tables: the plain form of a piece, one output
+// element each, and where the kernels split the work of an element over threads, the parts they run
+// (.._part, .._taps, .._sum), which a host check adds up against the plain form.  Complex values are
+// interleaved (re, im) doubles.
 //
 // The forward step n -> n+1 is linear in the state (sigma ring, S ring, alpha, alpha') and the
 // forcing, so the gradient of a loss of the receiver fields follows from the transposed pieces
@@ -113,6 +115,21 @@ WAVE1D_HD void receivers_T_source(int64_t l, const int64_t* ptr, const int32_t* 
     }
 }
 
+// One of kReceiverParts parts of that work, the m = part, part + kReceiverParts, ..: every ring entry belongs to one
+// part, which meets the receivers in order.
+constexpr int kReceiverParts = 8;
+template <class Add>
+WAVE1D_HD void receivers_T_part(int64_t l, int part, const int64_t* ptr, const int32_t* rcv, const int32_t* mrange,
+                                const int64_t* woff, const double* w, const double* ubar, int64_t q, int ring, Add add) {
+    for (int64_t e = ptr[l]; e < ptr[l + 1]; e++) {
+        const double coef = 0.5 * ubar[rcv[e]];
+        if (coef == 0.0) continue;
+        const int mlo = mrange[e] & 0xffff, cnt = mrange[e] >> 16;
+        for (int c = (part - mlo) & (kReceiverParts - 1); c < cnt; c += kReceiverParts)
+            add(slot(q - mlo - c, ring), w[woff[e] + c] * coef);
+    }
+}
+
 // Transposed block solve for member l of a block of s members (members m0 .. m0 + s - 1 of
 // blk_members, inverse stored column-major: invT[l s + i] = inverse[i][l]):
 //   rhsbar[member l] = sum_i inverse[i][l] sigbar[member i]
@@ -127,6 +144,28 @@ WAVE1D_HD double solve_T(const double* invT, const int32_t* members, int64_t m0,
     }
     if (i < s) a0 = fma(col[i], sigbar[members[m0 + i]], a0);
     return a0 + a1;
+}
+
+// complex value i of an array of the library's own (16-byte aligned), one load on the GPU
+struct Complex {
+    double x, y;
+};
+WAVE1D_HD Complex complex_at(const double* v, int64_t i) {
+#ifdef __CUDA_ARCH__
+    const double2 e = *((const double2*)v + i);
+    return {e.x, e.y};
+#else
+    return {v[2 * i], v[2 * i + 1]};
+#endif
+}
+
+WAVE1D_HD void set_complex(double* v, int64_t i, double x, double y) {
+#ifdef __CUDA_ARCH__
+    *((double2*)v + i) = make_double2(x, y);
+#else
+    v[2 * i] = x;
+    v[2 * i + 1] = y;
+#endif
 }
 
 // alphabar_k += w_k (2 pi S1_k + sum_r ubar_r e^{i k x_r}): the adjoints of the springs' u_H
@@ -167,36 +206,60 @@ WAVE1D_HD void rbc_grid_T(int ig, int K, const double* tw2K, const double* ab, c
     *vbar = (phi - 1.0) * Dv;
 }
 
+// the terms k = first, first + step, .. (1 <= k < K) of the two sums of rbc_grid_T, added to (su, sv); e^{i k x}
+// by stepping its index
+WAVE1D_HD void rbc_grid_sum(int ig, int K, int first, int step, const double* tw2K, const double* ab, const double* apb,
+                            double& su, double& sv) {
+    const int64_t twoK = 2 * (int64_t)K, inc = ((int64_t)step * ig) % twoK;
+    int64_t a = ((int64_t)first * ig) % twoK;
+    for (int k = first; k < K; k += step) {
+        const Complex e = complex_at(tw2K, a), u = complex_at(ab, k), v = complex_at(apb, k);
+        su += u.x * e.x + u.y * e.y;
+        sv += v.x * e.x + v.y * e.y;
+        a += inc;
+        if (a >= twoK) a -= twoK;
+    }
+}
+// the point's adjoints from the two whole sums
+WAVE1D_HD void rbc_grid_values(int K, double su, double sv, double phi, double dphi, double* uvbar) {
+    const double Du = su / (double)(2 * (int64_t)K), Dv = sv / (double)(2 * (int64_t)K);
+    uvbar[0] = fma(phi - 1.0, Du, dphi * Dv);
+    uvbar[1] = (phi - 1.0) * Dv;
+}
+
 // Transposed projection, mode part: the identity on k < K plus the grid values' dependence on
 // alpha (u = Re alpha_0 + 2 sum_{k=1}^{K-1} Re(alpha_k e^{-i k x})); alpha_K does not reach the
 // projected field, whose alpha_K is zero, so its adjoint is zero.
-WAVE1D_HD void rbc_update_T(int k, int K, int npts, const int32_t* idx, const double* tw2K,
-                            const double* uvbar, double* ab, double* apb) {
+// rbc_update_sum: the points first, first + step, .., added to (u, v); rbc_update_values: mode k from the whole sums.
+WAVE1D_HD void rbc_update_sum(int k, int K, int first, int step, int npts, const int32_t* idx, const double* tw2K,
+                              const double* uvbar, Complex& u, Complex& v) {
+    for (int pt = first; pt < npts; pt += step) {
+        const Complex e = complex_at(tw2K, ((int64_t)k * idx[pt]) % (2 * (int64_t)K)), w = complex_at(uvbar, pt);
+        u.x = fma(w.x, e.x, u.x);
+        u.y = fma(w.x, e.y, u.y);
+        v.x = fma(w.y, e.x, v.x);
+        v.y = fma(w.y, e.y, v.y);
+    }
+}
+WAVE1D_HD void rbc_update_values(int k, int K, const Complex& u, const Complex& v, double* ab, double* apb) {
     if (k == K) {
         ab[2 * k] = ab[2 * k + 1] = 0.0;
         apb[2 * k] = apb[2 * k + 1] = 0.0;
-        return;
-    }
-    const int64_t twoK = 2 * (int64_t)K;
-    double ur = 0.0, ui = 0.0, vr = 0.0, vi = 0.0;
-    for (int pt = 0; pt < npts; pt++) {
-        const int64_t a = ((int64_t)k * idx[pt]) % twoK;
-        const double c = tw2K[2 * a], s = tw2K[2 * a + 1];
-        const double u = uvbar[2 * pt], v = uvbar[2 * pt + 1];
-        ur = fma(u, c, ur);
-        ui = fma(u, s, ui);
-        vr = fma(v, c, vr);
-        vi = fma(v, s, vi);
-    }
-    if (k == 0) {                        // Re alpha_0 only
-        ab[0] += ur;
-        apb[0] += vr;
+    } else if (k == 0) {                 // Re alpha_0 only
+        ab[0] += u.x;
+        apb[0] += v.x;
     } else {
-        ab[2 * k] = fma(2.0, ur, ab[2 * k]);
-        ab[2 * k + 1] = fma(2.0, ui, ab[2 * k + 1]);
-        apb[2 * k] = fma(2.0, vr, apb[2 * k]);
-        apb[2 * k + 1] = fma(2.0, vi, apb[2 * k + 1]);
+        ab[2 * k] = fma(2.0, u.x, ab[2 * k]);
+        ab[2 * k + 1] = fma(2.0, u.y, ab[2 * k + 1]);
+        apb[2 * k] = fma(2.0, v.x, apb[2 * k]);
+        apb[2 * k + 1] = fma(2.0, v.y, apb[2 * k + 1]);
     }
+}
+WAVE1D_HD void rbc_update_T(int k, int K, int npts, const int32_t* idx, const double* tw2K,
+                            const double* uvbar, double* ab, double* apb) {
+    Complex u = {0.0, 0.0}, v = {0.0, 0.0};
+    if (k < K) rbc_update_sum(k, K, 0, 1, npts, idx, tw2K, uvbar, u, v);
+    rbc_update_values(k, K, u, v, ab, apb);
 }
 
 // Transposed mode update of step n for mode k (K1 = K + 1 modes):
@@ -225,6 +288,36 @@ WAVE1D_HD void modes_T(int k, int K1, int W, int64_t n, const double* rot, const
     a2[2 * k] = s[0] * scale;
     a2[2 * k + 1] = k == 0 ? 0.0 : s[1] * scale;
     s[0] = s[1] = 0.0;
+}
+
+// The taps m = ma .. ma + kModeTaps - 1 of that update, for threads side by side: every part reads the old (ab, apb)
+// and updates its own ring slots; part 0 also writes the rotated modes to (ab_out, apb_out), which must not
+// be (ab, apb), and takes Sbar^n out of its slot.
+constexpr int kModeTaps = 4;
+WAVE1D_HD void modes_T_taps(int k, int K1, int W, int64_t n, int ma, const double* rot, const double* pq, const double* ab,
+                            const double* apb, double* ab_out, double* apb_out, double* Sb, double* a2) {
+    const Complex h = complex_at(ab, k), g = complex_at(apb, k);
+    Complex w[kModeTaps], s[kModeTaps];
+    double* at[kModeTaps];
+    for (int u = 0; u < kModeTaps; u++) {
+        const int m = ma + u < W ? ma + u : W - 1;
+        at[u] = Sb + 2 * ((int64_t)slot(n - m, W) * K1 + k);
+        w[u] = complex_at(pq, (int64_t)m * K1 + k);
+        s[u] = complex_at(at[u], 0);
+    }
+    for (int u = 0; u < kModeTaps; u++) {
+        s[u].x = fma(w[u].x, h.x, fma(w[u].y, g.x, s[u].x));
+        s[u].y = fma(w[u].x, h.y, fma(w[u].y, g.y, s[u].y));
+        if (ma + u > 0 && ma + u < W) set_complex(at[u], 0, s[u].x, s[u].y);
+    }
+    if (ma > 0) return;
+    const double cs = rot[3 * k], so = rot[3 * k + 1], ks = rot[3 * k + 2];
+    set_complex(ab_out, k, fma(cs, h.x, -ks * g.x), fma(cs, h.y, -ks * g.y));
+    set_complex(apb_out, k, fma(so, h.x, cs * g.x), fma(so, h.y, cs * g.y));
+    const double scale = (k == 0 ? 1.0 : 0.5) / 6.283185307179586476925286766559;
+    a2[2 * k] = s[0].x * scale;
+    a2[2 * k + 1] = k == 0 ? 0.0 : s[0].y * scale;
+    set_complex(at[0], 0, 0.0, 0.0);
 }
 
 }  // namespace adj

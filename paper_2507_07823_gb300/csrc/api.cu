@@ -14,6 +14,7 @@
 #include <string>
 #include <vector>
 
+#include "adjoint.cuh"
 #include "adjoint_host.h"
 #include "internal.h"
 #include "plan_hooks.h"
@@ -1552,7 +1553,7 @@ struct Reverse {
                 }
                 k_rs_unfold_add<<<dim3(gM, (unsigned)P.m_max), 256, 0, sl>>>(d, rd, runs, n, usum, sb);
             } else {
-                if (have_rcv) k_adj_receivers<<<dim3(gM, 8), 256, 0, s>>>(M, ring, n, rptr, rrcv, rmr, rwoff, rw, ub, sb);
+                if (have_rcv) k_adj_receivers<<<dim3(gM, adj::kReceiverParts), 256, 0, s>>>(M, ring, n, rptr, rrcv, rmr, rwoff, rw, ub, sb);
                 k_adj_solve<<<gM, 256, 0, s>>>(d, dblk, sb + (int64_t)((n + 1) % ring) * M, sig_rows + (n - row0) * M, g ? g + n * M : nullptr,
                                                want_beta ? gsum : nullptr, grad_g ? grad_g + n * M : nullptr, cbar, uHbar);
                 if (n == 0) break;
@@ -1568,7 +1569,7 @@ struct Reverse {
                 k_adj_rbc_grid<<<npts, 256, 0, s>>>(K, npts, d.rbc_idx, d.tw2K, d.rbc_phi, d.rbc_dphi, ab, apb, uvbar);
                 k_adj_rbc_update<<<blocks_for(K1, 32, INT32_MAX), 256, 0, s>>>(K, npts, d.rbc_idx, d.tw2K, uvbar, ab, apb);
             }
-            k_adj_modes<<<dim3(blocks_for(K1, 128, INT32_MAX), (unsigned)(P.W + 3) / 4), 128, 0, s>>>(K, P.W, n, d.rot, d.pq, ab, apb,
+            k_adj_modes<<<dim3(blocks_for(K1, 128, INT32_MAX), (unsigned)(P.W + adj::kModeTaps - 1) / adj::kModeTaps), 128, 0, s>>>(K, P.W, n, d.rot, d.pq, ab, apb,
                                                                                                 ab2, apb2, Sb, a2);
             std::swap(ab, ab2);
             std::swap(apb, apb2);
