@@ -1309,8 +1309,7 @@ void build_range_tables(const Params& P, RangeTables& rt) {
     {
         // intervals wider than kRangeMaxWidth dt are cut into equal parts: the curvature
         // coefficients (single floats on the device) shrink with the width as width^r
-        const char* env = std::getenv("WAVE1D_RANGE_WIDTH");
-        const double cap = (env ? std::atof(env) : kRangeMaxWidth) * P.dt;
+        const double cap = kRangeMaxWidth * P.dt;
         std::vector<double> cut = {rt.bp[0]};
         for (size_t i = 1; i < rt.bp.size(); i++) {
             const double a = rt.bp[i - 1], b = rt.bp[i];

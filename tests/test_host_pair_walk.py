@@ -38,3 +38,11 @@ def test_every_pair_once_and_the_stored_weights_sums(checker, name, bar, part):
     wrong, err, terr, pairs = r.stdout.split()[1:]
     assert int(wrong) == 0 and int(pairs) >= x.size
     assert float(err) < bar and float(terr) < 1e-9, (err, terr)
+
+
+def test_tables_do_not_depend_on_the_environment(checker):
+    bc, dt, tol, x = _layout("coincident", np.random.default_rng(9))
+    text = f"{x.size} {dt!r} {tol!r} {bc} 0\n" + " ".join(repr(float(v)) for v in x) + "\n"
+    out = [subprocess.run([checker], input=text, capture_output=True, text=True, env=env).stdout
+           for env in (os.environ, dict(os.environ, WAVE1D_RANGE_WIDTH="0.45"))]
+    assert out[0].startswith("ok") and out[0] == out[1]
