@@ -506,21 +506,18 @@ int window_steps(double tol, double gamma, int W) {
     return W > 0 ? W : (int)std::ceil(2.0 * std::log(1.0 / tol) / (kPi * gamma));
 }
 
-// The range tables depend on dt, delta, b, W, N_L, m_max and p only (and the interval cap), so plans
+// The range tables depend on dt, delta, b, W, N_L, m_max and p only, so plans
 // that share them (the instances of a batched plan) build them once: the last few are kept.
 static void range_tables_cached(const Params& P, RangeTables& rt) {
     struct Entry {
-        double dt, delta, b, cap;
+        double dt, delta, b;
         int W, NL, m_max, p;
         RangeTables rt;
     };
     static std::mutex mu;
     static std::vector<Entry> cache;
-    const char* env = std::getenv("WAVE1D_RANGE_WIDTH");
-    const double cap = env ? std::atof(env) : -1.0;
     auto same = [&](const Entry& e) {
-        return e.dt == P.dt && e.delta == P.delta && e.b == P.b && e.cap == cap && e.W == P.W && e.NL == P.NL &&
-               e.m_max == P.m_max && e.p == P.p;
+        return e.dt == P.dt && e.delta == P.delta && e.b == P.b && e.W == P.W && e.NL == P.NL && e.m_max == P.m_max && e.p == P.p;
     };
     {
         std::lock_guard<std::mutex> lock(mu);
@@ -533,7 +530,7 @@ static void range_tables_cached(const Params& P, RangeTables& rt) {
     build_range_tables(P, rt);
     std::lock_guard<std::mutex> lock(mu);
     if (cache.size() >= 4) cache.erase(cache.begin());
-    cache.push_back(Entry{P.dt, P.delta, P.b, cap, P.W, P.NL, P.m_max, P.p, rt});
+    cache.push_back(Entry{P.dt, P.delta, P.b, P.W, P.NL, P.m_max, P.p, rt});
 }
 
 // History tables (eqs. pkqkcomp, hkcompdisc, the mode rotation, the NUFFT deconvolution, the FFT
