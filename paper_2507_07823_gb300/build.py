@@ -48,7 +48,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         o = os.path.join(OUT, src + ".o")
         objs.append(o)
         if force or _stale(o, [s] + headers):
-            jobs.append(["g++", "-O2", "-std=c++17", "-fPIC", "-pthread", "-c", s, "-o", o])
+            jobs.append(["g++", "-O2", "-std=c++17", "-fPIC", "-pthread", "-DWAVE1D_LIBRARY", "-c", s, "-o", o])
 
     def run(cmd):
         r = subprocess.run(cmd, capture_output=True, text=True)

@@ -81,22 +81,24 @@ struct RangeTables {
     std::vector<float> coef;           // [iv][m][12]: monomial coefficients of z, a0 .. a3 as (hi, lo)
                                        //   pairs, a4 .. a7 single
     std::vector<double> cheb;          // [iv][m][8]: Chebyshev coefficients in z (FP64)
-    // the same polynomials as slices of kRsSliceBits bits for the tensor-core fold (fold_index below):
-    // a_{iv,m,r} = 2^(e - 10) sum_j s_j 2^(-11 j), s_j whole numbers of at most 1024, e per (iv, r)
+    std::vector<uint16_t> fine;        // kRsFineCells: interval of the left end of each cell of [0, delta)
+    int fine_span = 0;                 // breakpoints in one of those cells at most
+    // The same polynomials as slices of 11 bits, a_{iv,m,r} = 2^(e - 10) sum_j s_j 2^(-11 j), s_j whole numbers of at
+    // most 1024, e per (iv, r): operands of a fold by half-precision matrix instructions.  Empty in the library: no
+    // kernel reads them, since units common to all m lose the small coefficients (range.cu); a host check
+    // measures what they hold of full windows.
     int nk = 0, nivp = 0;              // steps of 16 m (m = 1 .. 16 nk), intervals with padding
     std::vector<uint16_t> fold;        // half-precision s_j
     std::vector<float> fold_scale;     // [nivp][8]: 2^(e - 10)
-    int fold_shift = 0;                // the density slices' units are 2^shift larger, so that
-                                       //   1024 sum_m |s_0| stays below 2^(24 + shift) (long windows)
-    std::vector<uint16_t> fine;        // kRsFineCells: interval of the left end of each cell of [0, delta)
-    int fine_span = 0;                 // breakpoints in one of those cells at most
+    int fold_shift = 0;                // density units 2^shift larger keep 1024 sum_m |s_0| below 2^24 (the sums of the
+                                       //   later slices are not bounded by it)
     int nis = 0, nmp = 0;              // steps of 16 intervals, m = 1 .. nmp (a multiple of 8)
-    std::vector<uint16_t> unfold;      // the same s_j as operands of the transposed sum (unfold_index)
+    std::vector<uint16_t> unfold;      // the same s_j, intervals innermost (unfold_index)
     std::vector<int32_t> cell;         // kRsCells: interval of the left end of each cell of [0, delta)
     float cell_scale = 0.f;            // kRsCells / delta: cell of a distance d is floor(d cell_scale)
 };
 void build_range_tables(const Params& P, RangeTables& out);
-// Slices of the fold: the densities carry 4, the coefficients of power r kRsSlicesOf[r] (first index
+// Slices of that form: the densities carry 4, the coefficients of power r kRsSlicesOf[r] (first index
 // kRsFirstSlice[r]); products of slices i and j with i + j < kRsDiagonals[r] are kept.
 constexpr int kRsPowers = 8;
 constexpr int kRsSlices = 4;

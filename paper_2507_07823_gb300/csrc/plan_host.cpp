@@ -1207,7 +1207,7 @@ static uint16_t half_bits(int v) {
     return (uint16_t)(sign | ((e + 15) << 10) | (((a << 10) >> e) & 0x3ff));
 }
 
-// the coefficient slices of the tensor-core fold from a[iv][m][r] (FP64)
+// the coefficient slices of the sliced form (RangeTables::fold) from a[iv][m][r] (FP64)
 static void fold_slices(const std::vector<double>& a, RangeTables& rt) {
     const int n = rt.nint, nm = rt.nm;
     rt.nk = (nm - 1 + 15) / 16;
@@ -1241,6 +1241,11 @@ static void fold_slices(const std::vector<double>& a, RangeTables& rt) {
             most = std::max(most, sum);
         }
     while (most > std::ldexp(1.0, 14 + rt.fold_shift)) rt.fold_shift++;
+}
+
+// the pair kernel's table of fine cells
+static void fine_cells(RangeTables& rt) {
+    const int n = rt.nint;
     rt.fine.assign(kRsFineCells, 0);
     int last = 0;
     for (int c = 0; c < kRsFineCells; c++) {
@@ -1396,7 +1401,10 @@ void build_range_tables(const Params& P, RangeTables& rt) {
         rt.mr[2 * iv] = lo1;
         rt.mr[2 * iv + 1] = hi1;
     }
-    fold_slices(mono, rt);
+    fine_cells(rt);
+#ifndef WAVE1D_LIBRARY
+    fold_slices(mono, rt);                                // for its host check only; no kernel reads slices
+#endif
 }
 
 void receiver_columns(const LocalCSR& rloc, int64_t M, ReceiverColumns& out) {

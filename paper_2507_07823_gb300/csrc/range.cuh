@@ -119,7 +119,7 @@ WAVE1D_RS_HD Pair split(double v) {
     return {h, (float)(v - (double)h)};
 }
 
-// A density hi + lo as four slices of 11 bits, whole numbers s_i of magnitude at most 1024 (2048 where
+// (Host check of the sliced form, RangeTables::fold.)  A density hi + lo as four slices of 11 bits, whole numbers s_i of magnitude at most 1024 (2048 where
 // |hi| inv reaches it) with (hi + lo) inv = sum_i s_i 2^(-11 i) up to half a unit of the last slice;
 // inv: a power of two with |hi| inv < 1024.  The residues of hi are exact; lo (at most 2^-3 of a unit
 // of the second slice) joins the residue of that slice, with 2^-25 of its unit lost.
