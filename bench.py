@@ -45,7 +45,7 @@ L2_FLUSH_BYTES = 512 << 20
 STEP_KERNEL_SOURCES = ["step.cu", "grid_sync.cuh", "phases.cuh", "device_common.cuh", "internal.h"]
 STEP_TRAFFIC = {"sources_sha256": "7eb459635b849cfa2fd0795fbb4a3f1fbf3ae75954968e7d6afb630d826588d3", "bytes_per_launch": 317395712 + 5562880}
 L2_CLEAN_BYTES = 256 << 20
-# DRAM bytes of one step's local sum (k_rs_slices, k_rs_fold and k_rs_pairs over all slabs) from one ncu
+# DRAM bytes of one step's local sum (k_rs_fold and k_rs_pairs over all slabs) from one ncu
 # capture of the clustered layout at the springs below, for the kernel sources it was taken with (null
 # once they change)
 RS_LOCAL_SOURCES = ["range.cu", "range_dev.cuh", "range.cuh", "phases.cuh", "device_common.cuh", "internal.h"]
@@ -195,7 +195,7 @@ def run_ours(args):
     launches = K * range_launches_per_step(w)
 
     # --- per-stage device times (CUDA events between the stages, K steps): the local-sum stage is
-    # the density slices and, per slab of intervals, the fold and the pair kernel ------------------
+    # per slab of intervals the fold and the pair kernel ---------------------------------------------
     wave1d.wave1d_profile(plan.h, 1)
     for i in range(K):
         wave1d._check(wave1d.wave1d_step(plan.h), "wave1d_step")
@@ -220,15 +220,14 @@ def run_ours(args):
     e2e_value = w.M * K * world / e2e_s
     plan.close()
 
-    # --- roofline of the local sum (k_rs_fold on the tensor cores, k_rs_pairs in FP32, the larger part):
-    # bound by FP32 issue, not by HBM.  Algorithmic work per step: the local sum's multiply-adds
+    # --- roofline of the local sum (k_rs_fold, and k_rs_pairs, the larger part): FP32 work, not HBM.  Algorithmic work per step: the local sum's multiply-adds
     # Q_m(d) sigma (info.local_terms, 2 flops each),
     # the work the method does whatever the arithmetic; peak: 152 SMs x 128 FP32 lanes x 2 flops x
     # the maximum SM clock.
     fp32_peak, clk_src = _fp32_peak()
     ms_local = per_step["local"]
     achieved = 2.0 * info.local_terms / (ms_local * 1e-3) / 1e12
-    roof = {"kernel": "k_rs_slices + k_rs_fold + k_rs_pairs (one step)", "bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
+    roof = {"kernel": "k_rs_fold + k_rs_pairs (one step)", "bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
             "frac": achieved / fp32_peak, "traffic": rs_local_traffic(info),
             "peak_source": f"derived: 152 SMs x 128 FP32 lanes x 2 flops x {clk_src}",
             "algorithmic_flops_per_launch": 2.0 * info.local_terms, "launch_ms": ms_local,
@@ -247,8 +246,7 @@ def run_ours(args):
                    "local_pairs": info.local_pairs, "nearby_pairs": info.nearby_pairs,
                    "plan": "local_weights = 1: no pair lists (local sum over sorted index windows with "
                            "weights from distance polynomials, implicit part by Jacobi sweeps)",
-                   "arithmetic": "local sum in compensated FP32 pairs (k_rs_pairs) on e-vectors folded exactly on the "
-                                 "tensor cores (k_rs_fold, 11-bit integer slices); history part (NUFFTs, "
+                   "arithmetic": "local sum in compensated FP32 pairs (k_rs_fold, k_rs_pairs); history part (NUFFTs, "
                                  "FFTs, mode recurrence), implicit solve and receivers in FP64",
                    "parallelism": f"replicas x{world}",
                    "l2": "not flushed: every step reads the 3.6 GB of implicit-part weights and the 0.84 GB "
@@ -295,8 +293,8 @@ def run_ours(args):
 
 
 def range_launches_per_step(w, intervals=484):
-    """Kernel launches of one step of the clustered plan without pair lists: the density slices, a fold
-    and a pair launch per slab of intervals, five history-part launches (spreading + FFT columns, FIR
+    """Kernel launches of one step of the clustered plan without pair lists: a fold and a pair launch
+    per slab of intervals, five history-part launches (spreading + FFT columns, FIR
     tail, FFT rows + mode update, inverse FFT columns, interpolation), the solve's set-up, its 40 Jacobi
     sweep launches (those after convergence return at once), the store, the receivers' local part (with
     receivers) and the finishing launch.  Slabs: 64 intervals at a time (one part) of the 484 at dt =
@@ -304,7 +302,7 @@ def range_launches_per_step(w, intervals=484):
     part = 64
     slab = max(1, int(min(16384 * w.M, 4 << 30) / (48 * w.M)) // 16 * 16 // part) * part
     slabs = -(-intervals // slab)
-    return 1 + 2 * slabs + 5 + 1 + 40 + 1 + (1 if len(w.xr) else 0) + 1
+    return 2 * slabs + 5 + 1 + 40 + 1 + (1 if len(w.xr) else 0) + 1
 
 
 def periodic_gaussians(w, tt):
@@ -948,7 +946,7 @@ def run_free_only(args):
 
 
 def run_local_only(args):
-    """The local sum of the plan without pair lists alone (k_rs_slices, k_rs_fold, k_rs_pairs) on the clustered recipe at
+    """The local sum of the plan without pair lists alone (k_rs_fold, k_rs_pairs) on the clustered recipe at
     --local-M springs in --local-clusters clusters (50,000 springs per cluster keeps the million-
     spring workload's cluster density), or with --local-uniform on a uniform instance of the
     batched workload's recipe: 2 steps, then 3 profiled steps.  The small cases the kernel's full

@@ -69,3 +69,34 @@ def test_autotuner_cuts_what_the_spreading_runs(precision, tol, rel):
                    (cells in (60, 120, 240) and points in (512, 1024, 2048)) for cells, points in caps), caps
     finally:
         nu.close()
+
+
+def test_more_instances_than_one_group_of_ffts():
+    """1100 instances at K = 6283: the FFT passes take them in two groups (1024 fine grids of 32768 to a group).  The
+    instances beside the cut and at the ends against direct sums."""
+    import torch
+    from oracle import wfp
+    rng = np.random.default_rng(21)
+    K, n = 6283, 1100
+    sets = [rng.uniform(-np.pi, np.pi, 1 + i % 4) for i in range(n)]
+    nu = wave1d.Nufft(sets, K, 1e-10, 0)
+    try:
+        assert nu.nf == 32768
+        c = rng.standard_normal(nu.M)
+        a = rng.standard_normal((n, K + 1, 2))
+        a[:, 0, 1] = 0.0
+        S = torch.zeros(n, K + 1, 2, dtype=torch.float64, device="cuda")
+        ud = torch.zeros(nu.M, dtype=torch.float64, device="cuda")
+        nu.type1(torch.from_numpy(c[nu.perm]).cuda(), S)
+        nu.type2(torch.from_numpy(a).cuda(), ud)
+        u = np.empty(nu.M)
+        u[nu.perm] = ud.cpu().numpy()
+        off = nu.offsets
+        for i in (0, 511, 1022, 1023, 1024, 1025, n - 1):
+            ref = wfp.type1(c[off[i]:off[i + 1]], sets[i], K)
+            got = S[i].cpu().numpy() @ np.array([1.0, 1j])
+            assert np.max(np.abs(got - ref)) < 1e-8 * np.max(np.abs(ref))
+            ref = wfp.type2(a[i] @ np.array([1.0, 1j]), sets[i])
+            assert np.max(np.abs(u[off[i]:off[i + 1]] - ref)) < 1e-8 * np.sum(np.abs(a[i]))
+    finally:
+        nu.close()

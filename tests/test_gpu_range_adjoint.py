@@ -71,3 +71,26 @@ def test_reverse_march_of_a_mixed_plan():
     finally:
         for plan in (f64, mixed, ck):
             plan.close()
+
+
+@pytest.mark.parametrize("lw", [0, 1])
+def test_more_receivers_than_the_table_of_waves_holds(lw):
+    """1400 receivers at 3142 modes pass the 64 MB of the receivers' waves, which are then formed at each step: the
+    gradient is the sum of those of the two halves of the receivers (bar: 1e-12, the order of the sums)."""
+    rng = np.random.default_rng(2)
+    M, n, R = 40, 20, 1400
+    xr = np.sort(rng.uniform(-1.0, 1.0, R))
+    ubar = torch.from_numpy(rng.standard_normal((n, R))).cuda()
+    w = W.Workload(name="waves", bc=W.FREE, x=np.sort(rng.uniform(-0.5, 0.5, M)), beta=rng.uniform(0.5, 2.0, M), amp=np.array([1.0]),
+                   center=np.array([-0.2]), width=np.array([0.3]), dt=1e-3, Nt=n, tol=1e-8, p=4, xr=xr, seed=2)
+    out, sigma = [], None
+    for part in (slice(0, R), slice(0, R // 2), slice(R // 2, R)):
+        plan = wave1d.Plan.from_workload(w.with_(xr=xr[part]), local_weights=lw)
+        try:
+            if sigma is None:
+                sigma, _ = plan.solve_device(n)
+            out.append(plan.adjoint(sigma, ubar[:, part].contiguous(), forcing_gradient=True))
+        finally:
+            plan.close()
+    for whole, a, b in zip(*out):
+        assert float((a + b - whole).abs().max()) <= 1e-12 * max(float(a.abs().max()), float(b.abs().max()))
