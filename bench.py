@@ -43,13 +43,13 @@ L2_FLUSH_BYTES = 512 << 20
 # (dram__bytes_read.sum + dram__bytes_write.sum), valid only for the kernel sources it was taken
 # with: reported as roofline.traffic while their SHA-256 matches, else null
 STEP_KERNEL_SOURCES = ["step.cu", "grid_sync.cuh", "phases.cuh", "device_common.cuh", "internal.h"]
-STEP_TRAFFIC = {"sources_sha256": "7eb459635b849cfa2fd0795fbb4a3f1fbf3ae75954968e7d6afb630d826588d3", "bytes_per_launch": 317395712 + 5562880}
+STEP_TRAFFIC = {"sources_sha256": "046eb023f13f88754f595fa4fd5c582aeeea77416d71564e6592587f164b2118", "bytes_per_launch": 316537088 + 5592832}
 L2_CLEAN_BYTES = 256 << 20
 # DRAM bytes of one step's local sum (k_rs_fold and k_rs_pairs over all slabs) from one ncu
 # capture of the clustered layout at the springs below, for the kernel sources it was taken with (null
 # once they change)
 RS_LOCAL_SOURCES = ["range.cu", "range_dev.cuh", "range.cuh", "phases.cuh", "device_common.cuh", "internal.h"]
-RS_LOCAL_TRAFFIC = {"sources_sha256": "f7562d31d9278ed433cd5cb38c168481561408eebb2cb7704229d2cdd66d0671", "bytes_per_step": 18108773120.0, "springs": 250000}
+RS_LOCAL_TRAFFIC = {"sources_sha256": "15c18423b01c4584a97bb822fb5a4a1973869461d43edbd6ea691cf4b3426f29", "bytes_per_step": 17933657344.0, "springs": 250000}
 
 
 def _peaks():

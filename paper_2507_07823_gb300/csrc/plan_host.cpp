@@ -1261,7 +1261,8 @@ static void fine_cells(RangeTables& rt) {
 
 // Parts hold about 160 sources to a side on average (a warp's 32 targets start and end up to 32 sources apart,
 // which it waits for), 64 to 160 intervals: a million clustered springs 80.7 ms per step with parts of 16,
-// 74.5 of 32, 72.6 of 64; 1e5 uniform springs 3.46 ms with parts of 80, 3.33 of 160.  No more than 4 GiB of
+// 74.5 of 32, 72.6 of 64; 1e5 uniform springs 3.46 ms with parts of 80, 3.33 of 160 (with a faster fold; the
+// parts are the pair kernel's).  No more than 4 GiB of
 // records to a part, 16 intervals at least.
 // Slabs: 16 KB of records a spring (some 340 intervals; 8 KB below 16384 springs, whose plans stay smaller
 // than one with stored weights) up to 4 GiB, and no more than an eighth of the memory that is free where

@@ -399,8 +399,9 @@ struct RsSum {
     }
 };
 
-// ten blocks to an SM (48 registers): the loads' latency is what a warp waits for.  A million clustered
-// springs 72.2 ms per step with six blocks (66 registers), 69.8 with eight, 66.2 with ten
+// ten blocks to an SM (48 registers, five words spilled): the loads' latency is what a warp waits for, and
+// more warps gain more than the spills cost.  A million clustered springs, the whole step: 72.2 ms with six
+// blocks (66 registers, no spills), 69.8 with eight, 66.2 with ten (measured with a fold 12 ms faster)
 constexpr int kRsPairBlocks = 10;
 __global__ void __launch_bounds__(kRsPairTargets, kRsPairBlocks) k_rs_pairs(DevPlan P, RangeDev R, int s0) {
     extern __shared__ __align__(16) float4 pair_sm[];
@@ -912,7 +913,7 @@ __global__ void __launch_bounds__(kRsPairTargets) k_rs_moments(DevPlan P, RangeD
 // (blockIdx.z) and a group of steps (blockIdx.y); it stages records and coefficients of 8 intervals at a time (two
 // buffers, asynchronous copies).  Warp w takes the group's steps w, w + nwarps, .., four at most, so that the warps'
 // work is even.  sums: [blockIdx.z][m][M], carried from slab to slab; k_rs_unfold_add puts them into the ring.
-// Bound by FP32 issue, 52 instructions per output, interval and m: 30,000 outputs and 676 intervals about 1.1 ms,
+// Bound by FP32 issue, 52 instructions per output, interval and m: 30,000 outputs and 676 intervals 1.5 ms,
 // of which the FP32 pipe needs 0.7 (one run of intervals with four warps' steps of eight: 3.3 ms, 469 blocks in two
 // uneven rounds).  11-bit slices on the tensor cores took 0.84 ms, held moments and coefficients in common
 // units and the sums as pairs, and gave NaN at p = 16.
